@@ -24,10 +24,13 @@
 // (cell-centred), full weighting / trilinear (nodal).  Coarse densities are 8-cell means.
 // The coarsest level is solved by one block with conjugate gradients.  Norms use fixed-order
 // two-stage reductions, so results are deterministic.
+#include <cooperative_groups.h>
+
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "rmt_kernels.h"
@@ -225,6 +228,8 @@ __device__ __forceinline__ AT fe_op(const Lv& L, const XT* __restrict__ x, const
   diag = AT(4) * bs * s12;
   return (AT(4) * bs * (AT)x[nix(L, i, j, k)] - s) * s12;
 }
+
+#include "rmt_mg_coarse.cuh"
 
 // ----------------------------------------------------------------------------- two-float residual
 // A two-float number is an unevaluated sum hi + lo of floats.  Every rounding step is spelled
@@ -1419,9 +1424,11 @@ __global__ void k_add_to64(const T* __restrict__ a, double* __restrict__ b, long
   GRID_LOOP(i, n) b[i] = set ? (double)a[i] : b[i] + (double)a[i];
 }
 
-// coarsest level: one block solves it by conjugate gradients (the operator is symmetric
-// positive semi-definite with the constants as null space; the right-hand side is made
-// mean-free and so is the result)
+// coarsest level: conjugate gradients (the operator is symmetric positive semi-definite with the
+// constants as null space; the right-hand side is made mean-free and so is the result).  Levels
+// that fit a cluster's registers and shared memory take k_coarse_solve (rmt_mg_coarse.cuh); the
+// one-block kernel below is for those that do not (an odd grid of more than 32^3 cells, which has
+// one level only).
 constexpr int COARSE_TPB = 512;
 // relative tolerance of the coarsest solve: FP64 solves to 1e-10; an FP32 V-cycle needs its
 // coarse correction to well below its own convergence factor (about 0.1), and FP32 CG on the
@@ -1509,65 +1516,6 @@ __device__ void cg_block(const Lv& L, int kind, int max_it, double rtol, T* x, T
   __syncthreads();
 }
 
-// The same iteration run by one warp (the calling warp; small levels, where the block's barriers
-// would dominate): reductions by shuffles only.
-template <typename T>
-__device__ void cg_warp(const Lv& L, int kind, int max_it, double rtol, T* x, T* r, T* p, T* q, const T* rho) {
-  const int lane = threadIdx.x & 31;
-  const int n = (int)L.nunk;
-  auto wsum = [](T v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  };
-  T loc = T(0);
-  for (int u = lane; u < n; u += 32) loc += r[u];
-  const T mean = wsum(loc) / T(n);
-  loc = T(0);
-  for (int u = lane; u < n; u += 32) {
-    const T v = r[u] - mean;
-    r[u] = v;
-    p[u] = v;
-    x[u] = T(0);
-    loc += v * v;
-  }
-  T rr = wsum(loc);
-  const T stop = T(rtol * rtol) * rr;
-  const int ex = kind == 0 ? L.n[0] : L.nn[0], ey = kind == 0 ? L.n[1] : L.nn[1];
-  for (int it = 0; it < max_it && rr > stop; it++) {
-    __syncwarp();  // p complete
-    loc = T(0);
-    for (int u = lane; u < n; u += 32) {
-      const int rw = u / ex;
-      const int i = u - rw * ex, j = rw % ey, k = rw / ey;
-      T dg;
-      const T ap = kind == 0 ? mac_op<T>(L, p, rho, i, j, k, dg) : fe_op<T>(L, p, rho, i, j, k, dg);
-      q[u] = ap;
-      loc += p[u] * ap;
-    }
-    const T pq = wsum(loc);
-    if (!(pq > T(0))) break;
-    const T a = rr / pq;
-    loc = T(0);
-    for (int u = lane; u < n; u += 32) {
-      x[u] += a * p[u];
-      const T v = r[u] - a * q[u];
-      r[u] = v;
-      loc += v * v;
-    }
-    const T rr2 = wsum(loc);
-    const T beta = rr2 / rr;
-    rr = rr2;
-    __syncwarp();  // every lane has read p for its q before p changes
-    for (int u = lane; u < n; u += 32) p[u] = r[u] + beta * p[u];
-  }
-  __syncwarp();
-  loc = T(0);
-  for (int u = lane; u < n; u += 32) loc += x[u];
-  const T xm = wsum(loc) / T(n);
-  for (int u = lane; u < n; u += 32) x[u] = x[u] - xm;
-  __syncwarp();
-}
-
 template <typename T>
 __global__ void __launch_bounds__(COARSE_TPB) k_coarse_cg(Lv L, int kind, int max_it, double rtol, T* __restrict__ gx,
                                                          T* __restrict__ gp, T* __restrict__ gb,
@@ -1589,10 +1537,7 @@ __global__ void __launch_bounds__(COARSE_TPB) k_coarse_cg(Lv L, int kind, int ma
     rho = c;
     __syncthreads();
   }
-  if (blockDim.x == 32)
-    cg_warp(L, kind, max_it, rtol, x, r, p, q, rho);
-  else
-    cg_block(L, kind, max_it, rtol, x, r, p, q, rho, red);
+  cg_block(L, kind, max_it, rtol, x, r, p, q, rho, red);
   if (in_smem)
     for (long u = threadIdx.x; u < n; u += blockDim.x) gx[u] = x[u];
 }
@@ -1631,6 +1576,7 @@ struct MGSolver {
   int zc0_auto = 0;          // z-chunk of the finest level's fused sweep from the wave heuristic
   int fe_zc0 = 0;            // z-chunk of the finest level's FE tiles (0: the heuristic)
   size_t bytes = 0;          // device bytes requested
+  CoarseCfg cc;              // the coarsest level's cluster solve
 };
 
 void mg_set_hook(MGSolver* m, mg_hook_fn fn, void* ctx) {
@@ -1751,11 +1697,20 @@ MGSolver* mg_build(const Geo& g, int kind, int prec_fp32, bool dry, cudaError_t*
     if (e == cudaSuccess) e = cudaMallocHost((void**)&m->hpin, 8 * sizeof(double));
     // the coarsest level lives in shared memory during its solve (when it fits): opt in to its
     // size once, outside any stream capture
-    const size_t smem = coarse_smem(m->lv[m->nlev - 1], m->esz);
+    m->cc = coarse_cfg(kind, m->lv[m->nlev - 1], m->esz);
+    const size_t smem = m->cc.cs > 0 ? 0 : coarse_smem(m->lv[m->nlev - 1], m->esz);
     // the attribute belongs to the kernel, shared by every solver: it only ever grows
     static std::mutex mu;
-    static size_t opted[2] = {0, 0};
+    static size_t opted[2] = {0, 0}, opted_cl[2][2][COARSE_UPT + 1] = {};
     std::lock_guard<std::mutex> lock(mu);
+    if (e == cudaSuccess && m->cc.cs > 0) {
+      size_t& have = opted_cl[prec_fp32 ? 1 : 0][kind][m->cc.upt];
+      if (m->cc.smem > have) {
+        e = cudaFuncSetAttribute(coarse_fn(kind, !prec_fp32, m->cc.upt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)m->cc.smem);
+        if (e == cudaSuccess) have = m->cc.smem;
+      }
+    }
     if (e == cudaSuccess && smem > opted[prec_fp32 ? 1 : 0]) {
       if (prec_fp32)
         e = cudaFuncSetAttribute(k_coarse_cg<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1966,14 +1921,14 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
     // the launch, the tolerance ends it
     const int max_it = 8 * nmax + 64;
     const double tol = coarse_tol<T>();
-    const size_t smem = coarse_smem(L, sizeof(T));  // opted in at creation
-    // as many warps as the level has unknowns for, and a single warp (reductions by shuffles, no
-    // block barriers) up to 512 unknowns: a small level's iterations are bound by the reductions
-    const long want = (L.nunk + 31) / 32 * 32;
-    const int tpb = L.nunk <= 512 ? 32 : (want < COARSE_TPB ? (int)want : COARSE_TPB);
-    k_coarse_cg<T><<<1, tpb, smem, s>>>(L, m->kind, max_it, tol, (T*)m->x[l], (T*)m->xt[l], (T*)m->b[l],
-                                               (T*)m->r[l], (const T*)m->rho[l], smem > 0);
     rmt_count_launches(1);
+    if (m->cc.cs > 0) {
+      launch_coarse_solve<T>(m->cc, m->kind, L, max_it, tol, (T*)m->x[l], (const T*)m->b[l], (const T*)m->rho[l], s);
+      return;
+    }
+    const size_t smem = coarse_smem(L, sizeof(T));  // opted in at creation
+    k_coarse_cg<T><<<1, COARSE_TPB, smem, s>>>(L, m->kind, max_it, tol, (T*)m->x[l], (T*)m->xt[l], (T*)m->b[l],
+                                               (T*)m->r[l], (const T*)m->rho[l], smem > 0);
     return;
   }
   const int npre = l > 0 && m->cpre >= 0 ? m->cpre : m->pre, npost = l > 0 && m->cpost >= 0 ? m->cpost : m->post;

@@ -1,0 +1,62 @@
+"""Kernels whose variant depends on size, type or boundary, at the sizes where the rule or the tiling
+can go wrong, against the FP64 oracle or the general path."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2104_00095_gb300 import rmt, scenes as S
+from parity_util import compare_state, needs_gpu, pair, rel_l2
+
+pytestmark = [pytest.mark.gpu, needs_gpu]
+
+
+def _box(n, periodic):
+    """A flow without bodies on an n[0] x n[1] x n[2] grid: a lid between walls, or a smooth field
+    in a periodic box; varying density needs no body here (the coefficient is 1)."""
+    sc = S._box(max(n), periodic=periodic, lid=0.0 if periodic else 1.0)
+    sc.update(n=tuple(n), hi=tuple(v / max(n) for v in n), mu=0.02)
+    return sc
+
+
+def _with_body(n, periodic):
+    sc = _box(n, periodic)
+    c = [0.5 * v / max(n) for v in n]
+    r = 0.28 * min(n) / max(n)
+    sc["solids"] = [S.solid(S.ELLIPSOID, c, (r, 0.8 * r, 0.9 * r), S.random_rotation(np.random.default_rng(2)),
+                            rho_s=1.6, G=0.3, mu_a=0.02)]
+    return sc
+
+
+# coarsest levels of one block (3^3, 9 x 7 x 5, 11^3) and of a cluster with 1, 4 and 8 unknowns per
+# thread (17 x 15 x 19, 23^3, 27^3), with walls and periodic; 54^3 = 2 x 27^3
+@pytest.mark.parametrize("n,periodic", [((24, 24, 24), True), ((36, 28, 20), False), ((44, 44, 44), False),
+                                        ((34, 30, 38), False), ((34, 38, 30), True), ((46, 46, 46), True),
+                                        ((54, 54, 54), False)])
+def test_coarsest_level_solves_fp64(n, periodic):
+    """One step from a moving state, solved to 1e-13, against the oracle's conjugate gradients."""
+    g, o = pair(_with_body(n, periodic))
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    g.write(rmt.RMT_F_U, u)
+    assert o.write(O.F_U, u) == 0
+    g.step(1)
+    assert o.step(1) == 0, o.error()
+    assert max(g.cycles()) <= 40  # the V-cycle keeps its rate only with an accurate coarsest solve
+    compare_state(g, o, 1, 1e-10, tag=f"{n}")
+
+
+@pytest.mark.parametrize("n,periodic", [((48, 48, 48), True), ((34, 30, 38), False), ((46, 46, 46), True),
+                                        ((54, 54, 54), False)])
+def test_coarsest_level_solves_fp32(n, periodic):
+    """The FP32 form's adaptive solves to 1e-9 take about the cycles of the FP64 form's to 1e-9, and
+    reach its velocities to FP32 accuracy."""
+    out = []
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    for prec in ("fp64", "fp32"):
+        g = rmt.Grid(dict(_with_body(n, periodic), precision=prec, mg_rtol=1e-9, mg_max_cycles=60))
+        g.write(rmt.RMT_F_U, u)
+        g.step(1)
+        out.append((g.read(rmt.RMT_F_U), g.cycles()))
+        g.close()
+    (u64, c64), (u32, c32) = out
+    assert rel_l2(u32, u64) <= 1e-5
+    assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)
