@@ -287,21 +287,54 @@ template <typename T>
 __global__ void k_cvt_back(const double* __restrict__ a, T* __restrict__ b, long n) {
   GRID_LOOP(i, n) b[i] = (T)a[i];
 }
-__global__ void k_cvt_i8(const int8_t* __restrict__ a, double* __restrict__ b, long n) {
-  GRID_LOOP(i, n) b[i] = (double)a[i];
+template <typename OT>
+__global__ void k_cvt_i8(const int8_t* __restrict__ a, OT* __restrict__ b, long n) {
+  GRID_LOOP(i, n) b[i] = (OT)a[i];
 }
-// a reference map to FP64 xi (FP32 storage: the displacement plus the cell centre's image)
-template <typename T>
-__global__ void k_xi_out(Geo g, Body b, const T* __restrict__ x, double* __restrict__ out) {
-  GRID_LOOP(q, 3 * g.N) {
-    double v = (double)x[q];
-    if constexpr (disp_storage<T>()) {
-      const int a = (int)(q / g.N);
-      const long c = q - a * g.N;
-      const int ii[3] = {(int)(c % g.n[0]), (int)((c / g.n[0]) % g.n[1]), (int)(c / ((long)g.n[0] * g.n[1]))};
-      v += g.lo[a] + (img_u(g, b, a, ii[a]) + 0.5) * g.h;
+// A reference map stored as displacements to xi = S + x0, x0 = lo + (u + 1/2) h the cell centre's
+// image, as float or double.  Bound: HBM (one read and one write per value).  x0 depends on one index
+// per axis, so a thread marches up a column of XOZ cells with the x and y parts in registers and the
+// block's z parts in shared memory; for float output x0 is a two-float pair and the sum's rounding
+// error is carried (Knuth's two-sum), which leaves the FP64 pipe (two lanes per SM) idle.  A
+// linear loop with 64-bit divisions and FP64 sums took 484 us per 256^3 map plus 166 us of
+// conversion and copy (201 MB out); this takes 72 us.
+constexpr int XOZ = 16;
+template <typename OT>
+__global__ void __launch_bounds__(TILE_X* TILE_Y) k_xi_out(Geo g, Body b, const float* __restrict__ x,
+                                                           OT* __restrict__ out) {
+  __shared__ double z0[XOZ];
+  __shared__ float zh[XOZ], zl[XOZ];
+  const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
+  const int k0 = blockIdx.z * XOZ, k1 = min(k0 + XOZ, g.n[2]);
+  const int t = threadIdx.y * TILE_X + threadIdx.x;
+  auto image = [&](int a, int q) { return g.lo[a] + (img_u(g, b, a, q) + 0.5) * g.h; };
+  if (t < k1 - k0) {
+    z0[t] = image(2, k0 + t);
+    zh[t] = (float)z0[t];
+    zl[t] = (float)(z0[t] - (double)zh[t]);
+  }
+  __syncthreads();
+  if (i >= g.n[0] || j >= g.n[1]) return;
+  const double xy[2] = {image(0, i), image(1, j)};
+  const float h2[2] = {(float)xy[0], (float)xy[1]};
+  const float l2[2] = {(float)(xy[0] - (double)h2[0]), (float)(xy[1] - (double)h2[1])};
+  const long plane = (long)g.n[0] * g.n[1], c0 = cidx(g, i, j, k0);
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float* xa = x + a * g.N + c0;
+    OT* oa = out + a * g.N + c0;
+#pragma unroll 4
+    for (int k = 0; k < k1 - k0; k++) {
+      const float v = xa[k * plane];
+      if constexpr (sizeof(OT) == 8) {
+        oa[k * plane] = (double)v + (a < 2 ? xy[a & 1] : z0[k]);
+      } else {
+        const float h = a < 2 ? h2[a & 1] : zh[k], l = a < 2 ? l2[a & 1] : zl[k];
+        const float s = __fadd_rn(h, v), bb = __fsub_rn(s, h);
+        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb));
+        oa[k * plane] = __fadd_rn(s, __fadd_rn(e, l));
+      }
     }
-    out[q] = v;
   }
 }
 // FP64 xi to the stored form
@@ -790,40 +823,50 @@ rmt_status build_graph(rmt_grid* g) {
 }  // namespace
 
 namespace {
-template <typename T>
-rmt_status gather_t(rmt_grid* g, int field, int sid, double* out) {
+// field of a grid with storage T into the device array out, as OT
+template <typename T, typename OT>
+rmt_status gather_t(rmt_grid* g, int field, int sid, OT* out) {
   const Geo& G = g->g;
   const long N = G.N;
   cudaStream_t s = g->s;
-  auto cvt = [&](const void* src, long n, long off) { k_cvt<T><<<nbk(n), 256, 0, s>>>((const T*)src, out + off, n); rmt_count_launches(1); };
+  rmt_status st = RMT_OK;
+  auto cvt = [&](const void* src, long n, long off) {
+    if constexpr (sizeof(T) == sizeof(OT)) {
+      if (cudaMemcpyAsync(out + off, src, (size_t)n * sizeof(T), cudaMemcpyDefault, s) != cudaSuccess)
+        st = fail(g, RMT_ECUDA, "field copy: %s", cudaGetErrorString(cudaGetLastError()));
+    } else if constexpr (sizeof(OT) == 8) {
+      k_cvt<T><<<nbk(n), 256, 0, s>>>((const T*)src, out + off, n);
+      rmt_count_launches(1);
+    } else {
+      k_cvt_back<OT><<<nbk(n), 256, 0, s>>>((const double*)src, out + off, n);
+      rmt_count_launches(1);
+    }
+  };
+  auto xi = [&](const void* src) {
+    if constexpr (disp_storage<T>()) {
+      const dim3 gr((G.n[0] + TILE_X - 1) / TILE_X, (G.n[1] + TILE_Y - 1) / TILE_Y, (G.n[2] + XOZ - 1) / XOZ);
+      k_xi_out<OT><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(G, g->bodies[sid], (const float*)src, out);
+      rmt_count_launches(1);
+    } else {
+      cvt(src, 3 * N, 0);
+    }
+  };
   switch (field) {
     case RMT_F_U: cvt(g->u, 3 * N, 0); break;
     case RMT_F_P: cvt(g->p, G.NN, 0); break;
     case RMT_F_RHO: cvt(g->rho, N, 0); break;
-    case RMT_F_XI:
-      k_xi_out<T><<<nbk(3 * N), 256, 0, s>>>(G, g->bodies[sid], (const T*)g->bm[sid].X[g->par], out);
-      rmt_count_launches(1);
-      break;
+    case RMT_F_XI: xi(g->bm[sid].X[g->par]); break;
     case RMT_F_PHI: cvt(g->bm[sid].PHI[g->par], N, 0); break;
-    case RMT_F_LAYER: k_cvt_i8<<<nbk(N), 256, 0, s>>>(g->bm[sid].LAY[g->par], out, N); rmt_count_launches(1); break;
-    case RMT_F_XI_HALF:
-      k_xi_out<T><<<nbk(3 * N), 256, 0, s>>>(G, g->bodies[sid], (const T*)g->bm[sid].XH, out);
+    case RMT_F_LAYER:
+      k_cvt_i8<OT><<<nbk(N), 256, 0, s>>>(g->bm[sid].LAY[g->par], out, N);
       rmt_count_launches(1);
       break;
+    case RMT_F_XI_HALF: xi(g->bm[sid].XH); break;
     case RMT_F_DIVTAU_N: cvt(g->divn, 3 * N, 0); break;
     case RMT_F_DIVTAU_H: cvt(g->divh, 3 * N, 0); break;
     case RMT_F_ADV_U: cvt(g->adv, 3 * N, 0); break;
     case RMT_F_USTAR: cvt(g->ustar, 3 * N, 0); break;
     case RMT_F_RHO_HALF: cvt(g->rho_h, N, 0); break;
-    case RMT_F_REPULSION:  // from the last step's half-level bodies
-      launch_rep_field<T>(G, g->bodies_d, views<T>(g, 1 - g->par, 1), (int)g->bodies.size(), out, s);
-      break;
-    case RMT_F_MAC_Q:
-      CK(g, cudaMemcpyAsync(out, mg_solution64(g->mac, s), N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-      break;
-    case RMT_F_PSI:
-      CK(g, cudaMemcpyAsync(out, mg_solution64(g->fe, s), G.NN * sizeof(double), cudaMemcpyDeviceToDevice, s));
-      break;
     case RMT_F_UFACE_X: case RMT_F_UFACE_Y: case RMT_F_UFACE_Z: {
       const int d = field - RMT_F_UFACE_X;
       const long nf = nfaces(G, d);
@@ -835,10 +878,42 @@ rmt_status gather_t(rmt_grid* g, int field, int sid, double* out) {
       cvt(g->umac[d], nfaces(G, d), 0);
       break;
     }
+    // values that exist in FP64 only (see formed_in_fp64)
+    case RMT_F_REPULSION:  // from the last step's half-level bodies
+      if constexpr (sizeof(OT) == 8)
+        launch_rep_field<T>(G, g->bodies_d, views<T>(g, 1 - g->par, 1), (int)g->bodies.size(), out, s);
+      break;
+    case RMT_F_MAC_Q:
+      if constexpr (sizeof(OT) == 8)
+        CK(g, cudaMemcpyAsync(out, mg_solution64(g->mac, s), N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+      break;
+    case RMT_F_PSI:
+      if constexpr (sizeof(OT) == 8)
+        CK(g, cudaMemcpyAsync(out, mg_solution64(g->fe, s), G.NN * sizeof(double), cudaMemcpyDeviceToDevice, s));
+      break;
     default: return fail(g, RMT_EINVAL, "unknown field %d", field);
   }
+  if (st != RMT_OK) return st;
   CK(g, cudaGetLastError());
   return RMT_OK;
+}
+template <typename OT>
+rmt_status gather(rmt_grid* g, int field, int sid, OT* out) {
+  return g->fp32 ? gather_t<float, OT>(g, field, sid, out) : gather_t<double, OT>(g, field, sid, out);
+}
+// fields that a float read takes through the FP64 staging array
+bool formed_in_fp64(int field) { return field == RMT_F_REPULSION || field == RMT_F_MAC_Q || field == RMT_F_PSI; }
+// may a kernel write floats to dst: device memory of this device, aligned to a float (a copy has
+// neither condition)
+bool kernel_writable(const void* dst) {
+  cudaPointerAttributes at;
+  int dev = 0;
+  if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cudaGetDevice(&dev) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev &&
+         (uintptr_t)dst % sizeof(float) == 0;
 }
 
 template <typename T>
@@ -877,17 +952,20 @@ rmt_status read_field(rmt_grid* g, int field, int solid_id, void* dst, size_t ds
   if (f32 && g->fp32 && (field == RMT_F_U || field == RMT_F_P)) {
     // stored in this layout: one copy, no conversion
     CK(g, cudaMemcpyAsync(dst, field == RMT_F_U ? g->u : g->p, (size_t)n * sizeof(float), kind, g->s));
+  } else if (f32 && !formed_in_fp64(field)) {
+    // formed as floats, in place where a kernel may write there
+    float* out = dst_is_device && kernel_writable(dst) ? (float*)dst : (float*)g->stage;
+    if ((st = gather<float>(g, field, solid_id, out)) != RMT_OK) return st;
+    if (out != dst) CK(g, cudaMemcpyAsync(dst, out, (size_t)n * sizeof(float), kind, g->s));
   } else if (f32) {
-    st = g->fp32 ? gather_t<float>(g, field, solid_id, g->stage) : gather_t<double>(g, field, solid_id, g->stage);
-    if (st != RMT_OK) return st;
+    if ((st = gather<double>(g, field, solid_id, g->stage)) != RMT_OK) return st;
     if (!g->stage_f) CK(g, cudaMalloc((void**)&g->stage_f, (size_t)g->stage_len * sizeof(float)));
     k_cvt_back<float><<<nbk(n), 256, 0, g->s>>>(g->stage, g->stage_f, n);
     rmt_count_launches(1);
     CK(g, cudaMemcpyAsync(dst, g->stage_f, (size_t)n * sizeof(float), kind, g->s));
   } else {
     double* out = dst_is_device ? (double*)dst : g->stage;
-    st = g->fp32 ? gather_t<float>(g, field, solid_id, out) : gather_t<double>(g, field, solid_id, out);
-    if (st != RMT_OK) return st;
+    if ((st = gather<double>(g, field, solid_id, out)) != RMT_OK) return st;
     if (!dst_is_device) CK(g, cudaMemcpyAsync(dst, g->stage, (size_t)n * sizeof(double), kind, g->s));
   }
   CK(g, cudaStreamSynchronize(g->s));
@@ -1053,7 +1131,7 @@ rmt_status rmt_init_pressure(rmt_grid* g, int max_iters, double tol, int* iters_
   }
   std::vector<double> prev((size_t)G.NN), cur((size_t)G.NN);
   auto read_p = [&](std::vector<double>& dst) -> rmt_status {
-    rmt_status s2 = g->fp32 ? gather_t<float>(g, RMT_F_P, 0, g->stage) : gather_t<double>(g, RMT_F_P, 0, g->stage);
+    const rmt_status s2 = gather<double>(g, RMT_F_P, 0, g->stage);
     if (s2 != RMT_OK) return s2;
     CK(g, cudaMemcpyAsync(dst.data(), g->stage, G.NN * sizeof(double), cudaMemcpyDeviceToHost, g->s));
     CK(g, cudaStreamSynchronize(g->s));

@@ -60,3 +60,27 @@ def test_coarsest_level_solves_fp32(n, periodic):
     (u64, c64), (u32, c32) = out
     assert rel_l2(u32, u64) <= 1e-5
     assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)
+
+
+@pytest.mark.parametrize("n,periodic,precision", [((36, 40, 44), True, "fp32"), ((33, 35, 50), False, "fp32"),
+                                                  ((36, 40, 44), True, "fp64")])
+def test_float_reads_of_every_field(n, periodic, precision):
+    """Float reads to the host, to device memory and to a device address that is not aligned to a
+    float equal the rounded FP64 read; a reference map's is within one unit in the last place."""
+    import torch
+
+    g = rmt.Grid(dict(_with_body(n, periodic), precision=precision, mg_rtol=1e-6))
+    g.write(rmt.RMT_F_U, 0.1 * np.sin(np.arange(3 * np.prod(n)) * 0.37))
+    g.step(1)
+    for f in list(range(1, 7)) + list(range(20, 35)):
+        ref = g.read(f).astype(np.float32)
+        raw = torch.zeros(ref.size * 4 + 8, dtype=torch.uint8, device="cuda")
+        got = [g.read_float(f)]
+        for off in (0, 2):
+            g.read_float_ptr(f, raw.data_ptr() + off, ref.size * 4, 1)
+            got.append(raw.cpu().numpy()[off:off + 4 * ref.size].copy().view(np.float32))
+        for v in got:
+            assert np.array_equal(np.isnan(v), np.isnan(ref)), f
+            ok = ~np.isnan(ref)
+            assert np.all(np.abs(v[ok] - ref[ok]) <= (np.spacing(np.abs(ref[ok])) if f in (4, 30) else 0)), f
+    g.close()
