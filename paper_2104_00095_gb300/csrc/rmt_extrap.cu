@@ -319,38 +319,343 @@ __device__ int wls_cell_warp(const Geo& g, const Body& b, const T* __restrict__ 
   return wls_cell_try<AT>(g, b, x, lay, i, j, k, le, cd, out);
 }
 
-// FP32 fits run at six blocks per SM (80 registers a thread, 8 bytes spilled); FP64 fits take what
-// they need
-#define WLS_MINB(T, REDO) ((sizeof(T) == 4 && !(REDO)) ? 6 : 1)
+// ---- batches of cells ------------------------------------------------------------------
+// A warp fits up to 32 cells together: cell after cell the lanes sum the normal equations over the 125
+// candidates of the radius-2 box, and then every lane solves the 4 x 4 system of a cell of its own, so
+// that the solves (some 200 dependent operations each) cost a warp once per batch instead of once
+// per cell and fit.  What bounds it is the FP64 pipe (two lanes per SM: a warp instruction takes 16
+// cycles) in the FP64 form and instruction issue in the FP32 form, so the sums are cut to what cannot
+// be avoided:
+//  * the kernel-only fit's weights 2^-(|di|+|dj|+|dk|) and its products with the offsets are exact
+//    multiples of 2^-6: its normal matrix is summed in integers (one redux per entry), and the
+//    right-hand sides take one FMA per candidate and entry (the weight times the value is exact);
+//  * the normal-weighted fit's sums take one FMA each;
+//  * sums over the lanes are transposed: at every step a lane hands over half of its partial sums,
+//    16 + 8 + 4 + 2 + 1 additions for 22 totals instead of 110, added in the same tree.
+// One warp per cell with 66 multiplications and additions per candidate and fit and a solve by all
+// lanes took 32.2 ms per step of the 128^3 settling mixture in FP64 (20 bodies; 27.4 now) and 1.50 ms
+// per extrapolation of one body on 96^3 (0.78 now).
+constexpr int WB = 32;                 // cells of a batch at most
+constexpr int NSUM = 22, NPAD = 23;    // totals of a fit, padded against bank conflicts
+template <typename AT>
+struct WlsShared {
+  AT v[TPB / 32][WB][NPAD];
+};
 
-// one warp per cell of layer l (its segment of the band list).  REDO: the FP64 pass over the
-// cells whose FP32 fits were too ill-conditioned (redo[0 .. cnt[0]), filtered by layer);
-// otherwise the storage type's pass, which lists such cells in redo (FP32 storage).
-template <typename T, bool REDO>
-__global__ void __launch_bounds__(TPB, WLS_MINB(T, REDO)) k_wls(Geo g, Body b, int l, T* __restrict__ x, int8_t* __restrict__ lay, const int* __restrict__ list,
-                      int* __restrict__ cnt, int* __restrict__ redo, int* __restrict__ err) {
-  using AT = typename std::conditional<REDO || sizeof(T) == 8, double, float>::type;
+// this lane's candidates t = lane + 32 q of the 5^3 box
+struct Slots {
+  int off[NQ0];        // linear offset from the cell
+  signed char d[NQ0][3];
+  bool in[NQ0];
+};
+__device__ __forceinline__ Slots wls_slots(const Geo& g) {
+  Slots s;
+  const int lane = threadIdx.x & 31, w = 2 * RS0 + 1;
+#pragma unroll
+  for (int q = 0; q < NQ0; q++) {
+    const int t = lane + 32 * q;
+    const int di = t % w - RS0, dj = (t / w) % w - RS0, dk = t / (w * w) - RS0;
+    s.in[q] = t < NC0;
+    s.d[q][0] = (signed char)di;
+    s.d[q][1] = (signed char)dj;
+    s.d[q][2] = (signed char)dk;
+    s.off[q] = di + g.n[0] * (dj + g.n[1] * dk);
+  }
+  return s;
+}
+template <typename T>
+__device__ __forceinline__ void slot_cand(const Geo& g, const Slots& s, const T* __restrict__ x,
+                                          const int8_t* __restrict__ lay, long c, int i, int j, int k, int le,
+                                          Cand<T>& cd) {
+  long cc[NQ0];
+  int ld[NQ0];
+  const bool inner = i >= RS0 && i + RS0 < g.n[0] && j >= RS0 && j + RS0 < g.n[1] && k >= RS0 && k + RS0 < g.n[2];
+#pragma unroll
+  for (int q = 0; q < NQ0; q++) {
+    ld[q] = -1;
+    cc[q] = c;
+    bool in = s.in[q];
+    if (inner) cc[q] = c + s.off[q];
+    else if (in) in = cell_at(g, i + s.d[q][0], j + s.d[q][1], k + s.d[q][2], cc[q]);
+    if (in) ld[q] = lay[cc[q]];
+  }
+  cd.ok = 0u;
+#pragma unroll
+  for (int q = 0; q < NQ0; q++) {
+    cd.v[q][0] = cd.v[q][1] = cd.v[q][2] = T(0);
+    if (ld[q] >= 0 && ld[q] < le) {
+      cd.ok |= 1u << q;
+      cd.v[q][0] = x[cc[q]];
+      cd.v[q][1] = x[g.N + cc[q]];
+      cd.v[q][2] = x[2 * g.N + cc[q]];
+    }
+  }
+}
+__device__ __forceinline__ float fma_any(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_any(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// lane totals: v[q] summed over the warp ends in lane q (32 values) -- or, HALF (16 values), in lanes
+// 2 q and 2 q + 1
+template <typename AT, bool HALF>
+__device__ __forceinline__ AT warp_transpose_sum(AT* v) {
   const int lane = threadIdx.x & 31;
-  const int base = REDO ? 0 : layer_base(cnt, l), n = REDO ? cnt[0] : cnt[l];
-  const int* src = REDO ? redo : list + base;
+  constexpr int N = HALF ? 8 : 16;
+#pragma unroll
+  for (int h = N, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; q++) {
+      const AT give = up ? v[q] : v[q + h];
+      const AT keep = up ? v[q + h] : v[q];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  if (HALF) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  return v[0];
+}
+
+template <typename AT>
+__device__ __forceinline__ bool solve_totals(const AT* t, int npos, AT tolfac, AT sol[4][3]) {
+  if (npos < 4) return false;
+  AT A[4][4], B[4][3];
+  int q = 0;
+#pragma unroll
+  for (int r = 0; r < 4; r++)
+#pragma unroll
+    for (int c = r; c < 4; c++) {
+      A[r][c] = t[q];
+      A[c][r] = t[q];
+      q++;
+    }
+#pragma unroll
+  for (int r = 0; r < 4; r++)
+#pragma unroll
+    for (int d = 0; d < 3; d++) B[r][d] = t[10 + 3 * r + d];
+  return solve4<AT>(A, B, sol, tolfac);
+}
+
+// Fits this lane's cell c (none: c < 0) of layer le together with the other lanes' cells.  Returns 1 with
+// out, 0 when the radius-2 system is degenerate or (FP32) too ill-conditioned to trust.
+template <typename AT, typename T>
+__device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared<AT>& sh, const T* __restrict__ x,
+                         const int8_t* __restrict__ lay, long c, int le, AT out[3]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // FP64: the degeneracy threshold; FP32: also the point below which the fit is redone in FP64
+  const AT tolfac = sizeof(AT) == 8 ? AT(1e-12) : AT(1e-4);
+  const AT hid = disp_storage<T>() ? cv<AT>(g.h, g.f.h) : AT(0);
+  int i = 0, j = 0, k = 0;
+  if (c >= 0) decode(c, g.n[0], g.n[1], i, j, k);
+  const unsigned todo = __ballot_sync(0xffffffffu, c >= 0);
+  int npos = 0;
+  // kernel-only fit: normal matrix in units of 2^-6
+  for (unsigned m = todo; m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    const long cc = __shfl_sync(0xffffffffu, c, src);
+    const int ci = __shfl_sync(0xffffffffu, i, src), cj = __shfl_sync(0xffffffffu, j, src), ck = __shfl_sync(0xffffffffu, k, src);
+    Cand<T> cd;
+    slot_cand(g, sl, x, lay, cc, ci, cj, ck, le, cd);
+    int a[10];
+    AT bs[16];
+#pragma unroll
+    for (int q = 0; q < 10; q++) a[q] = 0;
+#pragma unroll
+    for (int q = 0; q < 16; q++) bs[q] = AT(0);
+#pragma unroll
+    for (int q = 0; q < NQ0; q++) {
+      if (!(cd.ok >> q & 1u)) continue;
+      const int di = sl.d[q][0], dj = sl.d[q][1], dk = sl.d[q][2];
+      const int w = 64 >> (abs(di) + abs(dj) + abs(dk));
+      const int v[4] = {1, di, dj, dk};
+      int e = 0;
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int s = r; s < 4; s++) a[e++] += w * v[r] * v[s];
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        const AT wv = (AT)((float)(w * v[r]) * (1.0f / 64.0f));
+#pragma unroll
+        for (int d = 0; d < 3; d++) bs[3 * r + d] = fma_any(wv, (AT)cd.v[q][d], bs[3 * r + d]);
+      }
+    }
+    const int np = __reduce_add_sync(0xffffffffu, __popc(cd.ok));
+    if (lane == src) npos = np;
+#pragma unroll
+    for (int q = 0; q < 10; q++) a[q] = __reduce_add_sync(0xffffffffu, a[q]);
+    const AT tot = warp_transpose_sum<AT, true>(bs);
+    if (lane < 24 && !(lane & 1)) sh.v[warp][src][10 + (lane >> 1)] = tot;
+    if (lane == 0) {
+#pragma unroll
+      for (int q = 0; q < 10; q++) sh.v[warp][src][q] = (AT)((float)a[q] * (1.0f / 64.0f));
+    }
+  }
+  __syncwarp();
+  int ok = 0;
+  AT s1[4][3], nrm[3] = {AT(0), AT(0), AT(0)};
+  if (c >= 0 && solve_totals<AT>(sh.v[warp][lane], npos, tolfac, s1)) {
+    ok = 1;
+#pragma unroll
+    for (int d = 0; d < 3; d++) out[d] = s1[0][d];
+    if (le <= 2) {
+      // n_e = normalised (grad xi)^T grad_X phi_0(xi_e); FP32 storage: the identity's part added back
+      AT gX[3], v[3];
+      if constexpr (disp_storage<T>()) {
+        const AT r0[3] = {cell_rel<AT>(g, b, 0, i) + s1[0][0], cell_rel<AT>(g, b, 1, j) + s1[0][1],
+                          cell_rel<AT>(g, b, 2, k) + s1[0][2]};
+        phi0_dir_r<AT>(b, r0, gX);
+      } else {
+        const AT c0[3] = {s1[0][0], s1[0][1], s1[0][2]};
+        phi0_dir<AT>(b, c0, gX);
+      }
+#pragma unroll
+      for (int q = 0; q < 3; q++)
+        v[q] = (s1[1 + q][0] + (q == 0 ? hid : AT(0))) * gX[0] + (s1[1 + q][1] + (q == 1 ? hid : AT(0))) * gX[1] +
+               (s1[1 + q][2] + (q == 2 ? hid : AT(0))) * gX[2];
+      const AT nv = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+      if (nv > AT(0)) {
+#pragma unroll
+        for (int q = 0; q < 3; q++) nrm[q] = v[q] / nv;
+      } else {
+        ok = 0;
+      }
+    }
+  }
+  __syncwarp();  // the totals have been read
+  if (le > 2) return ok;
+  // the fit weighted by max(0, cos) of the angle to the normal
+  AT kl[NQ0];  // 2^-sr / |d| of this lane's candidates
+#pragma unroll
+  for (int q = 0; q < NQ0; q++) {
+    const int di = sl.d[q][0], dj = sl.d[q][1], dk = sl.d[q][2], s2 = di * di + dj * dj + dk * dk;
+    kl[q] = s2 ? (AT)(64 >> (abs(di) + abs(dj) + abs(dk))) * AT(1.0 / 64.0) / sqrt((AT)s2) : AT(0);
+  }
+  for (unsigned m = __ballot_sync(0xffffffffu, ok != 0); m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    const long cc = __shfl_sync(0xffffffffu, c, src);
+    const int ci = __shfl_sync(0xffffffffu, i, src), cj = __shfl_sync(0xffffffffu, j, src), ck = __shfl_sync(0xffffffffu, k, src);
+    AT n[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) n[d] = __shfl_sync(0xffffffffu, nrm[d], src);
+    Cand<T> cd;
+    slot_cand(g, sl, x, lay, cc, ci, cj, ck, le, cd);
+    AT sum[32];
+#pragma unroll
+    for (int q = 0; q < 32; q++) sum[q] = AT(0);
+    int pos = 0;
+#pragma unroll
+    for (int q = 0; q < NQ0; q++) {
+      if (!(cd.ok >> q & 1u)) continue;
+      const AT di = (AT)(float)sl.d[q][0], dj = (AT)(float)sl.d[q][1], dk = (AT)(float)sl.d[q][2];
+      const AT wt = -(di * n[0] + dj * n[1] + dk * n[2]) * kl[q];
+      if (!(wt > AT(0))) continue;
+      pos++;
+      const AT wv[4] = {wt, wt * di, wt * dj, wt * dk}, v[4] = {AT(1), di, dj, dk};
+      int e = 0;
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int s = r; s < 4; s++, e++) sum[e] = s == 0 ? sum[e] + wt : fma_any(wv[r], v[s], sum[e]);
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int d = 0; d < 3; d++) sum[10 + 3 * r + d] = fma_any(wv[r], (AT)cd.v[q][d], sum[10 + 3 * r + d]);
+    }
+    const int np = __reduce_add_sync(0xffffffffu, pos);
+    if (lane == src) npos = np;
+    const AT tot = warp_transpose_sum<AT, false>(sum);
+    if (lane < NSUM) sh.v[warp][src][lane] = tot;
+  }
+  __syncwarp();
+  if (ok && solve_totals<AT>(sh.v[warp][lane], npos, tolfac, s1)) {
+#pragma unroll
+    for (int d = 0; d < 3; d++) out[d] = s1[0][d];
+  } else {
+    ok = 0;
+  }
+  __syncwarp();  // the totals have been read: the next batch may write
+  return ok;
+}
+
+// Cells per batch for n cells on the launch's warps.  FP64 fits want fuller batches, since the pipe is
+// busy with a few warps an SM: a quarter of the warps (a half: 28.9 ms per step of the 128^3 mixture, a
+// fifth 27.4, a tenth 27.0, but 0.72, 0.78 and 0.92 ms per 96^3 extrapolation).  FP32 fits want the
+// warps in flight (batches of at least 1, 2, 4, 8: 7.99, 8.11, 8.22, 8.33 ms per 4 steps at 112^3).
+template <typename AT>
+__device__ __forceinline__ int batch_size(int n, int warps) {
+  const int want = sizeof(AT) == 8 ? (warps + 3) / 4 : warps;
+  const int g = (n + want - 1) / want;
+  return g < 1 ? 1 : (g > WB ? WB : g);
+}
+
+// The cells of layer l (its segment of the band list) in the storage type, batch by batch.  FP32 storage:
+// cells whose fits were too ill-conditioned are listed in redo.  FP64 storage: a cell whose radius-2
+// system is degenerate is fitted again by the whole warp with the growing radius.
+template <typename T>
+__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, Body b, int l, T* __restrict__ x, int8_t* __restrict__ lay,
+                                             const int* __restrict__ list, int* __restrict__ cnt,
+                                             int* __restrict__ redo, int* __restrict__ err) {
+  __shared__ WlsShared<T> sh;
+  const int lane = threadIdx.x & 31;
+  const int base = layer_base(cnt, l), n = cnt[l];
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  const int G = batch_size<T>(n, warps);
+  const Slots sl = wls_slots(g);
+  for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; e0 < n; e0 += warps * G) {
+    const long c = lane < G && e0 + lane < n ? list[base + e0 + lane] : -1;
+    T out[3];
+    const int r = wls_batch<T>(g, b, sl, sh, x, lay, c, l, out);
+    if (c >= 0 && r) {
+      x[c] = out[0];
+      x[g.N + c] = out[1];
+      x[2 * g.N + c] = out[2];
+    }
+    if constexpr (sizeof(T) == 4) {
+      if (c >= 0 && !r) redo[atomicAdd(&cnt[0], 1)] = (int)c;
+    } else {
+      for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
+        const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
+        int i, j, k;
+        decode(cc, g.n[0], g.n[1], i, j, k);
+        double o[3];
+        const int q = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, o);
+        __syncwarp();
+        if (lane == 0) {
+          if (q == 1) {
+            x[cc] = (T)o[0];
+            x[g.N + cc] = (T)o[1];
+            x[2 * g.N + cc] = (T)o[2];
+          } else {
+            lay[cc] = -1;
+            atomicAdd(err, 1);
+          }
+        }
+      }
+    }
+  }
+}
+
+// FP32 storage: the FP64 pass over the cells of layer l that k_wls listed, one warp per cell
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_wls_redo(Geo g, Body b, int l, T* __restrict__ x, int8_t* __restrict__ lay,
+                                                  const int* __restrict__ cnt, const int* __restrict__ redo,
+                                                  int* __restrict__ err) {
+  const int lane = threadIdx.x & 31, n = cnt[0];
   for (int e = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5); e < n; e += (gridDim.x * blockDim.x) >> 5) {
-    const long c = src[e];
-    if (REDO && lay[c] != l) continue;  // listed by an earlier layer's pass
+    const long c = redo[e];
+    if (lay[c] != l) continue;  // listed by an earlier layer's pass
     int i, j, k;
     decode(c, g.n[0], g.n[1], i, j, k);
     double out[3];
-    const int r = wls_cell_warp<AT>(g, b, x, lay, i, j, k, l, out);
+    const int r = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, out);
     __syncwarp();
     if (lane == 0) {
       if (r == 1) {
         x[c] = (T)out[0];
         x[g.N + c] = (T)out[1];
         x[2 * g.N + c] = (T)out[2];
-      } else if (r == 0) {
+      } else {
         lay[c] = -1;
         atomicAdd(err, 1);
-      } else {
-        redo[atomicAdd(&cnt[0], 1)] = (int)c;
       }
     }
   }
@@ -404,37 +709,73 @@ __global__ void k_corr(Geo g, const int* __restrict__ bb, const T* __restrict__ 
 }
 
 // cells new to the band: xi^{n+1/2} by the same WLS from the corrected lower layers (layer l's
-// segment of the new band's list; REDO as for k_wls, with its own redo count cnt[9])
-template <typename T, bool REDO>
-__global__ void __launch_bounds__(TPB, WLS_MINB(T, REDO)) k_wls_half(Geo g, Body b, int l, const int8_t* __restrict__ lay, const int8_t* __restrict__ layn,
-                           const T* __restrict__ xn, T* __restrict__ xh, const int* __restrict__ list,
-                           int* __restrict__ cnt, int* __restrict__ redo, int* __restrict__ err) {
-  using AT = typename std::conditional<REDO || sizeof(T) == 8, double, float>::type;
+// segment of the new band's list).  Few of a segment's cells are new: a warp looks at 32 of them and
+// fits those in one batch; what fails is treated as in k_wls, with a redo count of its own, cnt[9].
+template <typename T>
+__device__ __forceinline__ void half_result(const Geo& g, long c, int r, const double out[3], const T* __restrict__ xn,
+                                            T* __restrict__ xh, int* __restrict__ err) {
+  if (r == 1) {
+    xh[c] = (T)out[0];
+    xh[g.N + c] = (T)out[1];
+    xh[2 * g.N + c] = (T)out[2];
+  } else {
+    xh[c] = xn[c];
+    xh[g.N + c] = xn[g.N + c];
+    xh[2 * g.N + c] = xn[2 * g.N + c];
+    atomicAdd(err, 1);
+  }
+}
+template <typename T>
+__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g, Body b, int l, const int8_t* __restrict__ lay,
+                                                  const int8_t* __restrict__ layn, const T* __restrict__ xn,
+                                                  T* __restrict__ xh, const int* __restrict__ list,
+                                                  int* __restrict__ cnt, int* __restrict__ redo, int* __restrict__ err) {
+  __shared__ WlsShared<T> sh;
   const int lane = threadIdx.x & 31;
-  const int base = REDO ? 0 : layer_base(cnt, l), n = REDO ? cnt[9] : cnt[l];
-  const int* src = REDO ? redo : list + base;
+  const int base = layer_base(cnt, l), n = cnt[l];
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  const Slots sl = wls_slots(g);
+  for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; e0 < n; e0 += warps * 32) {
+    long c = e0 + lane < n ? list[base + e0 + lane] : -1;
+    if (c >= 0 && (layn[c] != l || lay[c] >= 0)) c = -1;
+    if (!__any_sync(0xffffffffu, c >= 0)) continue;
+    T out[3];
+    const int r = wls_batch<T>(g, b, sl, sh, xh, layn, c, l, out);
+    if (c >= 0 && r) {
+      xh[c] = out[0];
+      xh[g.N + c] = out[1];
+      xh[2 * g.N + c] = out[2];
+    }
+    if constexpr (sizeof(T) == 4) {
+      if (c >= 0 && !r) redo[atomicAdd(&cnt[9], 1)] = (int)c;
+    } else {
+      for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
+        const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
+        int i, j, k;
+        decode(cc, g.n[0], g.n[1], i, j, k);
+        double o[3];
+        const int q = wls_cell_warp<double>(g, b, xh, layn, i, j, k, l, o);
+        __syncwarp();
+        if (lane == 0) half_result(g, cc, q, o, xn, xh, err);
+      }
+    }
+  }
+}
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_wls_half_redo(Geo g, Body b, int l, const int8_t* __restrict__ lay,
+                                                       const int8_t* __restrict__ layn, const T* __restrict__ xn,
+                                                       T* __restrict__ xh, const int* __restrict__ cnt,
+                                                       const int* __restrict__ redo, int* __restrict__ err) {
+  const int lane = threadIdx.x & 31, n = cnt[9];
   for (int e = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5); e < n; e += (gridDim.x * blockDim.x) >> 5) {
-    const long c = src[e];
+    const long c = redo[e];
     if (layn[c] != l || lay[c] >= 0) continue;
     int i, j, k;
     decode(c, g.n[0], g.n[1], i, j, k);
     double out[3];
-    const int r = wls_cell_warp<AT>(g, b, xh, layn, i, j, k, l, out);
+    const int r = wls_cell_warp<double>(g, b, xh, layn, i, j, k, l, out);
     __syncwarp();
-    if (lane == 0) {
-      if (r < 0) {
-        redo[atomicAdd(&cnt[9], 1)] = (int)c;
-      } else if (r == 1) {
-        xh[c] = (T)out[0];
-        xh[g.N + c] = (T)out[1];
-        xh[2 * g.N + c] = (T)out[2];
-      } else {
-        xh[c] = xn[c];
-        xh[g.N + c] = xn[g.N + c];
-        xh[2 * g.N + c] = xn[2 * g.N + c];
-        atomicAdd(err, 1);
-      }
-    }
+    if (lane == 0) half_result(g, c, r, out, xn, xh, err);
   }
 }
 
@@ -491,10 +832,10 @@ cudaError_t launch_extrapolate(const Geo& g, const Body& b, const int* bb_in, in
     rmt_count_launches(1);
   }
   for (int l = 1; l <= g.layers; l++) {
-    k_wls<T, false><<<wls_blocks, TPB, 0, s>>>(g, b, l, x, lay, list, cnt, redo, err);
+    k_wls<T><<<wls_blocks, TPB, 0, s>>>(g, b, l, x, lay, list, cnt, redo, err);
     rmt_count_launches(1);
     if (sizeof(T) == 4) {
-      k_wls<T, true><<<sm_count(), TPB, 0, s>>>(g, b, l, x, lay, list, cnt, redo, err);
+      k_wls_redo<T><<<sm_count(), TPB, 0, s>>>(g, b, l, x, lay, cnt, redo, err);
       rmt_count_launches(1);
     }
   }
@@ -514,10 +855,10 @@ void launch_corrector(const Geo& g, const Body& b, const int* bb_in, int blocks,
   k_corr<T><<<blocks, TPB, 0, s>>>(g, bb_in, x, lay, xn, layn, xh);
   rmt_count_launches(1);
   for (int l = 1; l <= g.layers; l++) {
-    k_wls_half<T, false><<<wls_blocks, TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, list, cnt, redo, err);
+    k_wls_half<T><<<wls_blocks, TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, list, cnt, redo, err);
     rmt_count_launches(1);
     if (sizeof(T) == 4) {
-      k_wls_half<T, true><<<sm_count(), TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, list, cnt, redo, err);
+      k_wls_half_redo<T><<<sm_count(), TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, cnt, redo, err);
       rmt_count_launches(1);
     }
   }
