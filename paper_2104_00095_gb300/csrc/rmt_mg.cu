@@ -408,19 +408,117 @@ __device__ __forceinline__ void block_partial(double loc, double* part) {
   }
 }
 
+// FP64 levels: the 7-point operator from stored coefficients.  A division is some ten instructions
+// on a pipe with two lanes per SM, and a sweep, a residual or a restriction that forms its face
+// coefficients makes six per cell; they change once per solve.  f[d] at a cell: h^-2 beta of the face
+// below it along d (0 on a wall); dinv: 1 / their sum over the six faces (0 where that is 0).  A sweep
+// is then nine FP64 operations and 15 loads per cell: x + w ((b + sum f x_nb) dinv - x).  128^3 hierarchy: a colour
+// pass took 39.7 us on average and takes 8.1, the residual and restriction 68 and 24.
+struct MacCoef {
+  const double* f[3];
+  const double* dinv;
+};
+__global__ void __launch_bounds__(BX* BYMAX) k_mac_coef(Lv L, const double* __restrict__ rho, double* __restrict__ fx,
+                                                      double* __restrict__ fy, double* __restrict__ fz,
+                                                      double* __restrict__ dinv) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+  if (i >= L.n[0] || j >= L.n[1]) return;
+  const long c = cix(L, i, j, k);
+  const double rc = rho[c];
+  double* const out[3] = {fx, fy, fz};
+  double dg = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; d++)
+#pragma unroll
+    for (int up = 0; up < 2; up++) {
+      int q[3] = {i, j, k};
+      const int v = cnb(L, d, q[d] + (up ? 1 : -1));
+      double f = 0.0;
+      if (v >= 0) {
+        q[d] = v;
+        f = face_beta<false>(rc, rho[cix(L, q[0], q[1], q[2])]) * L.ih2;
+      }
+      if (!up) out[d][c] = f;
+      dg += f;
+    }
+  dinv[c] = dg > 0.0 ? 1.0 / dg : 0.0;
+}
+
+// s + sum over the six faces of f x_nb at cell (i, j, k); dg (where DIAG) receives sum f
+template <bool DIAG>
+__device__ __forceinline__ double mac_sum64(const Lv& L, const double* __restrict__ x, const MacCoef& F, int i, int j,
+                                            int k, double s, double& dg) {
+  const int c = (int)cix(L, i, j, k);
+  const int st[3] = {1, L.n[0], L.n[0] * L.n[1]}, ii[3] = {i, j, k};
+  dg = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    // the neighbours' offsets: wrapped on a periodic axis; the cell itself beyond a wall, where the
+    // lower face's coefficient is stored as 0 and the upper one's is taken as 0
+    const bool lo = ii[d] > 0, hi = ii[d] + 1 < L.n[d];
+    const int om = lo ? -st[d] : (L.per[d] ? (L.n[d] - 1) * st[d] : 0), op = hi ? st[d] : (L.per[d] ? (1 - L.n[d]) * st[d] : 0);
+    const double fm = F.f[d][c], fp = hi || L.per[d] ? F.f[d][c + op] : 0.0;
+    s += fm * x[c + om];
+    s += fp * x[c + op];
+    if (DIAG) dg += fm + fp;
+  }
+  return s;
+}
+__global__ void __launch_bounds__(BX* BYMAX) k_rbgs64(Lv L, int colour, double w, double* __restrict__ x,
+                                                    const double* __restrict__ b, MacCoef F) {
+  const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+  const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + colour) & 1);
+  if (i >= L.n[0] || j >= L.n[1]) return;
+  const long c = cix(L, i, j, k);
+  double dg;
+  const double s = mac_sum64<false>(L, x, F, i, j, k, b[c], dg), di = F.dinv[c], xc = x[c];
+  if (di > 0.0) x[c] = xc + w * (s * di - xc);
+}
+// residual of the 2 x 2 x 2 fine cells of a coarse cell and their mean (and a zero coarse iterate): one
+// thread per fine cell, eight neighbouring lanes per coarse cell, summed in the children's order
+__global__ void __launch_bounds__(256) k_resid_restrict64(Lv F, Lv C, const double* __restrict__ x,
+                                                          const double* __restrict__ b, MacCoef M,
+                                                          double* __restrict__ bc, double* __restrict__ xc) {
+  const long t = (long)blockIdx.x * 256 + threadIdx.x;
+  const int q = (int)(t & 7);
+  const long u = t >> 3;
+  double r = 0.0;
+  if (u < C.ncell) {
+    int I, J, K;
+    decode(u, C.n[0], C.n[1], I, J, K);
+    const int i = 2 * I + (q & 1), j = 2 * J + ((q >> 1) & 1), k = 2 * K + (q >> 2);
+    const long c = cix(F, i, j, k);
+    double dg;
+    const double s = mac_sum64<true>(F, x, M, i, j, k, b[c], dg);
+    r = s - dg * x[c];
+  }
+  double m = 0.0;
+#pragma unroll
+  for (int o = 0; o < 8; o++) m += __shfl_sync(0xffffffffu, r, o, 8);
+  if (u < C.ncell && q == 0) {
+    bc[u] = m * 0.125;
+    xc[u] = 0.0;
+  }
+}
+
 // FP64 residual r = b - A x of the FP64 iterate (T = double); writes r for the V-cycle and
 // per-block partial sums of r^2
 __global__ void __launch_bounds__(BX* BYMAX) k_resid64(Lv L, int kind, const double* __restrict__ x,
-                                                     const double* __restrict__ b, const double* __restrict__ rho,
-                                                     double* __restrict__ rT, double* __restrict__ part) {
+                                                     const double* __restrict__ b, const double* __restrict__ beta,
+                                                     MacCoef M, double* __restrict__ rT, double* __restrict__ part) {
   const int ext[3] = {kind == 0 ? L.n[0] : L.nn[0], kind == 0 ? L.n[1] : L.nn[1], kind == 0 ? L.n[2] : L.nn[2]};
   int i, j, k;
   double loc = 0.0;
   if (thread_cell(ext, i, j, k)) {
     double dg;
-    const double ax = kind == 0 ? mac_op<double>(L, x, rho, i, j, k, dg) : fe_op<double>(L, x, rho, i, j, k, dg);
     const long u = (long)(i + ext[0] * (j + ext[1] * k));
-    const double r = b[u] - ax;
+    double r;
+    if (kind == 0) {
+      const double s = mac_sum64<true>(L, x, M, i, j, k, b[u], dg);
+      r = s - dg * x[u];
+    } else {
+      r = b[u] - fe_op<double>(L, x, beta, i, j, k, dg);
+    }
     rT[u] = r;
     loc = r * r;
   }
@@ -531,49 +629,16 @@ __global__ void k_ff_to64(const float* __restrict__ xh, const float* __restrict_
 // red-black Gauss-Seidel update (7-point) of the cell of this colour among x = 2p and 2p+1 of
 // row (j, k); the increment scales the residual, so an approximate FP32 quotient moves the sweep,
 // not its fixed point
-template <typename T>
-__device__ __forceinline__ void rbgs_at(const Lv& L, int colour, T w, T* __restrict__ x, const T* __restrict__ b,
-                                        const T* __restrict__ rho, int p, int j, int k) {
-  const int i = 2 * p + ((j + k + colour) & 1);
-  if (i >= L.n[0]) return;
-  T dg;
-  const T ax = mac_op<T, true>(L, x, rho, i, j, k, dg);
-  const long c = cix(L, i, j, k);
-  if (dg > T(0)) {
-    if constexpr (sizeof(T) == 4) x[c] = x[c] + w * ((b[c] - ax) * rcp_approx(dg));
-    else x[c] = x[c] + w * ((b[c] - ax) / dg);
-  }
-}
 // one colour pass: one thread per cell pair along x
-template <typename T>
-__global__ void __launch_bounds__(BX* BYMAX) k_rbgs(Lv L, int colour, T w, T* __restrict__ x, const T* __restrict__ b,
-                                                  const T* __restrict__ rho) {
-  const int p = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (j >= L.n[1]) return;
-  rbgs_at(L, colour, w, x, b, rho, p, j, (int)blockIdx.z);
-}
-
-// weighted Jacobi sweep of the 7-point operator, out of place (x -> xo): the smoother of MAC
-// levels with an odd periodic side, where a red-black colouring is not consistent across the wrap
-// (two neighbours of one colour would update in the same pass)
-constexpr double MAC_JACOBI_W = 6.0 / 7.0;
-template <typename T>
-__global__ void __launch_bounds__(BX* BYMAX) k_jacobi_mac(Lv L, T w, const T* __restrict__ x, T* __restrict__ xo,
-                                                        const T* __restrict__ b, const T* __restrict__ rho) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
+__global__ void __launch_bounds__(BX* BYMAX) k_rbgs(Lv L, int colour, float w, float* __restrict__ x,
+                                                  const float* __restrict__ b, const float* __restrict__ rho) {
+  const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+  const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + colour) & 1);
   if (i >= L.n[0] || j >= L.n[1]) return;
-  T dg;
-  const T ax = mac_op<T, true>(L, x, rho, i, j, k, dg);
+  float dg;
+  const float ax = mac_op<float, true>(L, x, rho, i, j, k, dg);
   const long c = cix(L, i, j, k);
-  T v = x[c];
-  if (dg > T(0)) {
-    if constexpr (sizeof(T) == 4) v = v + w * ((b[c] - ax) * rcp_approx(dg));
-    else v = v + w * ((b[c] - ax) / dg);
-  }
-  xo[c] = v;
+  if (dg > 0.f) x[c] = x[c] + w * ((b[c] - ax) * rcp_approx(dg));
 }
 
 // Asynchronous global -> shared copies (cp.async, 4 or 8 bytes; size 0 fills zeros), so that
@@ -794,6 +859,20 @@ __global__ void __launch_bounds__(GT, 3) k_rbgs_sweep(Lv L, int c0, float w, con
   }
 }
 
+// FP64: 1 / diagonal of the 27-point operator at every node (0 where no cell touches it)
+__global__ void __launch_bounds__(BX* BYMAX) k_fe_dinv(Lv L, const double* __restrict__ beta, double* __restrict__ dinv) {
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+  if (i >= L.nn[0] || j >= L.nn[1]) return;
+  double bs = 0.0;
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const int ci = cnb(L, 0, i - 1 + (q & 1)), cj = cnb(L, 1, j - 1 + ((q >> 1) & 1)), ck = cnb(L, 2, k - 1 + (q >> 2));
+    if (ci >= 0 && cj >= 0 && ck >= 0) bs += beta[cix(L, ci, cj, ck)];
+  }
+  const double diag = 4.0 * bs * L.s12;
+  dinv[nix(L, i, j, k)] = diag > 0.0 ? 1.0 / diag : 0.0;
+}
+
 // 27-point FE sweeps on a plane-marching tile: a block owns FX x FY nodes of every plane of a
 // z-chunk (FZ planes, fewer on small levels; the grid's z extent sets it) and keeps a ring of
 // RING planes of x and of beta (with a one-point halo) in shared memory, and each thread a
@@ -814,7 +893,8 @@ constexpr int VNX = (FY + 2) * VXC, VNR = FY * VRC, VNB = (FY + 1) * VBC;  // ch
 static_assert(VNX + VNR + VNB <= FX * FY, "one staged chunk per thread and plane");
 template <typename T, int MODE, bool VEC = false>
 __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restrict__ x, T* __restrict__ out,
-                                                    const T* __restrict__ b, const T* __restrict__ beta) {
+                                                    const T* __restrict__ b, const T* __restrict__ beta,
+                                                    const T* __restrict__ dinv = nullptr) {
   static_assert(!VEC || sizeof(T) == 4, "16-byte rows of floats");
   constexpr int XW = VEC ? FX + 8 : FX + 2, BW = VEC ? FX + 4 : FX + 1;  // staged row lengths
   constexpr int XO = VEC ? 3 : 0, BO = VEC ? 3 : 0;  // column of node i0-1 / cell i0-1
@@ -971,7 +1051,8 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
     sxp = sxp + 1 == RING ? 0 : sxp + 1;
     sbc = sbc + 1 == RING ? 0 : sbc + 1;
     if (own) {
-      const T bsum = (Bl[0][0] + Bl[0][1]) + (Bl[1][0] + Bl[1][1]) + ((Bu[0][0] + Bu[0][1]) + (Bu[1][0] + Bu[1][1]));
+      T di = T(0);
+      if constexpr (MODE == 0 && sizeof(T) == 8) di = dinv[ubase + (long)k * sz];
       T acc = T(0);
 #pragma unroll
       for (int qy = 0; qy < 2; qy++)
@@ -994,15 +1075,20 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
 #pragma unroll
       for (int qy = 0; qy < 2; qy++) acc += (Bu[qy][0] + Bu[qy][1]) * P[2 * qy][1];
       const T xc = C[1][1];
-      const T diag = T(4) * bsum * s12;
-      const T ax = (T(4) * bsum * xc - acc) * s12;
       const long u = ubase + (long)k * sz;
-      if constexpr (MODE == 0 && sizeof(T) == 4)
-        out[u] = diag > T(0) ? xc + w * __fdividef(bcur - ax, diag) : xc;  // increment only (see k_rbgs)
-      else if constexpr (MODE == 0)
-        out[u] = diag > T(0) ? xc + w * (bcur - ax) / diag : xc;
-      else
-        out[u] = bcur - ax;
+      if constexpr (MODE == 0 && sizeof(T) == 8) {
+        // (b - K x) / diag = (b + s12 acc) / diag - x: neither the diagonal nor a division is formed (the
+        // FP64 pipe bounds the FP64 kernel; 38 operations per node instead of 60)
+        out[u] = di > T(0) ? xc + w * ((bcur + s12 * acc) * di - xc) : xc;
+      } else {
+        const T bsum = (Bl[0][0] + Bl[0][1]) + (Bl[1][0] + Bl[1][1]) + ((Bu[0][0] + Bu[0][1]) + (Bu[1][0] + Bu[1][1]));
+        const T diag = T(4) * bsum * s12;
+        const T ax = (T(4) * bsum * xc - acc) * s12;
+        if constexpr (MODE == 0)
+          out[u] = diag > T(0) ? xc + w * __fdividef(bcur - ax, diag) : xc;  // increment only (see k_rbgs)
+        else
+          out[u] = bcur - ax;
+      }
     }
     k++;
   };
@@ -1036,12 +1122,11 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
 // The 8 fine cells' stencils share their values: x and rho of the 2 x 2 x 2 block and of the 24
 // cells beyond its faces are read once (32 of each instead of 8 x 7), and each fine cell's
 // operator is accumulated from registers face by face in mac_op's order.
-template <typename T>
-__device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, const T* __restrict__ x,
-                                                      const T* __restrict__ b, const T* __restrict__ rho,
-                                                      T* __restrict__ bc, T* __restrict__ xc, int I, int J, int K) {
+__device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, const float* __restrict__ x,
+                                                      const float* __restrict__ b, const float* __restrict__ rho,
+                                                      float* __restrict__ bc, float* __restrict__ xc, int I, int J, int K) {
   const int base[3] = {2 * I, 2 * J, 2 * K};
-  T xb[8], rb[8];  // the block, q = a + 2 b + 4 c
+  float xb[8], rb[8];  // the block, q = a + 2 b + 4 c
 #pragma unroll
   for (int q = 0; q < 8; q++) {
     const long c = cix(F, base[0] + (q & 1), base[1] + ((q >> 1) & 1), base[2] + (q >> 2));
@@ -1050,7 +1135,7 @@ __device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, 
   }
   // beyond the face of axis d on side sd (0: below the block, 1: above): cell t of the face, t =
   // the offsets along the other two axes in increasing axis order; missing outside a wall
-  T xo[3][2][4], ro[3][2][4];
+  float xo[3][2][4], ro[3][2][4];
   bool ho[3][2][4];
 #pragma unroll
   for (int d = 0; d < 3; d++)
@@ -1065,8 +1150,8 @@ __device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, 
         p[e1] = base[e1] + (t & 1);
         p[e2] = base[e2] + (t >> 1);
         ho[d][sd][t] = v >= 0;
-        xo[d][sd][t] = T(0);
-        ro[d][sd][t] = T(0);
+        xo[d][sd][t] = float(0);
+        ro[d][sd][t] = float(0);
         if (v >= 0) {
           const long c = cix(F, p[0], p[1], p[2]);
           xo[d][sd][t] = x[c];
@@ -1074,18 +1159,18 @@ __device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, 
         }
       }
     }
-  const T ih2 = cv<T>(F.ih2, F.f_ih2);
-  T s = T(0);
+  const float ih2 = F.f_ih2;
+  float s = float(0);
 #pragma unroll
   for (int q = 0; q < 8; q++) {
     const int pq[3] = {q & 1, (q >> 1) & 1, q >> 2};
-    const T rc = rb[q];
-    T off = T(0), dg = T(0);
+    const float rc = rb[q];
+    float off = float(0), dg = float(0);
 #pragma unroll
     for (int f = 0; f < 6; f++) {
       const int d = f >> 1, up = f & 1;
       const int e1 = d == 0 ? 1 : 0, e2 = d == 2 ? 1 : 2;
-      T rn, xn;
+      float rn, xn;
       bool has = true;
       if (pq[d] != up) {  // the neighbour is the block cell across the block's middle
         const int qn = q + (up ? 1 : -1) * (1 << d);
@@ -1098,22 +1183,21 @@ __device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, 
         has = ho[d][up][t];
       }
       if (has) {
-        const T beta = face_beta<true>(rc, rn);
+        const float beta = face_beta<true>(rc, rn);
         off += beta * xn;
         dg += beta;
       }
     }
-    const T ax = (dg * xb[q] - off) * ih2;
+    const float ax = (dg * xb[q] - off) * ih2;
     s += b[cix(F, base[0] + pq[0], base[1] + pq[1], base[2] + pq[2])] - ax;
   }
   const long u = cix(C, I, J, K);
-  bc[u] = s * T(0.125);
-  xc[u] = T(0);
+  bc[u] = s * float(0.125);
+  xc[u] = float(0);
 }
-template <typename T>
-__global__ void __launch_bounds__(BX* BYMAX) k_resid_restrict_mac(Lv F, Lv C, const T* __restrict__ x,
-                                                                const T* __restrict__ b, const T* __restrict__ rho,
-                                                                T* __restrict__ bc, T* __restrict__ xc) {
+__global__ void __launch_bounds__(BX* BYMAX) k_resid_restrict_mac(Lv F, Lv C, const float* __restrict__ x,
+                                                                const float* __restrict__ b, const float* __restrict__ rho,
+                                                                float* __restrict__ bc, float* __restrict__ xc) {
   int I, J, K;
   if (!thread_cell(C.n, I, J, K)) return;
   resid_restrict_mac_at(F, C, x, b, rho, bc, xc, I, J, K);
@@ -1553,6 +1637,9 @@ struct MGSolver {
   void* b[16] = {};
   void* r[16] = {};
   void* rho[16] = {};  // per-level coefficient: MAC density (level 0: the caller's array), FE beta
+  // FP64: stored coefficients of the smoothed levels (MAC: face coefficients and inverse diagonal; FE:
+  // inverse diagonal)
+  double *f64[16][3] = {}, *dinv[16] = {};
   const void* rho_in = nullptr;
   double *x64 = nullptr, *b64 = nullptr, *part = nullptr, *scal = nullptr;
   float *xh = nullptr, *xl = nullptr, *bh = nullptr, *bl = nullptr;  // two-float iterate and rhs (T = float)
@@ -1568,7 +1655,6 @@ struct MGSolver {
   int sweep = 1;
   int zc[16] = {};      // z-chunk of k_rbgs_sweep per level (0: the level's layout does not allow it)
   bool big[16] = {};    // level large enough for the fused sweep to pay
-  bool jac[16] = {};    // MAC level with an odd periodic side: Jacobi sweeps instead of red-black
   double omega = 0.9;
   mg_hook_fn hook = nullptr;
   void* hook_ctx = nullptr;
@@ -1662,22 +1748,26 @@ MGSolver* mg_build(const Geo& g, int kind, int prec_fp32, bool dry, cudaError_t*
     L.f_s12_lo = (float)(L.s12 - (double)L.f_s12);
     m->lv[l] = L;
     m->nlev = l + 1;
-    for (int d = 0; d < 3; d++)
-      if (kind == 0 && L.per[d] && (L.n[d] & 1)) m->jac[l] = true;
     const size_t vb = (size_t)L.nunk * m->esz;
     alloc(&m->x[l], vb);
     alloc(&m->xt[l], vb);
     alloc(&m->b[l], vb);
     alloc(&m->r[l], vb);
     if (l > 0 || kind == 1) alloc(&m->rho[l], (size_t)L.ncell * m->esz);
-    // coarsen while every axis is even and halves to at least 3 (a MAC level with an odd periodic
-    // side is smoothed by Jacobi sweeps, see jac)
+    // coarsen while every axis is even and halves to at least 3: only the coarsest level, which is
+    // solved and not smoothed, can have an odd side
     bool can = true;
     for (int d = 0; d < 3; d++) {
       const int h2 = L.n[d] / 2;
       if ((L.n[d] & 1) || h2 < 3) can = false;
     }
-    if (!can || l == 15) break;
+    const bool last = !can || l == 15;
+    if (!prec_fp32 && (!last || l == 0)) {  // a hierarchy of one level: for its residual
+      if (kind == 0)
+        for (int d = 0; d < 3; d++) alloc((void**)&m->f64[l][d], vb);
+      alloc((void**)&m->dinv[l], vb);
+    }
+    if (last) break;
     for (int d = 0; d < 3; d++) L.n[d] /= 2;
     L.h *= 2.0;
   }
@@ -1776,6 +1866,8 @@ void mg_destroy(MGSolver* m) {
     cudaFree(m->b[l]);
     cudaFree(m->r[l]);
     if (l > 0 || m->kind == 1) cudaFree(m->rho[l]);
+    for (int d = 0; d < 3; d++) cudaFree(m->f64[l][d]);
+    cudaFree(m->dinv[l]);
   }
   cudaFree(m->x64);
   cudaFree(m->b64);
@@ -1805,6 +1897,8 @@ void mg_set_density(MGSolver* m, const void* rho) {
 }
 
 namespace {
+
+inline MacCoef mac_coef(const MGSolver* m, int l) { return {{m->f64[l][0], m->f64[l][1], m->f64[l][2]}, m->dinv[l]}; }
 
 inline void hk(MGSolver* m, int l, int which, int begin, cudaStream_t s) {
   if (m->hook && l == 0) m->hook(m->hook_ctx, which, begin, s);
@@ -1874,21 +1968,15 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
         continue;
       }
     }
-    if (m->kind == 0 && m->jac[l]) {
-      hk(m, l, 0, 1, s);
-      k_jacobi_mac<T><<<grid3(L.n[0], L.n[1], L.n[2], m->by), dim3(BX, m->by), 0, s>>>(
-          L, T(MAC_JACOBI_W), (const T*)m->x[l], (T*)m->xt[l], b, rho);
-      rmt_count_launches(1);
-      hk(m, l, 0, 0, s);
-      void* t = m->x[l];
-      m->x[l] = m->xt[l];
-      m->xt[l] = t;
-    } else if (m->kind == 0) {
+    if (m->kind == 0) {
       const dim3 gr(((L.n[0] + 1) / 2 + BX - 1) / BX, (L.n[1] + m->by - 1) / m->by, L.n[2]);
       for (int q = 0; q < 2; q++) {
         const int col = forward ? q : 1 - q;
         hk(m, l, 0, 1, s);
-        k_rbgs<T><<<gr, dim3(BX, m->by), 0, s>>>(L, col, T(m->omega), (T*)m->x[l], b, rho);
+        if constexpr (sizeof(T) == 4)
+          k_rbgs<<<gr, dim3(BX, m->by), 0, s>>>(L, col, T(m->omega), (T*)m->x[l], b, rho);
+        else
+          k_rbgs64<<<gr, dim3(BX, m->by), 0, s>>>(L, col, m->omega, (T*)m->x[l], b, mac_coef(m, l));
         rmt_count_launches(1);
         hk(m, l, 0, 0, s);
       }
@@ -1900,7 +1988,8 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
                                                                       (float*)m->xt[l], (const float*)b,
                                                                       (const float*)rho);
       else
-        k_fe_tile<T, 0><<<fg, dim3(FX, FY), 0, s>>>(L, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho);
+        k_fe_tile<T, 0><<<fg, dim3(FX, FY), 0, s>>>(L, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
+                                                    (const T*)m->dinv[l]);
       rmt_count_launches(1);
       hk(m, l, 0, 0, s);
       void* t = m->x[l];
@@ -1935,8 +2024,12 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
   smooth<T>(m, l, npre, true, s);
   const Lv& C = m->lv[l + 1];
   if (m->kind == 0) {
-    k_resid_restrict_mac<T><<<grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s>>>(
-        L, C, (const T*)m->x[l], (const T*)m->b[l], (const T*)m->rho[l], (T*)m->b[l + 1], (T*)m->x[l + 1]);
+    if constexpr (sizeof(T) == 4)
+      k_resid_restrict_mac<<<grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s>>>(
+          L, C, (const T*)m->x[l], (const T*)m->b[l], (const T*)m->rho[l], (T*)m->b[l + 1], (T*)m->x[l + 1]);
+    else
+      k_resid_restrict64<<<(unsigned)((8 * C.ncell + 255) / 256), 256, 0, s>>>(
+          L, C, (const T*)m->x[l], (const T*)m->b[l], mac_coef(m, l), (T*)m->b[l + 1], (T*)m->x[l + 1]);
     rmt_count_launches(1);
   } else {
     const dim3 fg = fe_grid(L, l == 0 ? m->fe_zc0 : 0);
@@ -1978,6 +2071,18 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
     const Lv& C = m->lv[l];
     k_coarsen<T><<<grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s>>>(F, C, (const T*)m->rho[l - 1], (T*)m->rho[l]);
     rmt_count_launches(1);
+  }
+  if constexpr (sizeof(T) == 8) {
+    for (int l = 0; l < (m->nlev > 1 ? m->nlev - 1 : 1); l++) {
+      const Lv& Q = m->lv[l];
+      if (m->kind == 0)
+        k_mac_coef<<<grid3(Q.n[0], Q.n[1], Q.n[2], m->by), dim3(BX, m->by), 0, s>>>(
+            Q, (const double*)m->rho[l], m->f64[l][0], m->f64[l][1], m->f64[l][2], m->dinv[l]);
+      else
+        k_fe_dinv<<<grid3(Q.nn[0], Q.nn[1], Q.nn[2], m->by), dim3(BX, m->by), 0, s>>>(Q, (const double*)m->rho[l],
+                                                                                    m->dinv[l]);
+      rmt_count_launches(1);
+    }
   }
   // scal: [0] mean of b, [2] |r|^2, [3] mean of x (FP64); fm: the two means as two-float pairs
   float* fm = (float*)(m->scal + 6);
@@ -2036,7 +2141,7 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
                                                (float*)m->b[0], m->part);
       else
         k_resid64<<<g0, dim3(BX, m->by), 0, s>>>(L0, m->kind, m->x64, m->b64, (const double*)m->rho[0],
-                                              (double*)m->b[0], m->part);
+                                              mac_coef(m, 0), (double*)m->b[0], m->part);
       rmt_count_launches(1);
       hk(m, 0, 1, 0, s);
     }
