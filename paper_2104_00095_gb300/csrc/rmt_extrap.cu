@@ -94,7 +94,7 @@ __global__ void k_bfs(Geo g, const int* __restrict__ bb, int l, int8_t* __restri
 // when a pivot is not above tolfac * trace(A)/4 (tolfac = 1e-12 in FP64)
 template <typename AT>
 __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
-  AT L[4][4], D[4];
+  AT L[4][4], D[4], iD[4];
   for (int r = 0; r < 4; r++)
     for (int q = 0; q < 4; q++) L[r][q] = AT(0);
   const AT tr = A[0][0] + A[1][1] + A[2][2] + A[3][3];
@@ -104,11 +104,12 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
     for (int j = 0; j < k; j++) s -= L[k][j] * L[k][j] * D[j];
     D[k] = s;
     if (!(s > tol)) return false;
+    iD[k] = AT(1) / s;  // one division per pivot: each is some ten instructions
     L[k][k] = AT(1);
     for (int i = k + 1; i < 4; i++) {
       AT t = A[i][k];
       for (int j = 0; j < k; j++) t -= L[i][j] * L[k][j] * D[j];
-      L[i][k] = t / D[k];
+      L[i][k] = t * iD[k];
     }
   }
   for (int c = 0; c < 3; c++) {
@@ -118,7 +119,7 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
       for (int j = 0; j < i; j++) t -= L[i][j] * y[j];
       y[i] = t;
     }
-    for (int i = 0; i < 4; i++) y[i] /= D[i];
+    for (int i = 0; i < 4; i++) y[i] *= iD[i];
     for (int i = 3; i >= 0; i--) {
       AT t = y[i];
       for (int j = i + 1; j < 4; j++) t -= L[j][i] * X[j][c];
@@ -333,13 +334,45 @@ __device__ int wls_cell_warp(const Geo& g, const Body& b, const T* __restrict__ 
 //  * sums over the lanes are transposed: at every step a lane hands over half of its partial sums,
 //    16 + 8 + 4 + 2 + 1 additions for 22 totals instead of 110, added in the same tree.
 // One warp per cell with 66 multiplications and additions per candidate and fit and a solve by all
-// lanes took 32.2 ms per step of the 128^3 settling mixture in FP64 (20 bodies; 27.4 now) and 1.50 ms
-// per extrapolation of one body on 96^3 (0.78 now).
+// lanes took 136 us per layer and body of the 128^3 settling mixture in FP64, and 1.50 ms per
+// extrapolation of one body on 96^3 (0.66 now); with it a step of the mixture took 5.5 ms longer.
 constexpr int WB = 32;                 // cells of a batch at most
 constexpr int NSUM = 22, NPAD = 23;    // totals of a fit, padded against bank conflicts
+// 1 / sqrt(s), s = 0 .. 12 (the squared lengths of the 5^3 box's offsets)
+__constant__ double INV_SQRT[13] = {0.0,
+                                    1.0,
+                                    0.70710678118654752440,
+                                    0.57735026918962576451,
+                                    0.5,
+                                    0.44721359549995793928,
+                                    0.40824829046386301637,
+                                    0.37796447300922722721,
+                                    0.35355339059327376220,
+                                    0.33333333333333333333,
+                                    0.31622776601683793320,
+                                    0.30151134457776362265,
+                                    0.28867513459481288225};
 template <typename AT>
 struct WlsShared {
   AT v[TPB / 32][WB][NPAD];
+  // per candidate: 2^-sr, and times di, dj, dk; di, dj, dk; 2^-sr / |d| (an integer converted to FP64 per
+  // use would occupy the FP64 pipe)
+  AT k[NQ0][4][32], d[NQ0][3][32], kl[NQ0][32];
+  __device__ void fill() {
+    for (int t = threadIdx.x; t < 32 * NQ0; t += blockDim.x) {
+      const int q = t >> 5, lane = t & 31, w = 2 * RS0 + 1;
+      const int o[3] = {t % w - RS0, (t / w) % w - RS0, t / (w * w) - RS0};
+      const float wt = (float)(64 >> min(abs(o[0]) + abs(o[1]) + abs(o[2]), 6)) * (1.0f / 64.0f);
+      const int s2 = o[0] * o[0] + o[1] * o[1] + o[2] * o[2];
+      k[q][0][lane] = (AT)wt;
+      for (int d3 = 0; d3 < 3; d3++) {
+        k[q][1 + d3][lane] = (AT)(wt * (float)o[d3]);
+        d[q][d3][lane] = (AT)(float)o[d3];
+      }
+      kl[q][lane] = (AT)wt * (AT)INV_SQRT[s2 <= 12 ? s2 : 0];  // past the box's end: unused
+    }
+    __syncthreads();
+  }
 };
 
 // this lane's candidates t = lane + 32 q of the 5^3 box
@@ -473,7 +506,7 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
         for (int s = r; s < 4; s++) a[e++] += w * v[r] * v[s];
 #pragma unroll
       for (int r = 0; r < 4; r++) {
-        const AT wv = (AT)((float)(w * v[r]) * (1.0f / 64.0f));
+        const AT wv = sh.k[q][r][lane];
 #pragma unroll
         for (int d = 0; d < 3; d++) bs[3 * r + d] = fma_any(wv, (AT)cd.v[q][d], bs[3 * r + d]);
       }
@@ -513,8 +546,9 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
                (s1[1 + q][2] + (q == 2 ? hid : AT(0))) * gX[2];
       const AT nv = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
       if (nv > AT(0)) {
+        const AT in = AT(1) / nv;
 #pragma unroll
-        for (int q = 0; q < 3; q++) nrm[q] = v[q] / nv;
+        for (int q = 0; q < 3; q++) nrm[q] = v[q] * in;
       } else {
         ok = 0;
       }
@@ -523,12 +557,6 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
   __syncwarp();  // the totals have been read
   if (le > 2) return ok;
   // the fit weighted by max(0, cos) of the angle to the normal
-  AT kl[NQ0];  // 2^-sr / |d| of this lane's candidates
-#pragma unroll
-  for (int q = 0; q < NQ0; q++) {
-    const int di = sl.d[q][0], dj = sl.d[q][1], dk = sl.d[q][2], s2 = di * di + dj * dj + dk * dk;
-    kl[q] = s2 ? (AT)(64 >> (abs(di) + abs(dj) + abs(dk))) * AT(1.0 / 64.0) / sqrt((AT)s2) : AT(0);
-  }
   for (unsigned m = __ballot_sync(0xffffffffu, ok != 0); m; m &= m - 1) {
     const int src = __ffs(m) - 1;
     const long cc = __shfl_sync(0xffffffffu, c, src);
@@ -545,8 +573,8 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
 #pragma unroll
     for (int q = 0; q < NQ0; q++) {
       if (!(cd.ok >> q & 1u)) continue;
-      const AT di = (AT)(float)sl.d[q][0], dj = (AT)(float)sl.d[q][1], dk = (AT)(float)sl.d[q][2];
-      const AT wt = -(di * n[0] + dj * n[1] + dk * n[2]) * kl[q];
+      const AT di = sh.d[q][0][lane], dj = sh.d[q][1][lane], dk = sh.d[q][2][lane];
+      const AT wt = -(di * n[0] + dj * n[1] + dk * n[2]) * sh.kl[q][lane];
       if (!(wt > AT(0))) continue;
       pos++;
       const AT wv[4] = {wt, wt * di, wt * dj, wt * dk}, v[4] = {AT(1), di, dj, dk};
@@ -577,8 +605,8 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
 }
 
 // Cells per batch for n cells on the launch's warps.  FP64 fits want fuller batches, since the pipe is
-// busy with a few warps an SM: a quarter of the warps (a half: 28.9 ms per step of the 128^3 mixture, a
-// fifth 27.4, a tenth 27.0, but 0.72, 0.78 and 0.92 ms per 96^3 extrapolation).  FP32 fits want the
+// busy with a few warps an SM: a quarter of the warps (a half: 19.3 ms per step of the 128^3 mixture, a
+// quarter 18.9, an eighth 18.7, but 0.62, 0.66 and 0.81 ms per 96^3 extrapolation).  FP32 fits want the
 // warps in flight (batches of at least 1, 2, 4, 8: 7.99, 8.11, 8.22, 8.33 ms per 4 steps at 112^3).
 template <typename AT>
 __device__ __forceinline__ int batch_size(int n, int warps) {
@@ -599,6 +627,8 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, Body
   const int base = layer_base(cnt, l), n = cnt[l];
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int G = batch_size<T>(n, warps);
+  if (n == 0) return;
+  sh.fill();
   const Slots sl = wls_slots(g);
   for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; e0 < n; e0 += warps * G) {
     const long c = lane < G && e0 + lane < n ? list[base + e0 + lane] : -1;
@@ -734,6 +764,8 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g,
   const int lane = threadIdx.x & 31;
   const int base = layer_base(cnt, l), n = cnt[l];
   const int warps = (gridDim.x * blockDim.x) >> 5;
+  if (n == 0) return;
+  sh.fill();
   const Slots sl = wls_slots(g);
   for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; e0 < n; e0 += warps * 32) {
     long c = e0 + lane < n ? list[base + e0 + lane] : -1;
