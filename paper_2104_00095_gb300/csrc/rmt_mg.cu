@@ -385,6 +385,7 @@ __device__ __forceinline__ F2 fe_op_ff(const Lv& L, const float* __restrict__ xh
 // ----------------------------------------------------------------------------- kernels
 template <typename T>
 __global__ void k_zero(T* a, long n) {
+  wait_prior();
   GRID_LOOP(i, n) a[i] = T(0);
 }
 
@@ -421,6 +422,7 @@ struct MacCoef {
 __global__ void __launch_bounds__(BX* BYMAX) k_mac_coef(Lv L, const double* __restrict__ rho, double* __restrict__ fx,
                                                       double* __restrict__ fy, double* __restrict__ fz,
                                                       double* __restrict__ dinv) {
+  wait_prior();
   const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   if (i >= L.n[0] || j >= L.n[1]) return;
   const long c = cix(L, i, j, k);
@@ -466,6 +468,7 @@ __device__ __forceinline__ double mac_sum64(const Lv& L, const double* __restric
 }
 __global__ void __launch_bounds__(BX* BYMAX) k_rbgs64(Lv L, int colour, double w, double* __restrict__ x,
                                                     const double* __restrict__ b, MacCoef F) {
+  wait_prior();
   const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + colour) & 1);
   if (i >= L.n[0] || j >= L.n[1]) return;
@@ -479,6 +482,7 @@ __global__ void __launch_bounds__(BX* BYMAX) k_rbgs64(Lv L, int colour, double w
 __global__ void __launch_bounds__(256) k_resid_restrict64(Lv F, Lv C, const double* __restrict__ x,
                                                           const double* __restrict__ b, MacCoef M,
                                                           double* __restrict__ bc, double* __restrict__ xc) {
+  wait_prior();
   const long t = (long)blockIdx.x * 256 + threadIdx.x;
   const int q = (int)(t & 7);
   const long u = t >> 3;
@@ -506,6 +510,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict64(Lv F, Lv C, const doub
 __global__ void __launch_bounds__(BX* BYMAX) k_resid64(Lv L, int kind, const double* __restrict__ x,
                                                      const double* __restrict__ b, const double* __restrict__ beta,
                                                      MacCoef M, double* __restrict__ rT, double* __restrict__ part) {
+  wait_prior();
   const int ext[3] = {kind == 0 ? L.n[0] : L.nn[0], kind == 0 ? L.n[1] : L.nn[1], kind == 0 ? L.n[2] : L.nn[2]};
   int i, j, k;
   double loc = 0.0;
@@ -544,6 +549,7 @@ __device__ __forceinline__ void block_partial_f(float loc, double* part) {
 __global__ void __launch_bounds__(BX* BYMAX) k_first_resid64(Lv L, int kind, double* __restrict__ b,
                                                            const double* __restrict__ mean, double* __restrict__ rT,
                                                            double* __restrict__ part) {
+  wait_prior();
   const int ext[3] = {kind == 0 ? L.n[0] : L.nn[0], kind == 0 ? L.n[1] : L.nn[1], kind == 0 ? L.n[2] : L.nn[2]};
   int i, j, k;
   double loc = 0.0;
@@ -565,6 +571,7 @@ __global__ void __launch_bounds__(BX* BYMAX) k_first_resid_ff(Lv L, int kind, fl
                                                             float* __restrict__ bl, const float* __restrict__ mean,
                                                             float* __restrict__ rT, double* __restrict__ part,
                                                             int once, float* __restrict__ x) {
+  wait_prior();
   const int ext[3] = {kind == 0 ? L.n[0] : L.nn[0], kind == 0 ? L.n[1] : L.nn[1], kind == 0 ? L.n[2] : L.nn[2]};
   int i, j, k;
   float loc = 0.0f;
@@ -591,6 +598,7 @@ __global__ void __launch_bounds__(BX* BYMAX) k_resid_ff(Lv L, int kind, const fl
                                                       const float* __restrict__ xl, const float* __restrict__ bh,
                                                       const float* __restrict__ bl, const float* __restrict__ rho,
                                                       float* __restrict__ rT, double* __restrict__ part) {
+  wait_prior();
   const int ext[3] = {kind == 0 ? L.n[0] : L.nn[0], kind == 0 ? L.n[1] : L.nn[1], kind == 0 ? L.n[2] : L.nn[2]};
   int i, j, k;
   float loc = 0.0f;
@@ -608,6 +616,7 @@ __global__ void __launch_bounds__(BX* BYMAX) k_resid_ff(Lv L, int kind, const fl
 // two-float iterate update (xh + xl) += e; set: (xh, xl) = (e, 0)
 __global__ void k_add_ff(const float* __restrict__ e, float* __restrict__ xh, float* __restrict__ xl, long n,
                          int set) {
+  wait_prior();
   GRID_LOOP(i, n) {
     if (set) {
       xh[i] = e[i];
@@ -623,6 +632,7 @@ __global__ void k_add_ff(const float* __restrict__ e, float* __restrict__ xh, fl
 
 // FP64 value of a two-float array (read-back only)
 __global__ void k_ff_to64(const float* __restrict__ xh, const float* __restrict__ xl, double* __restrict__ x, long n) {
+  wait_prior();
   GRID_LOOP(i, n) x[i] = (double)xh[i] + (double)xl[i];
 }
 
@@ -632,6 +642,7 @@ __global__ void k_ff_to64(const float* __restrict__ xh, const float* __restrict_
 // one colour pass: one thread per cell pair along x
 __global__ void __launch_bounds__(BX* BYMAX) k_rbgs(Lv L, int colour, float w, float* __restrict__ x,
                                                   const float* __restrict__ b, const float* __restrict__ rho) {
+  wait_prior();
   const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + colour) & 1);
   if (i >= L.n[0] || j >= L.n[1]) return;
@@ -715,6 +726,7 @@ template <bool WALLS>
 __global__ void __launch_bounds__(GT, 3) k_rbgs_sweep(Lv L, int c0, float w, const float* __restrict__ xin,
                                                       float* __restrict__ xout, const float* __restrict__ b,
                                                       const float* __restrict__ rho, int zc) {
+  wait_prior();
   extern __shared__ float4 sweep_sm4[];
   float* const sm = reinterpret_cast<float*>(sweep_sm4);  // all shared reads index this base
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
@@ -861,6 +873,7 @@ __global__ void __launch_bounds__(GT, 3) k_rbgs_sweep(Lv L, int c0, float w, con
 
 // FP64: 1 / diagonal of the 27-point operator at every node (0 where no cell touches it)
 __global__ void __launch_bounds__(BX* BYMAX) k_fe_dinv(Lv L, const double* __restrict__ beta, double* __restrict__ dinv) {
+  wait_prior();
   const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   if (i >= L.nn[0] || j >= L.nn[1]) return;
   double bs = 0.0;
@@ -894,7 +907,8 @@ static_assert(VNX + VNR + VNB <= FX * FY, "one staged chunk per thread and plane
 template <typename T, int MODE, bool VEC = false>
 __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restrict__ x, T* __restrict__ out,
                                                     const T* __restrict__ b, const T* __restrict__ beta,
-                                                    const T* __restrict__ dinv = nullptr) {
+                                                    const T* __restrict__ dinv) {
+  wait_prior();
   static_assert(!VEC || sizeof(T) == 4, "16-byte rows of floats");
   constexpr int XW = VEC ? FX + 8 : FX + 2, BW = VEC ? FX + 4 : FX + 1;  // staged row lengths
   constexpr int XO = VEC ? 3 : 0, BO = VEC ? 3 : 0;  // column of node i0-1 / cell i0-1
@@ -1198,6 +1212,7 @@ __device__ __forceinline__ void resid_restrict_mac_at(const Lv& F, const Lv& C, 
 __global__ void __launch_bounds__(BX* BYMAX) k_resid_restrict_mac(Lv F, Lv C, const float* __restrict__ x,
                                                                 const float* __restrict__ b, const float* __restrict__ rho,
                                                                 float* __restrict__ bc, float* __restrict__ xc) {
+  wait_prior();
   int I, J, K;
   if (!thread_cell(C.n, I, J, K)) return;
   resid_restrict_mac_at(F, C, x, b, rho, bc, xc, I, J, K);
@@ -1214,6 +1229,7 @@ constexpr int RZ = 8;
 template <typename T>
 __global__ void __launch_bounds__(BX* BYMAX) k_restrict(Lv F, Lv C, int kind, const T* __restrict__ rf,
                                                       T* __restrict__ bc, T* __restrict__ xc, int zc) {
+  wait_prior();
   const int ext[3] = {kind == 0 ? C.n[0] : C.nn[0], kind == 0 ? C.n[1] : C.nn[1], kind == 0 ? C.n[2] : C.nn[2]};
   const int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   if (I >= ext[0] || J >= ext[1]) return;
@@ -1294,6 +1310,7 @@ constexpr int PZ = 8;  // coarse planes per thread column
 template <typename T>
 __global__ void __launch_bounds__(BX* BYMAX) k_prolong_mac(Lv F, Lv C, const T* __restrict__ xc, T* __restrict__ xf,
                                                          int zc) {
+  wait_prior();
   const int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   if (I >= C.n[0] || J >= C.n[1]) return;
   const int K0 = blockIdx.z * zc, K1 = min(K0 + zc, C.n[2]);
@@ -1387,6 +1404,7 @@ __device__ __forceinline__ void prolong_fe_at(const Lv& F, const Lv& C, const T*
 }
 template <typename T>
 __global__ void __launch_bounds__(BX* BYMAX) k_prolong_fe(Lv F, Lv C, const T* __restrict__ xc, T* __restrict__ xf) {
+  wait_prior();
   int I, J, K;
   if (!thread_cell(C.nn, I, J, K)) return;
   prolong_fe_at(F, C, xc, xf, I, J, K);
@@ -1395,12 +1413,14 @@ __global__ void __launch_bounds__(BX* BYMAX) k_prolong_fe(Lv F, Lv C, const T* _
 // FE coefficient beta = 1/rho per cell (finest level)
 template <typename T>
 __global__ void k_inv(long n, const T* __restrict__ rho, T* __restrict__ beta) {
+  wait_prior();
   GRID_LOOP(i, n) beta[i] = T(1) / rho[i];
 }
 
 // coarse coefficient (MAC: density, FE: beta) = mean of the 8 fine cells
 template <typename T>
 __global__ void __launch_bounds__(BX* BYMAX) k_coarsen(Lv F, Lv C, const T* __restrict__ rf, T* __restrict__ rc) {
+  wait_prior();
   int I, J, K;
   if (!thread_cell(C.n, I, J, K)) return;
   T s = T(0);
@@ -1412,6 +1432,7 @@ __global__ void __launch_bounds__(BX* BYMAX) k_coarsen(Lv F, Lv C, const T* __re
 // sum (mode 0) or sum of squares (mode 1): per-block partials
 template <typename XT>
 __global__ void k_partial(const XT* __restrict__ a, long n, int mode, double* __restrict__ part) {
+  wait_prior();
   __shared__ double sh[TPB / 32];
   double loc = 0.0;
   GRID_LOOP(i, n) {
@@ -1432,8 +1453,9 @@ __global__ void k_partial(const XT* __restrict__ a, long n, int mode, double* __
 // sets *nonfinite (when given): every solve takes the mean of its right-hand side and of its
 // solution, so a NaN or infinity anywhere in the velocity that feeds them is caught here
 __global__ void __launch_bounds__(1024) k_final(const double* __restrict__ part, int np, double scale,
-                                                double* __restrict__ out, float* __restrict__ out_ff = nullptr,
-                                                int* __restrict__ nonfinite = nullptr) {
+                                                double* __restrict__ out, float* __restrict__ out_ff,
+                                                int* __restrict__ nonfinite) {
+  wait_prior();
   __shared__ double sh[1024];
   double loc = 0.0;
   for (int i = threadIdx.x; i < np; i += blockDim.x) loc += part[i];
@@ -1458,6 +1480,7 @@ __global__ void __launch_bounds__(1024) k_final(const double* __restrict__ part,
 // accumulation per thread, FP64 across threads
 __global__ void k_partial_ff(const float* __restrict__ h, const float* __restrict__ l, long n,
                              double* __restrict__ part) {
+  wait_prior();
   __shared__ double sh[TPB / 32];
   float ah = 0.0f, al = 0.0f;
   GRID_LOOP(i, n) {
@@ -1479,6 +1502,7 @@ __global__ void k_partial_ff(const float* __restrict__ h, const float* __restric
 // (h, l) = (e, 0) - m: the two-float solution from a single FP32 solve, mean-free
 __global__ void k_set_ff_sub_mean(const float* __restrict__ e, float* __restrict__ h, float* __restrict__ l, long n,
                                   const float* __restrict__ m) {
+  wait_prior();
   GRID_LOOP(i, n) {
     float a = e[i], b = 0.0f;
     ff_sub_pair(a, b, m);
@@ -1488,6 +1512,7 @@ __global__ void k_set_ff_sub_mean(const float* __restrict__ e, float* __restrict
 }
 
 __global__ void k_ff_sub_mean(float* __restrict__ h, float* __restrict__ l, long n, const float* __restrict__ m) {
+  wait_prior();
   GRID_LOOP(i, n) {
     float a = h[i], b = l[i];
     ff_sub_pair(a, b, m);
@@ -1498,6 +1523,7 @@ __global__ void k_ff_sub_mean(float* __restrict__ h, float* __restrict__ l, long
 
 template <typename XT>
 __global__ void k_sub_scalar(XT* __restrict__ a, long n, const double* __restrict__ s) {
+  wait_prior();
   const double v = *s;
   GRID_LOOP(i, n) a[i] = (XT)((double)a[i] - v);
 }
@@ -1505,6 +1531,7 @@ __global__ void k_sub_scalar(XT* __restrict__ a, long n, const double* __restric
 // b += a (set: b = a)
 template <typename T>
 __global__ void k_add_to64(const T* __restrict__ a, double* __restrict__ b, long n, int set) {
+  wait_prior();
   GRID_LOOP(i, n) b[i] = set ? (double)a[i] : b[i] + (double)a[i];
 }
 
@@ -1605,6 +1632,7 @@ __global__ void __launch_bounds__(COARSE_TPB) k_coarse_cg(Lv L, int kind, int ma
                                                          T* __restrict__ gp, T* __restrict__ gb,
                                                          T* __restrict__ gq, const T* __restrict__ grho,
                                                          int in_smem) {
+  wait_prior();
   __shared__ double red[COARSE_TPB / 32];
   extern __shared__ unsigned char smem[];
   const long n = L.nunk;
@@ -1886,7 +1914,7 @@ MGVec mg_solution(MGSolver* m) { return m->fp32 ? MGVec{nullptr, m->xh, m->xl} :
 const double* mg_solution64(MGSolver* m, cudaStream_t s) {
   if (m->fp32) {
     const long n = m->lv[0].nunk;
-    k_ff_to64<<<nblocks(n), TPB, 0, s>>>(m->xh, m->xl, m->x64, n);
+    launch_after(k_ff_to64, nblocks(n), TPB, 0, s, m->xh, m->xl, m->x64, n);
     rmt_count_launches(1);
   }
   return m->x64;
@@ -1908,9 +1936,9 @@ template <typename T>
 void sum_into(MGSolver* m, const T* a, long n, int mode, double scale, double* out, cudaStream_t s) {
   int nb = nblocks(n);
   if (nb > RED_BLOCKS) nb = RED_BLOCKS;
-  k_partial<T><<<nb, TPB, 0, s>>>(a, n, mode, m->part);
+  launch_after(k_partial<T>, nb, TPB, 0, s, a, n, mode, m->part);
   rmt_count_launches(1);
-  k_final<<<1, 1024, 0, s>>>(m->part, nb, scale, out, nullptr, m->nonfinite);
+  launch_after(k_final, 1, 1024, 0, s, m->part, nb, scale, out, nullptr, m->nonfinite);
   rmt_count_launches(1);
 }
 
@@ -1919,9 +1947,9 @@ void sum_ff(MGSolver* m, const float* h, const float* l, long n, double scale, d
             cudaStream_t s) {
   int nb = nblocks(n);
   if (nb > RED_BLOCKS) nb = RED_BLOCKS;
-  k_partial_ff<<<nb, TPB, 0, s>>>(h, l, n, m->part);
+  launch_after(k_partial_ff, nb, TPB, 0, s, h, l, n, m->part);
   rmt_count_launches(1);
-  k_final<<<1, 1024, 0, s>>>(m->part, nb, scale, out, out_ff, m->nonfinite);
+  launch_after(k_final, 1, 1024, 0, s, m->part, nb, scale, out, out_ff, m->nonfinite);
   rmt_count_launches(1);
 }
 
@@ -1955,10 +1983,10 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
         const dim3 gr((L.n[0] + GX - 1) / GX, (L.n[1] + GY - 1) / GY, (L.n[2] + m->zc[l] - 1) / m->zc[l]);
         hk(m, l, 2, 1, s);
         if (L.per[0] && L.per[1] && L.per[2])
-          k_rbgs_sweep<false><<<gr, GT, SWEEP_SMEM, s>>>(L, forward ? 0 : 1, (float)m->omega, (const float*)m->x[l],
+          launch_after(k_rbgs_sweep<false>, gr, GT, SWEEP_SMEM, s, L, forward ? 0 : 1, (float)m->omega, (const float*)m->x[l],
                                                          (float*)m->xt[l], b, rho, m->zc[l]);
         else
-          k_rbgs_sweep<true><<<gr, GT, SWEEP_SMEM, s>>>(L, forward ? 0 : 1, (float)m->omega, (const float*)m->x[l],
+          launch_after(k_rbgs_sweep<true>, gr, GT, SWEEP_SMEM, s, L, forward ? 0 : 1, (float)m->omega, (const float*)m->x[l],
                                                         (float*)m->xt[l], b, rho, m->zc[l]);
         rmt_count_launches(1);
         hk(m, l, 2, 0, s);
@@ -1974,9 +2002,9 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
         const int col = forward ? q : 1 - q;
         hk(m, l, 0, 1, s);
         if constexpr (sizeof(T) == 4)
-          k_rbgs<<<gr, dim3(BX, m->by), 0, s>>>(L, col, T(m->omega), (T*)m->x[l], b, rho);
+          launch_after(k_rbgs, gr, dim3(BX, m->by), 0, s, L, col, T(m->omega), (T*)m->x[l], b, rho);
         else
-          k_rbgs64<<<gr, dim3(BX, m->by), 0, s>>>(L, col, m->omega, (T*)m->x[l], b, mac_coef(m, l));
+          launch_after(k_rbgs64, gr, dim3(BX, m->by), 0, s, L, col, m->omega, (T*)m->x[l], b, mac_coef(m, l));
         rmt_count_launches(1);
         hk(m, l, 0, 0, s);
       }
@@ -1984,11 +2012,11 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
       hk(m, l, 0, 1, s);
       const dim3 fg = fe_grid(L, l == 0 ? m->fe_zc0 : 0);
       if (fe_vec<T>(L))
-        k_fe_tile<float, 0, true><<<fg, dim3(FX, FY), 0, s>>>(L, (float)m->omega, (const float*)m->x[l],
+        launch_after(k_fe_tile<float, 0, true>, fg, dim3(FX, FY), 0, s, L, (float)m->omega, (const float*)m->x[l],
                                                                       (float*)m->xt[l], (const float*)b,
-                                                                      (const float*)rho);
+                                                                      (const float*)rho, nullptr);
       else
-        k_fe_tile<T, 0><<<fg, dim3(FX, FY), 0, s>>>(L, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
+        launch_after(k_fe_tile<T, 0>, fg, dim3(FX, FY), 0, s, L, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
                                                     (const T*)m->dinv[l]);
       rmt_count_launches(1);
       hk(m, l, 0, 0, s);
@@ -2016,7 +2044,7 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
       return;
     }
     const size_t smem = coarse_smem(L, sizeof(T));  // opted in at creation
-    k_coarse_cg<T><<<1, COARSE_TPB, smem, s>>>(L, m->kind, max_it, tol, (T*)m->x[l], (T*)m->xt[l], (T*)m->b[l],
+    launch_after(k_coarse_cg<T>, 1, COARSE_TPB, smem, s, L, m->kind, max_it, tol, (T*)m->x[l], (T*)m->xt[l], (T*)m->b[l],
                                                (T*)m->r[l], (const T*)m->rho[l], smem > 0);
     return;
   }
@@ -2025,33 +2053,33 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
   const Lv& C = m->lv[l + 1];
   if (m->kind == 0) {
     if constexpr (sizeof(T) == 4)
-      k_resid_restrict_mac<<<grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s>>>(
+      launch_after(k_resid_restrict_mac, grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s, 
           L, C, (const T*)m->x[l], (const T*)m->b[l], (const T*)m->rho[l], (T*)m->b[l + 1], (T*)m->x[l + 1]);
     else
-      k_resid_restrict64<<<(unsigned)((8 * C.ncell + 255) / 256), 256, 0, s>>>(
+      launch_after(k_resid_restrict64, (unsigned)((8 * C.ncell + 255) / 256), 256, 0, s, 
           L, C, (const T*)m->x[l], (const T*)m->b[l], mac_coef(m, l), (T*)m->b[l + 1], (T*)m->x[l + 1]);
     rmt_count_launches(1);
   } else {
     const dim3 fg = fe_grid(L, l == 0 ? m->fe_zc0 : 0);
     if (fe_vec<T>(L))
-      k_fe_tile<float, 1, true><<<fg, dim3(FX, FY), 0, s>>>(L, 0.f, (const float*)m->x[l], (float*)m->r[l],
-                                                                    (const float*)m->b[l], (const float*)m->rho[l]);
+      launch_after(k_fe_tile<float, 1, true>, fg, dim3(FX, FY), 0, s, L, 0.f, (const float*)m->x[l], (float*)m->r[l],
+                                                                    (const float*)m->b[l], (const float*)m->rho[l], nullptr);
     else
-      k_fe_tile<T, 1><<<fg, dim3(FX, FY), 0, s>>>(L, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l],
-                                                         (const T*)m->rho[l]);
+      launch_after(k_fe_tile<T, 1>, fg, dim3(FX, FY), 0, s, L, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l],
+                                                         (const T*)m->rho[l], nullptr);
     rmt_count_launches(1);
     const int zc = column_chunk(C.nnode, RZ);
-    k_restrict<T><<<grid3(C.nn[0], C.nn[1], (C.nn[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s>>>(
+    launch_after(k_restrict<T>, grid3(C.nn[0], C.nn[1], (C.nn[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s, 
         L, C, m->kind, (const T*)m->r[l], (T*)m->b[l + 1], (T*)m->x[l + 1], zc);
     rmt_count_launches(1);
   }
   vcycle<T>(m, l + 1, s);
   if (m->kind == 0) {
     const int zc = column_chunk(C.ncell, PZ);
-    k_prolong_mac<T><<<grid3(C.n[0], C.n[1], (C.n[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s>>>(
+    launch_after(k_prolong_mac<T>, grid3(C.n[0], C.n[1], (C.n[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s, 
         L, C, (const T*)m->x[l + 1], (T*)m->x[l], zc);
   } else
-    k_prolong_fe<T><<<grid3(C.nn[0], C.nn[1], C.nn[2], m->by), dim3(BX, m->by), 0, s>>>(L, C, (const T*)m->x[l + 1],
+    launch_after(k_prolong_fe<T>, grid3(C.nn[0], C.nn[1], C.nn[2], m->by), dim3(BX, m->by), 0, s, L, C, (const T*)m->x[l + 1],
                                                                                         (T*)m->x[l]);
   rmt_count_launches(1);
   smooth<T>(m, l, npost, false, s);
@@ -2063,23 +2091,23 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
   const long n = L0.nunk;
   // coefficients of every level
   if (m->kind == 1) {
-    k_inv<T><<<nblocks(L0.ncell), TPB, 0, s>>>(L0.ncell, (const T*)m->rho_in, (T*)m->rho[0]);
+    launch_after(k_inv<T>, nblocks(L0.ncell), TPB, 0, s, L0.ncell, (const T*)m->rho_in, (T*)m->rho[0]);
     rmt_count_launches(1);
   }
   for (int l = 1; l < m->nlev; l++) {
     const Lv& F = m->lv[l - 1];
     const Lv& C = m->lv[l];
-    k_coarsen<T><<<grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s>>>(F, C, (const T*)m->rho[l - 1], (T*)m->rho[l]);
+    launch_after(k_coarsen<T>, grid3(C.n[0], C.n[1], C.n[2], m->by), dim3(BX, m->by), 0, s, F, C, (const T*)m->rho[l - 1], (T*)m->rho[l]);
     rmt_count_launches(1);
   }
   if constexpr (sizeof(T) == 8) {
     for (int l = 0; l < (m->nlev > 1 ? m->nlev - 1 : 1); l++) {
       const Lv& Q = m->lv[l];
       if (m->kind == 0)
-        k_mac_coef<<<grid3(Q.n[0], Q.n[1], Q.n[2], m->by), dim3(BX, m->by), 0, s>>>(
+        launch_after(k_mac_coef, grid3(Q.n[0], Q.n[1], Q.n[2], m->by), dim3(BX, m->by), 0, s, 
             Q, (const double*)m->rho[l], m->f64[l][0], m->f64[l][1], m->f64[l][2], m->dinv[l]);
       else
-        k_fe_dinv<<<grid3(Q.nn[0], Q.nn[1], Q.nn[2], m->by), dim3(BX, m->by), 0, s>>>(Q, (const double*)m->rho[l],
+        launch_after(k_fe_dinv, grid3(Q.nn[0], Q.nn[1], Q.nn[2], m->by), dim3(BX, m->by), 0, s, Q, (const double*)m->rho[l],
                                                                                     m->dinv[l]);
       rmt_count_launches(1);
     }
@@ -2106,9 +2134,9 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
     // mean of b here, since the first residual is a full one
     have_x = true;
     if constexpr (ff) {
-      k_ff_sub_mean<<<nblocks(n), TPB, 0, s>>>(m->bh, m->bl, n, fm);
+      launch_after(k_ff_sub_mean, nblocks(n), TPB, 0, s, m->bh, m->bl, n, fm);
     } else {
-      k_sub_scalar<double><<<nblocks(n), TPB, 0, s>>>(m->b64, n, m->scal);
+      launch_after(k_sub_scalar<double>, nblocks(n), TPB, 0, s, m->b64, n, m->scal);
     }
     rmt_count_launches(1);
     if (fixed_cycles <= 0) {
@@ -2128,25 +2156,25 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
     if (!have_x) {
       // the residual of the zero iterate is b itself: remove its mean, no operator
       if constexpr (ff) {
-        k_first_resid_ff<<<g0, dim3(BX, m->by), 0, s>>>(L0, m->kind, m->bh, m->bl, fm, (float*)m->b[0], m->part,
+        launch_after(k_first_resid_ff, g0, dim3(BX, m->by), 0, s, L0, m->kind, m->bh, m->bl, fm, (float*)m->b[0], m->part,
                                                         once ? 1 : 0, (float*)m->x[0]);
         x_zeroed = once;
       } else
-        k_first_resid64<<<g0, dim3(BX, m->by), 0, s>>>(L0, m->kind, m->b64, m->scal, (double*)m->b[0], m->part);
+        launch_after(k_first_resid64, g0, dim3(BX, m->by), 0, s, L0, m->kind, m->b64, m->scal, (double*)m->b[0], m->part);
       rmt_count_launches(1);
     } else {
       hk(m, 0, 1, 1, s);
       if constexpr (ff)
-        k_resid_ff<<<g0, dim3(BX, m->by), 0, s>>>(L0, m->kind, m->xh, m->xl, m->bh, m->bl, (const float*)m->rho[0],
+        launch_after(k_resid_ff, g0, dim3(BX, m->by), 0, s, L0, m->kind, m->xh, m->xl, m->bh, m->bl, (const float*)m->rho[0],
                                                (float*)m->b[0], m->part);
       else
-        k_resid64<<<g0, dim3(BX, m->by), 0, s>>>(L0, m->kind, m->x64, m->b64, (const double*)m->rho[0],
+        launch_after(k_resid64, g0, dim3(BX, m->by), 0, s, L0, m->kind, m->x64, m->b64, (const double*)m->rho[0],
                                               mac_coef(m, 0), (double*)m->b[0], m->part);
       rmt_count_launches(1);
       hk(m, 0, 1, 0, s);
     }
     if (fixed_cycles <= 0) {
-      k_final<<<1, 1024, 0, s>>>(m->part, nbr, 1.0, m->scal + 2, nullptr, m->nonfinite);
+      launch_after(k_final, 1, 1024, 0, s, m->part, nbr, 1.0, m->scal + 2, nullptr, m->nonfinite);
       rmt_count_launches(1);
       cudaMemcpyAsync(m->hpin + 1, m->scal + 2, sizeof(double), cudaMemcpyDeviceToHost, s);
       if ((*err = cudaStreamSynchronize(s)) != cudaSuccess) return -1;
@@ -2164,7 +2192,7 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
       break;
     }
     if (!x_zeroed) {
-      k_zero<T><<<nblocks(n), TPB, 0, s>>>((T*)m->x[0], n);
+      launch_after(k_zero<T>, nblocks(n), TPB, 0, s, (T*)m->x[0], n);
       rmt_count_launches(1);
     }
     x_zeroed = false;
@@ -2179,9 +2207,9 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
       break;
     }
     if constexpr (ff)
-      k_add_ff<<<nblocks(n), TPB, 0, s>>>((const float*)m->x[0], m->xh, m->xl, n, have_x ? 0 : 1);
+      launch_after(k_add_ff, nblocks(n), TPB, 0, s, (const float*)m->x[0], m->xh, m->xl, n, have_x ? 0 : 1);
     else
-      k_add_to64<<<nblocks(n), TPB, 0, s>>>((const double*)m->x[0], m->x64, n, have_x ? 0 : 1);
+      launch_after(k_add_to64<T>, nblocks(n), TPB, 0, s, (const T*)m->x[0], m->x64, n, have_x ? 0 : 1);
     rmt_count_launches(1);
     have_x = true;
     if (fixed_cycles > 0 && cycles >= fixed_cycles) break;
@@ -2189,26 +2217,26 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
   // mean-free solution
   if constexpr (ff) {
     if (!have_x) {
-      k_zero<float><<<nblocks(n), TPB, 0, s>>>(m->xh, n);
-      k_zero<float><<<nblocks(n), TPB, 0, s>>>(m->xl, n);
+      launch_after(k_zero<float>, nblocks(n), TPB, 0, s, m->xh, n);
+      launch_after(k_zero<float>, nblocks(n), TPB, 0, s, m->xl, n);
       rmt_count_launches(2);
     } else if (single) {
       // the same values as setting (x, 0) and removing the two-float mean, in one pass
       sum_ff(m, (const float*)m->x[0], nullptr, n, 1.0 / (double)n, m->scal + 3, fm + 2, s);
-      k_set_ff_sub_mean<<<nblocks(n), TPB, 0, s>>>((const float*)m->x[0], m->xh, m->xl, n, fm + 2);
+      launch_after(k_set_ff_sub_mean, nblocks(n), TPB, 0, s, (const float*)m->x[0], m->xh, m->xl, n, fm + 2);
       rmt_count_launches(1);
     } else {
       sum_ff(m, m->xh, m->xl, n, 1.0 / (double)n, m->scal + 3, fm + 2, s);
-      k_ff_sub_mean<<<nblocks(n), TPB, 0, s>>>(m->xh, m->xl, n, fm + 2);
+      launch_after(k_ff_sub_mean, nblocks(n), TPB, 0, s, m->xh, m->xl, n, fm + 2);
       rmt_count_launches(1);
     }
   } else {
     if (!have_x) {
-      k_zero<double><<<nblocks(n), TPB, 0, s>>>(m->x64, n);
+      launch_after(k_zero<double>, nblocks(n), TPB, 0, s, m->x64, n);
       rmt_count_launches(1);
     } else {
       sum_into<double>(m, m->x64, n, 0, 1.0 / (double)n, m->scal + 3, s);
-      k_sub_scalar<double><<<nblocks(n), TPB, 0, s>>>(m->x64, n, m->scal + 3);
+      launch_after(k_sub_scalar<double>, nblocks(n), TPB, 0, s, m->x64, n, m->scal + 3);
       rmt_count_launches(1);
     }
   }

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
     k_coarse_solve(Lv L, int cs, int mplanes, int max_it, float tol,
                                                               double tol64, T* __restrict__ gx,
                                                               const T* __restrict__ gb, const T* __restrict__ grho) {
+  wait_prior();
   namespace cg = cooperative_groups;
   constexpr bool F64 = sizeof(T) == 8;
   extern __shared__ __align__(16) unsigned char coarse_sm[];
@@ -387,16 +388,18 @@ template <typename T>
 cudaError_t launch_coarse_solve(const CoarseCfg& c, int kind, const Lv& L, int max_it, double tol, T* x, const T* b,
                                 const T* rho, cudaStream_t s) {
   cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   lc.gridDim = dim3(c.cs);
   lc.blockDim = dim3(c.tpb);
   lc.dynamicSmemBytes = c.smem;
   lc.stream = s;
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = c.cs;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = c.cs;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   lc.attrs = at;
-  lc.numAttrs = c.cs > 1 ? 1 : 0;
+  lc.numAttrs = c.cs > 1 ? 2 : 1;
   Lv Lk = L;
   int cs = c.cs, mplanes = c.mcap / c.ps, mi = max_it;
   // FP64: an FP32 pass of 3e-4, three of which reach 1e-10
