@@ -92,7 +92,7 @@ struct rmt_grid {
   std::vector<BodyMem> bm;
   Body* bodies_d = nullptr;
   int* bb_all = nullptr;  // band boxes: body m, parity p at 12 m + 6 p
-  int *slist = nullptr, *scount = nullptr;  // cells some band reaches (stress pass 2)
+  StressList slist = {};                    // cells some band reaches (stress passes 2 and 3)
   double* t_d = nullptr;                      // simulated time (device copy of t)
   std::vector<cudaStream_t> body_s;           // one stream per body (re-extrapolation, corrector)
   std::vector<cudaEvent_t> ev_join;
@@ -457,8 +457,10 @@ rmt_status alloc_t(rmt_grid* g) {
     if (e == 4) AL(b.redo, N * sizeof(int));
   }
   AL(g->bb_all, (nb > 0 ? nb : 1) * 12 * sizeof(int));
-  AL(g->slist, (nb > 0 ? N : 1) * sizeof(int));
-  AL(g->scount, 16);
+  AL(g->slist.cell, (nb > 0 ? N : 1) * sizeof(int));
+  AL(g->slist.mask, (nb > 0 ? N : 1) * sizeof(uint64_t));
+  AL(g->slist.listed, nb > 0 ? N : 1);
+  AL(g->slist.count, 16);
   AL(g->t_d, 16);
   for (int m = 0; m < nb; m++) g->bm[m].bb = g->bb_all + 12 * m;
   AL(g->bodies_d, (nb > 0 ? nb : 1) * sizeof(Body));
@@ -575,7 +577,7 @@ rmt_status step_t(rmt_grid* g) {
   // 1. tau^n and its divergence
   pb(g, P_STRESS_N);
   CK(g, launch_stress_div<T>(G, u, g->bodies_d, views<T>(g, cur, 0), nb, g->bb_all + 6 * cur, 12, g->t_d, 0.0,
-                              (T*)g->divn, g->slist, g->scount, slopes, s));
+                              (T*)g->divn, g->slist, slopes, s));
   pe(g, P_STRESS_N);
   // 2. Godunov face states of u (transverse bar states first)
   pb(g, P_GODUNOV);
@@ -648,7 +650,7 @@ rmt_status step_t(rmt_grid* g) {
   // 8. tau^{n+1/2}; 9. rho^{n+1/2}; 10. u*
   pb(g, P_STRESS_H);
   CK(g, launch_stress_div<T>(G, u, g->bodies_d, views<T>(g, cur, 1), nb, g->bb_all + 6 * nxt, 12, g->t_d,
-                              0.5 * G.dt, (T*)g->divh, g->slist, g->scount, slopes, s));
+                              0.5 * G.dt, (T*)g->divh, g->slist, slopes, s));
   pe(g, P_STRESS_H);
   pb(g, P_USTAR);
   launch_density<T>(G, g->bodies_d, views<T>(g, cur, 1), nb, g->bb_all + 6 * nxt, 12, (T*)g->rho_h, s);

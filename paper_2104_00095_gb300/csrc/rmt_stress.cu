@@ -13,14 +13,6 @@
 
 namespace {
 
-constexpr int TPB = 256;
-
-inline int nblocks(long n) {
-  long b = (n + TPB - 1) / TPB;
-  if (b > (long)sm_count() * 64) b = (long)sm_count() * 64;  // grid-stride beyond 64 blocks per SM
-  return (int)(b < 1 ? 1 : b);
-}
-
 // ---------------------------------------------------------------------------------
 // stress: face-normal row of the blended deviatoric stress, then its divergence
 
@@ -36,10 +28,11 @@ __device__ __forceinline__ bool xget(const Geo& g, const BodyView<T>& v, int i, 
 }
 
 // Row tau . e_d at the d-face below cell (i,j,k) (cell a = (i,j,k) - e_d, b = (i,j,k)).
-// bmask: bodies that may have xi at a or b.
-template <typename T>
-__device__ __noinline__ void face_row(const Geo& g, const T* __restrict__ u, const Body* __restrict__ bodies,
-                         const BodyView<T>* __restrict__ views, uint64_t bmask, int d, int i, int j, int k,
+// bmask: bodies that may have xi at a or b.  The direction is a template argument: a runtime one indexes
+// every small array through local memory.
+template <typename T, int d>
+__device__ __forceinline__ void face_row(const Geo& g, const T* __restrict__ u, const Body* __restrict__ bodies,
+                         const BodyView<T>* __restrict__ views, uint64_t bmask, int i, int j, int k,
                          T tt, T row[3]) {
   const T ih = cv<T>(g.ih, g.f.ih);
   int ia[3] = {i, j, k};
@@ -157,29 +150,20 @@ __device__ __noinline__ void face_row(const Geo& g, const T* __restrict__ u, con
   for (int a = 0; a < 3; a++) row[a] = Hf * mu * du[a] + acc[a] * sc;
 }
 
-// bodies whose band holds cell (i,j,k): only they can contribute at its six faces
-template <typename T>
-__device__ __forceinline__ uint64_t cell_bodies(const Geo& g, const BodyView<T>* __restrict__ views, int nb,
-                                                const int* sbb, int i, int j, int k, long c) {
-  uint64_t bm = 0;
-  for (int m = 0; m < nb; m++)
-    if (in_box(g, sbb + 6 * m, i, j, k) && views[m].lay[c] >= 0) bm |= (1ull << m);
-  return bm;
-}
-
 // Pass 1, every cell: cells no body reaches take the pure-fluid divergence mu lap(u) here; the
 // others are appended to a list (one atomic per warp and plane) for pass 2.  A block marches
 // over SFZ planes of a TILE_X x TILE_Y column, so the body boxes and the tile's body mask are
 // set up once per column, and keeps u of the planes below and above in registers.  Every
 // neighbour comes from selects (periodic wrap, or the mirrored ghost 2 u_wall - u at a no-slip
-// wall), so no warp takes a separate path at the domain's edges.
+// wall), so no warp takes a separate path at the domain's edges.  The listed cells' body masks go with
+// the list and every cell gets a byte that says whether it is listed, so that the later passes do not
+// search the bodies again.
 constexpr int SFZ = 8;
 template <typename T>
 __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const T* __restrict__ u,
                                                                   const BodyView<T>* __restrict__ views, int nb,
                                                                   const int* __restrict__ bbs, int bstride,
-                                                                  T* __restrict__ out, int* __restrict__ list,
-                                                                  int* __restrict__ count) {
+                                                                  T* __restrict__ out, StressList L) {
   __shared__ int sbb[6 * RMT_MAX_BODIES];
   __shared__ unsigned long long tile_mask;
   stage_boxes(bbs, bstride, nb, sbb);
@@ -248,15 +232,18 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
       const int m = __ffsll((long long)r) - 1;
       if (in_box(g, sbb + 6 * m, i, j, k) && views[m].lay[c] >= 0) bm |= (1ull << m);
     }
+    if (nb > 0) L.listed[c] = bm != 0;
     const unsigned act = __activemask();
     const unsigned want = __ballot_sync(act, bm != 0);
     if (bm != 0) {
       const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
       const int leader = __ffs(want) - 1;
       int base = 0;
-      if (lane == leader) base = atomicAdd(count, __popc(want));
+      if (lane == leader) base = atomicAdd(L.count, __popc(want));
       base = __shfl_sync(want, base, leader);
-      list[base + __popc(want & ((1u << lane) - 1u))] = (int)c;
+      const int at = base + __popc(want & ((1u << lane) - 1u));
+      L.cell[at] = (int)c;
+      L.mask[at] = bm;
     } else {
       // pure fluid around this cell: every face row is mu (u_b - u_a)/h
 #pragma unroll
@@ -282,81 +269,92 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
   }
 }
 
-// Pass 2, the listed cells (a body's band reaches them): the blended face row of each listed
-// cell's three lower faces (the face below the cell along d), one thread per cell, into rows
-// (nine cell arrays, row component a of the d-face at 3d+a).  A face row depends only on the face:
-// a body contributes where it holds both cells of the face, and every such body is in the mask of
-// either cell, so each face is computed once.
+// Pass 2, the listed cells (a body's band reaches them): the blended row of each listed cell's lower face
+// along d = blockIdx.y, and of its upper face where the cell above is not listed, into rows (nine cell
+// arrays, component a of the d-face below a cell at 3d+a; an unlisted cell's slots are free).  A face row
+// depends only on the face: a body contributes where it holds both cells of the face, and every such
+// body is in the mask of either cell, so each face is computed once.  Bound by latency (the chain of a
+// face: band bytes, ten map values, two inverses, a sine), so the three directions are separate threads;
+// one thread per cell, with the upper faces in pass 3 and the bodies searched for every cell and neighbour,
+// made the stress stage 273 us on the 128^3 mixture (154 now), 385 on 256^3 (294) and 65 on 48^3 (46).
 struct Rows9 {
   void* r[9];
 };
-template <typename T>
-__global__ void __launch_bounds__(128) k_stress_rows(Geo g, const T* __restrict__ u, const Body* __restrict__ bodies,
-                                                      const BodyView<T>* __restrict__ views, int nb,
-                                                      const int* __restrict__ bbs, int bstride,
-                                                      const double* __restrict__ t, double toff,
-                                                      const int* __restrict__ list, const int* __restrict__ count,
-                                                      Rows9 R) {
-  __shared__ int sbb[6 * RMT_MAX_BODIES];
-  stage_boxes(bbs, bstride, nb, sbb);
-  const int n = *count;
-  const T tt = (T)(*t + toff);
+template <typename T, int d>
+__device__ __forceinline__ void stress_faces(const Geo& g, const T* __restrict__ u, const Body* __restrict__ bodies,
+                                             const BodyView<T>* __restrict__ views, T tt, const StressList& L,
+                                             const Rows9& R) {
+  const int n = *L.count;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const long c = list[e];
+    const long c = L.cell[e];
+    const uint64_t bm = L.mask[e];
     int i, j, k;
     decode(c, g.n[0], g.n[1], i, j, k);
-    const uint64_t bm = cell_bodies(g, views, nb, sbb, i, j, k, c);
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
+    int up[3] = {i, j, k};
+    up[d] += 1;
+    long cn = -1;
+    const bool above = cell_at(g, up[0], up[1], up[2], cn) && !L.listed[cn];
+    long at = c;
+#pragma unroll 1
+    for (int f = 0; f < 2; f++) {
       T rm[3];
-      face_row(g, u, bodies, views, bm, d, i, j, k, tt, rm);
+      face_row<T, d>(g, u, bodies, views, bm, i, j, k, tt, rm);
 #pragma unroll
-      for (int a = 0; a < 3; a++) ((T*)R.r[3 * d + a])[c] = rm[a];
+      for (int a = 0; a < 3; a++) ((T*)R.r[3 * d + a])[at] = rm[a];
+      if (!above) break;
+      i = up[0];
+      j = up[1];
+      k = up[2];
+      at = cn;
     }
   }
 }
+template <typename T>
+__global__ void __launch_bounds__(128) k_stress_rows(Geo g, const T* __restrict__ u, const Body* __restrict__ bodies,
+                                                      const BodyView<T>* __restrict__ views,
+                                                      const double* __restrict__ t, double toff, StressList L, Rows9 R) {
+  const T tt = (T)(*t + toff);
+  if (blockIdx.y == 0) stress_faces<T, 0>(g, u, bodies, views, tt, L, R);
+  else if (blockIdx.y == 1) stress_faces<T, 1>(g, u, bodies, views, tt, L, R);
+  else stress_faces<T, 2>(g, u, bodies, views, tt, L, R);
+}
 
-// Pass 3, the listed cells: divergence of the face rows.  The upper face along d is the lower
-// face of the neighbour above: its row is read from rows where that neighbour is listed, and
-// computed here otherwise (the band region's outer faces and the faces on a wall).
+// Pass 3, the listed cells: divergence of the face rows.  The upper face along d is the lower face of the
+// neighbour above; a face on a wall has no such cell and is computed here.
+template <typename T, int d>
+__device__ __forceinline__ void stress_div_axis(const Geo& g, const T* __restrict__ u, const Body* __restrict__ bodies,
+                                                const BodyView<T>* __restrict__ views, uint64_t bm, T tt, T ih,
+                                                const Rows9& R, long c, int i, int j, int k, T acc[3]) {
+  int up[3] = {i, j, k};
+  up[d] += 1;
+  T rp[3];
+  long cn;
+  if (cell_at(g, up[0], up[1], up[2], cn)) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) rp[a] = ((const T*)R.r[3 * d + a])[cn];
+  } else {
+    face_row<T, d>(g, u, bodies, views, bm, up[0], up[1], up[2], tt, rp);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; a++) acc[a] += (rp[a] - ((const T*)R.r[3 * d + a])[c]) * ih;
+}
 template <typename T>
 __global__ void __launch_bounds__(128) k_stress_band(Geo g, const T* __restrict__ u, const Body* __restrict__ bodies,
-                                                      const BodyView<T>* __restrict__ views, int nb,
-                                                      const int* __restrict__ bbs, int bstride,
-                                                      const double* __restrict__ t, double toff,
-                                                      const int* __restrict__ list, const int* __restrict__ count,
-                                                      Rows9 R, T* __restrict__ out) {
-  __shared__ int sbb[6 * RMT_MAX_BODIES];
-  stage_boxes(bbs, bstride, nb, sbb);
-  const int n = *count;
+                                                      const BodyView<T>* __restrict__ views,
+                                                      const double* __restrict__ t, double toff, StressList L, Rows9 R,
+                                                      T* __restrict__ out) {
+  const int n = *L.count;
   const T tt = (T)(*t + toff);
   const T ih = cv<T>(g.ih, g.f.ih);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const long c = list[e];
+    const long c = L.cell[e];
+    const uint64_t bm = L.mask[e];
     int i, j, k;
     decode(c, g.n[0], g.n[1], i, j, k);
-    uint64_t bm = 0;
-    bool have_bm = false;
     T acc[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      int ip[3] = {i, j, k};
-      ip[d] += 1;
-      T rp[3];
-      long cn;
-      if (cell_at(g, ip[0], ip[1], ip[2], cn) && cell_bodies(g, views, nb, sbb, ip[0], ip[1], ip[2], cn) != 0) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) rp[a] = ((const T*)R.r[3 * d + a])[cn];
-      } else {
-        if (!have_bm) {
-          bm = cell_bodies(g, views, nb, sbb, i, j, k, c);
-          have_bm = true;
-        }
-        face_row(g, u, bodies, views, bm, d, ip[0], ip[1], ip[2], tt, rp);
-      }
-#pragma unroll
-      for (int a = 0; a < 3; a++) acc[a] += (rp[a] - ((const T*)R.r[3 * d + a])[c]) * ih;
-    }
+    stress_div_axis<T, 0>(g, u, bodies, views, bm, tt, ih, R, c, i, j, k, acc);
+    stress_div_axis<T, 1>(g, u, bodies, views, bm, tt, ih, R, c, i, j, k, acc);
+    stress_div_axis<T, 2>(g, u, bodies, views, bm, tt, ih, R, c, i, j, k, acc);
 #pragma unroll
     for (int a = 0; a < 3; a++) out[a * g.N + c] = acc[a];
   }
@@ -366,29 +364,28 @@ __global__ void __launch_bounds__(128) k_stress_band(Geo g, const T* __restrict_
 
 template <typename T>
 cudaError_t launch_stress_div(const Geo& g, const T* u, const Body* bodies, const BodyView<T>* views, int nb,
-                              const int* bbs, int bstride, const double* t, double toff, T* out, int* list,
-                              int* count, T* const rows[9], cudaStream_t s) {
+                              const int* bbs, int bstride, const double* t, double toff, T* out, const StressList& L,
+                              T* const rows[9], cudaStream_t s) {
   const dim3 gr((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, (g.n[2] + SFZ - 1) / SFZ);
-  const cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
+  const cudaError_t e = cudaMemsetAsync(L.count, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  k_stress_fluid<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, views, nb, bbs, bstride, out, list, count);
+  k_stress_fluid<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, views, nb, bbs, bstride, out, L);
   rmt_count_launches(1);
   if (nb == 0) return cudaSuccess;
   Rows9 R;
   for (int q = 0; q < 9; q++) R.r[q] = rows[q];
-  k_stress_rows<T><<<sm_count() * 8, 128, 0, s>>>(g, u, bodies, views, nb, bbs, bstride, t, toff, list, count, R);
+  k_stress_rows<T><<<dim3(sm_count() * 8, 3), 128, 0, s>>>(g, u, bodies, views, t, toff, L, R);
   rmt_count_launches(1);
-  k_stress_band<T><<<sm_count() * 8, 128, 0, s>>>(g, u, bodies, views, nb, bbs, bstride, t, toff, list, count, R,
-                                                  out);
+  k_stress_band<T><<<sm_count() * 8, 128, 0, s>>>(g, u, bodies, views, t, toff, L, R, out);
   rmt_count_launches(1);
   return cudaSuccess;
 }
 
 template cudaError_t launch_stress_div<float>(const Geo&, const float*, const Body*, const BodyView<float>*, int,
-                                              const int*, int, const double*, double, float*, int*, int*,
+                                              const int*, int, const double*, double, float*, const StressList&,
                                               float* const[9], cudaStream_t);
 template cudaError_t launch_stress_div<double>(const Geo&, const double*, const Body*, const BodyView<double>*, int,
-                                               const int*, int, const double*, double, double*, int*, int*,
+                                               const int*, int, const double*, double, double*, const StressList&,
                                                double* const[9], cudaStream_t);
 
 // simulated time on the device: t += dt after each step (read by the stress kernels, so that a
