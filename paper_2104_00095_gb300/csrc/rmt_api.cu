@@ -38,8 +38,7 @@ struct BodyMem {
   int* bb = nullptr;  // band bounding boxes of the two parities (2 x 6 ints, device)
   int blocks = 1;     // launch width of the body's window kernels
   int* list = nullptr;   // compacted band cells of the current step (capacity N)
-  int* count = nullptr;  // per-layer counts of the list and the redo lists' lengths (device)
-  int* redo = nullptr;   // FP32: cells whose fits are redone in FP64 (device)
+  int* count = nullptr;  // per-layer counts of the list (device)
   void* X[2] = {nullptr, nullptr};
   void* PHI[2] = {nullptr, nullptr};
   int8_t* LAY[2] = {nullptr, nullptr};
@@ -94,10 +93,11 @@ struct rmt_grid {
   int* bb_all = nullptr;  // band boxes: body m, parity p at 12 m + 6 p
   StressList slist = {};                    // cells some band reaches (stress passes 2 and 3)
   double* t_d = nullptr;                      // simulated time (device copy of t)
-  std::vector<cudaStream_t> body_s;           // one stream per body (re-extrapolation, corrector)
-  std::vector<cudaEvent_t> ev_join;
-  cudaEvent_t ev_fork = nullptr;
+  cudaStream_t side_s = nullptr;              // the odd bodies' predictors
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  int win_blocks = 1;                         // launch width of the window kernels of all bodies together
   void* views_d = nullptr;  // BodyView<T>[2 parities][3 levels][nb]
+  void* bands_d = nullptr;  // Band<T>[nb]
   int par = 0;
   void *u = nullptr, *p = nullptr, *rho = nullptr, *rho_h = nullptr, *divn = nullptr, *divh = nullptr;
   void *adv = nullptr, *ustar = nullptr, *psi = nullptr;
@@ -152,8 +152,14 @@ struct rmt_grid {
 
 namespace {
 
-// launch width of the one-warp-per-band-cell fits: 4 resident blocks of 128 threads per SM
-inline int wls_blocks() { return sm_count() * 4; }
+// Launch width per body of the band fits of nb bodies in one launch: 4 blocks of 128 threads per SM for one
+// body, twice that in all for several (their bands are of unequal size; FP64: four times, 2.1 against 2.5 ms for eight
+// bodies in 128^3), at least 64 each
+template <typename T>
+int wls_blocks(int nb) {
+  const int all = sm_count() * (nb > 1 ? (sizeof(T) == 8 ? 16 : 8) : 4), each = all / (nb > 0 ? nb : 1);
+  return each > sm_count() * 4 ? sm_count() * 4 : (each < 64 ? 64 : each);
+}
 
 rmt_status fail(rmt_grid* g, rmt_status st, const char* fmt, ...) {
   if (g) {
@@ -373,7 +379,22 @@ rmt_status build_views(rmt_grid* g) {
       hv[(par * 3 + 1) * nb + m] = {(const T*)b.XH, (const T*)b.PHIH, b.LAY[1 - par]};
       hv[(par * 3 + 2) * nb + m] = {(const T*)b.X[1 - par], (const T*)b.PHI[1 - par], b.LAY[1 - par]};
     }
+  std::vector<Band<T>> ba((size_t)(nb > 0 ? nb : 1));
+  for (int m = 0; m < nb; m++) {
+    BodyMem& b = g->bm[m];
+    for (int q = 0; q < 2; q++) {
+      ba[m].X[q] = (T*)b.X[q];
+      ba[m].PHI[q] = (T*)b.PHI[q];
+      ba[m].LAY[q] = b.LAY[q];
+    }
+    ba[m].XH = (T*)b.XH;
+    ba[m].PHIH = (T*)b.PHIH;
+    ba[m].list = b.list;
+    ba[m].cnt = b.count;
+    ba[m].bb = b.bb;
+  }
   if (nb > 0) {
+    CK(g, cudaMemcpyAsync(g->bands_d, ba.data(), nb * sizeof(Band<T>), cudaMemcpyHostToDevice, g->s));
     CK(g, cudaMemcpyAsync(g->views_d, hv.data(), hv.size() * sizeof(BodyView<T>), cudaMemcpyHostToDevice, g->s));
     CK(g, cudaMemcpyAsync(g->bodies_d, g->bodies.data(), nb * sizeof(Body), cudaMemcpyHostToDevice, g->s));
     CK(g, cudaStreamSynchronize(g->s));
@@ -381,10 +402,30 @@ rmt_status build_views(rmt_grid* g) {
   return RMT_OK;
 }
 
-// launch width of each body's window kernels from its band box (the kernels stride over the
-// whole window, so this only sizes the launch)
+// count bodies from m0 on, with their device arrays; out, in: see BandSet
+template <typename T>
+BandSet<T> band_set(rmt_grid* g, int m0, int count, int out, int in) {
+  BandSet<T> S;
+  memset(&S, 0, sizeof S);
+  S.bodies = g->bodies_d;
+  S.bands = (const Band<T>*)g->bands_d;
+  S.m0 = m0;
+  S.count = count;
+  S.out = out;
+  S.in = in;
+  return S;
+}
+
+// Launch width of the window kernels from the band boxes (the kernels stride over the whole window, so this
+// only sizes the launch): one cell to a thread, and for all bodies together not much more than the chip holds
+// at a time (16 blocks of four warps to an SM): each block reads its body and its band first, which costs more
+// than a cell does.  Eight bodies in 256^3, all passes of a step: 554 us; with a thread to each cell 960 us.
 rmt_status size_windows(rmt_grid* g) {
   const Geo& G = g->g;
+  const long fill = (long)sm_count() * 16;
+  long most = fill / (long)(g->bm.empty() ? 1 : g->bm.size());
+  if (most < 1) most = 1;
+  g->win_blocks = 1;
   for (auto& b : g->bm) {
     int h[6];
     CK(g, cudaMemcpy(h, b.bb, sizeof h, cudaMemcpyDeviceToHost));
@@ -398,6 +439,8 @@ rmt_status size_windows(rmt_grid* g) {
     if (blocks < 1) blocks = 1;
     if (blocks > (long)sm_count() * 64) blocks = (long)sm_count() * 64;
     b.blocks = (int)blocks;
+    if (blocks > most) blocks = most;
+    if ((int)blocks > g->win_blocks) g->win_blocks = (int)blocks;
   }
   return RMT_OK;
 }
@@ -454,7 +497,6 @@ rmt_status alloc_t(rmt_grid* g) {
     b.bb = nullptr;  // set below: all bodies' boxes are contiguous
     AL(b.list, N * sizeof(int));
     AL(b.count, BAND_COUNTERS * sizeof(int));
-    if (e == 4) AL(b.redo, N * sizeof(int));
   }
   AL(g->bb_all, (nb > 0 ? nb : 1) * 12 * sizeof(int));
   AL(g->slist.cell, (nb > 0 ? N : 1) * sizeof(int));
@@ -465,6 +507,7 @@ rmt_status alloc_t(rmt_grid* g) {
   for (int m = 0; m < nb; m++) g->bm[m].bb = g->bb_all + 12 * m;
   AL(g->bodies_d, (nb > 0 ? nb : 1) * sizeof(Body));
   AL(g->views_d, (size_t)6 * (nb > 0 ? nb : 1) * sizeof(BodyView<T>));
+  AL(g->bands_d, (size_t)(nb > 0 ? nb : 1) * sizeof(Band<T>));
   AL(g->err_d, 16);
   long sl = 3 * N;
   for (int d = 0; d < 3; d++)
@@ -517,12 +560,8 @@ rmt_status init_t(rmt_grid* g) {
   rmt_status st = alloc_t<T>(g);
   if (st != RMT_OK) return st;
   CK(g, cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming));
-  g->body_s.assign(nb, nullptr);
-  g->ev_join.assign(nb, nullptr);
-  for (int m = 0; m < nb; m++) {
-    CK(g, cudaStreamCreateWithFlags(&g->body_s[m], cudaStreamNonBlocking));
-    CK(g, cudaEventCreateWithFlags(&g->ev_join[m], cudaEventDisableTiming));
-  }
+  CK(g, cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming));
+  CK(g, cudaStreamCreateWithFlags(&g->side_s, cudaStreamNonBlocking));
   // outside a body's band every per-body array reads "absent" (layer -1, NaN); the window
   // kernels rely on it, since they only ever touch the band's neighbourhood
   const T nanv = (T)NAN;
@@ -538,10 +577,8 @@ rmt_status init_t(rmt_grid* g) {
   // SI "Initialization": u^0 = 0, p = 0, xi^0 = x, extrapolation, phi, rho^0
   const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 64);
   for (int m = 0; m < nb; m++) {
-    BodyMem& b = g->bm[m];
-    launch_init_xi<T>(G, g->bodies[m], (T*)b.X[0], g->s);
-    CK(g, launch_extrapolate<T>(G, g->bodies[m], nullptr, b.bb, full_blocks, b.list, b.count, b.redo, wls_blocks(),
-                                (T*)b.X[0], (T*)b.PHI[0], b.LAY[0], g->err_d, g->s));
+    launch_init_xi<T>(G, g->bodies[m], (T*)g->bm[m].X[0], g->s);
+    launch_extrapolate<T>(G, band_set<T>(g, m, 1, 0, -1), full_blocks, wls_blocks<T>(1), g->err_d, g->s);
   }
   launch_density<T>(G, g->bodies_d, views<T>(g, 0, 0), nb, g->bb_all, 12, (T*)g->rho, g->s);
   CK(g, cudaGetLastError());
@@ -612,7 +649,7 @@ rmt_status step_t(rmt_grid* g) {
   // cell-state arrays (free from the Godunov stage until the half-step stress), so the even
   // bodies run one after another on the step's stream and the odd ones on a second stream
   pb(g, P_XI_PRED);
-  cudaStream_t s2 = nb > 1 ? g->body_s[1] : s;
+  cudaStream_t s2 = nb > 1 ? g->side_s : s;
   if (nb > 1) {
     CK(g, cudaEventRecord(g->ev_fork, s));
     CK(g, cudaStreamWaitEvent(s2, g->ev_fork, 0));
@@ -625,27 +662,14 @@ rmt_status step_t(rmt_grid* g) {
                          odd ? g->xscr_ok2 : g->xscr_ok, (T*)b.X[nxt], odd ? s2 : s);
   }
   if (nb > 1) {
-    CK(g, cudaEventRecord(g->ev_join[1], s2));
-    CK(g, cudaStreamWaitEvent(s, g->ev_join[1], 0));
+    CK(g, cudaEventRecord(g->ev_join, s2));
+    CK(g, cudaStreamWaitEvent(s, g->ev_join, 0));
   }
   pe(g, P_XI_PRED);
-  // 6.-7. re-extrapolation and corrector: the bodies are independent, so each runs on its own
-  // stream, forked from and joined back into the step's stream (parallel branches when the step
-  // is captured as a graph)
+  // 6.-7. re-extrapolation and corrector of all bodies, one launch per pass
   pb(g, P_EXTRAP);
-  if (nb > 0) CK(g, cudaEventRecord(g->ev_fork, s));
-  for (int m = 0; m < nb; m++) {
-    BodyMem& b = g->bm[m];
-    cudaStream_t bs = g->body_s[m];
-    CK(g, cudaStreamWaitEvent(bs, g->ev_fork, 0));
-    const int* bbc = b.bb + 6 * cur;
-    CK(g, launch_extrapolate<T>(G, g->bodies[m], bbc, b.bb + 6 * nxt, b.blocks, b.list, b.count, b.redo, wls_blocks(),
-                                (T*)b.X[nxt], (T*)b.PHI[nxt], b.LAY[nxt], g->err_d, bs));
-    launch_corrector<T>(G, g->bodies[m], bbc, b.blocks, b.list, b.count, b.redo, wls_blocks(), (const T*)b.X[cur], b.LAY[cur],
-                        (const T*)b.X[nxt], b.LAY[nxt], (T*)b.XH, (T*)b.PHIH, g->err_d, bs);
-    CK(g, cudaEventRecord(g->ev_join[m], bs));
-  }
-  for (int m = 0; m < nb; m++) CK(g, cudaStreamWaitEvent(s, g->ev_join[m], 0));
+  if (nb > 0)
+    launch_extrapolate_correct<T>(G, band_set<T>(g, 0, nb, nxt, cur), g->win_blocks, wls_blocks<T>(nb), g->err_d, s);
   pe(g, P_EXTRAP);
   // 8. tau^{n+1/2}; 9. rho^{n+1/2}; 10. u*
   pb(g, P_STRESS_H);
@@ -930,8 +954,7 @@ rmt_status scatter_t(rmt_grid* g, int field, int sid) {
     BodyMem& b = g->bm[sid];
     k_xi_in<T><<<nbk(3 * G.N), 256, 0, s>>>(G, g->bodies[sid], g->stage, (T*)b.X[g->par]); rmt_count_launches(1);
     const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 64);
-    CK(g, launch_extrapolate<T>(G, g->bodies[sid], nullptr, b.bb + 6 * g->par, full_blocks, b.list, b.count, b.redo,
-                                wls_blocks(), (T*)b.X[g->par], (T*)b.PHI[g->par], b.LAY[g->par], g->err_d, s));
+    launch_extrapolate<T>(G, band_set<T>(g, sid, 1, g->par, -1), full_blocks, wls_blocks<T>(1), g->err_d, s);
     launch_density<T>(G, g->bodies_d, views<T>(g, g->par, 0), (int)g->bodies.size(), g->bb_all + 6 * g->par, 12,
                       (T*)g->rho, s);
   }
@@ -1264,10 +1287,8 @@ rmt_status rmt_destroy_grid(rmt_grid* g) {
   else cudaDeviceSynchronize();
   drop_graphs(g);
   if (g->cap_s) cudaStreamDestroy(g->cap_s);
-  for (cudaStream_t b : g->body_s)
-    if (b) cudaStreamDestroy(b);
-  for (cudaEvent_t e : g->ev_join)
-    if (e) cudaEventDestroy(e);
+  if (g->side_s) cudaStreamDestroy(g->side_s);
+  if (g->ev_join) cudaEventDestroy(g->ev_join);
   if (g->ev_fork) cudaEventDestroy(g->ev_fork);
   for (void* p : g->allocs) cudaFree(p);
   if (g->stage_f) cudaFree(g->stage_f);

@@ -475,11 +475,9 @@ __device__ __forceinline__ void win_cell(const Geo& g, const Win& w, long t, int
   u[1] = w.lo[1] + b;
   u[2] = w.lo[2] + cc;
   int v[3];
+  // one wrap is enough: a window starts within dil cells of [0, n) and is at most n long
 #pragma unroll
-  for (int d = 0; d < 3; d++) {
-    v[d] = u[d] % g.n[d];
-    if (v[d] < 0) v[d] += g.n[d];
-  }
+  for (int d = 0; d < 3; d++) v[d] = u[d] < 0 ? u[d] + g.n[d] : (u[d] >= g.n[d] ? u[d] - g.n[d] : u[d]);
   i = v[0];
   j = v[1];
   k = v[2];
@@ -487,6 +485,32 @@ __device__ __forceinline__ void win_cell(const Geo& g, const Win& w, long t, int
 }
 #define WIN_LOOP(t, w) \
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < (w).vol; t += (long)gridDim.x * blockDim.x)
+
+// The window row by row: a warp takes rows of constant (j, k) and its lanes the cells along x, so that a row's
+// index arithmetic (a division, the wraps) is done once per row and not once per cell.  WIN_ROWS(w, row)
+// visits this warp's rows; WinRow(g, w, row) is one; ROW_CELLS(r, a) its cells, r.x(a) the wrapped x.
+struct WinRow {
+  int u1, u2, j, k, base;  // unwrapped and wrapped (y, z), linear index of (0, j, k)
+  int lo0, n0;
+  __device__ __forceinline__ WinRow(const Geo& g, const Win& w, int row) {
+    const int c = row / w.ext[1], b = row - c * w.ext[1];
+    u1 = w.lo[1] + b;
+    u2 = w.lo[2] + c;
+    j = u1 < 0 ? u1 + g.n[1] : (u1 >= g.n[1] ? u1 - g.n[1] : u1);
+    k = u2 < 0 ? u2 + g.n[2] : (u2 >= g.n[2] ? u2 - g.n[2] : u2);
+    base = g.n[0] * (j + g.n[1] * k);
+    lo0 = w.lo[0];
+    n0 = g.n[0];
+  }
+  __device__ __forceinline__ int x(int a) const {
+    const int u = lo0 + a;
+    return u < 0 ? u + n0 : (u >= n0 ? u - n0 : u);
+  }
+};
+#define WIN_ROWS(w, row)                                                                                          \
+  for (int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), row##_end = (w).vol > 0 ? (w).ext[1] * (w).ext[2] : 0; \
+       row < row##_end; row += (int)((gridDim.x * blockDim.x) >> 5))
+#define ROW_CELLS(w, a) for (int a = threadIdx.x & 31; a < (w).ext[0]; a += 32)
 
 // Band boxes of all bodies staged in shared memory (6 ints per body: inclusive min, max; min
 // above max for an empty band), so that a cell reads a body's layer byte only inside its box.

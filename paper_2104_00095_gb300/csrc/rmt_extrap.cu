@@ -41,19 +41,54 @@ __global__ void k_init_xi(Geo g, Body b, T* __restrict__ x) {
   }
 }
 
-// layer 0 = candidates (finite xi) with phi_0(xi) < 0; everything else unmarked
+// All bodies of a step run in one launch per pass (grid row y = body): a body of its own takes 27 launches a
+// step, most of them shorter than a launch, and streams beside each other overlap them only in part.  The
+// passes of one step, with a stream per body and so: 20 bodies in 128^3 879 -> 446 us, 3 in 48^3 170 -> 121 us,
+// 8 in 256^3 717 -> 554 us (FP32).  A block's body and its arrays, staged once:
 template <typename T>
-__global__ void k_classify(Geo g, Body b, const int* __restrict__ bb, const T* __restrict__ x,
-                           int8_t* __restrict__ lay) {
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int u[3], i, j, k;
-    long c;
-    win_cell(g, w, t, u, i, j, k, c);
-    const T x0 = x[c], x1 = x[g.N + c], x2 = x[2 * g.N + c];
-    int8_t l = -1;
-    if (isfinite(x0) && isfinite(x1) && isfinite(x2) && phi_stored(g, b, i, j, k, x0, x1, x2) < T(0)) l = 0;
-    lay[c] = l;
+struct BandCtx {
+  Body b;
+  Band<T> a;
+};
+template <typename T>
+__device__ __forceinline__ void load_ctx(const BandSet<T>& S, BandCtx<T>& c) {
+  const int m = S.m0 + blockIdx.y;
+  const int* bs = reinterpret_cast<const int*>(S.bodies ? S.bodies + m : &S.one);
+  const int* as = reinterpret_cast<const int*>(S.bodies ? S.bands + m : &S.oneb);
+  static_assert(sizeof(Body) % 4 == 0 && sizeof(Band<T>) % 4 == 0, "copied as words");
+  for (int t = threadIdx.x; t < (int)(sizeof(Body) / 4); t += blockDim.x) reinterpret_cast<int*>(&c.b)[t] = bs[t];
+  for (int t = threadIdx.x; t < (int)(sizeof(Band<T>) / 4); t += blockDim.x) reinterpret_cast<int*>(&c.a)[t] = as[t];
+  __syncthreads();
+}
+template <typename T>
+__device__ __forceinline__ Win band_win(const Geo& g, const BandSet<T>& S, const BandCtx<T>& c) {
+  return make_win(g, S.in >= 0 ? c.a.bb + 6 * S.in : nullptr, 2);
+}
+
+// layer 0 = candidates (finite xi) with phi_0(xi) < 0; everything else unmarked; the counters and the new
+// band's box start empty
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_classify(Geo g, const __grid_constant__ BandSet<T> S) {
+  __shared__ BandCtx<T> ctx;
+  load_ctx(S, ctx);
+  const Body& b = ctx.b;
+  const T* __restrict__ x = ctx.a.X[S.out];
+  int8_t* __restrict__ lay = ctx.a.LAY[S.out];
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < BAND_COUNTERS) ctx.a.cnt[threadIdx.x] = 0;
+    if (threadIdx.x < 6) ctx.a.bb[6 * S.out + threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : -0x7fffffff;
+  }
+  const Win w = band_win(g, S, ctx);
+  WIN_ROWS(w, row) {
+    const WinRow r(g, w, row);
+    ROW_CELLS(w, a) {
+      const int i = r.x(a);
+      const long c = r.base + i;
+      const T x0 = x[c], x1 = x[g.N + c], x2 = x[2 * g.N + c];
+      int8_t l = -1;
+      if (isfinite(x0) && isfinite(x1) && isfinite(x2) && phi_stored(g, b, i, r.j, r.k, x0, x1, x2) < T(0)) l = 0;
+      lay[c] = l;
+    }
   }
 }
 
@@ -68,23 +103,47 @@ __device__ __forceinline__ int layer_base(const int* __restrict__ cnt, int l) {
 // unmarked face neighbours of layer l-1 become layer l (walls stop, periodic axes wrap) and are
 // appended to layer l's segment of the band list; in place is race-free: only -1 -> l writes,
 // and only l-1 is tested
-__global__ void k_bfs(Geo g, const int* __restrict__ bb, int l, int8_t* __restrict__ lay, int* __restrict__ list,
-                      int* __restrict__ cnt) {
-  const Win w = make_win(g, bb, 2);
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_bfs(Geo g, const __grid_constant__ BandSet<T> S, int l) {
+  __shared__ BandCtx<T> ctx;
+  load_ctx(S, ctx);
+  int8_t* __restrict__ lay = ctx.a.LAY[S.out];
+  int* __restrict__ list = ctx.a.list;
+  int* __restrict__ cnt = ctx.a.cnt;
+  const Win w = band_win(g, S, ctx);
   const int base = layer_base(cnt, l);
-  WIN_LOOP(t, w) {
-    int u[3], i, j, k;
-    long c;
-    win_cell(g, w, t, u, i, j, k, c);
-    if (lay[c] != -1) continue;
-    const int off[6][3] = {{-1, 0, 0}, {1, 0, 0}, {0, -1, 0}, {0, 1, 0}, {0, 0, -1}, {0, 0, 1}};
-    for (int f = 0; f < 6; f++) {
-      long nb;
-      if (!cell_at(g, i + off[f][0], j + off[f][1], k + off[f][2], nb)) continue;
-      if (lay[nb] == l - 1) {
+  const int lane = threadIdx.x & 31, plane = g.n[0] * g.n[1];
+  WIN_ROWS(w, row) {
+    const WinRow r(g, w, row);
+    // the four neighbouring rows (-1: beyond a wall)
+    const int ym = r.j > 0 ? r.base - g.n[0] : (g.per[1] ? r.base + plane - g.n[0] : -1);
+    const int yp = r.j + 1 < g.n[1] ? r.base + g.n[0] : (g.per[1] ? r.base - plane + g.n[0] : -1);
+    const int zm = r.k > 0 ? r.base - plane : (g.per[2] ? r.base + (g.n[2] - 1) * plane : -1);
+    const int zp = r.k + 1 < g.n[2] ? r.base + plane : (g.per[2] ? r.base - (g.n[2] - 1) * plane : -1);
+    for (int a0 = 0; a0 < w.ext[0]; a0 += 32) {
+      const int a = a0 + lane;
+      bool hit = false;
+      int c = 0;
+      if (a < w.ext[0]) {
+        const int i = r.x(a);
+        c = r.base + i;
+        if (lay[c] == -1) {
+          const int im = i > 0 ? i - 1 : (g.per[0] ? g.n[0] - 1 : -1), ip = i + 1 < g.n[0] ? i + 1 : (g.per[0] ? 0 : -1);
+          const int v0 = im >= 0 ? lay[r.base + im] : -1, v1 = ip >= 0 ? lay[r.base + ip] : -1;
+          const int v2 = ym >= 0 ? lay[ym + i] : -1, v3 = yp >= 0 ? lay[yp + i] : -1;
+          const int v4 = zm >= 0 ? lay[zm + i] : -1, v5 = zp >= 0 ? lay[zp + i] : -1;
+          const int m = l - 1;
+          hit = v0 == m || v1 == m || v2 == m || v3 == m || v4 == m || v5 == m;
+        }
+      }
+      const unsigned want = __ballot_sync(0xffffffffu, hit);
+      if (!want) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&cnt[l], __popc(want));  // one counter update per warp and 32 cells
+      at = base + __shfl_sync(0xffffffffu, at, 0);
+      if (hit) {
         lay[c] = (int8_t)l;
-        list[base + atomicAdd(&cnt[l], 1)] = (int)c;
-        break;
+        list[at + __popc(want & ((1u << lane) - 1u))] = c;
       }
     }
   }
@@ -615,23 +674,39 @@ __device__ __forceinline__ int batch_size(int n, int warps) {
   return g < 1 ? 1 : (g > WB ? WB : g);
 }
 
-// The cells of layer l (its segment of the band list) in the storage type, batch by batch.  FP32 storage:
-// cells whose fits were too ill-conditioned are listed in redo.  FP64 storage: a cell whose radius-2
-// system is degenerate is fitted again by the whole warp with the growing radius.
+// A cell whose batched fit failed, fitted again by the whole warp in FP64 with the growing radius (FP32
+// storage: the system was too ill-conditioned for FP32; rare, so it is kept out of the callers' registers).
+// Returns 1 with the map at the cell in lane 0's out, 0 when degenerate.
 template <typename T>
-__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, Body b, int l, T* __restrict__ x, int8_t* __restrict__ lay,
-                                             const int* __restrict__ list, int* __restrict__ cnt,
-                                             int* __restrict__ redo, int* __restrict__ err) {
+__device__ __noinline__ int wls_again(const Geo& g, const Body& b, const T* x, const int8_t* lay, long c, int l,
+                                      double out[3]) {
+  int i, j, k;
+  decode(c, g.n[0], g.n[1], i, j, k);
+  const int q = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, out);
+  __syncwarp();
+  return q;
+}
+
+// The cells of layer l (its segment of the band list) in the storage type, batch by batch
+template <typename T>
+__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, const __grid_constant__ BandSet<T> S, int l,
+                                                                     int* __restrict__ err) {
   __shared__ WlsShared<T> sh;
+  __shared__ BandCtx<T> ctx;
+  load_ctx(S, ctx);
+  const Body& b = ctx.b;
+  T* x = ctx.a.X[S.out];
+  int8_t* lay = ctx.a.LAY[S.out];
   const int lane = threadIdx.x & 31;
-  const int base = layer_base(cnt, l), n = cnt[l];
+  const int base = layer_base(ctx.a.cnt, l), n = ctx.a.cnt[l];
+  const int* list = ctx.a.list + base;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int G = batch_size<T>(n, warps);
-  if (n == 0) return;
+  if ((int)blockIdx.x * (TPB / 32) * G >= n) return;
   sh.fill();
   const Slots sl = wls_slots(g);
   for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; e0 < n; e0 += warps * G) {
-    const long c = lane < G && e0 + lane < n ? list[base + e0 + lane] : -1;
+    const long c = lane < G && e0 + lane < n ? list[e0 + lane] : -1;
     T out[3];
     const int r = wls_batch<T>(g, b, sl, sh, x, lay, c, l, out);
     if (c >= 0 && r) {
@@ -639,136 +714,125 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, Body
       x[g.N + c] = out[1];
       x[2 * g.N + c] = out[2];
     }
-    if constexpr (sizeof(T) == 4) {
-      if (c >= 0 && !r) redo[atomicAdd(&cnt[0], 1)] = (int)c;
-    } else {
-      for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
-        const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
-        int i, j, k;
-        decode(cc, g.n[0], g.n[1], i, j, k);
-        double o[3];
-        const int q = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, o);
-        __syncwarp();
-        if (lane == 0) {
-          if (q == 1) {
-            x[cc] = (T)o[0];
-            x[g.N + cc] = (T)o[1];
-            x[2 * g.N + cc] = (T)o[2];
-          } else {
-            lay[cc] = -1;
-            atomicAdd(err, 1);
-          }
+    for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
+      const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
+      double o[3];
+      const int q = wls_again(g, b, x, lay, cc, l, o);
+      if (lane == 0) {
+        if (q == 1) {
+          x[cc] = (T)o[0];
+          x[g.N + cc] = (T)o[1];
+          x[2 * g.N + cc] = (T)o[2];
+        } else {
+          lay[cc] = -1;
+          atomicAdd(err, 1);
         }
       }
     }
   }
 }
 
-// FP32 storage: the FP64 pass over the cells of layer l that k_wls listed, one warp per cell
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_wls_redo(Geo g, Body b, int l, T* __restrict__ x, int8_t* __restrict__ lay,
-                                                  const int* __restrict__ cnt, const int* __restrict__ redo,
-                                                  int* __restrict__ err) {
-  const int lane = threadIdx.x & 31, n = cnt[0];
-  for (int e = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5); e < n; e += (gridDim.x * blockDim.x) >> 5) {
-    const long c = redo[e];
-    if (lay[c] != l) continue;  // listed by an earlier layer's pass
-    int i, j, k;
-    decode(c, g.n[0], g.n[1], i, j, k);
-    double out[3];
-    const int r = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, out);
-    __syncwarp();
-    if (lane == 0) {
-      if (r == 1) {
-        x[c] = (T)out[0];
-        x[g.N + c] = (T)out[1];
-        x[2 * g.N + c] = (T)out[2];
+// The end of the extrapolation: phi of the band cells, NaN elsewhere, the band's box (reduced per warp and
+// block before it reaches the six global words; shifted so that its minimum lies in [0, n) on a periodic axis
+// by the last block); FP32 storage: band cells near the seam of the body's image window are counted in *seam.
+// CORR: the corrector xi^{n+1/2} = (xi^n + xi^{n+1})/2 where both exist.
+template <typename T, bool CORR>
+__global__ void __launch_bounds__(TPB) k_finalize(Geo g, const __grid_constant__ BandSet<T> S, int* __restrict__ seam) {
+  __shared__ BandCtx<T> ctx;
+  __shared__ int box[6];
+  if (threadIdx.x < 6) box[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : -0x7fffffff;
+  load_ctx(S, ctx);
+  const Body& b = ctx.b;
+  T* __restrict__ x = ctx.a.X[S.out];
+  T* __restrict__ phi = ctx.a.PHI[S.out];
+  const int8_t* __restrict__ lay = ctx.a.LAY[S.out];
+  const T* __restrict__ xo = ctx.a.X[CORR ? S.in : 0];
+  const int8_t* __restrict__ layo = ctx.a.LAY[CORR ? S.in : 0];
+  T* __restrict__ xh = ctx.a.XH;
+  const T nanv = T(__longlong_as_double(0x7ff8000000000000ll));
+  int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+  const Win w = band_win(g, S, ctx);
+  WIN_ROWS(w, row) {
+    const WinRow r(g, w, row);
+    ROW_CELLS(w, a) {
+      const int i = r.x(a);
+      const long c = r.base + i;
+      if (lay[c] >= 0) {
+        lo[0] = min(lo[0], w.lo[0] + a);
+        hi[0] = max(hi[0], w.lo[0] + a);
+        lo[1] = min(lo[1], r.u1);
+        hi[1] = max(hi[1], r.u1);
+        lo[2] = min(lo[2], r.u2);
+        hi[2] = max(hi[2], r.u2);
+        const T x0 = x[c], x1 = x[g.N + c], x2 = x[2 * g.N + c];
+        phi[c] = phi_stored(g, b, i, r.j, r.k, x0, x1, x2);
+        if (disp_storage<T>() && near_seam(g, b, i, r.j, r.k)) atomicAdd(seam, 1);
+        if (CORR) {
+          if (layo[c] >= 0) {
+            xh[c] = T(0.5) * (xo[c] + x0);
+            xh[g.N + c] = T(0.5) * (xo[g.N + c] + x1);
+            xh[2 * g.N + c] = T(0.5) * (xo[2 * g.N + c] + x2);
+          } else {
+            xh[c] = xh[g.N + c] = xh[2 * g.N + c] = nanv;
+          }
+        }
       } else {
-        lay[c] = -1;
-        atomicAdd(err, 1);
+        x[c] = x[g.N + c] = x[2 * g.N + c] = nanv;
+        phi[c] = nanv;
+        if (CORR) xh[c] = xh[g.N + c] = xh[2 * g.N + c] = nanv;
       }
     }
   }
-}
-
-// phi of the band cells, NaN elsewhere, the band's box; FP32 storage: band cells near the seam of
-// the body's image window are counted in *seam
-template <typename T>
-__global__ void k_finalize(Geo g, Body b, const int* __restrict__ bb, T* __restrict__ x, T* __restrict__ phi,
-                           const int8_t* __restrict__ lay, int* __restrict__ bb_out, int* __restrict__ seam) {
-  const T nanv = T(__longlong_as_double(0x7ff8000000000000ll));
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int u[3], i, j, k;
-    long c;
-    win_cell(g, w, t, u, i, j, k, c);
-    if (lay[c] >= 0) {
 #pragma unroll
-      for (int d = 0; d < 3; d++) {
-        atomicMin(&bb_out[d], u[d]);
-        atomicMax(&bb_out[3 + d], u[d]);
-      }
+  for (int d = 0; d < 3; d++) {
+    lo[d] = __reduce_min_sync(0xffffffffu, lo[d]);
+    hi[d] = __reduce_max_sync(0xffffffffu, hi[d]);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&box[d], lo[d]);
+      atomicMax(&box[3 + d], hi[d]);
     }
-    if (lay[c] >= 0) {
-      phi[c] = phi_stored(g, b, i, j, k, x[c], x[g.N + c], x[2 * g.N + c]);
-      if (disp_storage<T>() && near_seam(g, b, i, j, k)) atomicAdd(seam, 1);
-    } else {
-      x[c] = x[g.N + c] = x[2 * g.N + c] = nanv;
-      phi[c] = nanv;
+  }
+  __syncthreads();
+  int* const bb = ctx.a.bb + 6 * S.out;
+  if (threadIdx.x < 3) atomicMin(&bb[threadIdx.x], box[threadIdx.x]);
+  else if (threadIdx.x < 6) atomicMax(&bb[threadIdx.x], box[threadIdx.x]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(&ctx.a.cnt[BAND_TICKET], 1) == (int)gridDim.x - 1) {
+    __threadfence();
+    for (int d = 0; d < 3; d++) {
+      const int l0 = ((volatile int*)bb)[d], h0 = ((volatile int*)bb)[3 + d];
+      if (!g.per[d] || l0 > h0) continue;
+      int q = l0 / g.n[d];
+      if (l0 < 0 && l0 % g.n[d]) q -= 1;
+      bb[d] = l0 - q * g.n[d];
+      bb[3 + d] = h0 - q * g.n[d];
     }
   }
 }
 
-// corrector xi^{n+1/2} = (xi^n + xi^{n+1})/2 where both exist
+// cells new to the band: xi^{n+1/2} by the same WLS from the corrected lower layers (layer l's segment of
+// the new band's list).  Few of a segment's cells are new: a warp looks at 32 of them and fits those in
+// one batch; where a fit stays degenerate xi^{n+1/2} = xi^{n+1}
 template <typename T>
-__global__ void k_corr(Geo g, const int* __restrict__ bb, const T* __restrict__ x, const int8_t* __restrict__ lay,
-                       const T* __restrict__ xn, const int8_t* __restrict__ layn, T* __restrict__ xh) {
-  const T nanv = T(__longlong_as_double(0x7ff8000000000000ll));
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int u[3], i, j, k;
-    long c;
-    win_cell(g, w, t, u, i, j, k, c);
-    if (layn[c] < 0 || lay[c] < 0) {
-      xh[c] = xh[g.N + c] = xh[2 * g.N + c] = nanv;
-      continue;
-    }
-#pragma unroll
-    for (int a = 0; a < 3; a++) xh[a * g.N + c] = T(0.5) * (x[a * g.N + c] + xn[a * g.N + c]);
-  }
-}
-
-// cells new to the band: xi^{n+1/2} by the same WLS from the corrected lower layers (layer l's
-// segment of the new band's list).  Few of a segment's cells are new: a warp looks at 32 of them and
-// fits those in one batch; what fails is treated as in k_wls, with a redo count of its own, cnt[9].
-template <typename T>
-__device__ __forceinline__ void half_result(const Geo& g, long c, int r, const double out[3], const T* __restrict__ xn,
-                                            T* __restrict__ xh, int* __restrict__ err) {
-  if (r == 1) {
-    xh[c] = (T)out[0];
-    xh[g.N + c] = (T)out[1];
-    xh[2 * g.N + c] = (T)out[2];
-  } else {
-    xh[c] = xn[c];
-    xh[g.N + c] = xn[g.N + c];
-    xh[2 * g.N + c] = xn[2 * g.N + c];
-    atomicAdd(err, 1);
-  }
-}
-template <typename T>
-__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g, Body b, int l, const int8_t* __restrict__ lay,
-                                                  const int8_t* __restrict__ layn, const T* __restrict__ xn,
-                                                  T* __restrict__ xh, const int* __restrict__ list,
-                                                  int* __restrict__ cnt, int* __restrict__ redo, int* __restrict__ err) {
+__global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g, const __grid_constant__ BandSet<T> S,
+                                                                          int l, int* __restrict__ err) {
   __shared__ WlsShared<T> sh;
+  __shared__ BandCtx<T> ctx;
+  load_ctx(S, ctx);
+  const Body& b = ctx.b;
+  const int8_t *lay = ctx.a.LAY[S.in], *layn = ctx.a.LAY[S.out];
+  const T* xn = ctx.a.X[S.out];
+  T* xh = ctx.a.XH;
   const int lane = threadIdx.x & 31;
-  const int base = layer_base(cnt, l), n = cnt[l];
+  const int base = layer_base(ctx.a.cnt, l), n = ctx.a.cnt[l];
+  const int* list = ctx.a.list + base;
   const int warps = (gridDim.x * blockDim.x) >> 5;
-  if (n == 0) return;
+  if ((int)blockIdx.x * TPB >= n) return;
   sh.fill();
   const Slots sl = wls_slots(g);
   for (int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; e0 < n; e0 += warps * 32) {
-    long c = e0 + lane < n ? list[base + e0 + lane] : -1;
+    long c = e0 + lane < n ? list[e0 + lane] : -1;
     if (c >= 0 && (layn[c] != l || lay[c] >= 0)) c = -1;
     if (!__any_sync(0xffffffffu, c >= 0)) continue;
     T out[3];
@@ -778,68 +842,42 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g,
       xh[g.N + c] = out[1];
       xh[2 * g.N + c] = out[2];
     }
-    if constexpr (sizeof(T) == 4) {
-      if (c >= 0 && !r) redo[atomicAdd(&cnt[9], 1)] = (int)c;
-    } else {
-      for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
-        const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
-        int i, j, k;
-        decode(cc, g.n[0], g.n[1], i, j, k);
-        double o[3];
-        const int q = wls_cell_warp<double>(g, b, xh, layn, i, j, k, l, o);
-        __syncwarp();
-        if (lane == 0) half_result(g, cc, q, o, xn, xh, err);
+    for (unsigned m = __ballot_sync(0xffffffffu, c >= 0 && !r); m; m &= m - 1) {
+      const long cc = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
+      double o[3];
+      const int q = wls_again(g, b, xh, layn, cc, l, o);
+      if (lane == 0) {
+        if (q == 1) {
+          xh[cc] = (T)o[0];
+          xh[g.N + cc] = (T)o[1];
+          xh[2 * g.N + cc] = (T)o[2];
+        } else {
+          xh[cc] = xn[cc];
+          xh[g.N + cc] = xn[g.N + cc];
+          xh[2 * g.N + cc] = xn[2 * g.N + cc];
+          atomicAdd(err, 1);
+        }
       }
     }
   }
 }
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_wls_half_redo(Geo g, Body b, int l, const int8_t* __restrict__ lay,
-                                                       const int8_t* __restrict__ layn, const T* __restrict__ xn,
-                                                       T* __restrict__ xh, const int* __restrict__ cnt,
-                                                       const int* __restrict__ redo, int* __restrict__ err) {
-  const int lane = threadIdx.x & 31, n = cnt[9];
-  for (int e = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5); e < n; e += (gridDim.x * blockDim.x) >> 5) {
-    const long c = redo[e];
-    if (layn[c] != l || lay[c] >= 0) continue;
-    int i, j, k;
-    decode(c, g.n[0], g.n[1], i, j, k);
-    double out[3];
-    const int r = wls_cell_warp<double>(g, b, xh, layn, i, j, k, l, out);
-    __syncwarp();
-    if (lane == 0) half_result(g, c, r, out, xn, xh, err);
-  }
-}
 
 template <typename T>
-__global__ void k_phi_half(Geo g, Body b, const int* __restrict__ bb, const T* __restrict__ xh,
-                           const int8_t* __restrict__ layn, T* __restrict__ phih) {
+__global__ void __launch_bounds__(TPB) k_phi_half(Geo g, const __grid_constant__ BandSet<T> S) {
+  __shared__ BandCtx<T> ctx;
+  load_ctx(S, ctx);
+  const T* __restrict__ xh = ctx.a.XH;
+  const int8_t* __restrict__ layn = ctx.a.LAY[S.out];
+  T* __restrict__ phih = ctx.a.PHIH;
   const T nanv = T(__longlong_as_double(0x7ff8000000000000ll));
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int u[3], i, j, k;
-    long c;
-    win_cell(g, w, t, u, i, j, k, c);
-    phih[c] = layn[c] >= 0 ? phi_stored(g, b, i, j, k, xh[c], xh[g.N + c], xh[2 * g.N + c]) : nanv;
-  }
-}
-
-// empty bounding box (min above max)
-__global__ void k_bb_reset(int* bb) {
-  if (threadIdx.x == 0) {
-    bb[0] = bb[1] = bb[2] = 0x7fffffff;
-    bb[3] = bb[4] = bb[5] = -0x7fffffff;
-  }
-}
-// shift the box of a periodic axis so that its minimum lies in [0, n)
-__global__ void k_bb_normalise(Geo g, int* bb) {
-  if (threadIdx.x != 0) return;
-  for (int d = 0; d < 3; d++) {
-    if (!g.per[d] || bb[d] > bb[3 + d]) continue;
-    int q = bb[d] / g.n[d];
-    if (bb[d] < 0 && bb[d] % g.n[d]) q -= 1;
-    bb[d] -= q * g.n[d];
-    bb[3 + d] -= q * g.n[d];
+  const Win w = band_win(g, S, ctx);
+  WIN_ROWS(w, row) {
+    const WinRow r(g, w, row);
+    ROW_CELLS(w, a) {
+      const int i = r.x(a);
+      const long c = r.base + i;
+      phih[c] = layn[c] >= 0 ? phi_stored(g, ctx.b, i, r.j, r.k, xh[c], xh[g.N + c], xh[2 * g.N + c]) : nanv;
+    }
   }
 }
 
@@ -850,59 +888,35 @@ void launch_init_xi(const Geo& g, const Body& b, T* x, cudaStream_t s) {
   k_init_xi<T><<<nblocks(g.N), TPB, 0, s>>>(g, b, x); rmt_count_launches(1);
 }
 
-// cnt: BAND_COUNTERS ints (see rmt_kernels.h); redo: FP32 storage, a list of the grid's size
+namespace {
+template <typename T, bool CORR>
+void extrapolate(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err, cudaStream_t s) {
+  const dim3 gw(blocks, S.count), gf(wls_blocks, S.count);
+  k_classify<T><<<gw, TPB, 0, s>>>(g, S);
+  for (int l = 1; l <= g.layers; l++) k_bfs<T><<<gw, TPB, 0, s>>>(g, S, l);
+  for (int l = 1; l <= g.layers; l++) k_wls<T><<<gf, TPB, 0, s>>>(g, S, l, err);
+  k_finalize<T, CORR><<<gw, TPB, 0, s>>>(g, S, err + 1);
+  rmt_count_launches(2 + 2 * g.layers);
+}
+}  // namespace
+
 template <typename T>
-cudaError_t launch_extrapolate(const Geo& g, const Body& b, const int* bb_in, int* bb_out, int blocks, int* list,
-                               int* cnt, int* redo, int wls_blocks, T* x, T* phi, int8_t* lay, int* err,
-                               cudaStream_t s) {
-  const cudaError_t e = cudaMemsetAsync(cnt, 0, BAND_COUNTERS * sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  k_classify<T><<<blocks, TPB, 0, s>>>(g, b, bb_in, x, lay);
-  rmt_count_launches(1);
-  for (int l = 1; l <= g.layers; l++) {
-    k_bfs<<<blocks, TPB, 0, s>>>(g, bb_in, l, lay, list, cnt);
-    rmt_count_launches(1);
-  }
-  for (int l = 1; l <= g.layers; l++) {
-    k_wls<T><<<wls_blocks, TPB, 0, s>>>(g, b, l, x, lay, list, cnt, redo, err);
-    rmt_count_launches(1);
-    if (sizeof(T) == 4) {
-      k_wls_redo<T><<<sm_count(), TPB, 0, s>>>(g, b, l, x, lay, cnt, redo, err);
-      rmt_count_launches(1);
-    }
-  }
-  k_bb_reset<<<1, 32, 0, s>>>(bb_out);
-  rmt_count_launches(1);
-  k_finalize<T><<<blocks, TPB, 0, s>>>(g, b, bb_in, x, phi, lay, bb_out, err + 1);
-  rmt_count_launches(1);
-  k_bb_normalise<<<1, 32, 0, s>>>(g, bb_out);
-  rmt_count_launches(1);
-  return cudaSuccess;
+void launch_extrapolate(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err, cudaStream_t s) {
+  extrapolate<T, false>(g, S, blocks, wls_blocks, err, s);
 }
 
 template <typename T>
-void launch_corrector(const Geo& g, const Body& b, const int* bb_in, int blocks, const int* list, int* cnt, int* redo,
-                      int wls_blocks, const T* x, const int8_t* lay, const T* xn, const int8_t* layn, T* xh, T* phih,
-                      int* err, cudaStream_t s) {
-  k_corr<T><<<blocks, TPB, 0, s>>>(g, bb_in, x, lay, xn, layn, xh);
-  rmt_count_launches(1);
-  for (int l = 1; l <= g.layers; l++) {
-    k_wls_half<T><<<wls_blocks, TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, list, cnt, redo, err);
-    rmt_count_launches(1);
-    if (sizeof(T) == 4) {
-      k_wls_half_redo<T><<<sm_count(), TPB, 0, s>>>(g, b, l, lay, layn, xn, xh, cnt, redo, err);
-      rmt_count_launches(1);
-    }
-  }
-  k_phi_half<T><<<blocks, TPB, 0, s>>>(g, b, bb_in, xh, layn, phih);
-  rmt_count_launches(1);
+void launch_extrapolate_correct(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err,
+                                cudaStream_t s) {
+  extrapolate<T, true>(g, S, blocks, wls_blocks, err, s);
+  for (int l = 1; l <= g.layers; l++) k_wls_half<T><<<dim3(wls_blocks, S.count), TPB, 0, s>>>(g, S, l, err);
+  k_phi_half<T><<<dim3(blocks, S.count), TPB, 0, s>>>(g, S);
+  rmt_count_launches(1 + g.layers);
 }
 
-#define INST(T)                                                                                                \
-  template void launch_init_xi<T>(const Geo&, const Body&, T*, cudaStream_t);                                   \
-  template cudaError_t launch_extrapolate<T>(const Geo&, const Body&, const int*, int*, int, int*, int*, int*, int, \
-                                             T*, T*, int8_t*, int*, cudaStream_t);                              \
-  template void launch_corrector<T>(const Geo&, const Body&, const int*, int, const int*, int*, int*, int,        \
-                                    const T*, const int8_t*, const T*, const int8_t*, T*, T*, int*, cudaStream_t);
+#define INST(T)                                                                                           \
+  template void launch_init_xi<T>(const Geo&, const Body&, T*, cudaStream_t);                              \
+  template void launch_extrapolate<T>(const Geo&, const BandSet<T>&, int, int, int*, cudaStream_t);        \
+  template void launch_extrapolate_correct<T>(const Geo&, const BandSet<T>&, int, int, int*, cudaStream_t);
 INST(float)
 INST(double)

@@ -124,27 +124,40 @@ template <typename T>
 void launch_fill(T* a, T v, long n, cudaStream_t s);
 
 // ---- extrapolation (rmt_extrap.cu) ------------------------------------------------
+// One body's arrays.  list: the band's cells sorted by layer (capacity: the grid), written by the layer
+// passes of launch_extrapolate and read by launch_corrector of the same step; cnt: BAND_COUNTERS ints,
+// cnt[l] the cells of layer l (l = 1..8), cnt[BAND_TICKET] the finished blocks of the last pass; bb: the
+// band's bounding boxes of the two parities (6 ints each)
+constexpr int BAND_COUNTERS = 10, BAND_TICKET = 9;
+template <typename T>
+struct Band {
+  T *X[2], *PHI[2];
+  int8_t* LAY[2];
+  T *XH, *PHIH;
+  int *list, *cnt, *bb;
+};
+// The bodies that a launch works on, one per grid row y: bodies m0, m0 + 1, ... of the device arrays, or
+// (bodies null) the one given here.  out: the parity that is written; in: the parity whose box bounds the
+// windows and whose map the corrector starts from (-1: the windows are the grid)
+template <typename T>
+struct BandSet {
+  const Body* bodies;
+  const Band<T>* bands;
+  int m0, count, out, in;
+  Body one;
+  Band<T> oneb;
+};
 template <typename T>
 void launch_init_xi(const Geo& g, const Body& b, T* x, cudaStream_t s);
-// bb_in: band bounding box of the step (null: whole grid); bb_out receives the new band's box;
-// blocks: launch width for the body's window (kernels stride over the whole window); list: the
-// band's cells sorted by layer (capacity: the grid), written by the layer passes of
-// launch_extrapolate and read by launch_corrector of the same step; cnt: BAND_COUNTERS ints,
-// cnt[l] the cells of layer l (l = 1..8), cnt[0] and cnt[9] the lengths of the FP64 redo lists
-// of the two fitting passes; redo: FP32 storage, a list of the grid's size for the cells whose
-// FP32 fits were too ill-conditioned (null for FP64 storage); wls_blocks: launch width of the
-// one-warp-per-cell fits.
-// err[0] counts degenerate fits, err[1] (FP32 storage) band cells near the seam of the body's
-// image window; returns the error of the one runtime call it makes besides launches
-constexpr int BAND_COUNTERS = 10;
+// blocks: launch width for a body's window (kernels stride over the whole window); wls_blocks: launch
+// width of the fits.  err[0] counts degenerate fits, err[1] (FP32 storage) band cells near the seam of
+// their body's image window
 template <typename T>
-cudaError_t launch_extrapolate(const Geo& g, const Body& b, const int* bb_in, int* bb_out, int blocks, int* list,
-                               int* cnt, int* redo, int wls_blocks, T* x, T* phi, int8_t* lay, int* err,
-                               cudaStream_t s);
+void launch_extrapolate(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err, cudaStream_t s);
+// the same for the map at out, followed by the corrector: xi^{n+1/2} from the maps at in and out
 template <typename T>
-void launch_corrector(const Geo& g, const Body& b, const int* bb_in, int blocks, const int* list, int* cnt, int* redo,
-                      int wls_blocks, const T* x, const int8_t* lay, const T* xn, const int8_t* layn, T* xh, T* phih,
-                      int* err, cudaStream_t s);
+void launch_extrapolate_correct(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err,
+                                cudaStream_t s);
 
 // ---- multigrid (rmt_mg.cu) ----------------------------------------------------------
 struct MGSolver;  // opaque

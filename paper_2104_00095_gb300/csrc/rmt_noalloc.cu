@@ -108,11 +108,20 @@ rmt_status rmt_extrapolate_noalloc(const rmt_grid_desc* d, const rmt_solid_desc*
   if (e != cudaSuccess) return RMT_ECUDA;
   const long wide = (long)sm_count() * 64;
   const int blocks = (int)((G.N + 127) / 128 < wide ? (G.N + 127) / 128 : wide);
-  e = launch_extrapolate<double>(G, b, nullptr, scr + SCR_BB, blocks, scr + SCR_LIST, scr + SCR_COUNT, nullptr,
-                                 sm_count() * 4,
-                                 xi_out, phi_out, (int8_t*)layer_out, scr + SCR_ERR, st);
+  BandSet<double> set;
+  memset(&set, 0, sizeof set);
+  set.count = 1;
+  set.in = -1;
+  set.one = b;
+  set.oneb.X[0] = xi_out;
+  set.oneb.PHI[0] = phi_out;
+  set.oneb.LAY[0] = (int8_t*)layer_out;
+  set.oneb.list = scr + SCR_LIST;
+  set.oneb.cnt = scr + SCR_COUNT;
+  set.oneb.bb = scr + SCR_BB;
+  launch_extrapolate<double>(G, set, blocks, sm_count() * 4, scr + SCR_ERR, st);
   int nbad = 0;
-  if (e == cudaSuccess) e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&nbad, scr + SCR_ERR, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return RMT_ECUDA;

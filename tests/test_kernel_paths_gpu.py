@@ -84,3 +84,35 @@ def test_float_reads_of_every_field(n, periodic, precision):
             ok = ~np.isnan(ref)
             assert np.all(np.abs(v[ok] - ref[ok]) <= (np.spacing(np.abs(ref[ok])) if f in (4, 30) else 0)), f
     g.close()
+
+
+@pytest.mark.parametrize("layers,periodic,precision", [(1, True, "fp64"), (4, False, "fp64"), (8, True, "fp64"),
+                                                       (4, True, "fp32")])
+def test_extrapolation_of_unequal_bodies(layers, periodic, precision):
+    """Bodies of unequal size extrapolated together: one across the seam, a small one, and a needle whose tip is
+    a single line of cells, where the fits of radius 2 and 3 are degenerate and a wider search is taken."""
+    n = (36, 28, 30)
+    sc = _box(n, periodic)
+    at = lambda i, j, k: tuple((v + 0.5) / max(n) for v in (i, j, k))
+    size = lambda *r: tuple(v / max(n) for v in r)
+    turn = S.random_rotation(np.random.default_rng(3))
+    edge = at(1.3, 20.2, 27.9) if periodic else at(8.3, 19.2, 21.9)
+    sc.update(band_layers=layers, precision=precision)
+    sc["solids"] = [S.solid(S.ELLIPSOID, edge, size(6.4, 5.2, 4.3), turn, rho_s=1.4, G=0.2, mu_a=0.02),
+                    S.solid(S.ELLIPSOID, at(18, 8, 8), size(7.6, 1.3, 1.3), rho_s=1.2, G=0.2, mu_a=0.02),
+                    S.solid(S.SPHERE, at(27.6, 19.4, 14.7), size(2.6, 2.6, 2.6), rho_s=1.6, G=0.2, mu_a=0.02)]
+    if precision == "fp32":
+        sc.update(mg_rtol=1e-9, mg_max_cycles=60)
+    g, o = pair(sc)
+    u = 0.1 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    g.write(rmt.RMT_F_U, u)
+    assert o.write(O.F_U, u) == 0
+    g.step(2)
+    assert o.step(2) == 0, o.error()
+    if precision == "fp64":
+        compare_state(g, o, 3, 1e-9)
+    else:
+        for m in range(3):
+            assert np.array_equal(g.read(rmt.RMT_F_LAYER, m), o.read(O.F_LAYER, m))
+            assert rel_l2(g.read(rmt.RMT_F_XI, m), o.read(O.F_XI, m)) <= 1e-5
+    g.close()
