@@ -36,7 +36,6 @@ namespace {
 
 struct BodyMem {
   int* bb = nullptr;  // band bounding boxes of the two parities (2 x 6 ints, device)
-  int blocks = 1;     // launch width of the body's window kernels
   int* list = nullptr;   // compacted band cells of the current step (capacity N)
   int* count = nullptr;  // per-layer counts of the list (device)
   void* X[2] = {nullptr, nullptr};
@@ -93,18 +92,13 @@ struct rmt_grid {
   int* bb_all = nullptr;  // band boxes: body m, parity p at 12 m + 6 p
   StressList slist = {};                    // cells some band reaches (stress passes 2 and 3)
   double* t_d = nullptr;                      // simulated time (device copy of t)
-  cudaStream_t side_s = nullptr;              // the odd bodies' predictors
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int win_blocks = 1;                         // launch width of the window kernels of all bodies together
+  int win_tiles = 1;                          // launch width per body of the predictors
   void* views_d = nullptr;  // BodyView<T>[2 parities][3 levels][nb]
   void* bands_d = nullptr;  // Band<T>[nb]
   int par = 0;
   void *u = nullptr, *p = nullptr, *rho = nullptr, *rho_h = nullptr, *divn = nullptr, *divh = nullptr;
   void *adv = nullptr, *ustar = nullptr, *psi = nullptr;
-  void* xscr_s[9] = {};
-  void* xscr_b[9] = {};
-  int8_t* xscr_ok[3] = {};
-  int8_t* xscr_ok2[3] = {};  // the second predictor scratch set's flags (its arrays: slopes, wcell)
   void* vadv[3] = {};
   void* ub[3][3] = {};
   void* slopes[9] = {};
@@ -426,21 +420,23 @@ rmt_status size_windows(rmt_grid* g) {
   long most = fill / (long)(g->bm.empty() ? 1 : g->bm.size());
   if (most < 1) most = 1;
   g->win_blocks = 1;
+  g->win_tiles = 1;
   for (auto& b : g->bm) {
     int h[6];
     CK(g, cudaMemcpy(h, b.bb, sizeof h, cudaMemcpyDeviceToHost));
-    long vol = 1;
+    long vol = 1, tiles = 1;
     for (int d = 0; d < 3; d++) {
       long e = h[d] <= h[3 + d] ? (long)(h[3 + d] - h[d] + 1) + 8 : 0;
       if (e > G.n[d]) e = G.n[d];
       vol *= e;
+      tiles *= (e + 7) / 8;
     }
     long blocks = (vol + 127) / 128;
     if (blocks < 1) blocks = 1;
-    if (blocks > (long)sm_count() * 64) blocks = (long)sm_count() * 64;
-    b.blocks = (int)blocks;
     if (blocks > most) blocks = most;
     if ((int)blocks > g->win_blocks) g->win_blocks = (int)blocks;
+    if (tiles > most) tiles = most;
+    if ((int)tiles > g->win_tiles) g->win_tiles = (int)tiles;
   }
   return RMT_OK;
 }
@@ -465,15 +461,6 @@ rmt_status alloc_t(rmt_grid* g) {
   AL(g->psi, G.NN * e);
   for (int q = 0; q < 9; q++) AL(g->slopes[q], N * e);
   for (int q = 0; q < 9; q++) AL(g->wcell[q], N * e);
-  if (!g->bodies.empty()) {
-    for (int q = 0; q < 9; q++) {
-      AL(g->xscr_s[q], N * e);
-      AL(g->xscr_b[q], N * e);
-    }
-    for (int q = 0; q < 3; q++) AL(g->xscr_ok[q], N);
-    if (g->bodies.size() > 1)
-      for (int q = 0; q < 3; q++) AL(g->xscr_ok2[q], N);
-  }
   for (int d = 0; d < 3; d++) {
     const long nf = nfaces(G, d);
     for (int a = 0; a < 3; a++) {
@@ -559,9 +546,6 @@ rmt_status init_t(rmt_grid* g) {
   const int nb = (int)g->bodies.size();
   rmt_status st = alloc_t<T>(g);
   if (st != RMT_OK) return st;
-  CK(g, cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming));
-  CK(g, cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming));
-  CK(g, cudaStreamCreateWithFlags(&g->side_s, cudaStreamNonBlocking));
   // outside a body's band every per-body array reads "absent" (layer -1, NaN); the window
   // kernels rely on it, since they only ever touch the band's neighbourhood
   const T nanv = (T)NAN;
@@ -645,26 +629,9 @@ rmt_status step_t(rmt_grid* g) {
   // 4. advective term
   launch_advect<T>(G, uf, umac, (T*)g->adv, s);
   pe(g, P_MAC_CORR_ADV);
-  // 5. predictor of every body.  Two scratch sets: the predictor's own and the Godunov slope and
-  // cell-state arrays (free from the Godunov stage until the half-step stress), so the even
-  // bodies run one after another on the step's stream and the odd ones on a second stream
+  // 5. predictor of every body
   pb(g, P_XI_PRED);
-  cudaStream_t s2 = nb > 1 ? g->side_s : s;
-  if (nb > 1) {
-    CK(g, cudaEventRecord(g->ev_fork, s));
-    CK(g, cudaStreamWaitEvent(s2, g->ev_fork, 0));
-  }
-  for (int m = 0; m < nb; m++) {
-    BodyMem& b = g->bm[m];
-    const bool odd = (m & 1) != 0;
-    launch_xi_predict<T>(G, u, vadv, uf, umac, b.bb + 6 * cur, b.blocks, (const T*)b.X[cur], b.LAY[cur],
-                         odd ? slopes : (T* const*)g->xscr_s, odd ? wcell : (T* const*)g->xscr_b,
-                         odd ? g->xscr_ok2 : g->xscr_ok, (T*)b.X[nxt], odd ? s2 : s);
-  }
-  if (nb > 1) {
-    CK(g, cudaEventRecord(g->ev_join, s2));
-    CK(g, cudaStreamWaitEvent(s, g->ev_join, 0));
-  }
+  if (nb > 0) CK(g, launch_xi_predict<T>(G, u, vadv, uf, umac, band_set<T>(g, 0, nb, nxt, cur), g->win_tiles, s));
   pe(g, P_XI_PRED);
   // 6.-7. re-extrapolation and corrector of all bodies, one launch per pass
   pb(g, P_EXTRAP);
@@ -1287,9 +1254,6 @@ rmt_status rmt_destroy_grid(rmt_grid* g) {
   else cudaDeviceSynchronize();
   drop_graphs(g);
   if (g->cap_s) cudaStreamDestroy(g->cap_s);
-  if (g->side_s) cudaStreamDestroy(g->side_s);
-  if (g->ev_join) cudaEventDestroy(g->ev_join);
-  if (g->ev_fork) cudaEventDestroy(g->ev_fork);
   for (void* p : g->allocs) cudaFree(p);
   if (g->stage_f) cudaFree(g->stage_f);
   if (g->err_h) cudaFreeHost(g->err_h);

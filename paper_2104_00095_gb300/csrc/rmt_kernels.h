@@ -91,12 +91,6 @@ void launch_mac_correct(const Geo& g, T* const uf[3][3], const T* rho, MGVec q, 
                         cudaStream_t s);
 template <typename T>
 void launch_advect(const Geo& g, T* const uf[3][3], T* const umac[3], T* adv, cudaStream_t s);
-// scratch_s, scratch_xb, scratch_ok: N-sized scratch (9 + 9 arrays of T, 3 of int8) reused by
-// every body in turn
-template <typename T>
-void launch_xi_predict(const Geo& g, const T* u, T* const vadv[3], T* const uf[3][3], T* const umac[3],
-                       const int* bb, int blocks, const T* x, const int8_t* lay, T* const scratch_s[9],
-                       T* const scratch_xb[9], int8_t* const scratch_ok[3], T* xn, cudaStream_t s);
 template <typename T>
 void launch_density(const Geo& g, const Body* bodies, const BodyView<T>* views, int nb, const int* bbs, int bstride,
                     T* rho, cudaStream_t s);
@@ -149,6 +143,11 @@ struct BandSet {
 };
 template <typename T>
 void launch_init_xi(const Geo& g, const Body& b, T* x, cudaStream_t s);
+// predictor of every body's map at layers 0 and 1, from the map at in to the map at out; tiles: launch width for
+// a body's tiles (the kernel strides over the whole window)
+template <typename T>
+cudaError_t launch_xi_predict(const Geo& g, const T* u, T* const vadv[3], T* const uf[3][3], T* const umac[3],
+                              const BandSet<T>& S, int tiles, cudaStream_t s);
 // blocks: launch width for a body's window (kernels stride over the whole window); wls_blocks: launch
 // width of the fits.  err[0] counts degenerate fits, err[1] (FP32 storage) band cells near the seam of
 // their body's image window

@@ -1,34 +1,32 @@
 // Predictor of the reference map (arXiv 2104.00095, eq. dis_xi_adv with the Godunov face
-// states of eq. xi_taylor_final and the tangential terms of SI "Tangential derivatives").
-// Three passes over a body's window: limited slopes of xi, transverse bar states on faces,
-// then the predictor at the cells of layers 0 and 1.
+// states of eq. xi_taylor_final and the tangential terms of SI "Tangential derivatives"):
+// limited slopes of xi, transverse bar states on faces, face states, then the predictor at the
+// cells of layers 0 and 1 -- for all bodies in one launch, without scratch.
 //
 // FP32 storage holds S = xi - x0 (rmt_common.cuh).  The slopes are those of xi (the limiter sees
 // differences of xi: h + dS along the component's own axis, dS across it); every face state
 // is stored as the displacement from the face centre's image, so where the FP64 form adds a
 // Taylor term (h/2) s to xi, the FP32 form adds (h/2)(s - 1) for the component along the
 // face's axis, and a difference of face states across a cell gains h on that component.
-#include "rmt_kernels.h"
+//
+// A block takes tiles of 8^3 cells of a body's window and one component of xi (the components
+// meet only in the velocities): it stages the component and the layers with a halo of three
+// cells, and slopes, bar states and face states stay in shared memory, 45 KB (FP64 87 KB).
+// Kept in memory instead, these 21 words per window cell bound the three passes that each
+// body needs, and a body's window leaves most of the chip idle.  The halo repeats about twice
+// the slopes of a full tile; the choice of the upwind side before the state is formed, and a
+// face's state formed once for both its cells, take half of the states away.  All bodies of a step, three
+// passes for each and this: 20 bodies in 128^3 501 -> 170 us (FP64 1333 -> 847 us, bound by its arithmetic),
+// 3 in 48^3 81 -> 31 us, 8 in 256^3 327 -> 230 us.
+#include "rmt_band.cuh"
 
 namespace {
 
-constexpr int TPB = 256;
-
-inline int nblocks(long n) {
-  long b = (n + TPB - 1) / TPB;
-  if (b > (long)sm_count() * 64) b = (long)sm_count() * 64;  // grid-stride beyond 64 blocks per SM
-  return (int)(b < 1 ? 1 : b);
-}
-
-template <typename T>
-__device__ __forceinline__ void cell_faces(const Geo& g, int e, int i, int j, int k, long& lo, long& hi) {
-  lo = fidx(g, e, i, j, k);
-  int ii[3] = {i, j, k};
-  ii[e] += 1;
-  hi = fidx(g, e, ii[0], ii[1], ii[2]);
-}
-// ---------------------------------------------------------------------------------
-// predictor of the reference map at the cells of layers 0 and 1 (eq. dis_xi_adv)
+constexpr int XT = 8;                  // tile width in cells
+constexpr int XL = XT + 6;             // with the halo of the staged map and layers
+constexpr int XR = XT + 2;             // with one cell around: slopes and bar states
+constexpr int XF = (XT + 1) * XT * XT; // faces of one direction
+constexpr int XTPB = 256;
 
 struct XiPredPtrs {
   const void* vadv[3];
@@ -36,249 +34,250 @@ struct XiPredPtrs {
   const void* umac[3];
 };
 
+// Shared arrays of a block: s[e], bar[e] at q = x + 1 + XR (y + 1 + XR (z + 1)) the limited slope along e and the
+// upwinded bar state on the e-face below tile cell (x, y, z); f[d] the state on the d-faces of the tile; x, lay the
+// staged component and layers (-1 beyond a wall).
 template <typename T>
-__device__ __forceinline__ bool xi3(const Geo& g, const T* __restrict__ x, const int8_t* __restrict__ lay, int i,
-                                    int j, int k, T v[3]) {
-  long c;
-  if (!cell_at(g, i, j, k, c) || lay[c] < 0) return false;
-  v[0] = x[c];
-  v[1] = x[g.N + c];
-  v[2] = x[2 * g.N + c];
-  return true;
-}
-
-template <typename T>
-__device__ __forceinline__ void slope_xi(const Geo& g, const T* __restrict__ x, const int8_t* __restrict__ lay, int d,
-                                         int i, int j, int k, T s[3]) {
-  T q[3][5];
-  unsigned ok = 0;
-#pragma unroll
-  for (int t = -2; t <= 2; t++) {
-    int ii[3] = {i, j, k};
-    ii[d] += t;
-    T v[3];
-    if (xi3(g, x, lay, ii[0], ii[1], ii[2], v)) {
-      ok |= 1u << (t + 2);
-      q[0][t + 2] = v[0]; q[1][t + 2] = v[1]; q[2][t + 2] = v[2];
-      // FP32 storage: the identity's part of xi_d along axis d, relative to the centre cell (the
-      // band never pairs cells across the seam of the body's image window)
-      if constexpr (disp_storage<T>()) q[d][t + 2] += T(t) * g.f.h;
-    } else {
-      q[0][t + 2] = q[1][t + 2] = q[2][t + 2] = T(0);
-    }
-  }
-  const T ih = cv<T>(g.ih, g.f.ih);
-#pragma unroll
-  for (int a = 0; a < 3; a++) s[a] = lim_slope(q[a], ok, ih);
-}
-
-// Per-body scratch shared by the three passes (N-sized arrays, reused body after body):
-// s[3d+a] limited slope of xi_a along d at a cell; xb[3e+a] the upwinded bar state of xi_a
-// on the e-face below a cell, ok[e] its availability.
-struct XiScratch {
-  void* s[9];
-  void* xb[9];
-  int8_t* ok[3];
+struct XiTile {
+  T x[XL * XL * XL], s[3][XR * XR * XR], bar[3][XR * XR * XR], f[3][XF];
+  int8_t lay[XL * XL * XL];
 };
+__device__ __forceinline__ int stage_at(int x, int y, int z) { return x + 3 + XL * (y + 3 + XL * (z + 3)); }
+__device__ __forceinline__ int ring_at(int x, int y, int z) { return x + 1 + XR * (y + 1 + XR * (z + 1)); }
+__device__ __forceinline__ int stage_step(int d) { return d == 0 ? 1 : (d == 1 ? XL : XL * XL); }
+__device__ __forceinline__ int ring_step(int d) { return d == 0 ? 1 : (d == 1 ? XR : XR * XR); }
 
-// pass 1: limited slopes of xi at every band cell of the window
+// Taylor state of component a from tile cell v toward its d-face (eq. xi_taylor_final): side 0 the face above
+// the cell (L state), side 1 the face below (R state)
 template <typename T>
-__global__ void k_xi_slopes(Geo g, const int* __restrict__ bb, const T* __restrict__ x, const int8_t* __restrict__ lay,
-                            XiScratch sc) {
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int uu[3], i, j, k;
-    long c;
-    win_cell(g, w, t, uu, i, j, k, c);
-    if (lay[c] < 0) continue;
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      T s3[3];
-      slope_xi(g, x, lay, d, i, j, k, s3);
-#pragma unroll
-      for (int a = 0; a < 3; a++) ((T*)sc.s[3 * d + a])[c] = s3[a];
-    }
-  }
-}
-
-// pass 2: transverse bar states of xi on the e-face below every window cell (SI "Tangential
-// derivatives"), upwinded with the velocity's advecting bar velocity; unavailable on walls
-// and where either cell lacks xi
-template <typename T>
-__global__ void k_xi_bar(Geo g, const int* __restrict__ bb, const T* __restrict__ u, XiPredPtrs pp,
-                         const T* __restrict__ x, const int8_t* __restrict__ lay, XiScratch sc) {
-  const T h = cv<T>(g.h, g.f.h), dt = cv<T>(g.dt, g.f.dt);
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int uu[3], i, j, k;
-    long c;
-    win_cell(g, w, t, uu, i, j, k, c);
-    const int cc[3] = {i, j, k};
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      int8_t ok = 0;
-      if ((g.per[e] || cc[e] > 0) && lay[c] >= 0) {
-        int lo[3] = {i, j, k};
-        lo[e] = cc[e] > 0 ? cc[e] - 1 : g.n[e] - 1;
-        const long cD = cidx(g, lo[0], lo[1], lo[2]);
-        if (lay[cD] >= 0) {
-          ok = 1;
-          const T uD = u[e * g.N + cD], uU = u[e * g.N + c];
-          const T va = ((const T*)pp.vadv[e])[fidx(g, e, i, j, k)];
-#pragma unroll
-          for (int a = 0; a < 3; a++) {
-            const T sD = ((const T*)sc.s[3 * e + a])[cD], sU = ((const T*)sc.s[3 * e + a])[c];
-            T L, R;
-            if constexpr (disp_storage<T>()) {
-              // displacements from the face centre's image x0_D + (h/2) e_e = x0_U - (h/2) e_e
-              const T id = a == e ? T(1) : T(0);
-              L = x[a * g.N + cD] + T(0.5) * h * (sD - id) - T(0.5) * dt * uD * sD;
-              R = x[a * g.N + c] - T(0.5) * h * (sU - id) - T(0.5) * dt * uU * sU;
-            } else {
-              L = x[a * g.N + cD] + (T(0.5) * h - T(0.5) * dt * uD) * sD;
-              R = x[a * g.N + c] - (T(0.5) * h + T(0.5) * dt * uU) * sU;
-            }
-            ((T*)sc.xb[3 * e + a])[c] = upwind(L, R, va, cv<T>(g.utol, g.f.utol));
-          }
-        }
-      }
-      sc.ok[e][c] = ok;
-    }
-  }
-}
-
-// Taylor state of xi from cell (i,j,k) (inside the grid) toward its d-face (eq. xi_taylor_final):
-// side 0 the face above the cell (L state), side 1 the face below (R state)
-template <typename T>
-__device__ __forceinline__ void xi_state(const Geo& g, const T* __restrict__ u, const T* __restrict__ x,
-                                         const XiPredPtrs& pp, const XiScratch& sc, int d, int side, int i, int j,
-                                         int k, T out[3]) {
+__device__ __forceinline__ T xi_state(const Geo& g, const T* __restrict__ u, const XiPredPtrs& pp, const XiTile<T>& t,
+                                      const int org[3], int a, int d, int side, int vx, int vy, int vz) {
   const T h = cv<T>(g.h, g.f.h), dt = cv<T>(g.dt, g.f.dt), ih = cv<T>(g.ih, g.f.ih);
-  const long c = cidx(g, i, j, k);
-  const T ud = u[d * g.N + c];
-  const T coef = side == 0 ? (T(0.5) * h - T(0.5) * dt * ud) : -(T(0.5) * h + T(0.5) * dt * ud);
-  T tr[3] = {T(0), T(0), T(0)};
-  const int cc[3] = {i, j, k};
+  int i = org[0] + vx, j = org[1] + vy, k = org[2] + vz;
+  wrap_axis(g, 0, i);
+  wrap_axis(g, 1, j);
+  wrap_axis(g, 2, k);
+  const int p = stage_at(vx, vy, vz), q = ring_at(vx, vy, vz);
+  const T ud = u[d * g.N + cidx(g, i, j, k)];
+  T tr = T(0);
 #pragma unroll
   for (int e = 0; e < 3; e++) {
-    if (e == d) continue;
-    // bar states on the e-faces below and above the cell; the one above is owned by the next
-    // cell along e (none past a wall)
-    if (!sc.ok[e][c]) continue;
-    if (!g.per[e] && cc[e] == g.n[e] - 1) continue;
-    int up[3] = {i, j, k};
-    up[e] = cc[e] + 1 < g.n[e] ? cc[e] + 1 : 0;
-    const long cu = cidx(g, up[0], up[1], up[2]);
-    if (!sc.ok[e][cu]) continue;
-    long lo, hi;
-    cell_faces<T>(g, e, i, j, k, lo, hi);
+    // bar states on the e-faces below and above the cell, where both are formed
+    if (e == d || t.lay[p - stage_step(e)] < 0 || t.lay[p + stage_step(e)] < 0) continue;
     const T* va = (const T*)pp.vadv[e];
-    const T vav = T(0.5) * (va[lo] + va[hi]);
-#pragma unroll
-    for (int a = 0; a < 3; a++)
-      tr[a] += vav * (((const T*)sc.xb[3 * e + a])[cu] - ((const T*)sc.xb[3 * e + a])[c]) * ih;
+    const long lo = fidx(g, e, i, j, k), up = fidx(g, e, i + (e == 0), j + (e == 1), k + (e == 2));
+    const T vav = T(0.5) * (va[lo] + va[up]);
+    tr += vav * (t.bar[e][q + ring_step(e)] - t.bar[e][q]) * ih;
     // FP32 storage: the two bar states are displacements from face centres h apart along e
-    if constexpr (disp_storage<T>()) tr[e] += vav;
+    if constexpr (disp_storage<T>()) {
+      if (a == e) tr += vav;
+    }
   }
+  const T s = t.s[d][q];
   if constexpr (disp_storage<T>()) {
     // displacement from the face centre's image x0_c +- (h/2) e_d
     const T sg = side == 0 ? T(0.5) * h : -T(0.5) * h;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      const T s = ((const T*)sc.s[3 * d + a])[c];
-      out[a] = x[a * g.N + c] + sg * (s - (a == d ? T(1) : T(0))) - T(0.5) * dt * ud * s - T(0.5) * dt * tr[a];
-    }
-    return;
+    return t.x[p] + sg * (s - (a == d ? T(1) : T(0))) - T(0.5) * dt * ud * s - T(0.5) * dt * tr;
+  } else {
+    const T coef = side == 0 ? (T(0.5) * h - T(0.5) * dt * ud) : -(T(0.5) * h + T(0.5) * dt * ud);
+    return t.x[p] + coef * s - T(0.5) * dt * tr;
   }
-#pragma unroll
-  for (int a = 0; a < 3; a++)
-    out[a] = x[a * g.N + c] + coef * ((const T*)sc.s[3 * d + a])[c] - T(0.5) * dt * tr[a];
 }
 
-// pass 3: xi^{n+1} = xi^n - dt [(u.grad) xi]^{n+1/2} at the cells of layers 0 and 1 whose six faces
-// carry xi^{n+1/2}; NaN at every other window cell
+// grid (tiles of a window, bodies, components).  A band cell's neighbours are at most one layer further out, so
+// the cells of layers 0 and 1 read states of layers up to 2 and bar states and slopes of layers up to 3.
 template <typename T>
-__global__ void k_xi_predict(Geo g, const T* __restrict__ u, XiPredPtrs pp, const int* __restrict__ bb,
-                             const T* __restrict__ x, const int8_t* __restrict__ lay, XiScratch sc,
-                             T* __restrict__ xn) {
-  const T ih = cv<T>(g.ih, g.f.ih), dt = cv<T>(g.dt, g.f.dt);
+__global__ void __launch_bounds__(XTPB) k_xi_predict(Geo g, const T* __restrict__ u,
+                                                     const __grid_constant__ XiPredPtrs pp,
+                                                     const __grid_constant__ BandSet<T> S) {
+  extern __shared__ double xi_smem[];
+  XiTile<T>& t = *reinterpret_cast<XiTile<T>*>(xi_smem);
+  const int m = S.m0 + blockIdx.y, a = blockIdx.z, tid = threadIdx.x;
+  const Band<T>& band = S.bands[m];
+  const T* __restrict__ x = band.X[S.in] + a * g.N;
+  const int8_t* __restrict__ lay = band.LAY[S.in];
+  T* __restrict__ xn = band.X[S.out] + a * g.N;
+  const Win w = make_win(g, band.bb + 6 * S.in, 2);
+  const T h = cv<T>(g.h, g.f.h), dt = cv<T>(g.dt, g.f.dt), ih = cv<T>(g.ih, g.f.ih), tol = cv<T>(g.utol, g.f.utol);
   const T nanv = T(__longlong_as_double(0x7ff8000000000000ll));
-  const Win w = make_win(g, bb, 2);
-  WIN_LOOP(t, w) {
-    int uu[3], i, j, k;
-    long c;
-    win_cell(g, w, t, uu, i, j, k, c);
-    const int l = lay[c];
-    if (l < 0 || l > 1) {
-      xn[c] = nanv; xn[g.N + c] = nanv; xn[2 * g.N + c] = nanv;
-      continue;
+  const int n0 = (w.ext[0] + XT - 1) / XT, n1 = (w.ext[1] + XT - 1) / XT, n2 = (w.ext[2] + XT - 1) / XT;
+  const int tiles = w.vol > 0 ? n0 * n1 * n2 : 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int o0 = tile % n0 * XT, o1 = tile / n0 % n1 * XT, o2 = tile / (n0 * n1) * XT;
+    const int org[3] = {w.lo[0] + o0, w.lo[1] + o1, w.lo[2] + o2};
+    // a tile without cells of layers 0 and 1 only gets its NaNs
+    bool live = false;
+    for (int q = tid; q < XT * XT * XT; q += XTPB) {
+      const int vx = q % XT, vy = q / XT % XT, vz = q / (XT * XT);
+      if (o0 + vx >= w.ext[0] || o1 + vy >= w.ext[1] || o2 + vz >= w.ext[2]) continue;
+      int i = org[0] + vx, j = org[1] + vy, k = org[2] + vz;
+      wrap_axis(g, 0, i);
+      wrap_axis(g, 1, j);
+      wrap_axis(g, 2, k);
+      const long c = cidx(g, i, j, k);
+      if ((unsigned)lay[c] <= 1u) live = true;
+      else xn[c] = nanv;
     }
-    T acc[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      T xf[2][3];
-#pragma unroll
-      for (int fs = 0; fs < 2; fs++) {
-        // fs = 0: face below c (a = c - e_d, b = c); fs = 1: face above (a = c, b = c + e_d)
-        int ca[3] = {i, j, k}, cb[3] = {i, j, k};
-        if (fs == 0) ca[d] -= 1; else cb[d] += 1;
-        const long f = fidx(g, d, cb[0], cb[1], cb[2]);  // face index: d-index of b, up to n_d
-        long la, lb;
-        const bool okA = cell_at(g, ca[0], ca[1], ca[2], la) && lay[la] >= 0;
-        const bool okB = cell_at(g, cb[0], cb[1], cb[2], lb) && lay[lb] >= 0;
-        wrap_axis(g, d, ca[d]);
-        wrap_axis(g, d, cb[d]);
-        const T un = ((const T*)pp.unpre[d])[f];
-        T L[3], R[3];
-        if (okA) xi_state(g, u, x, pp, sc, d, 0, ca[0], ca[1], ca[2], L);
-        if (okB) xi_state(g, u, x, pp, sc, d, 1, cb[0], cb[1], cb[2], R);
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-          xf[fs][a] = (okA && okB) ? upwind(L[a], R[a], un, cv<T>(g.utol, g.f.utol)) : (okA ? L[a] : R[a]);
+    if (!__syncthreads_or(live)) continue;  // also: the last tile's reads are done
+
+    for (int r = tid / 16; r < XL * XL; r += XTPB / 16) {
+      const int tx = tid % 16;
+      if (tx < XL) {
+        int i = org[0] + tx - 3, j = org[1] + r % XL - 3, k = org[2] + r / XL - 3;
+        int l = -1;
+        T v = T(0);
+        if (wrap_axis(g, 0, i) && wrap_axis(g, 1, j) && wrap_axis(g, 2, k)) {
+          const long c = cidx(g, i, j, k);
+          l = lay[c];
+          v = x[c];
+        }
+        t.lay[tx + XL * r] = (int8_t)l;
+        t.x[tx + XL * r] = l >= 0 ? v : T(0);
       }
-      long lo, hi;
-      cell_faces<T>(g, d, i, j, k, lo, hi);
-      const T* U = (const T*)pp.umac[d];
-      const T va = T(0.5) * (U[lo] + U[hi]);
-#pragma unroll
-      for (int a = 0; a < 3; a++) acc[a] += va * (xf[1][a] - xf[0][a]) * ih;
-      // FP32 storage: the face states are displacements from face centres h apart along d
-      if constexpr (disp_storage<T>()) acc[d] += va;
     }
+    __syncthreads();
+
+    // limited slopes
+    for (int q = tid; q < XR * XR * XR; q += XTPB) {
+      const int p = stage_at(q % XR - 1, q / XR % XR - 1, q / (XR * XR) - 1);
+      if ((unsigned)t.lay[p] > 3u) continue;
 #pragma unroll
-    for (int a = 0; a < 3; a++) xn[a * g.N + c] = x[a * g.N + c] - dt * acc[a];
+      for (int e = 0; e < 3; e++) {
+        T v[5];
+        unsigned ok = 0;
+#pragma unroll
+        for (int b = -2; b <= 2; b++) {
+          const int pb = p + b * stage_step(e);
+          if (t.lay[pb] >= 0) ok |= 1u << (b + 2);
+          v[b + 2] = t.x[pb];
+          // FP32 storage: the identity's part of xi_e along axis e, relative to the centre cell (the
+          // band never pairs cells across the seam of the body's image window)
+          if constexpr (disp_storage<T>()) v[b + 2] += a == e ? T(b) * h : T(0);
+        }
+        t.s[e][q] = lim_slope(v, ok, ih);
+      }
+    }
+    __syncthreads();
+
+    // transverse bar states (SI "Tangential derivatives"), upwinded with the velocity's advecting bar velocity;
+    // unavailable on walls and where either cell lacks xi
+    for (int q = tid; q < XR * XR * XR; q += XTPB) {
+      const int v[3] = {q % XR - 1, q / XR % XR - 1, q / (XR * XR) - 1};
+      const int p = stage_at(v[0], v[1], v[2]);
+      if ((unsigned)t.lay[p] > 3u) continue;
+      int cc[3] = {org[0] + v[0], org[1] + v[1], org[2] + v[2]};
+#pragma unroll
+      for (int d = 0; d < 3; d++) wrap_axis(g, d, cc[d]);
+#pragma unroll
+      for (int e = 0; e < 3; e++) {
+        const int pD = p - stage_step(e), qD = q - ring_step(e);
+        if (v[e] < 0 || (unsigned)t.lay[pD] > 3u) continue;
+        int lo[3] = {cc[0], cc[1], cc[2]};
+        lo[e] = cc[e] > 0 ? cc[e] - 1 : g.n[e] - 1;
+        const T va = ((const T*)pp.vadv[e])[fidx(g, e, cc[0], cc[1], cc[2])];
+        T L = T(0), R = T(0);
+        if (!(va < -tol)) {
+          const T uD = u[e * g.N + cidx(g, lo[0], lo[1], lo[2])], sD = t.s[e][qD];
+          if constexpr (disp_storage<T>())  // displacement from the face centre's image x0_D + (h/2) e_e
+            L = t.x[pD] + T(0.5) * h * (sD - (a == e ? T(1) : T(0))) - T(0.5) * dt * uD * sD;
+          else
+            L = t.x[pD] + (T(0.5) * h - T(0.5) * dt * uD) * sD;
+        }
+        if (!(va > tol)) {
+          const T uU = u[e * g.N + cidx(g, cc[0], cc[1], cc[2])], sU = t.s[e][q];
+          if constexpr (disp_storage<T>())  // x0_U - (h/2) e_e, the same point
+            R = t.x[p] - T(0.5) * h * (sU - (a == e ? T(1) : T(0))) - T(0.5) * dt * uU * sU;
+          else
+            R = t.x[p] - (T(0.5) * h + T(0.5) * dt * uU) * sU;
+        }
+        t.bar[e][q] = upwind(L, R, va, tol);
+      }
+    }
+    __syncthreads();
+
+    // face states next to cells of layers 0 and 1
+    for (int r = tid; r < 3 * XF; r += XTPB) {
+      const int d = r / XF, q = r - d * XF;
+      const int m0 = d == 0 ? XT + 1 : XT, m1 = d == 1 ? XT + 1 : XT;
+      const int vx = q % m0, vy = q / m0 % m1, vz = q / (m0 * m1);
+      const int pU = stage_at(vx, vy, vz), pD = pU - stage_step(d);
+      const int lU = t.lay[pU], lD = t.lay[pD];
+      if ((unsigned)lU > 1u && (unsigned)lD > 1u) continue;
+      const bool both = lU >= 0 && lD >= 0;
+      bool needL = lD >= 0, needR = lU >= 0;
+      T un = T(0);
+      if (both) {
+        int i = org[0] + vx, j = org[1] + vy, k = org[2] + vz;
+        wrap_axis(g, 0, i);
+        wrap_axis(g, 1, j);
+        wrap_axis(g, 2, k);
+        un = ((const T*)pp.unpre[d])[fidx(g, d, i, j, k)];
+        needL = !(un < -tol);
+        needR = !(un > tol);
+      }
+      T L = T(0), R = T(0);
+      // one state in the common case, from the cell on its side
+      const int side = needL ? 0 : 1;
+      const T first = xi_state(g, u, pp, t, org, a, d, side, vx - (side == 0 && d == 0), vy - (side == 0 && d == 1),
+                               vz - (side == 0 && d == 2));
+      if (needL) L = first;
+      else R = first;
+      if (needL && needR) R = xi_state(g, u, pp, t, org, a, d, 1, vx, vy, vz);
+      t.f[d][q] = both ? upwind(L, R, un, tol) : (lD >= 0 ? L : R);
+    }
+    __syncthreads();
+
+    // xi^{n+1} = xi^n - dt [(u.grad) xi]^{n+1/2}
+    for (int q = tid; q < XT * XT * XT; q += XTPB) {
+      const int vx = q % XT, vy = q / XT % XT, vz = q / (XT * XT);
+      const int p = stage_at(vx, vy, vz);
+      if ((unsigned)t.lay[p] > 1u || o0 + vx >= w.ext[0] || o1 + vy >= w.ext[1] || o2 + vz >= w.ext[2]) continue;
+      int i = org[0] + vx, j = org[1] + vy, k = org[2] + vz;
+      wrap_axis(g, 0, i);
+      wrap_axis(g, 1, j);
+      wrap_axis(g, 2, k);
+      T acc = T(0);
+#pragma unroll
+      for (int d = 0; d < 3; d++) {
+        const T* U = (const T*)pp.umac[d];
+        const long lo = fidx(g, d, i, j, k), up = fidx(g, d, i + (d == 0), j + (d == 1), k + (d == 2));
+        const T va = T(0.5) * (U[lo] + U[up]);
+        const int f = d == 0 ? vx + (XT + 1) * (vy + XT * vz) : vx + XT * (vy + (d == 1 ? XT + 1 : XT) * vz);
+        const int fs = d == 0 ? 1 : (d == 1 ? XT : XT * XT);
+        acc += va * (t.f[d][f + fs] - t.f[d][f]) * ih;
+        // FP32 storage: the face states are displacements from face centres h apart along d
+        if constexpr (disp_storage<T>()) {
+          if (a == d) acc += va;
+        }
+      }
+      xn[cidx(g, i, j, k)] = t.x[p] - dt * acc;
+    }
   }
 }
 
 }  // namespace
 
 template <typename T>
-void launch_xi_predict(const Geo& g, const T* u, T* const vadv[3], T* const uf[3][3], T* const umac[3], const int* bb,
-                       int blocks, const T* x, const int8_t* lay, T* const scratch_s[9], T* const scratch_xb[9],
-                       int8_t* const scratch_ok[3], T* xn, cudaStream_t s) {
+cudaError_t launch_xi_predict(const Geo& g, const T* u, T* const vadv[3], T* const uf[3][3], T* const umac[3],
+                              const BandSet<T>& S, int tiles, cudaStream_t s) {
   XiPredPtrs pp;
-  XiScratch sc;
   for (int d = 0; d < 3; d++) {
     pp.vadv[d] = vadv[d];
     pp.unpre[d] = uf[d][d];
     pp.umac[d] = umac[d];
-    sc.ok[d] = scratch_ok[d];
   }
-  for (int q = 0; q < 9; q++) {
-    sc.s[q] = scratch_s[q];
-    sc.xb[q] = scratch_xb[q];
+  const size_t smem = sizeof(XiTile<T>);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_xi_predict<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
   }
-  k_xi_slopes<T><<<blocks, TPB, 0, s>>>(g, bb, x, lay, sc);
+  k_xi_predict<T><<<dim3(tiles, S.count, 3), XTPB, smem, s>>>(g, u, pp, S);
   rmt_count_launches(1);
-  k_xi_bar<T><<<blocks, TPB, 0, s>>>(g, bb, u, pp, x, lay, sc);
-  rmt_count_launches(1);
-  k_xi_predict<T><<<blocks, TPB, 0, s>>>(g, u, pp, bb, x, lay, sc, xn);
-  rmt_count_launches(1);
+  return cudaSuccess;
 }
 
-template void launch_xi_predict<float>(const Geo&, const float*, float* const[3], float* const[3][3], float* const[3],
-                                       const int*, int, const float*, const int8_t*, float* const[9], float* const[9],
-                                       int8_t* const[3], float*, cudaStream_t);
-template void launch_xi_predict<double>(const Geo&, const double*, double* const[3], double* const[3][3],
-                                        double* const[3], const int*, int, const double*, const int8_t*,
-                                        double* const[9], double* const[9], int8_t* const[3], double*, cudaStream_t);
+#define INST(T)                                                                                                 \
+  template cudaError_t launch_xi_predict<T>(const Geo&, const T*, T* const[3], T* const[3][3], T* const[3],     \
+                                            const BandSet<T>&, int, cudaStream_t);
+INST(float)
+INST(double)
