@@ -100,8 +100,8 @@ struct rmt_grid {
   void *u = nullptr, *p = nullptr, *rho = nullptr, *rho_h = nullptr, *divn = nullptr, *divh = nullptr;
   void *adv = nullptr, *ustar = nullptr, *psi = nullptr;
   void* vadv[3] = {};
-  void* ub[3][3] = {};
   void* slopes[9] = {};
+  void* ub[3][3] = {};  // FP64: scratch of the Godunov passes
   void* wcell[9] = {};
   void* uf[3][3] = {};
   void* umac[3] = {};
@@ -459,13 +459,15 @@ rmt_status alloc_t(rmt_grid* g) {
   AL(g->adv, 3 * N * e);
   AL(g->ustar, 3 * N * e);
   AL(g->psi, G.NN * e);
-  for (int q = 0; q < 9; q++) AL(g->slopes[q], N * e);
-  for (int q = 0; q < 9; q++) AL(g->wcell[q], N * e);
+  for (int q = 0; q < 9; q++) {
+    AL(g->slopes[q], N * e);
+    if (e == 8) AL(g->wcell[q], N * e);
+  }
   for (int d = 0; d < 3; d++) {
     const long nf = nfaces(G, d);
     for (int a = 0; a < 3; a++) {
-      AL(g->ub[d][a], nf * e);
       AL(g->uf[d][a], nf * e);
+      if (e == 8) AL(g->ub[d][a], nf * e);
     }
     AL(g->vadv[d], nf * e);
     AL(g->umac[d], nf * e);
@@ -576,16 +578,16 @@ rmt_status step_t(rmt_grid* g) {
   cudaStream_t s = g->s;
   const int nb = (int)g->bodies.size();
   const int cur = g->par, nxt = 1 - g->par;
-  T* ub[3][3];
   T* slopes[9];
   T* wcell[9];
+  T* ub[3][3];
   T* vadv[3];
   T* uf[3][3];
   T* umac[3];
   for (int d = 0; d < 3; d++) {
     for (int a = 0; a < 3; a++) {
-      ub[d][a] = (T*)g->ub[d][a];
       uf[d][a] = (T*)g->uf[d][a];
+      ub[d][a] = (T*)g->ub[d][a];
     }
     vadv[d] = (T*)g->vadv[d];
     umac[d] = (T*)g->umac[d];
@@ -600,11 +602,10 @@ rmt_status step_t(rmt_grid* g) {
   CK(g, launch_stress_div<T>(G, u, g->bodies_d, views<T>(g, cur, 0), nb, g->bb_all + 6 * cur, 12, g->t_d, 0.0,
                               (T*)g->divn, g->slist, slopes, s));
   pe(g, P_STRESS_N);
-  // 2. Godunov face states of u (transverse bar states first)
+  // 2. Godunov face states of u
   pb(g, P_GODUNOV);
-  launch_bar_states<T>(G, u, slopes, ub, vadv, s);
-  launch_face_states<T>(G, u, (const T*)g->p, (const T*)g->rho, (const T*)g->divn, g->bodies_d, views<T>(g, cur, 0),
-                        nb, slopes, wcell, ub, vadv, uf, s);
+  CK(g, launch_godunov<T>(G, u, (const T*)g->p, (const T*)g->rho, (const T*)g->divn, g->bodies_d,
+                          views<T>(g, cur, 0), nb, vadv, uf, slopes, wcell, ub, s));
   pe(g, P_GODUNOV);
   // 3. MAC projection of the normal face velocities
   pb(g, P_MAC_SETUP);

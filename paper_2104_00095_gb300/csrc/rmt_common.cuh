@@ -342,15 +342,16 @@ __device__ __forceinline__ T dheavi(T phi, T eps) {
 __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
+// the smaller magnitude of the two one-sided differences where they agree in sign, else zero
 template <typename T>
-__device__ __forceinline__ T mc_lim(T qm, T q0, T qp) {
+__device__ __forceinline__ T mc_min(T qm, T q0, T qp) {
   const T a = qp - q0, b = q0 - qm;
   if constexpr (sizeof(T) == 8) {
     const unsigned long long ma = mag_bits(a), mb = mag_bits(b);
     const bool same = (__double2hiint(a) ^ __double2hiint(b)) >= 0 && max(ma, mb) <= 0x7ff0000000000000ull;
-    return T(2) * __longlong_as_double((long long)(same ? min(ma, mb) : 0ull));
+    return __longlong_as_double((long long)(same ? min(ma, mb) : 0ull));
   } else {
-    return (a * b > T(0)) ? T(2) * fmin(fabs(a), fabs(b)) : T(0);
+    return (a * b > T(0)) ? fmin(fabs(a), fabs(b)) : T(0);
   }
 }
 // sgn(s) min(|x|, y) for y >= 0, written as copysign(min(|x|, y), s): equal to the product form
@@ -364,23 +365,26 @@ __device__ __forceinline__ T sgn_min(T s, T x, T y) {
     return copysign(fmin(fabs(x), y), s);
   }
 }
+// twice the limited central difference (the factors of two are exact and are left to the end)
 template <typename T>
-__device__ __forceinline__ T dflim(T qm, T q0, T qp) {
-  const T dc = T(0.5) * (qp - qm);
-  return sgn_min(dc, dc, mc_lim(qm, q0, qp));
+__device__ __forceinline__ T dflim2(T qm, T q0, T qp) {
+  const T d = qp - qm;
+  return sgn_min(d, d, T(4) * mc_min(qm, q0, qp));
+}
+// h times the slope from the inner values and dflim2 of the two neighbours
+template <typename T>
+__device__ __forceinline__ T lim_slope4(T qm, T q0, T qp, T dfm2, T dfp2) {
+  const T d = qp - qm;
+  // the twelfth as a product (a division per slope would dominate the kernel)
+  const T d4 = T(2.0 / 3.0) * d - (dfp2 + dfm2) * T(1.0 / 12.0);
+  return sgn_min(d, d4, T(2) * mc_min(qm, q0, qp));
 }
 template <typename T>
 __device__ __forceinline__ T lim_slope(const T q[5], unsigned okmask, T inv_h) {
   // okmask bit s set when q[s] is present
   if ((okmask & 0xE) != 0xE) return T(0);
-  const T dc = T(0.5) * (q[3] - q[1]);
-  const T dl = mc_lim(q[1], q[2], q[3]);
-  if ((okmask & 0x11) != 0x11) return sgn_min(dc, dc, dl) * inv_h;
-  const T dfp = dflim(q[2], q[3], q[4]);
-  const T dfm = dflim(q[0], q[1], q[2]);
-  // the sixth as a product (a division per slope would dominate the kernel)
-  const T d4 = T(4.0 / 3.0) * dc - (dfp + dfm) * T(1.0 / 6.0);
-  return sgn_min(dc, d4, dl) * inv_h;
+  if ((okmask & 0x11) != 0x11) return T(0.5) * dflim2(q[1], q[2], q[3]) * inv_h;
+  return lim_slope4(q[1], q[2], q[3], dflim2(q[0], q[1], q[2]), dflim2(q[2], q[3], q[4])) * inv_h;
 }
 
 // Godunov choice of the normal velocity and upwinding of other quantities

@@ -21,223 +21,8 @@ __device__ __forceinline__ void cell_faces(const Geo& g, int e, int i, int j, in
   ii[e] += 1;
   hi = fidx(g, e, ii[0], ii[1], ii[2]);
 }
-// ---------------------------------------------------------------------------------
-// Godunov predictor
-
-template <typename T>
-__device__ __forceinline__ T slope_u(const Geo& g, const T* __restrict__ u, int a, int d, int i, int j, int k) {
-  T q[5];
-  if (d == 0 && g.per[0]) {
-    // periodic x: wrap by selects, one path for the whole row (no divergence at its ends)
-    const T* row = u + (long)a * g.N + cidx(g, 0, j, k);
-    const int n0 = g.n[0];
-#pragma unroll
-    for (int s = -2; s <= 2; s++) {
-      int ii = i + s;
-      ii += ii < 0 ? n0 : 0;
-      ii -= ii >= n0 ? n0 : 0;
-      q[s + 2] = row[ii];
-    }
-  } else if (inside<T>(g, d, i, j, k, 2)) {
-    const long c = (long)a * g.N + cidx(g, i, j, k);
-    const long st = d == 0 ? 1 : (d == 1 ? (long)g.n[0] : (long)g.n[0] * g.n[1]);
-#pragma unroll
-    for (int s = -2; s <= 2; s++) q[s + 2] = u[c + s * st];
-  } else {
-#pragma unroll
-    for (int s = -2; s <= 2; s++) {
-      int ii[3] = {i, j, k};
-      ii[d] += s;
-      q[s + 2] = uval(g, u, a, ii[0], ii[1], ii[2]);
-    }
-  }
-  return lim_slope(q, 0x1Fu, cv<T>(g.ih, g.f.ih));
-}
-
-// limited slopes of the three velocity components along the three axes at every cell
-// (SI "Normal derivatives"); S[3 * d + a] = d u_a / d x_d
-struct Slopes9 {
-  void* s[9];
-};
-// A cell whose five-point stencils reach no wall ghost (all points inside, or wrapped across
-// periodic sides: every cell of a periodic box) takes the offsets of its +-1, +-2 neighbours
-// along each axis once and reads the three components through them; the others go through
-// slope_u's boundary rules.  The same values reach the same limiter either way.
-template <typename T>
-__global__ void __launch_bounds__(TILE_X* TILE_Y) k_slopes(Geo g, const T* __restrict__ u, Slopes9 S) {
-  THREAD_XYZ(i, j, k);
-  if (i >= g.n[0] || j >= g.n[1]) return;
-  const long c = cidx(g, i, j, k);
-  const int ii[3] = {i, j, k};
-  const long st[3] = {1, (long)g.n[0], (long)g.n[0] * g.n[1]};
-  long off[3][4];  // neighbours -2, -1, +1, +2 along each axis
-  bool fast = true;
-#pragma unroll
-  for (int d = 0; d < 3; d++)
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int sft = q < 2 ? q - 2 : q - 1;
-      int v = ii[d] + sft;
-      if (v < 0 || v >= g.n[d]) {
-        fast = fast && g.per[d];
-        v += v < 0 ? g.n[d] : -g.n[d];
-      }
-      off[d][q] = (long)(v - ii[d]) * st[d];
-    }
-  if (fast) {
-    const T ih = cv<T>(g.ih, g.f.ih);
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      const T* pc = u + (long)a * g.N + c;
-      const T x0 = pc[0];
-#pragma unroll
-      for (int d = 0; d < 3; d++) {
-        const T q[5] = {pc[off[d][0]], pc[off[d][1]], x0, pc[off[d][2]], pc[off[d][3]]};
-        ((T*)S.s[3 * d + a])[c] = lim_slope(q, 0x1Fu, ih);
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int d = 0; d < 3; d++)
-#pragma unroll
-    for (int a = 0; a < 3; a++) ((T*)S.s[3 * d + a])[c] = slope_u(g, u, a, d, i, j, k);
-}
-
 __device__ __forceinline__ bool is_wall_face(const Geo& g, int d, int f) {
   return !g.per[d] && (f == 0 || f == g.n[d]);
-}
-
-// transverse bar states at every e-face (SI "Tangential derivatives")
-template <typename T, int e>
-__global__ void __launch_bounds__(TILE_X* TILE_Y) k_bar(Geo g, const T* __restrict__ u, Slopes9 S,
-                                                         T* __restrict__ ub0, T* __restrict__ ub1, T* __restrict__ ub2,
-                                                         T* __restrict__ vadv) {
-  const int ex = g.n[0] + (e == 0), ey = g.n[1] + (e == 1), ez = g.n[2] + (e == 2);
-  const T h = cv<T>(g.h, g.f.h), dt = cv<T>(g.dt, g.f.dt);
-  T* ub[3] = {ub0, ub1, ub2};
-  THREAD_XYZ(i, j, k);
-  if (i >= ex || j >= ey || k >= ez) return;
-  const long f = (long)(i + ex * (j + ey * k));
-  const int fi = e == 0 ? i : (e == 1 ? j : k);
-  if (is_wall_face(g, e, fi)) {
-    const int face = fi == 0 ? 2 * e : 2 * e + 1;
-#pragma unroll
-    for (int a = 0; a < 3; a++) ub[a][f] = cv<T>(g.wall[face][a], g.f.wall[face][a]);
-    vadv[f] = cv<T>(g.wall[face][e], g.f.wall[face][e]);
-    return;
-  }
-  // the two cells of an interior (or periodic) face: D below, U above
-  int lo[3] = {i, j, k}, hi[3] = {i, j, k};
-  lo[e] -= 1;
-  if (lo[e] < 0) lo[e] += g.n[e];
-  if (hi[e] >= g.n[e]) hi[e] -= g.n[e];
-  const long cD = cidx(g, lo[0], lo[1], lo[2]), cU = cidx(g, hi[0], hi[1], hi[2]);
-  const T uD = u[e * g.N + cD], uU = u[e * g.N + cU];
-  T qD[3], qU[3];
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    const T* Sa = (const T*)S.s[3 * e + a];
-    qD[a] = u[a * g.N + cD] + (T(0.5) * h - T(0.5) * dt * uD) * Sa[cD];
-    qU[a] = u[a * g.N + cU] - (T(0.5) * h + T(0.5) * dt * uU) * Sa[cU];
-  }
-  const T va = god_normal(qD[e], qU[e], cv<T>(g.utol, g.f.utol));
-  vadv[f] = va;
-#pragma unroll
-  for (int a = 0; a < 3; a++) ub[a][f] = upwind(qD[a], qU[a], va, cv<T>(g.utol, g.f.utol));
-}
-
-struct BarPtrs {
-  const void* ub[3][3];
-  const void* vadv[3];
-  void* uf[3];
-};
-
-// Side-independent part of the face states of every cell (eqs. left_final, right_final):
-// W[3d+a] = u_a - (dt/2) T_d(u_a) + dt/(2 rho) F_a, with T_d the tangential terms along the two
-// axes other than d (SI "Tangential derivatives") and F = -grad p^{n-1/2} + div tau^n + b^n,
-// b = (rho - rho_f) g.  A face state is then W + (+-h/2 - dt/2 u_d) * slope.
-template <typename T>
-__global__ void __launch_bounds__(TILE_X* TILE_Y) k_cellw(Geo g, const T* __restrict__ u, const T* __restrict__ p,
-                                                           const T* __restrict__ rho, const T* __restrict__ divtau,
-                                                           BarPtrs bp, Slopes9 W, const Body* __restrict__ bodies,
-                                                           const BodyView<T>* __restrict__ views, int nb) {
-  THREAD_XYZ(i, j, k);
-  if (i >= g.n[0] || j >= g.n[1]) return;
-  const T dt = cv<T>(g.dt, g.f.dt), ih = cv<T>(g.ih, g.f.ih);
-  const long c = cidx(g, i, j, k);
-  T gp[3] = {T(0), T(0), T(0)};
-#pragma unroll
-  for (int q = 0; q < 8; q++) {
-    const int sa = q & 1, sb = (q >> 1) & 1, sc = (q >> 2) & 1;
-    const T pv = p[node_at(g, i + sa, j + sb, k + sc)];
-    gp[0] += sa ? pv : -pv;
-    gp[1] += sb ? pv : -pv;
-    gp[2] += sc ? pv : -pv;
-  }
-  const T r = rho[c];
-  // wall repulsion joins b (SI "Contact with a wall"), from phi^n
-  T rep[3];
-  const bool has_rep = g.any_rep && rep_accel(g, bodies, views, nb, i, j, k, c, rep);
-  T vavg[3];
-  long lo[3], hi[3];
-#pragma unroll
-  for (int e = 0; e < 3; e++) {
-    cell_faces<T>(g, e, i, j, k, lo[e], hi[e]);
-    const T* vad = (const T*)bp.vadv[e];
-    vavg[e] = T(0.5) * (vad[lo[e]] + vad[hi[e]]);
-  }
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    T F = -gp[a] * (T(0.25) * ih) + divtau[a * g.N + c] + (r - cv<T>(g.rho_f, g.f.rho_f)) * cv<T>(g.grav[a], g.f.grav[a]);
-    if (has_rep) F = F + r * rep[a];
-    T term[3];
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      const T* ube = (const T*)bp.ub[e][a];
-      term[e] = vavg[e] * (ube[hi[e]] - ube[lo[e]]) * ih;
-    }
-    const T base = u[a * g.N + c] + T(0.5) * dt / r * F;
-    ((T*)W.s[a])[c] = base - T(0.5) * dt * (term[1] + term[2]);
-    ((T*)W.s[3 + a])[c] = base - T(0.5) * dt * (term[0] + term[2]);
-    ((T*)W.s[6 + a])[c] = base - T(0.5) * dt * (term[0] + term[1]);
-  }
-}
-
-// normal-face states of the velocity and the Godunov choice (SI "Godunov-type upwinding")
-template <typename T, int d>
-__global__ void __launch_bounds__(TILE_X* TILE_Y) k_face(Geo g, const T* __restrict__ u, Slopes9 S, Slopes9 W,
-                                                          BarPtrs bp) {
-  const int ex = g.n[0] + (d == 0), ey = g.n[1] + (d == 1), ez = g.n[2] + (d == 2);
-  const T h = cv<T>(g.h, g.f.h), dt = cv<T>(g.dt, g.f.dt);
-  T* uf[3] = {(T*)bp.uf[0], (T*)bp.uf[1], (T*)bp.uf[2]};
-  THREAD_XYZ(i, j, k);
-  if (i >= ex || j >= ey || k >= ez) return;
-  const long f = (long)(i + ex * (j + ey * k));
-  const int fi = d == 0 ? i : (d == 1 ? j : k);
-  if (is_wall_face(g, d, fi)) {
-    const int face = fi == 0 ? 2 * d : 2 * d + 1;
-#pragma unroll
-    for (int a = 0; a < 3; a++) uf[a][f] = cv<T>(g.wall[face][a], g.f.wall[face][a]);
-    return;
-  }
-  int lo[3] = {i, j, k}, hi[3] = {i, j, k};
-  lo[d] -= 1;
-  if (lo[d] < 0) lo[d] += g.n[d];
-  if (hi[d] >= g.n[d]) hi[d] -= g.n[d];
-  const long cc[2] = {cidx(g, lo[0], lo[1], lo[2]), cidx(g, hi[0], hi[1], hi[2])};
-  T st[2][3];
-#pragma unroll
-  for (int side = 0; side < 2; side++) {
-    const long c = cc[side];
-    const T ud = u[d * g.N + c];
-    const T coef = side == 0 ? (T(0.5) * h - T(0.5) * dt * ud) : -(T(0.5) * h + T(0.5) * dt * ud);
-#pragma unroll
-    for (int a = 0; a < 3; a++) st[side][a] = ((const T*)W.s[3 * d + a])[c] + coef * ((const T*)S.s[3 * d + a])[c];
-  }
-  const T un = god_normal(st[0][d], st[1][d], cv<T>(g.utol, g.f.utol));
-#pragma unroll
-  for (int a = 0; a < 3; a++) uf[a][f] = (a == d) ? un : upwind(st[0][a], st[1][a], un, cv<T>(g.utol, g.f.utol));
 }
 
 // ---------------------------------------------------------------------------------
@@ -691,48 +476,6 @@ __global__ void k_fill(T* a, T v, long n) {
 }  // namespace
 
 template <typename T>
-void launch_bar_states(const Geo& g, const T* u, T* const slopes[9], T* const ubar[3][3], T* const vadv[3],
-                       cudaStream_t s) {
-  Slopes9 S;
-  for (int q = 0; q < 9; q++) S.s[q] = slopes[q];
-  const dim3 gc((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, g.n[2]);
-  k_slopes<T><<<gc, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, S);
-  rmt_count_launches(1);
-  for (int e = 0; e < 3; e++) {
-    const dim3 gr((g.n[0] + (e == 0) + TILE_X - 1) / TILE_X, (g.n[1] + (e == 1) + TILE_Y - 1) / TILE_Y, g.n[2] + (e == 2));
-    // the direction is a template argument: a runtime index into the pointer bundles would
-    // copy them to local memory in every thread
-    auto kb = e == 0 ? k_bar<T, 0> : (e == 1 ? k_bar<T, 1> : k_bar<T, 2>);
-    kb<<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, S, ubar[e][0], ubar[e][1], ubar[e][2], vadv[e]);
-    rmt_count_launches(1);
-  }
-}
-template <typename T>
-void launch_face_states(const Geo& g, const T* u, const T* p, const T* rho, const T* divtau, const Body* bodies,
-                        const BodyView<T>* views, int nb, T* const slopes[9],
-                        T* const wcell[9], T* const ubar[3][3], T* const vadv[3], T* const uf[3][3], cudaStream_t s) {
-  BarPtrs bp;
-  Slopes9 S, W;
-  for (int q = 0; q < 9; q++) {
-    S.s[q] = slopes[q];
-    W.s[q] = wcell[q];
-  }
-  for (int e = 0; e < 3; e++) {
-    for (int a = 0; a < 3; a++) bp.ub[e][a] = ubar[e][a];
-    bp.vadv[e] = vadv[e];
-  }
-  const dim3 gc((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, g.n[2]);
-  k_cellw<T><<<gc, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, p, rho, divtau, bp, W, bodies, views, nb);
-  rmt_count_launches(1);
-  for (int d = 0; d < 3; d++) {
-    for (int a = 0; a < 3; a++) bp.uf[a] = uf[d][a];
-    const dim3 gr((g.n[0] + (d == 0) + TILE_X - 1) / TILE_X, (g.n[1] + (d == 1) + TILE_Y - 1) / TILE_Y, g.n[2] + (d == 2));
-    auto kf = d == 0 ? k_face<T, 0> : (d == 1 ? k_face<T, 1> : k_face<T, 2>);
-    kf<<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, S, W, bp);
-    rmt_count_launches(1);
-  }
-}
-template <typename T>
 void launch_mac_setup(const Geo& g, T* const uf[3][3], MGVec b64, cudaStream_t s) {
   FacePtrs3 un;
   for (int d = 0; d < 3; d++) un.p[d] = uf[d][d];
@@ -801,10 +544,6 @@ void launch_fill(T* a, T v, long n, cudaStream_t s) {
 }
 
 #define INST(T)                                                                                                   \
-  template void launch_bar_states<T>(const Geo&, const T*, T* const[9], T* const[3][3], T* const[3], cudaStream_t); \
-  template void launch_face_states<T>(const Geo&, const T*, const T*, const T*, const T*, const Body*,          \
-                                      const BodyView<T>*, int, T* const[9],                                   \
-                                      T* const[9], T* const[3][3], T* const[3], T* const[3][3], cudaStream_t);   \
   template void launch_mac_setup<T>(const Geo&, T* const[3][3], MGVec, cudaStream_t);                            \
   template void launch_mac_correct<T>(const Geo&, T* const[3][3], const T*, MGVec, T* const[3],                 \
                                       cudaStream_t);                                                             \

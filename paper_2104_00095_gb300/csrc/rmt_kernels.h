@@ -73,17 +73,13 @@ cudaError_t launch_stress_div(const Geo& g, const T* u, const Body* bodies, cons
                               const int* bbs, int bstride, const double* t, double toff, T* out, const StressList& L,
                               T* const rows[9], cudaStream_t s);
 void launch_tick(double* t, double dt, cudaStream_t s);
-// slopes: nine cell arrays, written by launch_bar_states (limited slope of u_a along d at 3d+a)
-// and read by launch_face_states
+// advecting velocities of the bar states and the upwinded face states of the velocity; bodies / views / nb: the
+// bodies at step n, for the wall-repulsion term of the forcing.  slopes, wcell (nine cell arrays each) and ubar
+// are scratch of the FP64 form; the FP32 form needs none
 template <typename T>
-void launch_bar_states(const Geo& g, const T* u, T* const slopes[9], T* const ubar[3][3], T* const vadv[3],
-                       cudaStream_t s);
-// wcell: nine cell arrays of scratch for the side-independent part of the face states
-template <typename T>
-// bodies / views / nb: the bodies at step n, for the wall-repulsion term of the forcing
-void launch_face_states(const Geo& g, const T* u, const T* p, const T* rho, const T* divtau, const Body* bodies,
-                        const BodyView<T>* views, int nb, T* const slopes[9], T* const wcell[9], T* const ubar[3][3],
-                        T* const vadv[3], T* const uf[3][3], cudaStream_t s);
+cudaError_t launch_godunov(const Geo& g, const T* u, const T* p, const T* rho, const T* divtau, const Body* bodies,
+                           const BodyView<T>* views, int nb, T* const vadv[3], T* const uf[3][3], T* const slopes[9],
+                           T* const wcell[9], T* const ubar[3][3], cudaStream_t s);
 template <typename T>
 void launch_mac_setup(const Geo& g, T* const uf[3][3], MGVec b, cudaStream_t s);
 template <typename T>

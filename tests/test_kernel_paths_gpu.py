@@ -116,3 +116,24 @@ def test_extrapolation_of_unequal_bodies(layers, periodic, precision):
             assert np.array_equal(g.read(rmt.RMT_F_LAYER, m), o.read(O.F_LAYER, m))
             assert rel_l2(g.read(rmt.RMT_F_XI, m), o.read(O.F_XI, m)) <= 1e-5
     g.close()
+
+
+@pytest.mark.parametrize("n,periodic,precision", [((30, 12, 20), True, "fp32"), ((31, 13, 9), False, "fp32"),
+                                                  ((62, 8, 44), True, "fp32"), ((4, 5, 6), False, "fp32"),
+                                                  ((59, 6, 8), False, "fp32"), ((33, 9, 17), False, "fp64")])
+def test_godunov_states_at_tile_edges(n, periodic, precision):
+    """Face states where tiles of 30 x 6 columns end at, before and after the grid's last faces, against the
+    oracle's (FP32 after one step from the same fields: rounding of the fields and of some hundred operations)."""
+    sc = _box(n, periodic)
+    sc.update(precision=precision)
+    if precision == "fp32":
+        sc.update(mg_rtol=1e-6, mg_max_cycles=60)
+    g, o = pair(sc)
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    g.write(rmt.RMT_F_U, u)
+    assert o.write(O.F_U, u) == 0
+    g.step(1)
+    assert o.step(1) == 0, o.error()
+    for f, of in ((rmt.RMT_F_UFACE_X, O.F_UFACE_X), (rmt.RMT_F_UFACE_Y, O.F_UFACE_Y), (rmt.RMT_F_UFACE_Z, O.F_UFACE_Z)):
+        assert rel_l2(g.read(f), o.read(of)) <= (1e-12 if precision == "fp64" else 1e-5)
+    g.close()
