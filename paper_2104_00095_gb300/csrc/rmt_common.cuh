@@ -336,20 +336,28 @@ __device__ __forceinline__ T dheavi(T phi, T eps) {
 // Fourth-order monotonicity-limited slope (after Colella 1990); q[0..4] = q_{i-2..i+2}.
 // Missing outer values fall back to the second-order limited slope, a missing inner
 // neighbour gives zero.
-// The limiters choose by sign and magnitude.  In FP64 both are read from the bits, as integers: the FP64 units
-// issue a warp's compare or minimum in 16 cycles, the integer units in one or two.  (Magnitudes order as their
-// bits do; a NaN's lie above those of infinity.)
-__device__ __forceinline__ unsigned long long mag_bits(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+// The limiters choose by sign and magnitude.  In FP64 both are read from the bits, with integer additions and
+// masks: the FP64 units issue a warp's compare or minimum in 16 cycles, the integer units in one or two.
+// (Magnitudes order as their bits do; a NaN's lie above those of infinity.)
+__device__ __forceinline__ long long mag_bits(double x) {
+  // spelled out: the compiler turns a masked sign bit back into an FP64 absolute value
+  long long r;
+  asm("{\n\t.reg .b32 lo, hi;\n\tmov.b64 {lo, hi}, %1;\n\tand.b32 hi, hi, 0x7fffffff;\n\tmov.b64 %0, {lo, hi};\n\t}"
+      : "=l"(r)
+      : "d"(x));
+  return r;
+}
+__device__ __forceinline__ long long mag_min(long long a, long long b) {
+  return b ^ ((a ^ b) & ((a - b) >> 63));
 }
 // the smaller magnitude of the two one-sided differences where they agree in sign, else zero
 template <typename T>
 __device__ __forceinline__ T mc_min(T qm, T q0, T qp) {
   const T a = qp - q0, b = q0 - qm;
   if constexpr (sizeof(T) == 8) {
-    const unsigned long long ma = mag_bits(a), mb = mag_bits(b);
-    const bool same = (__double2hiint(a) ^ __double2hiint(b)) >= 0 && max(ma, mb) <= 0x7ff0000000000000ull;
-    return __longlong_as_double((long long)(same ? min(ma, mb) : 0ull));
+    const long long ma = mag_bits(a), mb = mag_bits(b), inf = 0x7ff0000000000000ll;
+    const long long none = ((__double_as_longlong(a) ^ __double_as_longlong(b)) | (inf - ma) | (inf - mb)) >> 63;
+    return __longlong_as_double(mag_min(ma, mb) & ~none);
   } else {
     return (a * b > T(0)) ? fmin(fabs(a), fabs(b)) : T(0);
   }
@@ -359,8 +367,8 @@ __device__ __forceinline__ T mc_min(T qm, T q0, T qp) {
 template <typename T>
 __device__ __forceinline__ T sgn_min(T s, T x, T y) {
   if constexpr (sizeof(T) == 8) {
-    const unsigned long long sign = (unsigned long long)__double_as_longlong(s) & 0x8000000000000000ull;
-    return __longlong_as_double((long long)(min(mag_bits(x), mag_bits(y)) | sign));
+    const long long sign = __double_as_longlong(s) & (long long)0x8000000000000000ull;
+    return __longlong_as_double(mag_min(mag_bits(x), mag_bits(y)) | sign);
   } else {
     return copysign(fmin(fabs(x), y), s);
   }
