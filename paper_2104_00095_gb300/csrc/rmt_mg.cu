@@ -895,27 +895,40 @@ __global__ void __launch_bounds__(BX* BYMAX) k_fe_dinv(Lv L, const double* __res
 // wall carry beta = 0, which makes the stencil uniform (the clamped x of an outside node always
 // meets a zero weight).  MODE 0: weighted Jacobi, out = x + w (b - K x) / diag (x where
 // diag = 0); MODE 1: residual, out = b - K x.
-// VEC (FP32, periodic x with n_x % 4 == 0): planes arrive as 16-byte rows, one copy per thread
+// STG 1 (FP32, periodic x with n_x % 4 == 0): planes arrive as 16-byte rows, one copy per thread
 // per plane (x rows widened to 4 halo nodes on each side, beta rows to 4 halo cells on the left)
 // instead of one 4-byte copy per element.
+// STG 2 (FP32, walls in x): rows of n_x + 1 nodes start at every alignment, so a row is staged from
+// the 16-byte boundary at or below its window, and its reader shifts by the same remainder (plane and
+// row each give theirs); what lies beyond a row's ends is its neighbour row's or zero and meets zero
+// weights (cells beyond a wall are masked when read).  A ninth warp has a node column of its own, the
+// last one of a grid of 32 m + 1 nodes.  The FE solve of a step (four cycles) on 129^3 nodes, element by element
+// and so: 1224 -> 975 us, on 49^3 477 -> 429 us.
 constexpr int FX = 32, FY = 8, FZ = 32, RING = 5;
 constexpr int XH = (FX + 2) * (FY + 2) - FX * FY;  // halo nodes of an x plane (84)
 constexpr int BH = (FX + 1) * (FY + 1) - FX * FY;  // halo cells of a beta plane (41)
 constexpr int VXC = (FX + 8) / 4, VBC = (FX + 4) / 4, VRC = FX / 4;  // 16-byte chunks per staged row (VEC)
 constexpr int VNX = (FY + 2) * VXC, VNR = FY * VRC, VNB = (FY + 1) * VBC;  // chunks per plane (VEC)
 static_assert(VNX + VNR + VNB <= FX * FY, "one staged chunk per thread and plane");
-template <typename T, int MODE, bool VEC = false>
-__global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restrict__ x, T* __restrict__ out,
+constexpr int SXC = (FX + 3 + 3 + 3) / 4, SRC = (FX + 1 + 3 + 3) / 4, SBC = (FX + 2 + 3 + 3) / 4;  // (STG 2)
+constexpr int SNX = (FY + 2) * SXC, SNR = FY * SRC, SNB = (FY + 1) * SBC;
+static_assert(SNX + SNR + SNB <= FX * (FY + 1), "one staged chunk per thread and plane");
+template <typename T, int MODE, int STG = 0>
+__global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T w, const T* __restrict__ x, T* __restrict__ out,
                                                     const T* __restrict__ b, const T* __restrict__ beta,
                                                     const T* __restrict__ dinv) {
   wait_prior();
-  static_assert(!VEC || sizeof(T) == 4, "16-byte rows of floats");
-  constexpr int XW = VEC ? FX + 8 : FX + 2, BW = VEC ? FX + 4 : FX + 1;  // staged row lengths
+  static_assert(!STG || sizeof(T) == 4, "16-byte rows of floats");
+  constexpr bool VEC = STG == 1;
+  constexpr int XW = STG == 2 ? 4 * SXC : (VEC ? FX + 8 : FX + 2);  // staged row lengths
+  constexpr int BW = STG == 2 ? 4 * SBC : (VEC ? FX + 4 : FX + 1), RW = STG == 2 ? 4 * SRC : FX;
   constexpr int XO = VEC ? 3 : 0, BO = VEC ? 3 : 0;  // column of node i0-1 / cell i0-1
   __shared__ __align__(16) T xs[RING][FY + 2][XW];
   __shared__ __align__(16) T bs[RING][FY + 1][BW];
-  __shared__ __align__(16) T rs[RING][FY][FX];  // right-hand side b of the tile's nodes
-  const int tx = threadIdx.x, ty = threadIdx.y, t = ty * FX + tx;
+  __shared__ __align__(16) T rs[RING][FY][RW];  // right-hand side b of the tile's nodes
+  const int t = threadIdx.y * FX + threadIdx.x;
+  const bool last_col = STG == 2 && threadIdx.y == FY;  // the ninth warp: rows of the column FX
+  const int tx = last_col ? FX : threadIdx.x, ty = last_col ? threadIdx.x & (FY - 1) : threadIdx.y;
   const int i0 = blockIdx.x * FX, j0 = blockIdx.y * FY;
   const int fz = (L.nn[2] + (int)gridDim.z - 1) / (int)gridDim.z;  // planes per block (FZ, or fewer on small levels)
   const int k0 = blockIdx.z * fz, k1 = min(k0 + fz, L.nn[2]);
@@ -986,6 +999,61 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
       vslot = (size_t)(FY + 1) * BW;
     }
   }
+  // STG 2: this thread's chunk of its array's planes: its row's first element in plane 0, how far along it lies, the
+  // plane's and the array's lengths, the plane to copy next and its shared address; and the remainders that the
+  // thread's own rows add to a plane's when it reads: x (bits 0-5), beta (6-9), b (10-11)
+  const T* ssrc = nullptr;
+  int soff = 0, scc = 0, sstride = 0, slen = 0, splanes = 0, snext = k0 - 1;
+  unsigned sdst = 0, sbytes = 0, rxb = 0;
+  int sslot = 0;
+  const int szi = L.nn[0] * L.nn[1], czi = L.n[0] * L.n[1];
+  if constexpr (STG == 2) {
+    const int syi = L.nn[0], cyi = L.n[0];
+    sstride = szi;
+    slen = (int)L.nnode;
+    splanes = L.nn[2];
+    if (t < SNX) {
+      const int r = t / SXC;
+      ssrc = x;
+      scc = 4 * (t % SXC);
+      soff = nnb(L, 1, j0 - 1 + r) * syi + i0 - 1;
+      sdst = (unsigned)__cvta_generic_to_shared(&xs[0][r][scc]);
+      sbytes = sizeof(xs[0]);
+    } else if (t < SNX + SNR) {
+      const int u = t - SNX, r = u / SRC;
+      ssrc = b;
+      scc = 4 * (u % SRC);
+      soff = nnb(L, 1, j0 + r) * syi + i0;
+      sdst = (unsigned)__cvta_generic_to_shared(&rs[0][r][scc]);
+      sbytes = sizeof(rs[0]);
+    } else if (t < SNX + SNR + SNB) {
+      const int u = t - SNX - SNR, r = u / SBC, cj = cnb(L, 1, j0 - 1 + r);
+      ssrc = beta;
+      scc = 4 * (u % SBC);
+      soff = max(cj, 0) * cyi + i0 - 1;
+      sstride = czi;
+      slen = cj >= 0 ? (int)L.ncell : 0;  // a row beyond a wall is zeros
+      splanes = L.n[2];
+      sdst = (unsigned)__cvta_generic_to_shared(&bs[0][r][scc]);
+      sbytes = sizeof(bs[0]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) rxb |= (unsigned)((nnb(L, 1, j0 - 1 + ty + c) * syi + i0 - 1) & 3) << (2 * c);
+#pragma unroll
+    for (int c = 0; c < 2; c++) rxb |= (unsigned)((max(cnb(L, 1, j0 - 1 + ty + c), 0) * cyi + i0 - 1) & 3) << (6 + 2 * c);
+    rxb |= (unsigned)((nnb(L, 1, j0 + ty) * syi + i0) & 3) << 10;
+  }
+  auto copy_next = [&]() {  // the next plane of this thread's chunk; planes beyond a wall are zeros
+    if (ssrc) {
+      const int pz = !L.per[2] ? snext : (snext < 0 ? snext + splanes : (snext >= splanes ? snext - splanes : snext));
+      const int at = ((pz * sstride + soff) & ~3) + scc;  // from the 16-byte boundary at or below the row's first element
+      const int len = pz >= 0 && pz < splanes && at >= 0 ? min(max(slen - at, 0), 4) : 0;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sdst + sslot * sbytes),
+                   "l"(ssrc + (len > 0 ? at : 0)), "r"(4 * len));
+      snext++;
+      sslot = sslot + 1 == RING ? 0 : sslot + 1;
+    }
+  };
   auto cp16 = [&](T* dst, const T* src, bool valid) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(src), "r"(valid ? 16 : 0));
@@ -1014,20 +1082,33 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
     }
   };
   // group 0: x planes k0-1 .. k0+1, cell planes k0-1, k0; then one group per further plane
-  issue_x(k0 - 1);
-  issue_x(k0);
-  issue_x(k0 + 1);
-  issue_b(k0 - 1);
-  issue_b(k0);
-  cp_async_commit();
-  issue_x(k0 + 2);
-  issue_b(k0 + 1);
-  cp_async_commit();
-  issue_x(k0 + 3);
-  issue_b(k0 + 2);
-  cp_async_commit();
+  if constexpr (STG == 2) {
+    copy_next();
+    copy_next();
+    if (t < SNX + SNR) copy_next();  // x and b run one plane ahead of beta; b begins at plane k0 - 1 too
+    cp_async_commit();
+    copy_next();
+    cp_async_commit();
+    copy_next();
+    cp_async_commit();
+  } else {
+    issue_x(k0 - 1);
+    issue_x(k0);
+    issue_x(k0 + 1);
+    issue_b(k0 - 1);
+    issue_b(k0);
+    cp_async_commit();
+    issue_x(k0 + 2);
+    issue_b(k0 + 1);
+    cp_async_commit();
+    issue_x(k0 + 3);
+    issue_b(k0 + 2);
+    cp_async_commit();
+  }
   const int i = i0 + tx, j = j0 + ty;
-  const bool own = i < L.nn[0] && j < L.nn[1];
+  const bool own = i < L.nn[0] && j < L.nn[1] &&
+                   (!last_col || (threadIdx.x < FY && blockIdx.x == gridDim.x - 1 && i == L.nn[0] - 1));
+  const bool cell_lo = i > 0, cell_hi = i < L.n[0];  // the cells beside the node exist (STG 2)
   const T s12 = cv<T>(L.s12, L.f_s12);
   // Register window of the thread's column: three x planes (i-1..i+1, j-1..j+1) and two beta
   // cell planes (the cells around the node below / above it).  The window moves up one plane
@@ -1035,32 +1116,45 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
   // not DRAM, is the next limit of this kernel); the loop is unrolled so that the arrays change
   // roles instead of being copied.
   T Xa[3][3], Xb[3][3], Xc[3][3], Ba[2][2], Bb[2][2];
-  auto rd_x = [&](T (&P)[3][3], int slot) {
+  auto rd_x = [&](T (&P)[3][3], int slot, unsigned q) {  // q: the plane's remainder (STG 2)
 #pragma unroll
-    for (int c = 0; c < 3; c++)
+    for (int c = 0; c < 3; c++) {
+      const T* row = &xs[slot][ty + c][tx + XO + (STG == 2 ? ((rxb >> (2 * c)) + q) & 3u : 0u)];
 #pragma unroll
-      for (int a = 0; a < 3; a++) P[c][a] = xs[slot][ty + c][tx + XO + a];
+      for (int a = 0; a < 3; a++) P[c][a] = row[a];
+    }
   };
-  auto rd_b = [&](T (&P)[2][2], int slot) {
+  auto rd_b = [&](T (&P)[2][2], int slot, unsigned q) {
 #pragma unroll
-    for (int c = 0; c < 2; c++)
+    for (int c = 0; c < 2; c++) {
+      const T* row = &bs[slot][ty + c][tx + BO + (STG == 2 ? ((rxb >> (6 + 2 * c)) + q) & 3u : 0u)];
 #pragma unroll
-      for (int a = 0; a < 2; a++) P[c][a] = bs[slot][ty + c][tx + BO + a];
+      for (int a = 0; a < 2; a++) P[c][a] = STG != 2 || (a ? cell_hi : cell_lo) ? row[a] : T(0);
+    }
   };
   const long ubase = (long)i + (long)j * sy;
   int k = k0;
   int sxp = 2, sbc = 1;  // ring slots of x plane k+1 and of cell plane k
+  unsigned qx = (unsigned)(k0 * szi), qb = (unsigned)(k0 * czi);  // (STG 2) of x plane k, of cell plane k
   // one plane: M, C, P = x planes k-1, k, k+1 (P is filled here), Bl, Bu = cell planes k-1, k
   // (Bu is filled here)
   auto plane = [&](T (&M)[3][3], T (&C)[3][3], T (&P)[3][3], T (&Bl)[2][2], T (&Bu)[2][2]) {
     cp_async_wait<2>();  // x plane k+1 and cell plane k have landed (two newer groups may fly)
     __syncthreads();     // ... for every thread; the slots refilled below were last read at
                          // least one iteration ago, before this barrier
-    rd_x(P, sxp);
-    rd_b(Bu, sbc);
-    const T bcur = rs[sxp == 0 ? RING - 1 : sxp - 1][ty][tx];  // b of plane k (slot before k+1)
-    issue_x(k + 4);
-    issue_b(k + 3);
+    const unsigned qr = qx;  // of plane k
+    qx = k + 1 == L.nn[2] ? 0u : qx + (unsigned)szi;
+    rd_x(P, sxp, qx);
+    rd_b(Bu, sbc, qb);
+    qb += (unsigned)czi;
+    // b of plane k (slot before k+1)
+    const T bcur = rs[sxp == 0 ? RING - 1 : sxp - 1][ty][tx + (STG == 2 ? ((rxb >> 10) + qr) & 3u : 0u)];
+    if constexpr (STG == 2) {
+      copy_next();
+    } else {
+      issue_x(k + 4);
+      issue_b(k + 3);
+    }
     cp_async_commit();
     sxp = sxp + 1 == RING ? 0 : sxp + 1;
     sbc = sbc + 1 == RING ? 0 : sbc + 1;
@@ -1109,9 +1203,9 @@ __global__ void __launch_bounds__(FX* FY) k_fe_tile(Lv L, T w, const T* __restri
   // planes k0-1, k0 and cell plane k0-1 start the window
   cp_async_wait<2>();
   __syncthreads();
-  rd_x(Xa, 0);
-  rd_x(Xb, 1);
-  rd_b(Ba, 0);
+  rd_x(Xa, 0, (unsigned)((k0 > 0 ? k0 - 1 : L.nn[2] - 1) * szi));
+  rd_x(Xb, 1, qx);
+  rd_b(Ba, 0, (unsigned)((k0 > 0 ? k0 - 1 : L.n[2] - 1) * czi));
   while (k < k1) {
     plane(Xa, Xb, Xc, Ba, Bb);
     if (k >= k1) break;
@@ -1953,22 +2047,38 @@ void sum_ff(MGSolver* m, const float* h, const float* l, long n, double scale, d
   rmt_count_launches(1);
 }
 
-// the FE tile kernel stages 16-byte rows on FP32 levels with a periodic x axis of n_x % 4 == 0
+// How the FE tile kernel stages a level's planes: FP32 levels as 16-byte rows, aligned ones with a periodic x axis of
+// n_x % 4 == 0, shifted ones with walls in x; element by element otherwise (a periodic row of another length wraps
+// inside a copy; FP64 is bound by its arithmetic)
 template <typename T>
-inline bool fe_vec(const Lv& L) {
-  return sizeof(T) == 4 && L.per[0] && L.n[0] % 4 == 0;
+inline int fe_staging(const Lv& L) {
+  return sizeof(T) == 4 ? (L.per[0] ? (L.n[0] % 4 == 0 ? 1 : 0) : 2) : 0;
 }
-inline dim3 fe_grid(const Lv& L, int zchunk = 0) {
+inline dim3 fe_grid(const Lv& L, int zchunk = 0, int stg = 0) {
   // z-chunks of FZ planes, or more and shorter chunks on small levels, so that at least two
   // blocks per SM march concurrently (a block's planes follow one another); zchunk > 0 sets the
   // chunk length instead (the autotuner's choice); the kernel takes its chunk from the grid
-  const int tx = (L.nn[0] + FX - 1) / FX, ty = (L.nn[1] + FY - 1) / FY;
+  // (STG 2 blocks hold one more column: the last of 32 m + 1)
+  const int tx = stg == 2 && L.nn[0] > FX && L.nn[0] % FX == 1 ? L.nn[0] / FX : (L.nn[0] + FX - 1) / FX;
+  const int ty = (L.nn[1] + FY - 1) / FY;
   int nch = (L.nn[2] + FZ - 1) / FZ;
   const int want = (2 * sm_count() + tx * ty - 1) / (tx * ty);
   if (want > nch) nch = want < L.nn[2] ? want : L.nn[2];
   if (zchunk > 0) nch = (L.nn[2] + zchunk - 1) / zchunk;
   const int fz = (L.nn[2] + nch - 1) / nch;
   return dim3(tx, ty, (L.nn[2] + fz - 1) / fz);
+}
+
+template <typename T, int MODE>
+void launch_fe_tile(const Lv& L, int zchunk, T w, const T* x, T* out, const T* b, const T* beta, const T* dinv,
+                    cudaStream_t s) {
+  const int stg = fe_staging<T>(L);
+  const dim3 grid = fe_grid(L, zchunk, stg);
+  if constexpr (sizeof(T) == 4) {
+    if (stg == 1) return launch_after(k_fe_tile<T, MODE, 1>, grid, dim3(FX, FY), 0, s, L, w, x, out, b, beta, dinv);
+    if (stg == 2) return launch_after(k_fe_tile<T, MODE, 2>, grid, dim3(FX, FY + 1), 0, s, L, w, x, out, b, beta, dinv);
+  }
+  launch_after(k_fe_tile<T, MODE, 0>, grid, dim3(FX, FY), 0, s, L, w, x, out, b, beta, dinv);
 }
 
 template <typename T>
@@ -2010,14 +2120,8 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
       }
     } else {
       hk(m, l, 0, 1, s);
-      const dim3 fg = fe_grid(L, l == 0 ? m->fe_zc0 : 0);
-      if (fe_vec<T>(L))
-        launch_after(k_fe_tile<float, 0, true>, fg, dim3(FX, FY), 0, s, L, (float)m->omega, (const float*)m->x[l],
-                                                                      (float*)m->xt[l], (const float*)b,
-                                                                      (const float*)rho, nullptr);
-      else
-        launch_after(k_fe_tile<T, 0>, fg, dim3(FX, FY), 0, s, L, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
-                                                    (const T*)m->dinv[l]);
+      launch_fe_tile<T, 0>(L, l == 0 ? m->fe_zc0 : 0, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
+                           (const T*)m->dinv[l], s);
       rmt_count_launches(1);
       hk(m, l, 0, 0, s);
       void* t = m->x[l];
@@ -2060,13 +2164,8 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
           L, C, (const T*)m->x[l], (const T*)m->b[l], mac_coef(m, l), (T*)m->b[l + 1], (T*)m->x[l + 1]);
     rmt_count_launches(1);
   } else {
-    const dim3 fg = fe_grid(L, l == 0 ? m->fe_zc0 : 0);
-    if (fe_vec<T>(L))
-      launch_after(k_fe_tile<float, 1, true>, fg, dim3(FX, FY), 0, s, L, 0.f, (const float*)m->x[l], (float*)m->r[l],
-                                                                    (const float*)m->b[l], (const float*)m->rho[l], nullptr);
-    else
-      launch_after(k_fe_tile<T, 1>, fg, dim3(FX, FY), 0, s, L, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l],
-                                                         (const T*)m->rho[l], nullptr);
+    launch_fe_tile<T, 1>(L, l == 0 ? m->fe_zc0 : 0, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l],
+                         (const T*)m->rho[l], (const T*)nullptr, s);
     rmt_count_launches(1);
     const int zc = column_chunk(C.nnode, RZ);
     launch_after(k_restrict<T>, grid3(C.nn[0], C.nn[1], (C.nn[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s, 
@@ -2262,7 +2361,7 @@ void mg_set_zchunk(MGSolver* m, int zchunk) {
 int mg_zchunk(const MGSolver* m) {
   if (m->kind == 0) return mac_fused0(m) ? m->zc[0] : 0;
   const Lv& L = m->lv[0];
-  const dim3 g = fe_grid(L, m->fe_zc0);
+  const dim3 g = fe_grid(L, m->fe_zc0, m->fp32 ? fe_staging<float>(L) : 0);
   return (L.nn[2] + (int)g.z - 1) / (int)g.z;
 }
 

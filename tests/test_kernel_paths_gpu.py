@@ -137,3 +137,20 @@ def test_godunov_states_at_tile_edges(n, periodic, precision):
     for f, of in ((rmt.RMT_F_UFACE_X, O.F_UFACE_X), (rmt.RMT_F_UFACE_Y, O.F_UFACE_Y), (rmt.RMT_F_UFACE_Z, O.F_UFACE_Z)):
         assert rel_l2(g.read(f), o.read(of)) <= (1e-12 if precision == "fp64" else 1e-5)
     g.close()
+
+
+@pytest.mark.parametrize("n", [(32, 30, 34), (33, 30, 32), (64, 40, 36), (34, 62, 30), (47, 33, 39)])
+def test_fe_solve_with_walls_fp32(n):
+    """Walled FE levels whose rows end at, before and after the last block's columns and begin at every alignment:
+    the FP32 form's solves take the cycles of the FP64 form's and reach its velocities to FP32 accuracy."""
+    out = []
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    for prec in ("fp64", "fp32"):
+        g = rmt.Grid(dict(_box(n, False), precision=prec, mg_rtol=1e-9, mg_max_cycles=60))
+        g.write(rmt.RMT_F_U, u)
+        g.step(1)
+        out.append((g.read(rmt.RMT_F_U), g.cycles()))
+        g.close()
+    (u64, c64), (u32, c32) = out
+    assert rel_l2(u32, u64) <= 1e-5
+    assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)

@@ -306,3 +306,62 @@ def test_fe_tile_16_byte_staging_covers_the_window(nn, ny, i0, j0):
         for c, a in itertools.product(range(2), range(2)):
             assert 0 <= ty + c < FY + 1 and 0 <= tx + 3 + a < FX + 4
             assert (i0 - 4 + tx + 3 + a) == i0 + tx - 1 + a  # cell i-1+a
+
+
+SXC, SRC, SBC = (FX + 9) // 4, (FX + 7) // 4, (FX + 8) // 4
+SNX, SNR, SNB = (FY + 2) * SXC, FY * SRC, (FY + 1) * SBC
+
+
+@pytest.mark.parametrize("n,pery", [((32, 9, 3), False), ((33, 8, 4), True), ((64, 7, 2), False), ((7, 6, 5), True),
+                                    ((31, 17, 3), False), ((6, 5, 4), False)])
+def test_fe_tile_shifted_staging_reads_the_window(n, pery):
+    """Walls along x, rows of n0 + 1 nodes at every alignment: each staged row begins at the 16-byte boundary at or
+    below its window.  Every source lies in its array, every node has one owner, and the owner's window holds its
+    neighbours or, beyond a wall, cells of weight zero."""
+    n0, n1, n2 = n
+    nn = (n0 + 1, n1 if pery else n1 + 1, n2 + 1)
+    nnode, ncell = nn[0] * nn[1] * nn[2], n0 * n1 * n2
+    assert SNX + SNR + SNB <= FX * (FY + 1)
+    nnb = lambda d, v: ((nn[d] - 1 if v < 0 else 0 if v >= nn[d] else v) if (pery and d == 1)
+                        else min(max(v, 0), nn[d] - 1))
+    cnb = lambda d, v: (v % n[d] if (pery and d == 1 and (v < 0 or v >= n[d])) else v if 0 <= v < n[d] else -1)
+    owners = np.zeros(nn, int)
+    tiles = nn[0] // FX if nn[0] > FX and nn[0] % FX == 1 else -(-nn[0] // FX)
+
+    def stage(rows, chunks, first, size, valid):
+        out = np.zeros((rows, 4 * chunks), int)  # element id + 1; 0 where nothing is copied
+        for r, c in itertools.product(range(rows), range(chunks)):
+            at = first(r) - (first(r) & 3) + 4 * c
+            k = min(size - at, 4) if valid(r) and 0 <= at < size else 0
+            for e in range(max(k, 0)):
+                assert 0 <= at + e < size
+                out[r, 4 * c + e] = at + e + 1
+        return out
+
+    for bx, j0 in itertools.product(range(tiles), range(0, nn[1], FY)):
+        i0 = bx * FX
+        for k in range(nn[2]):
+            xrow = lambda r, p: nnb(2, p) * nn[0] * nn[1] + nnb(1, j0 - 1 + r) * nn[0] + i0 - 1
+            crow = lambda r, p: max(cnb(2, p), 0) * n0 * n1 + max(cnb(1, j0 - 1 + r), 0) * n0 + i0 - 1
+            xs = {p: stage(FY + 2, SXC, lambda r: xrow(r, p), nnode, lambda r: True) for p in (k - 1, k, k + 1)}
+            bs = {p: stage(FY + 1, SBC, lambda r: crow(r, p), ncell,
+                           lambda r: cnb(1, j0 - 1 + r) >= 0 and cnb(2, p) >= 0) for p in (k - 1, k)}
+            rrow = lambda r: nnb(2, k) * nn[0] * nn[1] + nnb(1, j0 + r) * nn[0] + i0
+            rs = stage(FY, SRC, rrow, nnode, lambda r: True)
+            for tx, ty in itertools.product(range(FX + 1), range(FY)):
+                i, j = i0 + tx, j0 + ty
+                if i >= nn[0] or j >= nn[1] or (tx == FX and not (bx == tiles - 1 and i == nn[0] - 1)):
+                    continue
+                owners[i, j, k] += 1
+                node = lambda a, b, c: a + nn[0] * (nnb(1, b) + nn[1] * nnb(2, c)) + 1
+                assert rs[ty, tx + (rrow(ty) & 3)] == node(i, j, k)
+                for a, c, p in itertools.product(range(3), range(3), (k - 1, k, k + 1)):
+                    got = xs[p][ty + c, tx + a + (xrow(ty + c, p) & 3)]
+                    if 0 <= i - 1 + a < nn[0]:
+                        assert got == node(i - 1 + a, j - 1 + c, p)
+                for a, c, p in itertools.product(range(2), range(2), (k - 1, k)):
+                    got = bs[p][ty + c, tx + a + (crow(ty + c, p) & 3)] if (i < n0 if a else i > 0) else 0
+                    ci, cj, ck = i - 1 + a, cnb(1, j - 1 + c), cnb(2, p)
+                    want = ci + n0 * (cj + n1 * ck) + 1 if 0 <= ci < n0 and cj >= 0 and ck >= 0 else 0
+                    assert got == want
+    assert (owners == 1).all()
