@@ -1523,74 +1523,85 @@ __global__ void __launch_bounds__(BX* BYMAX) k_coarsen(Lv F, Lv C, const T* __re
   rc[cix(C, I, J, K)] = T(0.125) * s;
 }
 
-// sum (mode 0) or sum of squares (mode 1): per-block partials
+// Sums of a solve.  The last block of a pass adds the blocks' partial sums itself, in their order, so that a mean
+// takes one launch, and by shuffles (48^3, cold caches: 7.7 us for a mean; a launch for each half and a barrier for
+// each halving 11.3 us).
+struct SumOut {
+  double scale;
+  double* out;       // scale * sum
+  float* out_ff;     // the same value as a two-float pair, or null
+  int* nonfinite;    // set by a non-finite result, or null: every solve takes the mean of its right-hand side and of
+                     // its solution, so a NaN or infinity anywhere in the velocity that feeds them is caught here
+  unsigned* ticket;  // counts the blocks of a pass; 0 between passes
+};
+// the block's sum of loc, in thread 0 (FP64 across threads, at most 32 warps)
+__device__ __forceinline__ double block_sum(double loc) {
+  __shared__ double sh[32];
+  for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = loc;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    loc = threadIdx.x < blockDim.x / 32 ? sh[threadIdx.x] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
+  }
+  __syncthreads();
+  return loc;
+}
+__device__ __forceinline__ void final_sum(const double* part, int np, const SumOut& o) {
+  double loc = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) loc += __ldcg(part + i);
+  loc = block_sum(loc);
+  if (threadIdx.x == 0) {
+    const double v = loc * o.scale;
+    *o.out = v;
+    if (o.nonfinite && !isfinite(v)) *o.nonfinite = 1;
+    if (o.out_ff) {
+      o.out_ff[0] = (float)v;
+      o.out_ff[1] = (float)(v - (double)o.out_ff[0]);
+    }
+  }
+}
+__device__ __forceinline__ void finish_sum(double loc, double* part, const SumOut& o) {
+  __shared__ bool last;
+  const double s = block_sum(loc);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = s;
+    __threadfence();
+    last = atomicInc(o.ticket, gridDim.x - 1) == gridDim.x - 1;  // the last one winds it back to 0
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    final_sum(part, gridDim.x, o);
+  }
+}
+// sum of a (mode 1: of a^2)
 template <typename XT>
-__global__ void k_partial(const XT* __restrict__ a, long n, int mode, double* __restrict__ part) {
+__global__ void k_sum(const XT* __restrict__ a, long n, int mode, double* __restrict__ part, SumOut o) {
   wait_prior();
-  __shared__ double sh[TPB / 32];
   double loc = 0.0;
   GRID_LOOP(i, n) {
     const double v = (double)a[i];
     loc += mode ? v * v : v;
   }
-  for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = loc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < TPB / 32; w++) s += sh[w];
-    part[blockIdx.x] = s;
-  }
+  finish_sum(loc, part, o);
 }
-
-// final fixed-order sum of the partials (one block); out = scale * sum; a non-finite result
-// sets *nonfinite (when given): every solve takes the mean of its right-hand side and of its
-// solution, so a NaN or infinity anywhere in the velocity that feeds them is caught here
-__global__ void __launch_bounds__(1024) k_final(const double* __restrict__ part, int np, double scale,
-                                                double* __restrict__ out, float* __restrict__ out_ff,
-                                                int* __restrict__ nonfinite) {
+// sum of partial sums that another kernel left (one block)
+__global__ void __launch_bounds__(1024) k_final(const double* __restrict__ part, int np, SumOut o) {
   wait_prior();
-  __shared__ double sh[1024];
-  double loc = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) loc += part[i];
-  sh[threadIdx.x] = loc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double v = sh[0] * scale;
-    *out = v;
-    if (nonfinite && !isfinite(v)) *nonfinite = 1;
-    if (out_ff) {  // the same value as a two-float pair
-      out_ff[0] = (float)v;
-      out_ff[1] = (float)(v - (double)out_ff[0]);
-    }
-  }
+  final_sum(part, np, o);
 }
-
-// per-block partial sums of the two-float array h + l (l null: all zero): two-float
-// accumulation per thread, FP64 across threads
-__global__ void k_partial_ff(const float* __restrict__ h, const float* __restrict__ l, long n,
-                             double* __restrict__ part) {
+// sum of the two-float array h + l (l null: all zero): two-float accumulation per thread, FP64 across threads
+__global__ void k_sum_ff(const float* __restrict__ h, const float* __restrict__ l, long n, double* __restrict__ part,
+                         SumOut o) {
   wait_prior();
-  __shared__ double sh[TPB / 32];
   float ah = 0.0f, al = 0.0f;
   GRID_LOOP(i, n) {
     const F2 t = two_sum(ah, h[i]);
     ah = t.h;
     al = __fadd_rn(al, __fadd_rn(t.l, l ? l[i] : 0.0f));
   }
-  double loc = (double)ah + (double)al;
-  for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = loc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < TPB / 32; w++) s += sh[w];
-    part[blockIdx.x] = s;
-  }
+  finish_sum((double)ah + (double)al, part, o);
 }
 
 // (h, l) = (e, 0) - m: the two-float solution from a single FP32 solve, mean-free
@@ -1904,7 +1915,7 @@ MGSolver* mg_build(const Geo& g, int kind, int prec_fp32, bool dry, cudaError_t*
     alloc((void**)&m->bl, L0.nunk * sizeof(float));
   }
   alloc((void**)&m->part, (size_t)(nbr > RED_BLOCKS ? nbr : RED_BLOCKS) * sizeof(double));
-  alloc((void**)&m->scal, 8 * sizeof(double));
+  alloc((void**)&m->scal, 8 * sizeof(double));  // ([4]: the blocks counted in a sum)
   if (!dry) {
     if (e == cudaSuccess) e = cudaMallocHost((void**)&m->hpin, 8 * sizeof(double));
     // the coarsest level lives in shared memory during its solve (when it fits): opt in to its
@@ -2026,13 +2037,15 @@ inline void hk(MGSolver* m, int l, int which, int begin, cudaStream_t s) {
   if (m->hook && l == 0) m->hook(m->hook_ctx, which, begin, s);
 }
 
+inline SumOut sum_out(const MGSolver* m, double scale, double* out, float* out_ff) {
+  return {scale, out, out_ff, m->nonfinite, (unsigned*)(m->scal + 4)};
+}
+
 template <typename T>
 void sum_into(MGSolver* m, const T* a, long n, int mode, double scale, double* out, cudaStream_t s) {
   int nb = nblocks(n);
   if (nb > RED_BLOCKS) nb = RED_BLOCKS;
-  launch_after(k_partial<T>, nb, TPB, 0, s, a, n, mode, m->part);
-  rmt_count_launches(1);
-  launch_after(k_final, 1, 1024, 0, s, m->part, nb, scale, out, nullptr, m->nonfinite);
+  launch_after(k_sum<T>, nb, TPB, 0, s, a, n, mode, m->part, sum_out(m, scale, out, nullptr));
   rmt_count_launches(1);
 }
 
@@ -2041,9 +2054,7 @@ void sum_ff(MGSolver* m, const float* h, const float* l, long n, double scale, d
             cudaStream_t s) {
   int nb = nblocks(n);
   if (nb > RED_BLOCKS) nb = RED_BLOCKS;
-  launch_after(k_partial_ff, nb, TPB, 0, s, h, l, n, m->part);
-  rmt_count_launches(1);
-  launch_after(k_final, 1, 1024, 0, s, m->part, nb, scale, out, out_ff, m->nonfinite);
+  launch_after(k_sum_ff, nb, TPB, 0, s, h, l, n, m->part, sum_out(m, scale, out, out_ff));
   rmt_count_launches(1);
 }
 
@@ -2273,7 +2284,7 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
       hk(m, 0, 1, 0, s);
     }
     if (fixed_cycles <= 0) {
-      launch_after(k_final, 1, 1024, 0, s, m->part, nbr, 1.0, m->scal + 2, nullptr, m->nonfinite);
+      launch_after(k_final, 1, 1024, 0, s, m->part, nbr, sum_out(m, 1.0, m->scal + 2, nullptr));
       rmt_count_launches(1);
       cudaMemcpyAsync(m->hpin + 1, m->scal + 2, sizeof(double), cudaMemcpyDeviceToHost, s);
       if ((*err = cudaStreamSynchronize(s)) != cudaSuccess) return -1;
