@@ -101,8 +101,7 @@ struct rmt_grid {
   void *adv = nullptr, *ustar = nullptr, *psi = nullptr;
   void* vadv[3] = {};
   void* slopes[9] = {};
-  void* ub[3][3] = {};  // FP64: scratch of the Godunov passes
-  void* wcell[9] = {};
+  void* wcell[9] = {};  // FP64: scratch of the Godunov passes
   void* uf[3][3] = {};
   void* umac[3] = {};
   MGSolver* mac = nullptr;
@@ -467,7 +466,6 @@ rmt_status alloc_t(rmt_grid* g) {
     const long nf = nfaces(G, d);
     for (int a = 0; a < 3; a++) {
       AL(g->uf[d][a], nf * e);
-      if (e == 8) AL(g->ub[d][a], nf * e);
     }
     AL(g->vadv[d], nf * e);
     AL(g->umac[d], nf * e);
@@ -580,14 +578,12 @@ rmt_status step_t(rmt_grid* g) {
   const int cur = g->par, nxt = 1 - g->par;
   T* slopes[9];
   T* wcell[9];
-  T* ub[3][3];
   T* vadv[3];
   T* uf[3][3];
   T* umac[3];
   for (int d = 0; d < 3; d++) {
     for (int a = 0; a < 3; a++) {
       uf[d][a] = (T*)g->uf[d][a];
-      ub[d][a] = (T*)g->ub[d][a];
     }
     vadv[d] = (T*)g->vadv[d];
     umac[d] = (T*)g->umac[d];
@@ -605,7 +601,7 @@ rmt_status step_t(rmt_grid* g) {
   // 2. Godunov face states of u
   pb(g, P_GODUNOV);
   CK(g, launch_godunov<T>(G, u, (const T*)g->p, (const T*)g->rho, (const T*)g->divn, g->bodies_d,
-                          views<T>(g, cur, 0), nb, vadv, uf, slopes, wcell, ub, s));
+                          views<T>(g, cur, 0), nb, vadv, uf, slopes, wcell, s));
   pe(g, P_GODUNOV);
   // 3. MAC projection of the normal face velocities
   pb(g, P_MAC_SETUP);

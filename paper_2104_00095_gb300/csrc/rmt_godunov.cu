@@ -538,8 +538,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_face(Geo g, const double* __
 template <>
 cudaError_t launch_godunov<float>(const Geo& g, const float* u, const float* p, const float* rho, const float* divtau,
                                   const Body* bodies, const BodyView<float>* views, int nb, float* const vadv[3],
-                                  float* const uf[3][3], float* const[9], float* const[9], float* const[3][3],
-                                  cudaStream_t s) {
+                                  float* const uf[3][3], float* const[9], float* const[9], cudaStream_t s) {
   GodOut o;
   for (int d = 0; d < 3; d++) {
     o.vadv[d] = vadv[d];
@@ -571,7 +570,7 @@ template <>
 cudaError_t launch_godunov<double>(const Geo& g, const double* u, const double* p, const double* rho,
                                    const double* divtau, const Body* bodies, const BodyView<double>* views, int nb,
                                    double* const vadv[3], double* const uf[3][3], double* const slopes[9],
-                                   double* const wcell[9], double* const ubar[3][3], cudaStream_t s) {
+                                   double* const wcell[9], cudaStream_t s) {
   Slopes9 S, W;
   BarPtrs bp;
   for (int q = 0; q < 9; q++) {
@@ -591,9 +590,9 @@ cudaError_t launch_godunov<double>(const Geo& g, const double* u, const double* 
     // the direction is a template argument: a runtime index into the pointer bundles would
     // copy them to local memory in every thread
     auto kb = e == 0 ? k_bar<0> : (e == 1 ? k_bar<1> : k_bar<2>);
-    kb<<<grid(e), tile, 0, s>>>(g, u, S, ubar[e][0], ubar[e][1], ubar[e][2], vadv[e]);
+    kb<<<grid(e), tile, 0, s>>>(g, u, S, uf[e][0], uf[e][1], uf[e][2], vadv[e]);
     rmt_count_launches(1);
-    for (int a = 0; a < 3; a++) bp.ub[e][a] = ubar[e][a];
+    for (int a = 0; a < 3; a++) bp.ub[e][a] = uf[e][a];  // the bar states give way to the face states
     bp.vadv[e] = vadv[e];
   }
   k_cellw<<<gc, tile, 0, s>>>(g, u, p, rho, divtau, bp, W, bodies, views, nb);

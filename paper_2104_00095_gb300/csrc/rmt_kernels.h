@@ -74,12 +74,12 @@ cudaError_t launch_stress_div(const Geo& g, const T* u, const Body* bodies, cons
                               T* const rows[9], cudaStream_t s);
 void launch_tick(double* t, double dt, cudaStream_t s);
 // advecting velocities of the bar states and the upwinded face states of the velocity; bodies / views / nb: the
-// bodies at step n, for the wall-repulsion term of the forcing.  slopes, wcell (nine cell arrays each) and ubar
-// are scratch of the FP64 form; the FP32 form needs none
+// bodies at step n, for the wall-repulsion term of the forcing.  slopes and wcell (nine cell arrays each) are
+// scratch of the FP64 form; the FP32 form needs none
 template <typename T>
 cudaError_t launch_godunov(const Geo& g, const T* u, const T* p, const T* rho, const T* divtau, const Body* bodies,
                            const BodyView<T>* views, int nb, T* const vadv[3], T* const uf[3][3], T* const slopes[9],
-                           T* const wcell[9], T* const ubar[3][3], cudaStream_t s);
+                           T* const wcell[9], cudaStream_t s);
 template <typename T>
 void launch_mac_setup(const Geo& g, T* const uf[3][3], MGVec b, cudaStream_t s);
 template <typename T>

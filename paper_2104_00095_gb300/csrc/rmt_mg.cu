@@ -871,19 +871,27 @@ __global__ void __launch_bounds__(GT, 3) k_rbgs_sweep(Lv L, int c0, float w, con
   }
 }
 
-// FP64: 1 / diagonal of the 27-point operator at every node (0 where no cell touches it)
-__global__ void __launch_bounds__(BX* BYMAX) k_fe_dinv(Lv L, const double* __restrict__ beta, double* __restrict__ dinv) {
+// FP64 coefficients of the 27-point operator, formed once per solve: at every node 1 / diagonal (0 where no cell
+// touches it) and, per direction d, the sum of beta over the four cells around the edge to the next node along d
+__global__ void __launch_bounds__(BX* BYMAX) k_fe_coef(Lv L, const double* __restrict__ beta, double* __restrict__ e0,
+                                                     double* __restrict__ e1, double* __restrict__ e2,
+                                                     double* __restrict__ dinv) {
   wait_prior();
   const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   if (i >= L.nn[0] || j >= L.nn[1]) return;
-  double bs = 0.0;
+  double v[8];
 #pragma unroll
   for (int q = 0; q < 8; q++) {
     const int ci = cnb(L, 0, i - 1 + (q & 1)), cj = cnb(L, 1, j - 1 + ((q >> 1) & 1)), ck = cnb(L, 2, k - 1 + (q >> 2));
-    if (ci >= 0 && cj >= 0 && ck >= 0) bs += beta[cix(L, ci, cj, ck)];
+    v[q] = ci >= 0 && cj >= 0 && ck >= 0 ? beta[cix(L, ci, cj, ck)] : 0.0;
   }
-  const double diag = 4.0 * bs * L.s12;
-  dinv[nix(L, i, j, k)] = diag > 0.0 ? 1.0 / diag : 0.0;
+  const long u = nix(L, i, j, k);
+  const double lo = (v[0] + v[2]) + (v[4] + v[6]), hi = (v[1] + v[3]) + (v[5] + v[7]);
+  e0[u] = hi;
+  e1[u] = (v[2] + v[3]) + (v[6] + v[7]);
+  e2[u] = (v[4] + v[5]) + (v[6] + v[7]);
+  const double diag = 4.0 * (lo + hi) * L.s12;
+  dinv[u] = diag > 0.0 ? 1.0 / diag : 0.0;
 }
 
 // 27-point FE sweeps on a plane-marching tile: a block owns FX x FY nodes of every plane of a
@@ -913,19 +921,17 @@ static_assert(VNX + VNR + VNB <= FX * FY, "one staged chunk per thread and plane
 constexpr int SXC = (FX + 3 + 3 + 3) / 4, SRC = (FX + 1 + 3 + 3) / 4, SBC = (FX + 2 + 3 + 3) / 4;  // (STG 2)
 constexpr int SNX = (FY + 2) * SXC, SNR = FY * SRC, SNB = (FY + 1) * SBC;
 static_assert(SNX + SNR + SNB <= FX * (FY + 1), "one staged chunk per thread and plane");
-template <typename T, int MODE, int STG = 0>
-__global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T w, const T* __restrict__ x, T* __restrict__ out,
-                                                    const T* __restrict__ b, const T* __restrict__ beta,
-                                                    const T* __restrict__ dinv) {
+template <int MODE, int STG>
+__global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, float w, const float* __restrict__ x, float* __restrict__ out,
+                                                    const float* __restrict__ b, const float* __restrict__ beta) {
   wait_prior();
-  static_assert(!STG || sizeof(T) == 4, "16-byte rows of floats");
   constexpr bool VEC = STG == 1;
   constexpr int XW = STG == 2 ? 4 * SXC : (VEC ? FX + 8 : FX + 2);  // staged row lengths
   constexpr int BW = STG == 2 ? 4 * SBC : (VEC ? FX + 4 : FX + 1), RW = STG == 2 ? 4 * SRC : FX;
   constexpr int XO = VEC ? 3 : 0, BO = VEC ? 3 : 0;  // column of node i0-1 / cell i0-1
-  __shared__ __align__(16) T xs[RING][FY + 2][XW];
-  __shared__ __align__(16) T bs[RING][FY + 1][BW];
-  __shared__ __align__(16) T rs[RING][FY][RW];  // right-hand side b of the tile's nodes
+  __shared__ __align__(16) float xs[RING][FY + 2][XW];
+  __shared__ __align__(16) float bs[RING][FY + 1][BW];
+  __shared__ __align__(16) float rs[RING][FY][RW];  // right-hand side b of the tile's nodes
   const int t = threadIdx.y * FX + threadIdx.x;
   const bool last_col = STG == 2 && threadIdx.y == FY;  // the ninth warp: rows of the column FX
   const int tx = last_col ? FX : threadIdx.x, ty = last_col ? threadIdx.x & (FY - 1) : threadIdx.y;
@@ -972,7 +978,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
   int vk = -1;
   long voff = 0;
   bool vok = true;
-  T* vdst = nullptr;
+  float* vdst = nullptr;
   size_t vslot = 0;  // elements between ring slots of the chunk's array
   if constexpr (VEC) {
     const int nx0 = L.n[0];  // = nn[0] on a periodic x axis
@@ -1002,7 +1008,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
   // STG 2: this thread's chunk of its array's planes: its row's first element in plane 0, how far along it lies, the
   // plane's and the array's lengths, the plane to copy next and its shared address; and the remainders that the
   // thread's own rows add to a plane's when it reads: x (bits 0-5), beta (6-9), b (10-11)
-  const T* ssrc = nullptr;
+  const float* ssrc = nullptr;
   int soff = 0, scc = 0, sstride = 0, slen = 0, splanes = 0, snext = k0 - 1;
   unsigned sdst = 0, sbytes = 0, rxb = 0;
   int sslot = 0;
@@ -1054,7 +1060,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
       sslot = sslot + 1 == RING ? 0 : sslot + 1;
     }
   };
-  auto cp16 = [&](T* dst, const T* src, bool valid) {
+  auto cp16 = [&](float* dst, const float* src, bool valid) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(src), "r"(valid ? 16 : 0));
   };
@@ -1109,27 +1115,27 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
   const bool own = i < L.nn[0] && j < L.nn[1] &&
                    (!last_col || (threadIdx.x < FY && blockIdx.x == gridDim.x - 1 && i == L.nn[0] - 1));
   const bool cell_lo = i > 0, cell_hi = i < L.n[0];  // the cells beside the node exist (STG 2)
-  const T s12 = cv<T>(L.s12, L.f_s12);
+  const float s12 = L.f_s12;
   // Register window of the thread's column: three x planes (i-1..i+1, j-1..j+1) and two beta
   // cell planes (the cells around the node below / above it).  The window moves up one plane
   // per iteration by reading only the new plane from shared memory (shared-memory bandwidth,
   // not DRAM, is the next limit of this kernel); the loop is unrolled so that the arrays change
   // roles instead of being copied.
-  T Xa[3][3], Xb[3][3], Xc[3][3], Ba[2][2], Bb[2][2];
-  auto rd_x = [&](T (&P)[3][3], int slot, unsigned q) {  // q: the plane's remainder (STG 2)
+  float Xa[3][3], Xb[3][3], Xc[3][3], Ba[2][2], Bb[2][2];
+  auto rd_x = [&](float (&P)[3][3], int slot, unsigned q) {  // q: the plane's remainder (STG 2)
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      const T* row = &xs[slot][ty + c][tx + XO + (STG == 2 ? ((rxb >> (2 * c)) + q) & 3u : 0u)];
+      const float* row = &xs[slot][ty + c][tx + XO + (STG == 2 ? ((rxb >> (2 * c)) + q) & 3u : 0u)];
 #pragma unroll
       for (int a = 0; a < 3; a++) P[c][a] = row[a];
     }
   };
-  auto rd_b = [&](T (&P)[2][2], int slot, unsigned q) {
+  auto rd_b = [&](float (&P)[2][2], int slot, unsigned q) {
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-      const T* row = &bs[slot][ty + c][tx + BO + (STG == 2 ? ((rxb >> (6 + 2 * c)) + q) & 3u : 0u)];
+      const float* row = &bs[slot][ty + c][tx + BO + (STG == 2 ? ((rxb >> (6 + 2 * c)) + q) & 3u : 0u)];
 #pragma unroll
-      for (int a = 0; a < 2; a++) P[c][a] = STG != 2 || (a ? cell_hi : cell_lo) ? row[a] : T(0);
+      for (int a = 0; a < 2; a++) P[c][a] = STG != 2 || (a ? cell_hi : cell_lo) ? row[a] : 0.f;
     }
   };
   const long ubase = (long)i + (long)j * sy;
@@ -1138,7 +1144,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
   unsigned qx = (unsigned)(k0 * szi), qb = (unsigned)(k0 * czi);  // (STG 2) of x plane k, of cell plane k
   // one plane: M, C, P = x planes k-1, k, k+1 (P is filled here), Bl, Bu = cell planes k-1, k
   // (Bu is filled here)
-  auto plane = [&](T (&M)[3][3], T (&C)[3][3], T (&P)[3][3], T (&Bl)[2][2], T (&Bu)[2][2]) {
+  auto plane = [&](float (&M)[3][3], float (&C)[3][3], float (&P)[3][3], float (&Bl)[2][2], float (&Bu)[2][2]) {
     cp_async_wait<2>();  // x plane k+1 and cell plane k have landed (two newer groups may fly)
     __syncthreads();     // ... for every thread; the slots refilled below were last read at
                          // least one iteration ago, before this barrier
@@ -1148,7 +1154,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
     rd_b(Bu, sbc, qb);
     qb += (unsigned)czi;
     // b of plane k (slot before k+1)
-    const T bcur = rs[sxp == 0 ? RING - 1 : sxp - 1][ty][tx + (STG == 2 ? ((rxb >> 10) + qr) & 3u : 0u)];
+    const float bcur = rs[sxp == 0 ? RING - 1 : sxp - 1][ty][tx + (STG == 2 ? ((rxb >> 10) + qr) & 3u : 0u)];
     if constexpr (STG == 2) {
       copy_next();
     } else {
@@ -1159,9 +1165,7 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
     sxp = sxp + 1 == RING ? 0 : sxp + 1;
     sbc = sbc + 1 == RING ? 0 : sbc + 1;
     if (own) {
-      T di = T(0);
-      if constexpr (MODE == 0 && sizeof(T) == 8) di = dinv[ubase + (long)k * sz];
-      T acc = T(0);
+      float acc = 0.f;
 #pragma unroll
       for (int qy = 0; qy < 2; qy++)
 #pragma unroll
@@ -1182,21 +1186,15 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
       for (int qy = 0; qy < 2; qy++) acc += (Bl[qy][0] + Bl[qy][1]) * M[2 * qy][1];
 #pragma unroll
       for (int qy = 0; qy < 2; qy++) acc += (Bu[qy][0] + Bu[qy][1]) * P[2 * qy][1];
-      const T xc = C[1][1];
+      const float xc = C[1][1];
       const long u = ubase + (long)k * sz;
-      if constexpr (MODE == 0 && sizeof(T) == 8) {
-        // (b - K x) / diag = (b + s12 acc) / diag - x: neither the diagonal nor a division is formed (the
-        // FP64 pipe bounds the FP64 kernel; 38 operations per node instead of 60)
-        out[u] = di > T(0) ? xc + w * ((bcur + s12 * acc) * di - xc) : xc;
-      } else {
-        const T bsum = (Bl[0][0] + Bl[0][1]) + (Bl[1][0] + Bl[1][1]) + ((Bu[0][0] + Bu[0][1]) + (Bu[1][0] + Bu[1][1]));
-        const T diag = T(4) * bsum * s12;
-        const T ax = (T(4) * bsum * xc - acc) * s12;
-        if constexpr (MODE == 0)
-          out[u] = diag > T(0) ? xc + w * __fdividef(bcur - ax, diag) : xc;  // increment only (see k_rbgs)
-        else
-          out[u] = bcur - ax;
-      }
+      const float bsum = (Bl[0][0] + Bl[0][1]) + (Bl[1][0] + Bl[1][1]) + ((Bu[0][0] + Bu[0][1]) + (Bu[1][0] + Bu[1][1]));
+      const float diag = 4.f * bsum * s12;
+      const float ax = (4.f * bsum * xc - acc) * s12;
+      if constexpr (MODE == 0)
+        out[u] = diag > 0.f ? xc + w * __fdividef(bcur - ax, diag) : xc;  // increment only (see k_rbgs)
+      else
+        out[u] = bcur - ax;
     }
     k++;
   };
@@ -1218,6 +1216,183 @@ __global__ void __launch_bounds__(FX*(STG == 2 ? FY + 1 : FY)) k_fe_tile(Lv L, T
     plane(Xb, Xc, Xa, Ba, Bb);
     if (k >= k1) break;
     plane(Xc, Xa, Xb, Bb, Ba);
+  }
+  cp_async_wait<0>();
+}
+
+// The FE sweeps in FP64, where the arithmetic bounds them.  With S_c the sum of a cell's eight nodes, the operator's
+// row is 12 h^2-scaled  5 B x - sum_c beta_c S_c + sum_edges E x_nb  (B the sum of beta over the node's cells, E the
+// stored edge sums): the products beta_c S_c are formed once per cell and shared, so a sweep takes 20 operations
+// per node, where gathering the 20 weighted neighbours takes 38.  128^3 with walls: 217 -> 124 us a sweep.
+// Tiles, ring and copies are k_fe_tile's; in iteration m the products of cell plane m are formed, and the nodes
+// of plane m - 1 are finished with those of the plane before, which a barrier has made visible.
+struct FeCoef {
+  const double *e[3], *dinv;
+};
+template <int MODE>
+__global__ void __launch_bounds__(FX* FY) k_fe_tile64(Lv L, double w, const double* __restrict__ x,
+                                                      double* __restrict__ out, const double* __restrict__ b,
+                                                      const double* __restrict__ beta, FeCoef E) {
+  wait_prior();
+  __shared__ double xs[RING][FY + 2][FX + 2];
+  __shared__ double bs[RING][FY + 1][FX + 1];
+  __shared__ double rs[RING][FY][FX];
+  __shared__ double vs[2][FY + 1][FX + 1];  // beta_c S_c of the last two cell planes
+  const int tx = threadIdx.x, ty = threadIdx.y, t = ty * FX + tx;
+  const int i0 = blockIdx.x * FX, j0 = blockIdx.y * FY;
+  const int fz = (L.nn[2] + (int)gridDim.z - 1) / (int)gridDim.z;
+  const int k0 = blockIdx.z * fz, k1 = min(k0 + fz, L.nn[2]);
+  const long sy = L.nn[0], sz = (long)L.nn[0] * L.nn[1];
+  const long cy = L.n[0], cz = (long)L.n[0] * L.n[1];
+  int hxa = 0, hxc = 0, hba = 0, hbc = 0;
+  if (t < XH) {
+    // halo ring of the (FX+2) x (FY+2) plane: row 0, row FY+1, then columns 0 and FX+1
+    if (t < FX + 2) {
+      hxa = t;
+    } else if (t < 2 * (FX + 2)) {
+      hxa = t - (FX + 2);
+      hxc = FY + 1;
+    } else {
+      const int r = t - 2 * (FX + 2);
+      hxa = (r & 1) ? FX + 1 : 0;
+      hxc = 1 + (r >> 1);
+    }
+  }
+  if (t < BH) {
+    // row 0 of the (FX+1) x (FY+1) cell plane, then column 0
+    if (t < FX + 1) hba = t;
+    else hbc = t - FX;
+  }
+  const long xo_own = nnb(L, 0, i0 + tx) + nnb(L, 1, j0 + ty) * sy;
+  const long xo_halo = nnb(L, 0, i0 - 1 + hxa) + nnb(L, 1, j0 - 1 + hxc) * sy;
+  const int ci_own = cnb(L, 0, i0 + tx), cj_own = cnb(L, 1, j0 + ty);
+  const int ci_halo = cnb(L, 0, i0 - 1 + hba), cj_halo = cnb(L, 1, j0 - 1 + hbc);
+  const bool b_own_ok = ci_own >= 0 && cj_own >= 0, b_halo_ok = ci_halo >= 0 && cj_halo >= 0;
+  const long bo_own = b_own_ok ? ci_own + cj_own * cy : 0, bo_halo = b_halo_ok ? ci_halo + cj_halo * cy : 0;
+  // x plane p lives in ring slot (p - k0 + 1) % RING, beta cell plane c in (c - k0 + 1) % RING
+  auto issue_x = [&](int p) {
+    const int slot = (p - k0 + 1 + RING) % RING;
+    const long base = nnb(L, 2, p) * sz;
+    cp_async_elem(&xs[slot][ty + 1][tx + 1], x + xo_own + base, true);
+    if (t < XH) cp_async_elem(&xs[slot][hxc][hxa], x + xo_halo + base, true);
+    cp_async_elem(&rs[slot][ty][tx], b + xo_own + base, true);
+  };
+  auto issue_b = [&](int c) {
+    const int slot = (c - k0 + 1 + RING) % RING;
+    const int ck = cnb(L, 2, c);
+    const long base = ck >= 0 ? ck * cz : 0;
+    cp_async_elem(&bs[slot][ty + 1][tx + 1], beta + bo_own + base, b_own_ok && ck >= 0);
+    if (t < BH) cp_async_elem(&bs[slot][hbc][hba], beta + bo_halo + base, b_halo_ok && ck >= 0);
+  };
+  // group 0: x planes k0-1 .. k0+1, cell planes k0-1, k0; then one group per further plane
+  issue_x(k0 - 1);
+  issue_x(k0);
+  issue_x(k0 + 1);
+  issue_b(k0 - 1);
+  issue_b(k0);
+  cp_async_commit();
+  issue_x(k0 + 2);
+  issue_b(k0 + 1);
+  cp_async_commit();
+  issue_x(k0 + 3);
+  issue_b(k0 + 2);
+  cp_async_commit();
+  const int i = i0 + tx, j = j0 + ty;
+  const bool own = i < L.nn[0] && j < L.nn[1];
+  const bool wall_x = !L.per[0] && i == 0, wall_y = !L.per[1] && j == 0;  // no edge below the node
+  const long u0 = own ? (long)i + (long)j * sy : 0;
+  const long u0x = own ? (long)nnb(L, 0, i - 1) + (long)j * sy : 0, u0y = own ? (long)i + (long)nnb(L, 1, j - 1) * sy : 0;
+  // sums over the four nodes of this thread's cell column, and of its halo cell's, in a plane
+  auto sum4 = [&](int slot, int a, int c) {
+    return (xs[slot][c][a] + xs[slot][c][a + 1]) + (xs[slot][c + 1][a] + xs[slot][c + 1][a + 1]);
+  };
+  double po, ph = 0.0;         // those sums in plane m
+  double xm, xc, xe[4];        // the node's column: x in planes m-2, m-1 and the four neighbours in plane m-1
+  double bc, tl, ez;           // b of plane m-1; sum of the four products below it; the edge sum below it along z
+  double co[5];                // of plane m-1: edge sums -x, +x, -y, +y, +z
+  double di = 0.0;
+  auto coefs = [&](int k, double (&q)[5], double& dv) {
+    const long o = (long)k * sz;
+    q[0] = wall_x ? 0.0 : E.e[0][u0x + o];
+    q[1] = E.e[0][u0 + o];
+    q[2] = wall_y ? 0.0 : E.e[1][u0y + o];
+    q[3] = E.e[1][u0 + o];
+    q[4] = E.e[2][u0 + o];
+    if (MODE == 0) dv = E.dinv[u0 + o];
+  };
+  cp_async_wait<2>();
+  __syncthreads();
+  po = sum4(1, tx + 1, ty + 1);
+  vs[1][ty + 1][tx + 1] = bs[0][ty + 1][tx + 1] * (sum4(0, tx + 1, ty + 1) + po);
+  if (t < BH) {
+    ph = sum4(1, hba, hbc);
+    vs[1][hbc][hba] = bs[0][hbc][hba] * (sum4(0, hba, hbc) + ph);
+  }
+  xm = xs[0][ty + 1][tx + 1];
+  xc = xs[1][ty + 1][tx + 1];
+  xe[0] = xs[1][ty + 1][tx];
+  xe[1] = xs[1][ty + 1][tx + 2];
+  xe[2] = xs[1][ty][tx + 1];
+  xe[3] = xs[1][ty + 2][tx + 1];
+  bc = rs[1][ty][tx];
+  ez = !L.per[2] && k0 == 0 ? 0.0 : E.e[2][u0 + (k0 > 0 ? k0 - 1 : L.nn[2] - 1) * sz];
+  coefs(k0, co, di);
+  // here the names hold plane m-1 = k0 as the first iteration below (m = k0) finds plane k0 - 1 finished
+  tl = 0.0;
+  int sx = 2, sb = 1, cur = 0;  // slots of x plane m+1 and cell plane m; half of vs of cell plane m
+  for (int m = k0; m <= k1; m++) {
+    cp_async_wait<2>();  // x plane m+1 and cell plane m have landed
+    __syncthreads();     // ... for every thread, and the products of cell plane m-1 are stored
+    const int prev = cur ^ 1;
+    const double tu = (vs[prev][ty][tx] + vs[prev][ty][tx + 1]) + (vs[prev][ty + 1][tx] + vs[prev][ty + 1][tx + 1]);
+    if (m > k0 && own) {
+      // finish plane m - 1: xm, xc, xp its column, tl and tu the products below and above it
+      const int k = m - 1;
+      const long u = u0 + (long)k * sz;
+      const double xp = xs[sx == 0 ? RING - 1 : sx - 1][ty + 1][tx + 1];
+      double acc = tl + tu;
+      acc -= co[0] * xe[0];
+      acc -= co[1] * xe[1];
+      acc -= co[2] * xe[2];
+      acc -= co[3] * xe[3];
+      acc -= ez * xm;
+      acc -= co[4] * xp;
+      if (MODE == 0) {
+        // (b - K x) / diag = (b + s12 acc) / diag - 5/4 x
+        const double v = xc + w * ((bc + L.s12 * acc) * di - 1.25 * xc);
+        out[u] = __double2hiint(di) > 0 ? v : xc;
+      } else {
+        out[u] = bc + L.s12 * (acc - 5.0 * (co[0] + co[1]) * xc);
+      }
+    }
+    if (m == k1) break;
+    tl = tu;
+    const int sc = sx == 0 ? RING - 1 : sx - 1;  // slot of x plane m
+    if (m > k0) {
+      xm = xc;
+      ez = co[4];
+      xc = xs[sc][ty + 1][tx + 1];
+      xe[0] = xs[sc][ty + 1][tx];
+      xe[1] = xs[sc][ty + 1][tx + 2];
+      xe[2] = xs[sc][ty][tx + 1];
+      xe[3] = xs[sc][ty + 2][tx + 1];
+      bc = rs[sc][ty][tx];
+      if (own) coefs(m, co, di);
+    }
+    const double pn = sum4(sx, tx + 1, ty + 1);
+    vs[cur][ty + 1][tx + 1] = bs[sb][ty + 1][tx + 1] * (po + pn);
+    po = pn;
+    if (t < BH) {
+      const double pq = sum4(sx, hba, hbc);
+      vs[cur][hbc][hba] = bs[sb][hbc][hba] * (ph + pq);
+      ph = pq;
+    }
+    issue_x(m + 4);
+    issue_b(m + 3);
+    cp_async_commit();
+    sx = sx + 1 == RING ? 0 : sx + 1;
+    sb = sb + 1 == RING ? 0 : sb + 1;
+    cur = prev;
   }
   cp_async_wait<0>();
 }
@@ -1896,8 +2071,7 @@ MGSolver* mg_build(const Geo& g, int kind, int prec_fp32, bool dry, cudaError_t*
     }
     const bool last = !can || l == 15;
     if (!prec_fp32 && (!last || l == 0)) {  // a hierarchy of one level: for its residual
-      if (kind == 0)
-        for (int d = 0; d < 3; d++) alloc((void**)&m->f64[l][d], vb);
+      for (int d = 0; d < 3; d++) alloc((void**)&m->f64[l][d], vb);
       alloc((void**)&m->dinv[l], vb);
     }
     if (last) break;
@@ -2061,9 +2235,8 @@ void sum_ff(MGSolver* m, const float* h, const float* l, long n, double scale, d
 // How the FE tile kernel stages a level's planes: FP32 levels as 16-byte rows, aligned ones with a periodic x axis of
 // n_x % 4 == 0, shifted ones with walls in x; element by element otherwise (a periodic row of another length wraps
 // inside a copy; FP64 is bound by its arithmetic)
-template <typename T>
-inline int fe_staging(const Lv& L) {
-  return sizeof(T) == 4 ? (L.per[0] ? (L.n[0] % 4 == 0 ? 1 : 0) : 2) : 0;
+inline int fe_staging(const Lv& L, bool fp32) {
+  return fp32 ? (L.per[0] ? (L.n[0] % 4 == 0 ? 1 : 0) : 2) : 0;
 }
 inline dim3 fe_grid(const Lv& L, int zchunk = 0, int stg = 0) {
   // z-chunks of FZ planes, or more and shorter chunks on small levels, so that at least two
@@ -2080,16 +2253,23 @@ inline dim3 fe_grid(const Lv& L, int zchunk = 0, int stg = 0) {
   return dim3(tx, ty, (L.nn[2] + fz - 1) / fz);
 }
 
-template <typename T, int MODE>
-void launch_fe_tile(const Lv& L, int zchunk, T w, const T* x, T* out, const T* b, const T* beta, const T* dinv,
-                    cudaStream_t s) {
-  const int stg = fe_staging<T>(L);
-  const dim3 grid = fe_grid(L, zchunk, stg);
-  if constexpr (sizeof(T) == 4) {
-    if (stg == 1) return launch_after(k_fe_tile<T, MODE, 1>, grid, dim3(FX, FY), 0, s, L, w, x, out, b, beta, dinv);
-    if (stg == 2) return launch_after(k_fe_tile<T, MODE, 2>, grid, dim3(FX, FY + 1), 0, s, L, w, x, out, b, beta, dinv);
+template <int MODE, typename T>
+void launch_fe_tile(const MGSolver* m, int l, T w, const T* x, T* out, const T* b, cudaStream_t s) {
+  const Lv& L = m->lv[l];
+  const T* beta = (const T*)m->rho[l];
+  const int stg = fe_staging(L, sizeof(T) == 4);
+  const dim3 grid = fe_grid(L, l == 0 ? m->fe_zc0 : 0, stg), tile(FX, FY), more(FX, FY + 1);
+  if constexpr (sizeof(T) == 8) {
+    const FeCoef E = {{m->f64[l][0], m->f64[l][1], m->f64[l][2]}, m->dinv[l]};
+    launch_after(k_fe_tile64<MODE>, grid, tile, 0, s, L, w, x, out, b, beta, E);
+  } else if (stg == 1) {
+    launch_after(k_fe_tile<MODE, 1>, grid, tile, 0, s, L, w, x, out, b, beta);
+  } else if (stg == 2) {
+    launch_after(k_fe_tile<MODE, 2>, grid, more, 0, s, L, w, x, out, b, beta);
+  } else {
+    launch_after(k_fe_tile<MODE, 0>, grid, tile, 0, s, L, w, x, out, b, beta);
   }
-  launch_after(k_fe_tile<T, MODE, 0>, grid, dim3(FX, FY), 0, s, L, w, x, out, b, beta, dinv);
+  rmt_count_launches(1);
 }
 
 template <typename T>
@@ -2131,9 +2311,7 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
       }
     } else {
       hk(m, l, 0, 1, s);
-      launch_fe_tile<T, 0>(L, l == 0 ? m->fe_zc0 : 0, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, rho,
-                           (const T*)m->dinv[l], s);
-      rmt_count_launches(1);
+      launch_fe_tile<0>(m, l, T(m->omega), (const T*)m->x[l], (T*)m->xt[l], b, s);
       hk(m, l, 0, 0, s);
       void* t = m->x[l];
       m->x[l] = m->xt[l];
@@ -2175,9 +2353,7 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
           L, C, (const T*)m->x[l], (const T*)m->b[l], mac_coef(m, l), (T*)m->b[l + 1], (T*)m->x[l + 1]);
     rmt_count_launches(1);
   } else {
-    launch_fe_tile<T, 1>(L, l == 0 ? m->fe_zc0 : 0, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l],
-                         (const T*)m->rho[l], (const T*)nullptr, s);
-    rmt_count_launches(1);
+    launch_fe_tile<1>(m, l, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l], s);
     const int zc = column_chunk(C.nnode, RZ);
     launch_after(k_restrict<T>, grid3(C.nn[0], C.nn[1], (C.nn[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s, 
         L, C, m->kind, (const T*)m->r[l], (T*)m->b[l + 1], (T*)m->x[l + 1], zc);
@@ -2217,8 +2393,8 @@ int solve_t(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStre
         launch_after(k_mac_coef, grid3(Q.n[0], Q.n[1], Q.n[2], m->by), dim3(BX, m->by), 0, s, 
             Q, (const double*)m->rho[l], m->f64[l][0], m->f64[l][1], m->f64[l][2], m->dinv[l]);
       else
-        launch_after(k_fe_dinv, grid3(Q.nn[0], Q.nn[1], Q.nn[2], m->by), dim3(BX, m->by), 0, s, Q, (const double*)m->rho[l],
-                                                                                    m->dinv[l]);
+        launch_after(k_fe_coef, grid3(Q.nn[0], Q.nn[1], Q.nn[2], m->by), dim3(BX, m->by), 0, s, Q, (const double*)m->rho[l],
+                     m->f64[l][0], m->f64[l][1], m->f64[l][2], m->dinv[l]);
       rmt_count_launches(1);
     }
   }
@@ -2372,7 +2548,7 @@ void mg_set_zchunk(MGSolver* m, int zchunk) {
 int mg_zchunk(const MGSolver* m) {
   if (m->kind == 0) return mac_fused0(m) ? m->zc[0] : 0;
   const Lv& L = m->lv[0];
-  const dim3 g = fe_grid(L, m->fe_zc0, m->fp32 ? fe_staging<float>(L) : 0);
+  const dim3 g = fe_grid(L, m->fe_zc0, fe_staging(L, m->fp32));
   return (L.nn[2] + (int)g.z - 1) / (int)g.z;
 }
 
