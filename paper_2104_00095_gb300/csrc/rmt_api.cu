@@ -559,7 +559,7 @@ rmt_status init_t(rmt_grid* g) {
   }
   if ((st = build_views<T>(g)) != RMT_OK) return st;
   // SI "Initialization": u^0 = 0, p = 0, xi^0 = x, extrapolation, phi, rho^0
-  const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 64);
+  const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 16);
   for (int m = 0; m < nb; m++) {
     launch_init_xi<T>(G, g->bodies[m], (T*)g->bm[m].X[0], g->s);
     launch_extrapolate<T>(G, band_set<T>(g, m, 1, 0, -1), full_blocks, wls_blocks<T>(1), g->err_d, g->s);
@@ -917,7 +917,7 @@ rmt_status scatter_t(rmt_grid* g, int field, int sid) {
   } else {
     BodyMem& b = g->bm[sid];
     k_xi_in<T><<<nbk(3 * G.N), 256, 0, s>>>(G, g->bodies[sid], g->stage, (T*)b.X[g->par]); rmt_count_launches(1);
-    const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 64);
+    const int full_blocks = (int)std::min((G.N + 127) / 128, (long)sm_count() * 16);
     launch_extrapolate<T>(G, band_set<T>(g, sid, 1, g->par, -1), full_blocks, wls_blocks<T>(1), g->err_d, s);
     launch_density<T>(G, g->bodies_d, views<T>(g, g->par, 0), (int)g->bodies.size(), g->bb_all + 6 * g->par, 12,
                       (T*)g->rho, s);

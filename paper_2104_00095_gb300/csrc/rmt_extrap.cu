@@ -25,6 +25,7 @@ inline int nblocks(long n) {
 // storage: the displacement from the cell's image, zero)
 template <typename T>
 __global__ void k_init_xi(Geo g, Body b, T* __restrict__ x) {
+  wait_prior();
   GRID_LOOP(c, g.N) {
     if constexpr (disp_storage<T>()) {
       x[c] = x[g.N + c] = x[2 * g.N + c] = T(0);
@@ -45,6 +46,7 @@ __global__ void k_init_xi(Geo g, Body b, T* __restrict__ x) {
 // band's box start empty
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_classify(Geo g, const __grid_constant__ BandSet<T> S) {
+  wait_prior();
   __shared__ BandCtx<T> ctx;
   load_ctx(S, ctx);
   const Body& b = ctx.b;
@@ -81,6 +83,7 @@ __device__ __forceinline__ int layer_base(const int* __restrict__ cnt, int l) {
 // and only l-1 is tested
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_bfs(Geo g, const __grid_constant__ BandSet<T> S, int l) {
+  wait_prior();
   __shared__ BandCtx<T> ctx;
   load_ctx(S, ctx);
   int8_t* __restrict__ lay = ctx.a.LAY[S.out];
@@ -667,6 +670,7 @@ __device__ __noinline__ int wls_again(const Geo& g, const Body& b, const T* x, c
 template <typename T>
 __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, const __grid_constant__ BandSet<T> S, int l,
                                                                      int* __restrict__ err) {
+  wait_prior();
   __shared__ WlsShared<T> sh;
   __shared__ BandCtx<T> ctx;
   load_ctx(S, ctx);
@@ -714,6 +718,7 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls(Geo g, cons
 // CORR: the corrector xi^{n+1/2} = (xi^n + xi^{n+1})/2 where both exist.
 template <typename T, bool CORR>
 __global__ void __launch_bounds__(TPB) k_finalize(Geo g, const __grid_constant__ BandSet<T> S, int* __restrict__ seam) {
+  wait_prior();
   __shared__ BandCtx<T> ctx;
   __shared__ int box[6];
   if (threadIdx.x < 6) box[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : -0x7fffffff;
@@ -793,6 +798,7 @@ __global__ void __launch_bounds__(TPB) k_finalize(Geo g, const __grid_constant__
 template <typename T>
 __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g, const __grid_constant__ BandSet<T> S,
                                                                           int l, int* __restrict__ err) {
+  wait_prior();
   __shared__ WlsShared<T> sh;
   __shared__ BandCtx<T> ctx;
   load_ctx(S, ctx);
@@ -840,6 +846,7 @@ __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 4 : 2) k_wls_half(Geo g,
 
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_phi_half(Geo g, const __grid_constant__ BandSet<T> S) {
+  wait_prior();
   __shared__ BandCtx<T> ctx;
   load_ctx(S, ctx);
   const T* __restrict__ xh = ctx.a.XH;
@@ -861,17 +868,17 @@ __global__ void __launch_bounds__(TPB) k_phi_half(Geo g, const __grid_constant__
 
 template <typename T>
 void launch_init_xi(const Geo& g, const Body& b, T* x, cudaStream_t s) {
-  k_init_xi<T><<<nblocks(g.N), TPB, 0, s>>>(g, b, x); rmt_count_launches(1);
+  launch_after(k_init_xi<T>, nblocks(g.N), TPB, 0, s, g, b, x); rmt_count_launches(1);
 }
 
 namespace {
 template <typename T, bool CORR>
 void extrapolate(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err, cudaStream_t s) {
   const dim3 gw(blocks, S.count), gf(wls_blocks, S.count);
-  k_classify<T><<<gw, TPB, 0, s>>>(g, S);
-  for (int l = 1; l <= g.layers; l++) k_bfs<T><<<gw, TPB, 0, s>>>(g, S, l);
-  for (int l = 1; l <= g.layers; l++) k_wls<T><<<gf, TPB, 0, s>>>(g, S, l, err);
-  k_finalize<T, CORR><<<gw, TPB, 0, s>>>(g, S, err + 1);
+  launch_after(k_classify<T>, gw, TPB, 0, s, g, S);
+  for (int l = 1; l <= g.layers; l++) launch_after(k_bfs<T>, gw, TPB, 0, s, g, S, l);
+  for (int l = 1; l <= g.layers; l++) launch_after(k_wls<T>, gf, TPB, 0, s, g, S, l, err);
+  launch_after(k_finalize<T, CORR>, gw, TPB, 0, s, g, S, err + 1);
   rmt_count_launches(2 + 2 * g.layers);
 }
 }  // namespace
@@ -885,8 +892,8 @@ template <typename T>
 void launch_extrapolate_correct(const Geo& g, const BandSet<T>& S, int blocks, int wls_blocks, int* err,
                                 cudaStream_t s) {
   extrapolate<T, true>(g, S, blocks, wls_blocks, err, s);
-  for (int l = 1; l <= g.layers; l++) k_wls_half<T><<<dim3(wls_blocks, S.count), TPB, 0, s>>>(g, S, l, err);
-  k_phi_half<T><<<dim3(blocks, S.count), TPB, 0, s>>>(g, S);
+  for (int l = 1; l <= g.layers; l++) launch_after(k_wls_half<T>, dim3(wls_blocks, S.count), TPB, 0, s, g, S, l, err);
+  launch_after(k_phi_half<T>, dim3(blocks, S.count), TPB, 0, s, g, S);
   rmt_count_launches(1 + g.layers);
 }
 

@@ -58,6 +58,7 @@ __device__ __forceinline__ void store_prod(MGVec b, long i, float x, float ch, f
 
 template <typename T>
 __global__ void k_mac_rhs(Geo g, FacePtrs3 un, MGVec b) {
+  wait_prior();
   const T ih = cv<T>(g.ih, g.f.ih);
   GRID_LOOP(c, g.N) {
     int i, j, k;
@@ -93,6 +94,7 @@ constexpr int MCZ = 8;
 template <typename T>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_mac_correct3(Geo g, Umac3 F, const T* __restrict__ rho, MGVec q,
                                                                  int zc) {
+  wait_prior();
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   if (i > g.n[0] || j > g.n[1]) return;
   const int k0 = blockIdx.z * zc, k1 = min(k0 + zc, g.n[2] + 1);
@@ -199,6 +201,7 @@ struct AdvPtrs {
 
 template <typename T>
 __global__ void k_adv(Geo g, AdvPtrs ap, T* __restrict__ adv) {
+  wait_prior();
   const T ih = cv<T>(g.ih, g.f.ih);
   GRID_LOOP(c, g.N) {
     int i, j, k;
@@ -232,6 +235,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_density(Geo g, const Body* _
                                                              const BodyView<T>* __restrict__ views, int nb,
                                                              const int* __restrict__ bbs, int bstride,
                                                              T* __restrict__ rho, int zc) {
+  wait_prior();
   __shared__ int sbb[6 * RMT_MAX_BODIES];
   __shared__ unsigned long long tile_mask;
   stage_boxes(bbs, bstride, nb, sbb);
@@ -261,6 +265,7 @@ template <typename T>
 __global__ void k_ustar(Geo g, const T* __restrict__ u, const T* __restrict__ adv, const T* __restrict__ p,
                         const T* __restrict__ rho_h, const T* __restrict__ divtau_h, T* __restrict__ ustar,
                         const Body* __restrict__ bodies, const BodyView<T>* __restrict__ views, int nb) {
+  wait_prior();
   const T dt = cv<T>(g.dt, g.f.dt), q4 = cv<T>(g.q4, g.f.q4);
   GRID_LOOP(c, g.N) {
     int i, j, k;
@@ -299,6 +304,7 @@ constexpr int FEZ = 16;
 template <typename T>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_fe_rhs(Geo g, const T* __restrict__ u,
                                                            const T* __restrict__ ustar, MGVec b, int zc) {
+  wait_prior();
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   if (i >= g.nn[0] || j >= g.nn[1]) return;
   const int k0 = blockIdx.z * zc, k1 = min(k0 + zc, g.nn[2]);
@@ -367,6 +373,7 @@ template <typename T>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_fe_update_u(Geo g, const T* __restrict__ ustar,
                                                                 const T* __restrict__ rho_h, MGVec psi,
                                                                 T* __restrict__ u, int zc) {
+  wait_prior();
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   if (i >= g.n[0] || j >= g.n[1]) return;
   const int k0 = blockIdx.z * zc, k1 = min(k0 + zc, g.n[2]);
@@ -443,6 +450,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_fe_update_u(Geo g, const T* 
 
 template <typename T>
 __global__ void k_fe_update_p(long nn, MGVec psi, T* __restrict__ p, T* __restrict__ psi_out) {
+  wait_prior();
   GRID_LOOP(i, nn) {
     T v;
     if constexpr (sizeof(T) == 8)
@@ -479,7 +487,7 @@ template <typename T>
 void launch_mac_setup(const Geo& g, T* const uf[3][3], MGVec b64, cudaStream_t s) {
   FacePtrs3 un;
   for (int d = 0; d < 3; d++) un.p[d] = uf[d][d];
-  k_mac_rhs<T><<<nblocks(g.N), TPB, 0, s>>>(g, un, b64);
+  launch_after(k_mac_rhs<T>, nblocks(g.N), TPB, 0, s, g, un, b64);
   rmt_count_launches(1);
 }
 template <typename T>
@@ -492,7 +500,7 @@ void launch_mac_correct(const Geo& g, T* const uf[3][3], const T* rho, MGVec q, 
   }
   const int zc = column_chunk(g.N, MCZ);
   const dim3 gr((g.n[0] + 1 + TILE_X - 1) / TILE_X, (g.n[1] + 1 + TILE_Y - 1) / TILE_Y, (g.n[2] + 1 + zc - 1) / zc);
-  k_mac_correct3<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, F, rho, q, zc);
+  launch_after(k_mac_correct3<T>, gr, dim3(TILE_X, TILE_Y), 0, s, g, F, rho, q, zc);
   rmt_count_launches(1);
 }
 template <typename T>
@@ -502,14 +510,14 @@ void launch_advect(const Geo& g, T* const uf[3][3], T* const umac[3], T* adv, cu
     ap.umac[d] = umac[d];
     for (int a = 0; a < 3; a++) ap.uf[d][a] = uf[d][a];
   }
-  k_adv<T><<<nblocks(g.N), TPB, 0, s>>>(g, ap, adv); rmt_count_launches(1);
+  launch_after(k_adv<T>, nblocks(g.N), TPB, 0, s, g, ap, adv); rmt_count_launches(1);
 }
 template <typename T>
 void launch_density(const Geo& g, const Body* bodies, const BodyView<T>* views, int nb, const int* bbs, int bstride,
                     T* rho, cudaStream_t s) {
   const int zc = column_chunk(g.N, DZ);
   const dim3 gr((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, (g.n[2] + zc - 1) / zc);
-  k_density<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, bodies, views, nb, bbs, bstride, rho, zc);
+  launch_after(k_density<T>, gr, dim3(TILE_X, TILE_Y), 0, s, g, bodies, views, nb, bbs, bstride, rho, zc);
   rmt_count_launches(1);
 }
 template <typename T>
@@ -520,14 +528,14 @@ void launch_rep_field(const Geo& g, const Body* bodies, const BodyView<T>* views
 template <typename T>
 void launch_ustar(const Geo& g, const T* u, const T* adv, const T* p, const T* rho_h, const T* divtau_h, T* ustar,
                   const Body* bodies, const BodyView<T>* views, int nb, cudaStream_t s) {
-  k_ustar<T><<<nblocks(g.N), TPB, 0, s>>>(g, u, adv, p, rho_h, divtau_h, ustar, bodies, views, nb);
+  launch_after(k_ustar<T>, nblocks(g.N), TPB, 0, s, g, u, adv, p, rho_h, divtau_h, ustar, bodies, views, nb);
   rmt_count_launches(1);
 }
 template <typename T>
 void launch_fe_setup(const Geo& g, const T* u, const T* ustar, MGVec b64, cudaStream_t s) {
   const int zc = column_chunk(g.NN, FEZ);
   const dim3 gr((g.nn[0] + TILE_X - 1) / TILE_X, (g.nn[1] + TILE_Y - 1) / TILE_Y, (g.nn[2] + zc - 1) / zc);
-  k_fe_rhs<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, ustar, b64, zc);
+  launch_after(k_fe_rhs<T>, gr, dim3(TILE_X, TILE_Y), 0, s, g, u, ustar, b64, zc);
   rmt_count_launches(1);
 }
 template <typename T>
@@ -535,8 +543,8 @@ void launch_fe_update(const Geo& g, const T* ustar, const T* rho_h, MGVec psi, T
                       cudaStream_t s) {
   const int zc = column_chunk(g.N, FEZ);
   const dim3 gr((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, (g.n[2] + zc - 1) / zc);
-  k_fe_update_u<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, ustar, rho_h, psi, u, zc); rmt_count_launches(1);
-  k_fe_update_p<T><<<nblocks(g.NN), TPB, 0, s>>>(g.NN, psi, p, psi_out); rmt_count_launches(1);
+  launch_after(k_fe_update_u<T>, gr, dim3(TILE_X, TILE_Y), 0, s, g, ustar, rho_h, psi, u, zc); rmt_count_launches(1);
+  launch_after(k_fe_update_p<T>, nblocks(g.NN), TPB, 0, s, g.NN, psi, p, psi_out); rmt_count_launches(1);
 }
 template <typename T>
 void launch_fill(T* a, T v, long n, cudaStream_t s) {

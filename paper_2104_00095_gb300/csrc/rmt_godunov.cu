@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(GX* GY, 2)
     k_godunov(Geo g, const float* __restrict__ u, const float* __restrict__ p, const float* __restrict__ rho,
               const float* __restrict__ divtau, const __grid_constant__ GodOut out, const Body* __restrict__ bodies,
               const BodyView<float>* __restrict__ views, int nb, int zc) {
+  wait_prior();
   extern __shared__ float god_smem[];
   GodSmem& sm = *reinterpret_cast<GodSmem*>(god_smem);
   const float hh = 0.5f * g.f.h, hdt = 0.5f * g.f.dt, ih = g.f.ih, tol = g.f.utol;
@@ -352,6 +353,7 @@ struct Slopes9 {
 // with a separate path at the walls 1.5 ms with the limiters of the time).
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_slopes64(Geo g, const double* __restrict__ u,
                                                              const __grid_constant__ Slopes9 S, int zc, int chunks) {
+  wait_prior();
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   if (i >= g.n[0] || j >= g.n[1]) return;
   const int a = blockIdx.z / chunks, k0 = blockIdx.z % chunks * zc, k1 = min(k0 + zc, g.n[2]);
@@ -407,6 +409,7 @@ template <int e>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_bar(Geo g, const double* __restrict__ u, Slopes9 S,
                                                          double* __restrict__ ub0, double* __restrict__ ub1, double* __restrict__ ub2,
                                                          double* __restrict__ vadv) {
+  wait_prior();
   const int ex = g.n[0] + (e == 0), ey = g.n[1] + (e == 1), ez = g.n[2] + (e == 2);
   const double h = g.h, dt = g.dt;
   double* ub[3] = {ub0, ub1, ub2};
@@ -455,6 +458,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_cellw(Geo g, const double* _
                                                            const double* __restrict__ rho, const double* __restrict__ divtau,
                                                            BarPtrs bp, Slopes9 W, const Body* __restrict__ bodies,
                                                            const BodyView<double>* __restrict__ views, int nb) {
+  wait_prior();
   THREAD_XYZ(i, j, k);
   if (i >= g.n[0] || j >= g.n[1]) return;
   const double dt = g.dt, ih = g.ih;
@@ -501,6 +505,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_cellw(Geo g, const double* _
 template <int d>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_face(Geo g, const double* __restrict__ u, Slopes9 S, Slopes9 W,
                                                           BarPtrs bp) {
+  wait_prior();
   const int ex = g.n[0] + (d == 0), ey = g.n[1] + (d == 1), ez = g.n[2] + (d == 2);
   const double h = g.h, dt = g.dt;
   double* uf[3] = {(double*)bp.uf[0], (double*)bp.uf[1], (double*)bp.uf[2]};
@@ -561,7 +566,7 @@ cudaError_t launch_godunov<float>(const Geo& g, const float* u, const float* p, 
       zc = len;
     }
   }
-  k_godunov<<<dim3(bx, by, (nz + zc - 1) / zc), dim3(GX, GY), smem, s>>>(g, u, p, rho, divtau, o, bodies, views, nb, zc);
+  launch_after(k_godunov, dim3(bx, by, (nz + zc - 1) / zc), dim3(GX, GY), smem, s, g, u, p, rho, divtau, o, bodies, views, nb, zc);
   rmt_count_launches(1);
   return cudaSuccess;
 }
@@ -581,7 +586,7 @@ cudaError_t launch_godunov<double>(const Geo& g, const double* u, const double* 
   // about 16 blocks to an SM, and no less than eight planes to a chunk where the grid has them
   const int want = (16 * sm_count() + 3 * (int)(gc.x * gc.y) - 1) / (3 * (int)(gc.x * gc.y));
   const int most = (g.n[2] + 7) / 8, chunks = want < most ? want : most, zc = (g.n[2] + chunks - 1) / chunks;
-  k_slopes64<<<dim3(gc.x, gc.y, 3 * chunks), tile, 0, s>>>(g, u, S, zc, chunks);
+  launch_after(k_slopes64, dim3(gc.x, gc.y, 3 * chunks), tile, 0, s, g, u, S, zc, chunks);
   rmt_count_launches(1);
   auto grid = [&](int d) {
     return dim3((g.n[0] + (d == 0) + TILE_X - 1) / TILE_X, (g.n[1] + (d == 1) + TILE_Y - 1) / TILE_Y, g.n[2] + (d == 2));
@@ -590,17 +595,17 @@ cudaError_t launch_godunov<double>(const Geo& g, const double* u, const double* 
     // the direction is a template argument: a runtime index into the pointer bundles would
     // copy them to local memory in every thread
     auto kb = e == 0 ? k_bar<0> : (e == 1 ? k_bar<1> : k_bar<2>);
-    kb<<<grid(e), tile, 0, s>>>(g, u, S, uf[e][0], uf[e][1], uf[e][2], vadv[e]);
+    launch_after(kb, grid(e), tile, 0, s, g, u, S, uf[e][0], uf[e][1], uf[e][2], vadv[e]);
     rmt_count_launches(1);
     for (int a = 0; a < 3; a++) bp.ub[e][a] = uf[e][a];  // the bar states give way to the face states
     bp.vadv[e] = vadv[e];
   }
-  k_cellw<<<gc, tile, 0, s>>>(g, u, p, rho, divtau, bp, W, bodies, views, nb);
+  launch_after(k_cellw, gc, tile, 0, s, g, u, p, rho, divtau, bp, W, bodies, views, nb);
   rmt_count_launches(1);
   for (int d = 0; d < 3; d++) {
     for (int a = 0; a < 3; a++) bp.uf[a] = uf[d][a];
     auto kf = d == 0 ? k_face<0> : (d == 1 ? k_face<1> : k_face<2>);
-    kf<<<grid(d), tile, 0, s>>>(g, u, S, W, bp);
+    launch_after(kf, grid(d), tile, 0, s, g, u, S, W, bp);
     rmt_count_launches(1);
   }
   return cudaGetLastError();

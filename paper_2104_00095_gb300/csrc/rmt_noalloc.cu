@@ -106,7 +106,7 @@ rmt_status rmt_extrapolate_noalloc(const rmt_grid_desc* d, const rmt_solid_desc*
   e = cudaMemsetAsync(scr + SCR_ERR, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(xi_out, xi_in, 3 * G.N * sizeof(double), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return RMT_ECUDA;
-  const long wide = (long)sm_count() * 64;
+  const long wide = (long)sm_count() * 16;
   const int blocks = (int)((G.N + 127) / 128 < wide ? (G.N + 127) / 128 : wide);
   BandSet<double> set;
   memset(&set, 0, sizeof set);

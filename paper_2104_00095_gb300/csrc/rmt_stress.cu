@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
                                                                   const BodyView<T>* __restrict__ views, int nb,
                                                                   const int* __restrict__ bbs, int bstride,
                                                                   T* __restrict__ out, StressList L) {
+  wait_prior();
   __shared__ int sbb[6 * RMT_MAX_BODIES];
   __shared__ unsigned long long tile_mask;
   stage_boxes(bbs, bstride, nb, sbb);
@@ -313,6 +314,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_stress_rows(Geo g, const T* __restrict__ u, const Body* __restrict__ bodies,
                                                       const BodyView<T>* __restrict__ views,
                                                       const double* __restrict__ t, double toff, StressList L, Rows9 R) {
+  wait_prior();
   const T tt = (T)(*t + toff);
   if (blockIdx.y == 0) stress_faces<T, 0>(g, u, bodies, views, tt, L, R);
   else if (blockIdx.y == 1) stress_faces<T, 1>(g, u, bodies, views, tt, L, R);
@@ -343,6 +345,7 @@ __global__ void __launch_bounds__(128) k_stress_band(Geo g, const T* __restrict_
                                                       const BodyView<T>* __restrict__ views,
                                                       const double* __restrict__ t, double toff, StressList L, Rows9 R,
                                                       T* __restrict__ out) {
+  wait_prior();
   const int n = *L.count;
   const T tt = (T)(*t + toff);
   const T ih = cv<T>(g.ih, g.f.ih);
@@ -369,14 +372,14 @@ cudaError_t launch_stress_div(const Geo& g, const T* u, const Body* bodies, cons
   const dim3 gr((g.n[0] + TILE_X - 1) / TILE_X, (g.n[1] + TILE_Y - 1) / TILE_Y, (g.n[2] + SFZ - 1) / SFZ);
   const cudaError_t e = cudaMemsetAsync(L.count, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  k_stress_fluid<T><<<gr, dim3(TILE_X, TILE_Y), 0, s>>>(g, u, views, nb, bbs, bstride, out, L);
+  launch_after(k_stress_fluid<T>, gr, dim3(TILE_X, TILE_Y), 0, s, g, u, views, nb, bbs, bstride, out, L);
   rmt_count_launches(1);
   if (nb == 0) return cudaSuccess;
   Rows9 R;
   for (int q = 0; q < 9; q++) R.r[q] = rows[q];
-  k_stress_rows<T><<<dim3(sm_count() * 8, 3), 128, 0, s>>>(g, u, bodies, views, t, toff, L, R);
+  launch_after(k_stress_rows<T>, dim3(sm_count() * 8, 3), 128, 0, s, g, u, bodies, views, t, toff, L, R);
   rmt_count_launches(1);
-  k_stress_band<T><<<sm_count() * 8, 128, 0, s>>>(g, u, bodies, views, t, toff, L, R, out);
+  launch_after(k_stress_band<T>, sm_count() * 8, 128, 0, s, g, u, bodies, views, t, toff, L, R, out);
   rmt_count_launches(1);
   return cudaSuccess;
 }
@@ -391,9 +394,10 @@ template cudaError_t launch_stress_div<double>(const Geo&, const double*, const 
 // simulated time on the device: t += dt after each step (read by the stress kernels, so that a
 // captured step graph needs no per-step parameter)
 __global__ void k_tick(double* t, double dt) {
+  wait_prior();
   if (threadIdx.x == 0 && blockIdx.x == 0) t[0] = t[0] + dt;
 }
 void launch_tick(double* t, double dt, cudaStream_t s) {
-  k_tick<<<1, 32, 0, s>>>(t, dt);
+  launch_after(k_tick, 1, 32, 0, s, t, dt);
   rmt_count_launches(1);
 }

@@ -90,6 +90,7 @@ template <typename T>
 __global__ void __launch_bounds__(XTPB) k_xi_predict(Geo g, const T* __restrict__ u,
                                                      const __grid_constant__ XiPredPtrs pp,
                                                      const __grid_constant__ BandSet<T> S) {
+  wait_prior();
   extern __shared__ double xi_smem[];
   XiTile<T>& t = *reinterpret_cast<XiTile<T>*>(xi_smem);
   const int m = S.m0 + blockIdx.y, a = blockIdx.z, tid = threadIdx.x;
@@ -271,7 +272,7 @@ cudaError_t launch_xi_predict(const Geo& g, const T* u, T* const vadv[3], T* con
     const cudaError_t e = cudaFuncSetAttribute(k_xi_predict<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_xi_predict<T><<<dim3(tiles, S.count, 3), XTPB, smem, s>>>(g, u, pp, S);
+  launch_after(k_xi_predict<T>, dim3(tiles, S.count, 3), XTPB, smem, s, g, u, pp, S);
   rmt_count_launches(1);
   return cudaSuccess;
 }
