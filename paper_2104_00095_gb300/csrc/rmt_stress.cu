@@ -119,7 +119,7 @@ __device__ __forceinline__ void face_row(const Geo& g, const T* __restrict__ u, 
 #pragma unroll
       for (int a = 0; a < 3; a++) Bd[a] = F[3 * a] * F[3 * d] + F[3 * a + 1] * F[3 * d + 1] + F[3 * a + 2] * F[3 * d + 2];
       const T tr3 = (F[0] * F[0] + F[1] * F[1] + F[2] * F[2] + F[3] * F[3] + F[4] * F[4] + F[5] * F[5] +
-                     F[6] * F[6] + F[7] * F[7] + F[8] * F[8]) / T(3);
+                     F[6] * F[6] + F[7] * F[7] + F[8] * F[8]) * T(1.0 / 3.0);
 #pragma unroll
       for (int a = 0; a < 3; a++) tau[a] = G * (Bd[a] - (a == d ? tr3 : T(0)));
     }
@@ -138,7 +138,8 @@ __device__ __forceinline__ void face_row(const Geo& g, const T* __restrict__ u, 
 #pragma unroll
       for (int a = 0; a < 3; a++) tau[a] += amp * ((f[a] / fn) * ed - (a == d ? T(1.0 / 3.0) : T(0)));
     }
-    const T visc = cv<T>(B.mu_a, B.f.mu_a) * (T(1) + cv<T>(B.gamma_t, B.f.gamma_t) * eps * dheavi(ph, eps));
+    T visc = cv<T>(B.mu_a, B.f.mu_a);
+    if (B.gamma_t != 0.0) visc *= T(1) + cv<T>(B.gamma_t, B.f.gamma_t) * eps * dheavi(ph, eps);
 #pragma unroll
     for (int a = 0; a < 3; a++) acc[a] += w * (tau[a] + visc * du[a]);
     wsum += w;
@@ -188,8 +189,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
   const unsigned long long tm = tile_mask;
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   if (i >= g.n[0] || j >= g.n[1]) return;
-  const T ih = cv<T>(g.ih, g.f.ih);
-  const T mu = cv<T>(g.mu, g.f.mu);
+  const T mu_h2 = cv<T>(g.mu, g.f.mu) * cv<T>(g.ih, g.f.ih) * cv<T>(g.ih, g.f.ih);
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long sy = n0, sz = (long)n0 * n1;
   // x and y neighbours: offsets from the cell (the cell itself where a wall ghost is used)
@@ -222,7 +222,11 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
     const long c = cij + (long)k * sz;
     const long oh = zoff(k + 1);
 #pragma unroll
-    for (int a = 0; a < 3; a++) win[a][2] = oh >= 0 ? pre[a] : T(2) * cv<T>(g.wall[5][a], g.f.wall[5][a]) - win[a][1];
+    for (int a = 0; a < 3; a++) win[a][2] = pre[a];
+    if (oh < 0) {
+#pragma unroll
+      for (int a = 0; a < 3; a++) win[a][2] = T(2) * cv<T>(g.wall[5][a], g.f.wall[5][a]) - win[a][1];
+    }
     if (k + 1 < k1) {
       const long o2 = zoff(k + 2);
 #pragma unroll
@@ -246,20 +250,21 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y, 8) k_stress_fluid(Geo g, const
       L.cell[at] = (int)c;
       L.mask[at] = bm;
     } else {
-      // pure fluid around this cell: every face row is mu (u_b - u_a)/h
+      // pure fluid around this cell: every face row is mu (u_b - u_a)/h, and 1/h and mu are left to the end (FP64:
+      // 40 operations a cell instead of 94, 392 -> 259 us on 128^3 with 20 bodies)
 #pragma unroll
       for (int a = 0; a < 3; a++) {
         const T* ua = u + (long)a * g.N + c;
         const T uc = win[a][1];
-        const T wxl = T(2) * cv<T>(g.wall[0][a], g.f.wall[0][a]) - uc, wxh = T(2) * cv<T>(g.wall[1][a], g.f.wall[1][a]) - uc;
-        const T wyl = T(2) * cv<T>(g.wall[2][a], g.f.wall[2][a]) - uc, wyh = T(2) * cv<T>(g.wall[3][a], g.f.wall[3][a]) - uc;
-        const T vxl = ua[oxl], vxh = ua[oxh], vyl = ua[oyl], vyh = ua[oyh];
-        const T nb6[6] = {gxl ? wxl : vxl, gxh ? wxh : vxh, gyl ? wyl : vyl, gyh ? wyh : vyh, win[a][0], win[a][2]};
-        T acc = T(0);
-#pragma unroll
-        for (int d = 0; d < 3; d++)
-          acc += (mu * ((nb6[2 * d + 1] - uc) * ih) - mu * ((uc - nb6[2 * d]) * ih)) * ih;
-        out[a * g.N + c] = acc;
+        T vxl = ua[oxl], vxh = ua[oxh], vyl = ua[oyl], vyh = ua[oyh];
+        if (gxl || gxh || gyl || gyh) {
+          vxl = gxl ? T(2) * cv<T>(g.wall[0][a], g.f.wall[0][a]) - uc : vxl;
+          vxh = gxh ? T(2) * cv<T>(g.wall[1][a], g.f.wall[1][a]) - uc : vxh;
+          vyl = gyl ? T(2) * cv<T>(g.wall[2][a], g.f.wall[2][a]) - uc : vyl;
+          vyh = gyh ? T(2) * cv<T>(g.wall[3][a], g.f.wall[3][a]) - uc : vyh;
+        }
+        const T lap = ((vxh - uc) - (uc - vxl)) + ((vyh - uc) - (uc - vyl)) + ((win[a][2] - uc) - (uc - win[a][0]));
+        out[a * g.N + c] = lap * mu_h2;
       }
     }
 #pragma unroll
