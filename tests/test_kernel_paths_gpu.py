@@ -154,3 +154,29 @@ def test_fe_solve_with_walls_fp32(n):
     (u64, c64), (u32, c32) = out
     assert rel_l2(u32, u64) <= 1e-5
     assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)
+
+
+@pytest.mark.parametrize("n,periodic", [((32, 32, 16), True), ((24, 20, 28), False), ((32, 16, 16), False),
+                                        ((28, 32, 12), True), ((36, 32, 16), False)])
+def test_small_mac_levels_in_one_block(n, periodic):
+    """Levels of one block's cells (16 x 16 x 8 and 16 x 8 x 8 fill it in FP32 and FP64, 18 x 16 x 8 does not fit, odd
+    rows): FP64 against the oracle, FP32 in the cycles of FP64 and to FP32 accuracy, the fused sweep's included."""
+    sc = _box(n, periodic)
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    g, o = pair(sc)
+    g.write(rmt.RMT_F_U, u)
+    assert o.write(O.F_U, u) == 0
+    g.step(1)
+    assert o.step(1) == 0, o.error()
+    compare_state(g, o, 0, 1e-10, tag=f"{n}")
+    g.close()
+    out = []
+    for prec, sweep in (("fp64", 0), ("fp32", 0), ("fp32", 2)):
+        g = rmt.Grid(dict(sc, precision=prec, mg_rtol=1e-9, mg_max_cycles=60, options={"mac_sweep": sweep}))
+        g.write(rmt.RMT_F_U, u)
+        g.step(1)
+        out.append((g.read(rmt.RMT_F_U), g.cycles()))
+        g.close()
+    for v, c in out[1:]:
+        assert rel_l2(v, out[0][0]) <= 1e-5
+        assert all(abs(a - b) <= 3 for a, b in zip(out[0][1], c)), (out[0][1], c)
