@@ -667,28 +667,30 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
-// All sweeps of a small level in one block: x in shared memory, and each thread with the face weights of its cells
-// of both colours in registers (pairs along x as in the colour passes, whose operations and order these are).  A colour
+// All sweeps of a small level in one block: x in shared memory, and each thread with the face weights of its C cells
+// of each colour in registers (pairs along x as in the colour passes, whose operations and order these are).  A colour
 // pass of such a level is a launch of some 2 us for 0.1 us of work; the limit is what the registers hold (FP32 1024
-// pairs, FP64 512).  A step with five pressure cycles in 48^3 1103 -> 1003 us, two levels of it so; the adaptive FP64 32^3
-// cavity 3% shorter.
+// pairs, FP64 512; with four cells of each colour to a thread, for 16^3, 128^3 cases took the same time).  A step with
+// five pressure cycles in 48^3, two levels of it so, 1103 -> 995 us; the adaptive FP64 32^3 cavity 4% shorter.
 constexpr int SMALL_TPB = 512;
+// cells of a colour per thread, 0 for a level that is too large
 template <typename T>
-constexpr int small_cells() { return sizeof(T) == 4 ? 2 : 1; }  // cells of a colour per thread
-template <typename T>
-inline bool mac_small(const Lv& L) {
-  return (long)((L.n[0] + 1) / 2) * L.n[1] * L.n[2] <= SMALL_TPB * small_cells<T>();
+inline int small_cells(const Lv& L) {
+  const long pairs = (long)((L.n[0] + 1) / 2) * L.n[1] * L.n[2];
+  const int most = sizeof(T) == 4 ? 2 : 1;
+  for (int c = 1; c <= most; c *= 2)
+    if (pairs <= (long)c * SMALL_TPB) return c;
+  return 0;
 }
-template <typename T>
+template <typename T, int C>
 __global__ void __launch_bounds__(SMALL_TPB) k_rbgs_block(Lv L, int sweeps, int first, T w, T* __restrict__ x,
                                                         const T* __restrict__ b, const T* __restrict__ rho, MacCoef F) {
   wait_prior();
-  constexpr int C = small_cells<T>();
   __shared__ T xs[2 * C * SMALL_TPB];
   const int ncell = (int)L.ncell, hx = (L.n[0] + 1) / 2, npair = hx * L.n[1] * L.n[2];
   for (int c = threadIdx.x; c < ncell; c += SMALL_TPB) xs[c] = x[c];
-  int at[2][C], nb[2][C][6];
-  T wt[2][C][6], dg[2][C], rd[2][C], bb[2][C];
+  unsigned short at[2][C], nb[2][C][6];
+  T wt[2][C][6], rd[2][C], bb[2][C];
 #pragma unroll
   for (int q = 0; q < 2; q++)
 #pragma unroll
@@ -698,23 +700,24 @@ __global__ void __launch_bounds__(SMALL_TPB) k_rbgs_block(Lv L, int sweeps, int 
       const bool in = u < npair && i < L.n[0];
       const int ii[3] = {i, j, k}, st[3] = {1, L.n[0], L.n[0] * L.n[1]};
       const int c = in ? i + L.n[0] * (j + L.n[1] * k) : 0;
-      at[q][t] = c;
-      dg[q][t] = rd[q][t] = bb[q][t] = T(0);
+      at[q][t] = (unsigned short)c;
+      rd[q][t] = bb[q][t] = T(0);
+      T dg = T(0);
 #pragma unroll
       for (int f = 0; f < 6; f++) {
         const int d = f >> 1, v = in ? cnb(L, d, ii[d] + (f & 1 ? 1 : -1)) : -1;
         const int cn = v >= 0 ? c + (v - ii[d]) * st[d] : c;
-        nb[q][t][f] = cn;
+        nb[q][t][f] = (unsigned short)cn;
         if constexpr (sizeof(T) == 4)
           wt[q][t][f] = v >= 0 ? face_beta<true>(rho[c], rho[cn]) : T(0);
         else
           wt[q][t][f] = v >= 0 ? F.f[d][f & 1 ? cn : c] : T(0);
-        dg[q][t] += wt[q][t][f];
+        dg += wt[q][t][f];
       }
       if (in) {
         bb[q][t] = b[c];
         if constexpr (sizeof(T) == 4) {
-          const float diag = dg[q][t] * L.f_ih2;
+          const float diag = dg * L.f_ih2;
           rd[q][t] = diag > 0.f ? rcp_approx(diag) : 0.f;
         } else {
           rd[q][t] = F.dinv[c];
@@ -730,10 +733,13 @@ __global__ void __launch_bounds__(SMALL_TPB) k_rbgs_block(Lv L, int sweeps, int 
         if (!(rd[q][t] > T(0))) continue;  // (also a pair past the level's end)
         const T xc = xs[at[q][t]];
         if constexpr (sizeof(T) == 4) {
-          float off = 0.f;
+          float off = 0.f, dg = 0.f;
 #pragma unroll
-          for (int f = 0; f < 6; f++) off += wt[q][t][f] * xs[nb[q][t][f]];
-          const float ax = (dg[q][t] * xc - off) * L.f_ih2;
+          for (int f = 0; f < 6; f++) {
+            off += wt[q][t][f] * xs[nb[q][t][f]];
+            dg += wt[q][t][f];
+          }
+          const float ax = (dg * xc - off) * L.f_ih2;
           xs[at[q][t]] = xc + w * ((bb[q][t] - ax) * rd[q][t]);
         } else {
           double v = bb[q][t];
@@ -2358,10 +2364,12 @@ void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
   const Lv& L = m->lv[l];
   const T* b = (const T*)m->b[l];
   const T* rho = (const T*)m->rho[l];
-  if (m->kind == 0 && m->sweep != 2 && sweeps > 0 && mac_small<T>(L)) {
+  const int small = m->kind == 0 && m->sweep != 2 && sweeps > 0 ? small_cells<T>(L) : 0;
+  if (small > 0) {
     hk(m, l, 0, 1, s);
-    launch_after(k_rbgs_block<T>, 1, SMALL_TPB, 0, s, L, sweeps, forward ? 0 : 1, T(m->omega), (T*)m->x[l], b, rho,
-                 mac_coef(m, l));
+    auto kernel = k_rbgs_block<T, 1>;
+    if constexpr (sizeof(T) == 4) kernel = small == 1 ? k_rbgs_block<T, 1> : k_rbgs_block<T, 2>;
+    launch_after(kernel, 1, SMALL_TPB, 0, s, L, sweeps, forward ? 0 : 1, T(m->omega), (T*)m->x[l], b, rho, mac_coef(m, l));
     rmt_count_launches(1);
     hk(m, l, 0, 0, s);
     return;

@@ -157,10 +157,11 @@ def test_fe_solve_with_walls_fp32(n):
 
 
 @pytest.mark.parametrize("n,periodic", [((32, 32, 16), True), ((24, 20, 28), False), ((32, 16, 16), False),
-                                        ((28, 32, 12), True), ((36, 32, 16), False)])
+                                        ((28, 32, 12), True), ((36, 32, 16), False),
+                                        ((32, 32, 32), True), ((36, 32, 28), False)])
 def test_small_mac_levels_in_one_block(n, periodic):
-    """Levels of one block's cells (16 x 16 x 8 and 16 x 8 x 8 fill it in FP32 and FP64, 18 x 16 x 8 does not fit, odd
-    rows): FP64 against the oracle, FP32 in the cycles of FP64 and to FP32 accuracy, the fused sweep's included."""
+    """Levels of one block's cells (16 x 16 x 8 and 16 x 8 x 8 fill it in FP32 and FP64, 18 x 16 x 8 and 16^3 do not
+    fit, odd rows): FP64 against the oracle, FP32 in the cycles of FP64 and to FP32 accuracy, the fused sweep's included."""
     sc = _box(n, periodic)
     u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
     g, o = pair(sc)
