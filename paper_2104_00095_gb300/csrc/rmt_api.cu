@@ -101,7 +101,7 @@ struct rmt_grid {
   void *adv = nullptr, *ustar = nullptr, *psi = nullptr;
   void* vadv[3] = {};
   void* slopes[9] = {};
-  void* wcell[9] = {};  // FP64: scratch of the Godunov passes
+  void* wcell[6] = {};  // FP64: scratch of the Godunov passes (with the advective term's array)
   void* uf[3][3] = {};
   void* umac[3] = {};
   MGSolver* mac = nullptr;
@@ -460,7 +460,7 @@ rmt_status alloc_t(rmt_grid* g) {
   AL(g->psi, G.NN * e);
   for (int q = 0; q < 9; q++) {
     AL(g->slopes[q], N * e);
-    if (e == 8) AL(g->wcell[q], N * e);
+    if (e == 8 && q < 6) AL(g->wcell[q], N * e);
   }
   for (int d = 0; d < 3; d++) {
     const long nf = nfaces(G, d);
@@ -590,7 +590,7 @@ rmt_status step_t(rmt_grid* g) {
   }
   for (int q = 0; q < 9; q++) {
     slopes[q] = (T*)g->slopes[q];
-    wcell[q] = (T*)g->wcell[q];
+    wcell[q] = q < 6 ? (T*)g->wcell[q] : (T*)g->adv + (q - 6) * G.N;  // (the advective term comes later)
   }
   T* u = (T*)g->u;
   // 1. tau^n and its divergence

@@ -115,7 +115,7 @@ void launch_fill(T* a, T v, long n, cudaStream_t s);
 
 // ---- extrapolation (rmt_extrap.cu) ------------------------------------------------
 // One body's arrays.  list: the band's cells sorted by layer (capacity: the grid), written by the layer
-// passes of launch_extrapolate and read by launch_corrector of the same step; cnt: BAND_COUNTERS ints,
+// passes and read by the fits and the corrector of the same step; cnt: BAND_COUNTERS ints,
 // cnt[l] the cells of layer l (l = 1..8), cnt[BAND_TICKET] the finished blocks of the last pass; bb: the
 // band's bounding boxes of the two parities (6 ints each)
 constexpr int BAND_COUNTERS = 10, BAND_TICKET = 9;
