@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(TPB) k_classify(Geo g, const __grid_constant__
       const long c = r.base + i;
       const T x0 = x[c], x1 = x[g.N + c], x2 = x[2 * g.N + c];
       int8_t l = -1;
-      if (isfinite(x0) && isfinite(x1) && isfinite(x2) && phi_stored(g, b, i, r.j, r.k, x0, x1, x2) < T(0)) l = 0;
+      if (finite_bits(x0) && finite_bits(x1) && finite_bits(x2) && phi_stored_neg(g, b, i, r.j, r.k, x0, x1, x2)) l = 0;
       lay[c] = l;
     }
   }

@@ -181,3 +181,23 @@ def test_small_mac_levels_in_one_block(n, periodic):
     for v, c in out[1:]:
         assert rel_l2(v, out[0][0]) <= 1e-5
         assert all(abs(a - b) <= 3 for a, b in zip(out[0][1], c)), (out[0][1], c)
+
+
+@pytest.mark.parametrize("shape,size,turn,precision", [(S.SPHERE, (8, 8, 8), False, "fp64"),
+                                                       (S.ELLIPSOID, (8, 5, 3), False, "fp64"),
+                                                       (S.ELLIPSOID, (11, 7.3, 2.2), True, "fp64"),
+                                                       (S.ELLIPSOID, (11, 7.3, 2.2), True, "fp32"),
+                                                       (S.SPHERE, (8.3, 8.3, 8.3), False, "fp32")])
+def test_layer_zero_is_the_sign_of_the_level_set(shape, size, turn, precision):
+    """Bodies whose surface passes through cell centres exactly (phi_0 = 0 there: not inside), and turned ones: the
+    layers are the oracle's at every cell."""
+    n = 32
+    sc = S._box(n, periodic=False)
+    sc.update(dt=0.2 / n, precision=precision)
+    sc["solids"] = [S.solid(shape, (16.5 / n,) * 3, tuple(v / n for v in size),
+                            S.random_rotation(np.random.default_rng(5)) if turn else None)]
+    g, o = pair(sc)
+    g.step(0)
+    assert o.step(0) == 0, o.error()
+    assert np.array_equal(g.read(rmt.RMT_F_LAYER, 0), o.read(O.F_LAYER, 0))
+    g.close()
