@@ -209,15 +209,6 @@ __device__ __forceinline__ T uval(const Geo& g, const T* __restrict__ u, int a, 
   return add + s * u[a * g.N + cidx(g, ii[0], ii[1], ii[2])];
 }
 
-// u component a at (i,j,k) along with its +-r neighbours on axis d: direct loads when the whole
-// stencil lies inside the grid (the common case), the boundary rules otherwise
-template <typename T>
-__device__ __forceinline__ bool inside(const Geo& g, int d, int i, int j, int k, int r) {
-  const int ii[3] = {i, j, k};
-  if (ii[0] < 0 || ii[0] >= g.n[0] || ii[1] < 0 || ii[1] >= g.n[1] || ii[2] < 0 || ii[2] >= g.n[2]) return false;
-  return ii[d] - r >= 0 && ii[d] + r < g.n[d];
-}
-
 // 3-D launch geometry for cell/face/node kernels: 32 x 4 threads per block in x and y, one
 // block layer per z index
 #define TILE_X 32
@@ -562,26 +553,6 @@ __device__ __forceinline__ void split3(long t, int n0, int n1, int& a, int& b, i
 }
 // cell or node coordinates of a linear index on an nx x ny x .. grid
 __device__ __forceinline__ void decode(long c, int nx, int ny, int& i, int& j, int& k) { split3(c, nx, ny, i, j, k); }
-
-// t-th cell of a window: unwrapped coordinates u[] and the wrapped cell index c
-__device__ __forceinline__ void win_cell(const Geo& g, const Win& w, long t, int u[3], int& i, int& j, int& k,
-                                         long& c) {
-  int a, b, cc;
-  split3(t, w.ext[0], w.ext[1], a, b, cc);
-  u[0] = w.lo[0] + a;
-  u[1] = w.lo[1] + b;
-  u[2] = w.lo[2] + cc;
-  int v[3];
-  // one wrap is enough: a window starts within dil cells of [0, n) and is at most n long
-#pragma unroll
-  for (int d = 0; d < 3; d++) v[d] = u[d] < 0 ? u[d] + g.n[d] : (u[d] >= g.n[d] ? u[d] - g.n[d] : u[d]);
-  i = v[0];
-  j = v[1];
-  k = v[2];
-  c = cidx(g, i, j, k);
-}
-#define WIN_LOOP(t, w) \
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < (w).vol; t += (long)gridDim.x * blockDim.x)
 
 // The window row by row: a warp takes rows of constant (j, k) and its lanes the cells along x, so that a row's
 // index arithmetic (a division, the wraps) is done once per row and not once per cell.  WIN_ROWS(w, row)
