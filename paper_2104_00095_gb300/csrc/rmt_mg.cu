@@ -2425,7 +2425,7 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
     if (L.n[1] > nmax) nmax = L.n[1];
     if (L.n[2] > nmax) nmax = L.n[2];
     // conjugate gradients converge in O(nmax) iterations on this level; the cap only bounds
-    // the launch, the tolerance ends it
+    // the launch (FP64 refinement: COARSE_WORK times as many in FP32), the tolerance ends it
     const int max_it = 8 * nmax + 64;
     const double tol = coarse_tol<T>();
     rmt_count_launches(1);

@@ -11,9 +11,12 @@
 // shared memory.
 //
 // FP64 levels: FP32 solves inside FP64 refinement.  The FP64 residual of the solution is updated
-// as r -= A e with FP64 coefficients and sums until it is 1e-10 of the right-hand side, the same
-// criterion as an FP64 CG; four refinements replace some 25 FP64 iterations, and GB300 has 2
-// FP64 lanes per SM against 128 FP32 ones, which the one-block FP64 CG was bound by.
+// as r -= A e with FP64 coefficients and sums until it is 1e-10 of the right-hand side, the
+// criterion of an FP64 CG (it ends at 1e-11 to 3e-11, the CG at 3e-11 to 1e-10); three refinements
+// replace 20 to 200 FP64 iterations, and GB300 has 2 FP64 lanes per SM against 128 FP32 ones,
+// which the one-block FP64 CG was bound by.  A level whose FP32 solves stall on rounding, or that needs
+// more iterations than the launch allows, is left above the criterion, as the CG left it at its
+// iteration limit; the outer solve measures its own residual.
 //
 // Bound: the latency chain of an iteration (shared loads, butterfly, barriers; about 0.3 us in one
 // block, 1 us in a cluster).  Against the one-block CG that formed its coefficients in every
@@ -26,6 +29,7 @@ constexpr int COARSE_CL = 8;         // largest cluster (the portable limit)
 constexpr int COARSE_ONE = 1024;     // unknowns of a single-block solve (FP32)
 constexpr int COARSE_ONE64 = 256;    // ... FP64: its operator is bound by one SM's FP64 lanes
 constexpr int COARSE_UPT = 8;        // unknowns per thread at most
+constexpr int COARSE_WORK = 8;       // FP64: FP32 iterations of all passes together, in units of max_it
 // threads of a block: one unknown each up to 1024, else 4 or 8 on 512 (128 registers a thread)
 constexpr int COARSE_MAXT = 1024, COARSE_MULTT = 512;
 
@@ -254,8 +258,9 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
     if (last[q]) dhi[in - (np - 1) * ps] = v;
   };
   float x[UPT], r[UPT], p[UPT], s[UPT];
-  // FP32 CG of A x = r from x = 0 to the relative residual tol; r is used up
-  auto solve32 = [&]() {
+  // FP32 CG of A x = r from x = 0 to the relative residual tol, in at most left iterations; r is used up.  Returns
+  // the iterations taken
+  auto solve32 = [&](int left) {
     float g = 0.f, dummy = 0.f;
 #pragma unroll
     for (int q = 0; q < UPT; q++) {
@@ -266,7 +271,8 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
     sum2(g, dummy);
     const float stop = tol * tol * g;
     float gamma = g, alpha = 0.f;
-    for (int it = 0; it < max_it && gamma > stop; it++) {
+    int it = 0;
+    for (; it < left && gamma > stop; it++) {
       if (it > 0) {
 #pragma unroll
         for (int q = 0; q < UPT; q++) publish(q, r[q]);
@@ -282,11 +288,12 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
       }
       sum2(rr, rw);
       if (it > 0 && !(rr > stop)) break;
-      const float beta = it > 0 ? __fdividef(rr, gamma) : 0.f;
-      const float den = it > 0 ? rw - __fdividef(beta * rr, alpha) : rw;
+      // (whole divisions: an approximate quotient's two units more would enter every later iterate)
+      const float beta = it > 0 ? rr / gamma : 0.f, back = it > 0 ? rr / alpha : 0.f;
+      const float den = rw - beta * back;
       if (!(den > 0.f)) break;
       gamma = rr;
-      alpha = __fdividef(rr, den);
+      alpha = rr / den;
 #pragma unroll
       for (int q = 0; q < UPT; q++) {
         p[q] = r[q] + beta * p[q];
@@ -295,6 +302,7 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
         r[q] -= alpha * s[q];
       }
     }
+    return it;
   };
   const long u0 = (long)k0 * ps;
   const double inv_n = 1.0 / (double)L.nunk;
@@ -309,7 +317,7 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
     mean *= (float)inv_n;
 #pragma unroll
     for (int q = 0; q < UPT; q++) r[q] = own[q] ? r[q] - mean : 0.f;
-    solve32();
+    solve32(max_it);
     dummy = 0.f;
 #pragma unroll
     for (int q = 0; q < UPT; q++) xm_ += x[q];
@@ -337,12 +345,17 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
     }
     sum2(rr, dummy);
     const double stop = tol64 * tol64 * rr;
-    // each pass gains the FP32 solve's factor tol; the cap bounds the launch
-    for (int it = 0; it < 24 && rr > stop; it++) {
+    // Each pass gains the FP32 solve's factor tol, or what rounding leaves of it: on to the next one while a pass takes
+    // a tenth off the residual.  A pass that does not lower the residual is dropped.  COARSE_WORK max_it iterations in
+    // all bound the launch.  With a body of 1/1000 to 1000 times the fluid's density, levels of 4^3 to 27^3 cells or
+    // nodes (restated on the CPU): the residual is at or below that of an FP64 CG of max_it iterations everywhere, and
+    // 1e-10 of the right-hand side up to a ratio of 100 either way on 17 x 15 x 16; 1/1000 ends at 1e-4 .. 3e-3
+    // (the FP64 CG at 0.1 .. 0.6).
+    for (int left = COARSE_WORK * max_it; left > 0 && rr > stop;) {
       const double nrm = sqrt(rr), inv = 1.0 / nrm;
 #pragma unroll
       for (int q = 0; q < UPT; q++) r[q] = (float)(rd[q] * inv);
-      solve32();
+      left -= max(solve32(left), 1);
       sync_all();  // the last operator has read the published vector
 #pragma unroll
       for (int q = 0; q < UPT; q++) publish(q, x[q]);
@@ -351,14 +364,14 @@ __global__ void __launch_bounds__(UPT == 1 ? COARSE_MAXT : COARSE_MULTT)
       dummy = 0.0;
 #pragma unroll
       for (int q = 0; q < UPT; q++) {
-        if (own[q]) {
-          rd[q] -= nrm * apply(q, (const double*)cd, 0.0);
-          xd[q] += nrm * (double)x[q];
-        }
+        if (own[q]) rd[q] -= nrm * apply(q, (const double*)cd, 0.0);
         rn += rd[q] * rd[q];
       }
       sum2(rn, dummy);
-      if (!(rn < 0.25 * rr)) break;  // rounding has the last word
+      if (!(rn < rr)) break;
+#pragma unroll
+      for (int q = 0; q < UPT; q++) xd[q] += nrm * (double)x[q];
+      if (!(rn < 0.81 * rr)) break;
       rr = rn;
     }
     double xs = 0.0;
@@ -402,7 +415,7 @@ cudaError_t launch_coarse_solve(const CoarseCfg& c, int kind, const Lv& L, int m
   lc.numAttrs = c.cs > 1 ? 2 : 1;
   Lv Lk = L;
   int cs = c.cs, mplanes = c.mcap / c.ps, mi = max_it;
-  // FP64: an FP32 pass of 3e-4, three of which reach 1e-10
+  // FP64: FP32 passes of 3e-4; three reach 1e-10 where none of them runs out of iterations
   float tf = sizeof(T) == 8 ? 3e-4f : (float)tol;
   double td = tol;
   void* args[] = {&Lk, &cs, &mplanes, &mi, &tf, &td, &x, (void*)&b, (void*)&rho};

@@ -62,6 +62,22 @@ def test_coarsest_level_solves_fp32(n, periodic):
     assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)
 
 
+@pytest.mark.parametrize("n", [(17, 15, 16), (23, 23, 23), (9, 7, 5)])
+@pytest.mark.parametrize("ratio", [0.001, 0.01, 100.0, 1000.0])
+def test_one_level_solves_at_density_ratios_fp64(n, ratio):
+    """Grids of one level (an odd side) with a body far lighter or heavier than the fluid, solved to 1e-12.  Restated
+    on the CPU, a solve leaves at most 2.7e-3 of its right-hand side at these ratios, so five gain twelve digits; one that
+    left when a pass no longer halved the residual kept 0.3 to 0.5 of it at a ratio of 1/1000 and took above twenty."""
+    sc = _with_body(n, False)
+    sc["solids"][0]["rho_s"] = ratio
+    sc.update(mg_rtol=1e-12, mg_max_cycles=60)
+    g = rmt.Grid(sc)
+    g.write(rmt.RMT_F_U, 0.1 * np.sin(np.arange(3 * np.prod(n)) * 0.37))
+    g.step(1)
+    assert max(g.cycles()) <= 8, g.cycles()
+    g.close()
+
+
 @pytest.mark.parametrize("n,periodic,precision", [((36, 40, 44), True, "fp32"), ((33, 35, 50), False, "fp32"),
                                                   ((36, 40, 44), True, "fp64")])
 def test_float_reads_of_every_field(n, periodic, precision):
