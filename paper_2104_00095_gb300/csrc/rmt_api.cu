@@ -291,12 +291,16 @@ __global__ void k_cvt_i8(const int8_t* __restrict__ a, OT* __restrict__ b, long 
   GRID_LOOP(i, n) b[i] = (OT)a[i];
 }
 // A reference map stored as displacements to xi = S + x0, x0 = lo + (u + 1/2) h the cell centre's
-// image, as float or double.  Bound: HBM (one read and one write per value).  x0 depends on one index
-// per axis, so a thread marches up a column of XOZ cells with the x and y parts in registers and the
-// block's z parts in shared memory; for float output x0 is a two-float pair and the sum's rounding
-// error is carried (Knuth's two-sum), which leaves the FP64 pipe (two lanes per SM) idle.  A
-// linear loop with 64-bit divisions and FP64 sums took 484 us per 256^3 map plus 166 us of
-// conversion and copy (201 MB out); this takes 72 us.
+// image, as float or double; a float is the rounded FP64 sum.  Bound: HBM (one read and one write per value).  x0
+// depends on one index per axis, so a thread marches up a column of XOZ cells with the x and y parts in
+// registers and the block's z parts in shared memory.  For float output x0 is a two-float pair h + l and the sum's
+// rounding error is carried (Knuth's two-sum), which leaves the FP64 pipe (two lanes per SM) idle: s + t with
+// t = fl(e + l) is off by at most 2^-24 |t| (t), 2^-48 |h| (l) and 2^-53 (|h| + |v|) (the FP64 sum's own rounding),
+// together less than half of m below, and t -+ m are off by a quarter of m at most; where s + (t - m) and s + (t + m)
+// round alike, so does the FP64 sum between them, and where they do not (one value in some 10^5) it is formed.  With
+// l = 0 the pair is x0 and s the rounded sum.
+// A linear loop with 64-bit divisions and FP64 sums took 484 us per 256^3 map plus 166 us of
+// conversion and copy (201 MB out); this takes 86 us (72 with the pair alone, not always the rounded sum).
 constexpr int XOZ = 16;
 template <typename OT>
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_xi_out(Geo g, Body b, const float* __restrict__ x,
@@ -305,12 +309,12 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_xi_out(Geo g, Body b, const 
   __shared__ float zh[XOZ], zl[XOZ];
   const int i = blockIdx.x * TILE_X + threadIdx.x, j = blockIdx.y * TILE_Y + threadIdx.y;
   const int k0 = blockIdx.z * XOZ, k1 = min(k0 + XOZ, g.n[2]);
-  const int t = threadIdx.y * TILE_X + threadIdx.x;
+  const int tid = threadIdx.y * TILE_X + threadIdx.x;
   auto image = [&](int a, int q) { return g.lo[a] + (img_u(g, b, a, q) + 0.5) * g.h; };
-  if (t < k1 - k0) {
-    z0[t] = image(2, k0 + t);
-    zh[t] = (float)z0[t];
-    zl[t] = (float)(z0[t] - (double)zh[t]);
+  if (tid < k1 - k0) {
+    z0[tid] = image(2, k0 + tid);
+    zh[tid] = (float)z0[tid];
+    zl[tid] = (float)(z0[tid] - (double)zh[tid]);
   }
   __syncthreads();
   if (i >= g.n[0] || j >= g.n[1]) return;
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_xi_out(Geo g, Body b, const 
   for (int a = 0; a < 3; a++) {
     const float* xa = x + a * g.N + c0;
     OT* oa = out + a * g.N + c0;
+    unsigned unsure = 0;
 #pragma unroll 4
     for (int k = 0; k < k1 - k0; k++) {
       const float v = xa[k * plane];
@@ -330,9 +335,16 @@ __global__ void __launch_bounds__(TILE_X* TILE_Y) k_xi_out(Geo g, Body b, const 
       } else {
         const float h = a < 2 ? h2[a & 1] : zh[k], l = a < 2 ? l2[a & 1] : zl[k];
         const float s = __fadd_rn(h, v), bb = __fsub_rn(s, h);
-        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb));
-        oa[k * plane] = __fadd_rn(s, __fadd_rn(e, l));
+        const float t = __fadd_rn(__fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb)), l);
+        const float m = l != 0.f ? __fmaf_rn(fabsf(h) + fabsf(v), 0x1p-46f, fabsf(t) * 0x1p-22f) : 0.f;
+        const float r = __fadd_rn(s, __fsub_rn(t, m));
+        oa[k * plane] = r;
+        if (r != __fadd_rn(s, __fadd_rn(t, m)) && v == v) unsure |= 1u << k;
       }
+    }
+    for (; unsure; unsure &= unsure - 1) {  // (after the column: predicated FP64 sums would be issued for every value)
+      const int k = __ffs(unsure) - 1;
+      oa[k * plane] = (OT)((double)xa[k * plane] + (a < 2 ? xy[a & 1] : z0[k]));
     }
   }
 }

@@ -102,6 +102,24 @@ def test_float_reads_of_every_field(n, periodic, precision):
     g.close()
 
 
+@pytest.mark.parametrize("n,periodic", [((100, 98, 96), True), ((100, 74, 66), False)])
+def test_float_reads_of_a_map_are_the_rounded_fp64_reads(n, periodic):
+    """Every value of a body whose cell centres, from a corner at -0.3 in steps of 0.01, are not floats (of some 10^3
+    displacements one makes a sum of a two-float centre round the other way)."""
+    sc = dict(_with_body(n, periodic), precision="fp32", mg_rtol=1e-6, lo=(-0.3,) * 3)
+    sc["hi"] = tuple(v / 100 - 0.3 for v in n)
+    sc["solids"][0]["center"] = tuple(v - 0.3 for v in sc["solids"][0]["center"])
+    g = rmt.Grid(sc)
+    z, y, x = np.meshgrid(*[(np.arange(v) + 0.5) / 100 - 0.3 for v in n[::-1]], indexing="ij")
+    for seed in range(4):
+        w = np.random.default_rng(seed).uniform(5, 9, 3)
+        xi = np.stack([c + 0.02 * np.sin(f * (x + 2 * y - z)) for c, f in zip((x, y, z), w)])
+        g.write(rmt.RMT_F_XI, xi.reshape(-1))
+        a, b = g.read_float(rmt.RMT_F_XI), g.read(rmt.RMT_F_XI).astype(np.float32)
+        assert np.array_equal(a, b, equal_nan=True), np.count_nonzero((a != b) & ~np.isnan(b))
+    g.close()
+
+
 @pytest.mark.parametrize("layers,periodic,precision", [(1, True, "fp64"), (4, False, "fp64"), (8, True, "fp64"),
                                                        (4, True, "fp32")])
 def test_extrapolation_of_unequal_bodies(layers, periodic, precision):
