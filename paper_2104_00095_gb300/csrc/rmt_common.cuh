@@ -361,6 +361,17 @@ __device__ __forceinline__ bool near_seam(const Geo& g, const Body& b, int i, in
   return false;
 }
 
+__device__ __forceinline__ float fma_any(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_any(double a, double b, double c) { return __fma_rn(a, b, c); }
+// a / d where id = 1 / d, rounded, is at hand: the product's exact remainder corrects it, which rounds the quotient as a
+// division does but for cases beside a tie (Markstein 1990; the product alone is off by up to one unit and a half).
+// Two multiply-adds for the ten and more instructions of a division.
+template <typename T>
+__device__ __forceinline__ T quot(T a, T d, T id) {
+  const T q = a * id;
+  return fma_any(fma_any(-q, d, a), id, q);
+}
+
 // smoothed Heaviside (eq. sm_heavi) and its derivative
 template <typename T>
 __device__ __forceinline__ T heavi(T phi, T eps) {
@@ -368,7 +379,7 @@ __device__ __forceinline__ T heavi(T phi, T eps) {
   if (phi >= eps) return T(1);
   if constexpr (sizeof(T) == 8) {  // (an FP64 division takes 20 instructions of the FP64 units)
     const T x = phi / eps;
-    return T(0.5) * (T(1) + x + sin(T(RMT_PI) * x) * T(1.0 / RMT_PI));
+    return T(0.5) * (T(1) + x + quot(sin(T(RMT_PI) * x), T(RMT_PI), T(1.0 / RMT_PI)));
   } else {
     return T(0.5) * (T(1) + phi / eps + sin(T(RMT_PI) * phi / eps) / T(RMT_PI));
   }
@@ -429,8 +440,10 @@ __device__ __forceinline__ T dflim2(T qm, T q0, T qp) {
 template <typename T>
 __device__ __forceinline__ T lim_slope4(T qm, T q0, T qp, T dfm2, T dfp2) {
   const T d = qp - qm;
-  // the twelfth as a product (a division per slope would dominate the kernel)
-  const T d4 = T(2.0 / 3.0) * d - (dfp2 + dfm2) * T(1.0 / 12.0);
+  // FP32: the twelfth as a product (a division per slope would dominate the kernel)
+  T d4;
+  if constexpr (sizeof(T) == 4) d4 = T(2.0 / 3.0) * d - (dfp2 + dfm2) * T(1.0 / 12.0);
+  else d4 = T(2.0 / 3.0) * d - quot(dfp2 + dfm2, T(12), T(1.0 / 12.0));
   return sgn_min(d, d4, T(2) * mc_min(qm, q0, qp));
 }
 template <typename T>
@@ -474,18 +487,20 @@ __device__ __forceinline__ bool inv3(const T A[9], T F[9]) {
   const T det = A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) +
                 A[2] * (A[3] * A[7] - A[4] * A[6]);
   if (det == T(0) || !isfinite(det)) return false;
-  if constexpr (sizeof(T) == 8) {  // one division instead of nine: 29 FP64 instructions for 180
+  if constexpr (sizeof(T) == 8) {  // one division instead of nine: 47 FP64 instructions for 180
     const T id = T(1) / det;
-    F[0] = (A[4] * A[8] - A[5] * A[7]) * id;
-    F[1] = (A[2] * A[7] - A[1] * A[8]) * id;
-    F[2] = (A[1] * A[5] - A[2] * A[4]) * id;
-    F[3] = (A[5] * A[6] - A[3] * A[8]) * id;
-    F[4] = (A[0] * A[8] - A[2] * A[6]) * id;
-    F[5] = (A[2] * A[3] - A[0] * A[5]) * id;
-    F[6] = (A[3] * A[7] - A[4] * A[6]) * id;
-    F[7] = (A[1] * A[6] - A[0] * A[7]) * id;
-    F[8] = (A[0] * A[4] - A[1] * A[3]) * id;
-    return true;
+    if (finite_bits(id)) {
+      F[0] = quot(A[4] * A[8] - A[5] * A[7], det, id);
+      F[1] = quot(A[2] * A[7] - A[1] * A[8], det, id);
+      F[2] = quot(A[1] * A[5] - A[2] * A[4], det, id);
+      F[3] = quot(A[5] * A[6] - A[3] * A[8], det, id);
+      F[4] = quot(A[0] * A[8] - A[2] * A[6], det, id);
+      F[5] = quot(A[2] * A[3] - A[0] * A[5], det, id);
+      F[6] = quot(A[3] * A[7] - A[4] * A[6], det, id);
+      F[7] = quot(A[1] * A[6] - A[0] * A[7], det, id);
+      F[8] = quot(A[0] * A[4] - A[1] * A[3], det, id);
+      return true;
+    }
   }
   F[0] = (A[4] * A[8] - A[5] * A[7]) / det;
   F[1] = (A[2] * A[7] - A[1] * A[8]) / det;

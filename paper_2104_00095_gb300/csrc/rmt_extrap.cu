@@ -147,7 +147,7 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
     for (int i = k + 1; i < 4; i++) {
       AT t = A[i][k];
       for (int j = 0; j < k; j++) t -= L[i][j] * L[k][j] * D[j];
-      L[i][k] = t * iD[k];
+      L[i][k] = quot(t, s, iD[k]);
     }
   }
   for (int c = 0; c < 3; c++) {
@@ -157,7 +157,7 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
       for (int j = 0; j < i; j++) t -= L[i][j] * y[j];
       y[i] = t;
     }
-    for (int i = 0; i < 4; i++) y[i] *= iD[i];
+    for (int i = 0; i < 4; i++) y[i] = quot(y[i], D[i], iD[i]);
     for (int i = 3; i >= 0; i--) {
       AT t = y[i];
       for (int j = i + 1; j < 4; j++) t -= L[j][i] * X[j][c];
@@ -462,8 +462,6 @@ __device__ __forceinline__ void slot_cand(const Geo& g, const Slots& s, const T*
     }
   }
 }
-__device__ __forceinline__ float fma_any(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_any(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // lane totals: v[q] summed over the warp ends in lane q (32 values) -- or, HALF (16 values), in lanes
 // 2 q and 2 q + 1
@@ -586,7 +584,7 @@ __device__ int wls_batch(const Geo& g, const Body& b, const Slots& sl, WlsShared
       if (nv > AT(0)) {
         const AT in = AT(1) / nv;
 #pragma unroll
-        for (int q = 0; q < 3; q++) nrm[q] = v[q] * in;
+        for (int q = 0; q < 3; q++) nrm[q] = quot(v[q], nv, in);
       } else {
         ok = 0;
       }

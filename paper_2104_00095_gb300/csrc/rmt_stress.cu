@@ -118,8 +118,9 @@ __device__ __forceinline__ void face_row(const Geo& g, const T* __restrict__ u, 
       T Bd[3];
 #pragma unroll
       for (int a = 0; a < 3; a++) Bd[a] = F[3 * a] * F[3 * d] + F[3 * a + 1] * F[3 * d + 1] + F[3 * a + 2] * F[3 * d + 2];
-      const T tr3 = (F[0] * F[0] + F[1] * F[1] + F[2] * F[2] + F[3] * F[3] + F[4] * F[4] + F[5] * F[5] +
-                     F[6] * F[6] + F[7] * F[7] + F[8] * F[8]) * T(1.0 / 3.0);
+      const T tr3 = quot(F[0] * F[0] + F[1] * F[1] + F[2] * F[2] + F[3] * F[3] + F[4] * F[4] + F[5] * F[5] +
+                             F[6] * F[6] + F[7] * F[7] + F[8] * F[8],
+                         T(3), T(1.0 / 3.0));
 #pragma unroll
       for (int a = 0; a < 3; a++) tau[a] = G * (Bd[a] - (a == d ? tr3 : T(0)));
     }

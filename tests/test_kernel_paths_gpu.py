@@ -152,6 +152,37 @@ def test_extrapolation_of_unequal_bodies(layers, periodic, precision):
     g.close()
 
 
+def test_extrapolation_rounds_no_more_than_with_divisions():
+    """Affine maps, which the fits reproduce but for rounding: the rms error of layers 1 and 3 over four bodies, in
+    units of 2^-53.  Fits that divide have 5.16 and 6.91 of them, fits that multiply by a rounded reciprocal pivot 5.62 and
+    7.77: the bounds lie midway."""
+    import ctypes as C
+
+    import torch
+
+    wide, rms = np.longdouble, []
+    for n, layers, r, seed in ((61, 5, 0.3, 1), (47, 4, 0.18, 4), (80, 5, 0.22, 5), (33, 3, 0.2, 2)):
+        rng = np.random.default_rng(seed)
+        sc = S._box(n, periodic=False)
+        sc["band_layers"] = layers
+        body = S.solid(S.ELLIPSOID, 0.5 + rng.uniform(-0.05, 0.05, 3), r * rng.uniform(0.6, 1.0, 3), S.random_rotation(rng))
+        x = (np.arange(n) + 0.5) / n
+        z, y, x = (v.reshape(-1).astype(wide) for v in np.meshgrid(x, x, x, indexing="ij"))
+        m = np.eye(3) + 0.02 * rng.normal(size=(3, 3))
+        exact = [wide(a) * x + wide(b) * y + wide(c) * z for a, b, c in m]
+        xi = torch.tensor(np.stack([v.astype(np.float64) for v in exact])).cuda()
+        out, phi = torch.empty_like(xi), torch.empty(n**3, dtype=torch.float64, device="cuda")
+        lay = torch.empty(n**3, dtype=torch.int8, device="cuda")
+        d, b = rmt.make_grid_desc(sc), rmt.make_solid_desc(body)
+        assert rmt.load().rmt_extrapolate_noalloc(C.byref(d), C.byref(b), xi.data_ptr(), out.data_ptr(), phi.data_ptr(),
+                                                  lay.data_ptr(), torch.cuda.current_stream().cuda_stream) == rmt.RMT_OK
+        lay, out = lay.cpu().numpy(), out.cpu().numpy()
+        err = lambda l: np.concatenate([(out[a][lay == l].astype(wide) - exact[a][lay == l]) for a in range(3)])
+        rms.append([np.sqrt(np.mean(err(l).astype(np.float64)**2)) * 2.0**53 for l in (1, 3)])
+    got = np.mean(rms, axis=0)
+    assert got[0] <= 5.39 and got[1] <= 7.34, got
+
+
 @pytest.mark.parametrize("n,periodic,precision", [((30, 12, 20), True, "fp32"), ((31, 13, 9), False, "fp32"),
                                                   ((62, 8, 44), True, "fp32"), ((4, 5, 6), False, "fp32"),
                                                   ((59, 6, 8), False, "fp32"), ((33, 9, 17), False, "fp64")])
