@@ -29,11 +29,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
 #include "rmt_kernels.h"
+#include "rmt_smem.h"
 
 namespace {
 
@@ -2183,38 +2183,24 @@ MGSolver* mg_build(const Geo& g, int kind, int prec_fp32, bool dry, cudaError_t*
     // size once, outside any stream capture
     m->cc = coarse_cfg(kind, m->lv[m->nlev - 1], m->esz);
     const size_t smem = m->cc.cs > 0 ? 0 : coarse_smem(m->lv[m->nlev - 1], m->esz);
-    // the attribute belongs to the kernel, shared by every solver: it only ever grows
-    static std::mutex mu;
-    static size_t opted[2] = {0, 0}, opted_cl[2][2][COARSE_UPT + 1] = {};
-    std::lock_guard<std::mutex> lock(mu);
-    if (e == cudaSuccess && m->cc.cs > 0) {
-      size_t& have = opted_cl[prec_fp32 ? 1 : 0][kind][m->cc.upt];
-      if (m->cc.smem > have) {
-        e = cudaFuncSetAttribute(coarse_fn(kind, !prec_fp32, m->cc.upt), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)m->cc.smem);
-        if (e == cudaSuccess) have = m->cc.smem;
-      }
-    }
-    if (e == cudaSuccess && smem > opted[prec_fp32 ? 1 : 0]) {
-      if (prec_fp32)
-        e = cudaFuncSetAttribute(k_coarse_cg<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      else
-        e = cudaFuncSetAttribute(k_coarse_cg<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) opted[prec_fp32 ? 1 : 0] = smem;
-    }
-
+    static SmemGrants grants;
+    int dev = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    auto opt_in = [&](const void* fn, size_t bytes, bool carveout) {
+      if (e == cudaSuccess)
+        e = grants.grant(dev, fn, bytes, [&] {
+          const cudaError_t r = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+          if (r != cudaSuccess || !carveout) return r;
+          return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        });
+    };
+    if (m->cc.cs > 0) opt_in(coarse_fn(kind, !prec_fp32, m->cc.upt), m->cc.smem, false);
+    if (smem > 0) opt_in(prec_fp32 ? (const void*)k_coarse_cg<float> : (const void*)k_coarse_cg<double>, smem, false);
     // the fused sweep's staging ring (beyond the 48 KB default) with the largest shared-memory
-    // carveout, so that three blocks fit on an SM; once per process
-    static bool sweep_opted = false;
-    if (e == cudaSuccess && kind == 0 && prec_fp32 && !sweep_opted) {
-      for (int v = 0; v < 2 && e == cudaSuccess; v++) {
-        const void* fn = v ? (const void*)k_rbgs_sweep<true> : (const void*)k_rbgs_sweep<false>;
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                   (int)cudaSharedmemCarveoutMaxShared);
-      }
-      if (e == cudaSuccess) sweep_opted = true;
+    // carveout, so that three blocks fit on an SM
+    if (kind == 0 && prec_fp32) {
+      opt_in((const void*)k_rbgs_sweep<false>, SWEEP_SMEM, true);
+      opt_in((const void*)k_rbgs_sweep<true>, SWEEP_SMEM, true);
     }
     if (e == cudaSuccess && kind == 0 && prec_fp32) {
       // levels that take the fused sweep: rows of whole 16-byte chunks and even periodic sides (a
