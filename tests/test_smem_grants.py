@@ -41,4 +41,4 @@ def test_solvers_opt_in_through_the_record():
     """Every opt-in of the multigrid solvers goes through the record; none is remembered for the process."""
     text = open(os.path.join(B.CSRC, "rmt_mg.cu")).read()
     assert text.count("grants.grant(dev, fn") == 1
-    assert text.count("cudaFuncSetAttribute") == 2 and "static bool" not in text
+    assert text.count("cudaFuncSetAttribute") == 2 and "static size_t" not in text
