@@ -357,11 +357,11 @@ long rmt_kernel_launches(void);
 /* Timing of the step's stages and of the finest-level multigrid kernels with CUDA events on
  * the grid's stream.  rmt_profile(g, 1) clears and starts collecting, rmt_profile(g, 0) stops.
  * Entries: 0..12 are stages of the timestep (each a group of kernels), 13..17 single kernels
- * (7-point smoother colour, 7-point high-precision residual, 27-point smoother colour, 27-point
- * high-precision residual, fused red-black sweep; high precision is FP64 in the FP64 form and
- * two-float in the FP32 form).  rmt_profile_read synchronises the stream and returns the
- * accumulated time, the number of timed launches and, for 13..17, the algorithmic bytes of one
- * launch (0 else). */
+ * (7-point smoother colour, or all sweeps of a smoothing call on a finest level small enough for one
+ * block, 7-point high-precision residual, 27-point smoother pass, 27-point high-precision residual,
+ * fused red-black sweep; high precision is FP64 in the FP64 form and two-float in the FP32 form).
+ * rmt_profile_read synchronises the stream and returns the accumulated time, the number of timed
+ * launches and, for 13..17, the algorithmic bytes of one launch (0 else). */
 rmt_status rmt_profile(rmt_grid* g, int enable);
 int rmt_profile_entries(void);
 const char* rmt_profile_name(int entry);

@@ -222,16 +222,21 @@ void mg_hook(void* ctx, int which, int begin, cudaStream_t) {
   else pe(h->g, e);
 }
 // algorithmic bytes of one launch of the profiled multigrid kernels (w = bytes per word, N
-// cells, NN nodes): red-black colour pass (7-point): x and rho read once, b read and x written
-// for half the cells; Jacobi pass (27-point): x, b read and x written per node, rho per cell;
-// FP64 residual: x and b 8 bytes each, rho, and the residual copy in the storage type; fused
-// red-black sweep: x, rho and b read and x written once per cell.
+// cells, NN nodes), each array read or written once: red-black colour pass (7-point): x and the coefficient, b
+// read and x written for half the cells, the coefficient being rho (FP32) or three face arrays and, for half the
+// cells, the inverse diagonal (FP64); a small level's passes in one block: x read and written, b and the
+// coefficients, whatever the sweeps; Jacobi pass (27-point): x, b read and x written per node, beta per cell, and FP64
+// three edge sums and the inverse diagonal per node; high-precision residual: x and b 8 bytes each, rho (FP64 7-point:
+// the face arrays), and the residual in the storage type; fused red-black sweep: x, rho and b read and x written.
 double prof_bytes(const rmt_grid* g, int e) {
   const double w = (double)g->esz, N = (double)g->g.N, NN = (double)g->g.NN;
+  const bool f64 = !g->fp32;
   switch (e) {
-    case P_MAC_SMOOTH: return 3.0 * N * w;
-    case P_MAC_RESID: return 16.0 * N + 2.0 * N * w;
-    case P_FE_SMOOTH: return 3.0 * NN * w + N * w;
+    case P_MAC_SMOOTH:
+      if (g->mac && mg_block_sweeps(g->mac)) return (f64 ? 7.0 : 4.0) * N * w;
+      return (f64 ? 5.5 : 3.0) * N * w;
+    case P_MAC_RESID: return 16.0 * N + (f64 ? 4.0 : 2.0) * N * w;
+    case P_FE_SMOOTH: return (f64 ? 7.0 : 3.0) * NN * w + N * w;
     case P_FE_RESID: return 16.0 * NN + N * w + NN * w;
     case P_MAC_SWEEP: return 4.0 * N * w;
   }

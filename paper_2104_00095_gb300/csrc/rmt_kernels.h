@@ -192,9 +192,11 @@ int mg_zchunk(const MGSolver* m);
 // default; 2: on every level that allows it; 0: never), else one pass per colour
 void mg_set_sweep(MGSolver* m, int fused);
 // Optional timing hook around the finest-level smoother and FP64-residual launches:
-// hook(ctx, which, begin, stream) with which = 0 (smoother colour), 1 (FP64 residual) or 2 (fused
-// red-black sweep).
+// hook(ctx, which, begin, stream) with which = 0 (smoother colour, or all sweeps of a smoothing call where
+// mg_block_sweeps), 1 (FP64 residual) or 2 (fused red-black sweep).
 typedef void (*mg_hook_fn)(void* ctx, int which, int begin, cudaStream_t s);
 void mg_set_hook(MGSolver* m, mg_hook_fn fn, void* ctx);
+// whether the finest level (MAC) is small enough that one launch makes all sweeps of a smoothing call
+bool mg_block_sweeps(const MGSolver* m);
 // Solves to rtol (or a fixed cycle count); returns cycles used, -1 on non-convergence.
 int mg_solve(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStream_t s, cudaError_t* err);

@@ -2345,12 +2345,18 @@ void launch_fe_tile(const MGSolver* m, int l, T w, const T* x, T* out, const T* 
   rmt_count_launches(1);
 }
 
+// cells of a colour per thread where level l's sweeps run in one block, else 0
+template <typename T>
+int block_cells(const MGSolver* m, int l) {
+  return m->kind == 0 && m->sweep != 2 ? small_cells<T>(m->lv[l]) : 0;
+}
+
 template <typename T>
 void smooth(MGSolver* m, int l, int sweeps, bool forward, cudaStream_t s) {
   const Lv& L = m->lv[l];
   const T* b = (const T*)m->b[l];
   const T* rho = (const T*)m->rho[l];
-  const int small = m->kind == 0 && m->sweep != 2 && sweeps > 0 ? small_cells<T>(L) : 0;
+  const int small = sweeps > 0 ? block_cells<T>(m, l) : 0;
   if (small > 0) {
     hk(m, l, 0, 1, s);
     auto kernel = k_rbgs_block<T, 1>;
@@ -2633,6 +2639,10 @@ int mg_zchunk(const MGSolver* m) {
   const Lv& L = m->lv[0];
   const dim3 g = fe_grid(L, m->fe_zc0, fe_staging(L, m->fp32));
   return (L.nn[2] + (int)g.z - 1) / (int)g.z;
+}
+
+bool mg_block_sweeps(const MGSolver* m) {
+  return m->nlev > 1 && (m->fp32 ? block_cells<float>(m, 0) : block_cells<double>(m, 0)) > 0;
 }
 
 int mg_solve(MGSolver* m, double rtol, int max_cycles, int fixed_cycles, cudaStream_t s, cudaError_t* err) {

@@ -266,3 +266,24 @@ def test_layer_zero_is_the_sign_of_the_level_set(shape, size, turn, precision):
     assert o.step(0) == 0, o.error()
     assert np.array_equal(g.read(rmt.RMT_F_LAYER, 0), o.read(O.F_LAYER, 0))
     g.close()
+
+
+@pytest.mark.parametrize("n,precision,smooth", [((24, 20, 16), "fp32", 12.0), ((12, 12, 12), "fp32", 16.0),
+                                                ((24, 20, 16), "fp64", 44.0), ((8, 8, 16), "fp64", 56.0)])
+def test_profile_counts_the_bytes_of_the_kernels_that_run(n, precision, smooth):
+    """Bytes per cell of a 7-point smoothing launch: a colour pass of x, the coefficient and half of b and x (FP32 one
+    array, FP64 three and half the inverse diagonal), or a small level's sweeps in one block, every array once;
+    the FP64 7-point residual's (x, b, three face arrays, r) and 27-point pass's (four stored arrays more)."""
+    g = rmt.Grid(dict(_box(n, False), precision=precision, mg_rtol=1e-6))
+    g.step(1)
+    g.profile(True)
+    g.step(1)
+    g.profile(False)
+    got = {p[0]: p[2:] for p in g.profile_read()}
+    cells, nodes = np.prod(n), np.prod([v + 1 for v in n])
+    names = list(got)
+    assert got[names[13]][0] > 0 and got[names[13]][1] == smooth * cells
+    if precision == "fp64":
+        assert got[names[14]][1] == 48 * cells
+        assert got[names[15]][1] == 56 * nodes + 8 * cells
+    g.close()
