@@ -287,3 +287,55 @@ def test_profile_counts_the_bytes_of_the_kernels_that_run(n, precision, smooth):
         assert got[names[14]][1] == 48 * cells
         assert got[names[15]][1] == 56 * nodes + 8 * cells
     g.close()
+
+
+@pytest.mark.parametrize("n,periodic", [((30, 28, 34), (0, 0, 0)), ((32, 36, 30), (0, 1, 0)), ((62, 30, 28), (0, 0, 1)),
+                                        ((64, 28, 32), (0, 1, 1)), ((66, 30, 36), (0, 0, 0)), ((34, 28, 30), (1, 0, 0))])
+def test_fe_tiles_of_two_levels_with_walls(n, periodic):
+    """Even sides, so that the finest level is smoothed by the FE tiles: node rows that end before, at and after a block's
+    last column (31, 33, 63, 65, 67), at every alignment, with periodic axes beside the walls.  FP64 against the oracle;
+    FP32 in the cycles of FP64 and to FP32 accuracy."""
+    assert all(v % 2 == 0 and v // 2 >= 3 for v in n)  # two levels at least
+    sc = _box(n, False)
+    sc["bc"] = [S.PERIODIC if periodic[d // 2] else S.NOSLIP for d in range(6)]
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    g, o = pair(sc)
+    g.write(rmt.RMT_F_U, u)
+    assert o.write(O.F_U, u) == 0
+    g.step(1)
+    assert o.step(1) == 0, o.error()
+    compare_state(g, o, 0, 1e-10, tag=f"{n}")
+    g.close()
+    out = []
+    for prec in ("fp64", "fp32"):
+        g = rmt.Grid(dict(sc, precision=prec, mg_rtol=1e-9, mg_max_cycles=60))
+        g.write(rmt.RMT_F_U, u)
+        g.step(1)
+        out.append((g.read(rmt.RMT_F_U), g.cycles()))
+        g.close()
+    (u64, c64), (u32, c32) = out
+    assert rel_l2(u32, u64) <= 1e-5
+    assert all(abs(a - b) <= 3 for a, b in zip(c64, c32)), (c64, c32)
+
+
+@pytest.mark.parametrize("n,precision", [((90, 90, 10), "fp64"), ((58, 58, 58), "fp64"), ((70, 66, 66), "fp32")])
+def test_coarsest_levels_beyond_a_cluster(n, precision):
+    """Two-level grids whose coarsest level is solved by one block on global memory: 45 x 45 x 5 and 29^3 cells in FP64
+    (their coefficients exceed a cluster's shared memory), 35 x 33 x 33 (more unknowns than a cluster holds)."""
+    sc = _with_body(n, False)
+    sc.update(precision=precision)
+    u = 0.3 * np.sin(np.arange(3 * np.prod(n)) * 0.37)
+    if precision == "fp64":
+        g, o = pair(sc)
+        g.write(rmt.RMT_F_U, u)
+        assert o.write(O.F_U, u) == 0
+        g.step(1)
+        assert o.step(1) == 0, o.error()
+        assert max(g.cycles()) <= 40
+        compare_state(g, o, 1, 1e-10, tag=f"{n}")
+    else:
+        g = rmt.Grid(dict(sc, mg_rtol=1e-9, mg_max_cycles=60))
+        g.write(rmt.RMT_F_U, u)
+        g.step(1)
+        assert max(g.cycles()) <= 40
+    g.close()
