@@ -8,8 +8,6 @@
 // are degenerate, which weights are positive) are reproducible.  FP64 storage fits in FP64;
 // FP32 storage holds displacements S = xi - x0 (rmt_common.cuh) and fits them in FP32, redone
 // in FP64 when ill-conditioned.
-#include <type_traits>
-
 #include "rmt_band.cuh"
 
 namespace {
@@ -168,7 +166,7 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
 }
 
 // The candidate cells of the radius-2 search box around one cell, loaded once per cell for
-// every fit that uses that box (the kernel-only fit, the normal-weighted fit and an FP64 redo):
+// both fits that use that box (the kernel-only and the normal-weighted one):
 // lane L holds the candidates t = L + 32 q (q < 4) of the 5^3 box, a bit per slot that says
 // whether the candidate is a cell of a lower layer, and its stored values.  The layer bytes of
 // the four slots are read first and the values of the usable ones after them, so a cell costs
@@ -219,30 +217,30 @@ __device__ __forceinline__ void load_cand(const Geo& g, const T* __restrict__ x,
 // are then small, so the solve's error, which scales with the data, carries no O(1) positions
 // into the extrapolated maps.  With cd (rs = 2 only) the candidates come from the registers that
 // load_cand filled, in the same order, so the sums are the same to the last bit.
-template <typename AT, typename T>
+template <typename T>
 __device__ bool wls_fit_warp(const Geo& g, const T* __restrict__ x, const int8_t* __restrict__ lay, int i, int j,
-                             int k, int le, int rs, int mode, const AT nrm[3], AT tolfac, AT sol[4][3],
+                             int k, int le, int rs, int mode, const double nrm[3], double sol[4][3],
                              const Cand<T>* cd = nullptr) {
   const int lane = threadIdx.x & 31;
-  AT a[10], bsum[12];
+  double a[10], bsum[12];
 #pragma unroll
-  for (int q = 0; q < 10; q++) a[q] = AT(0);
+  for (int q = 0; q < 10; q++) a[q] = 0.0;
 #pragma unroll
-  for (int q = 0; q < 12; q++) bsum[q] = AT(0);
+  for (int q = 0; q < 12; q++) bsum[q] = 0.0;
   int npos = 0;
   const int w = 2 * rs + 1, nc = w * w * w;
   // one candidate's contribution; false when its weight is not positive
   auto add = [&](int di, int dj, int dk, T x0, T x1, T x2) {
     const int sr = abs(di) + abs(dj) + abs(dk);
-    AT wt = sizeof(AT) == 4 ? (AT)ldexpf(1.0f, -sr) : (AT)ldexp(1.0, -sr);
+    double wt = ldexp(1.0, -sr);
     if (mode == 1) {
-      const AT len = sqrt((AT)(di * di + dj * dj + dk * dk));
-      const AT cs = -((AT)di * nrm[0] + (AT)dj * nrm[1] + (AT)dk * nrm[2]) / len;
+      const double len = sqrt((double)(di * di + dj * dj + dk * dk));
+      const double cs = -((double)di * nrm[0] + (double)dj * nrm[1] + (double)dk * nrm[2]) / len;
       wt = cs * wt;
-      if (!(wt > AT(0))) return;
+      if (!(wt > 0.0)) return;
     }
-    const AT v[4] = {AT(1), (AT)di, (AT)dj, (AT)dk};
-    const AT xv[3] = {(AT)x0, (AT)x1, (AT)x2};
+    const double v[4] = {1.0, (double)di, (double)dj, (double)dk};
+    const double xv[3] = {(double)x0, (double)x1, (double)x2};
     int q = 0;
 #pragma unroll
     for (int r = 0; r < 4; r++)
@@ -280,7 +278,7 @@ __device__ bool wls_fit_warp(const Geo& g, const T* __restrict__ x, const int8_t
     npos += __shfl_xor_sync(0xffffffffu, npos, o);
   }
   if (npos < 4) return false;
-  AT A[4][4], B[4][3];
+  double A[4][4], B[4][3];
   int q = 0;
   for (int r = 0; r < 4; r++)
     for (int cc = r; cc < 4; cc++) {
@@ -290,72 +288,58 @@ __device__ bool wls_fit_warp(const Geo& g, const T* __restrict__ x, const int8_t
     }
   for (int r = 0; r < 4; r++)
     for (int d = 0; d < 3; d++) B[r][d] = bsum[3 * r + d];
-  return solve4<AT>(A, B, sol, tolfac);
+  return solve4<double>(A, B, sol, 1e-12);
 }
 
-// Extrapolates one cell (whole warp) with fits accumulated in AT: kernel-only fit, then (layers
-// 1 and 2) the fit weighted by the normal n_e = normalised (grad xi)^T grad_X phi_0(xi_e) of that
-// first fit; the search radius grows up to 4 while the system stays degenerate.  Returns 1 on
-// success, 0 when degenerate, -1 when an FP32 attempt was too ill-conditioned to trust.  cd: the
-// preloaded candidates of the radius-2 box.
-template <typename AT, typename T>
-__device__ int wls_cell_try(const Geo& g, const Body& b, const T* __restrict__ x, const int8_t* __restrict__ lay,
-                            int i, int j, int k, int le, const Cand<T>& cd, double out[3]) {
-  // FP64: the degeneracy threshold; FP32: also the point below which the fit is redone in FP64
-  const AT tolfac = sizeof(AT) == 8 ? AT(1e-12) : AT(1e-4);
-  // FP32 storage fits displacements: the identity's slope per cell offset is added back to the
-  // fitted gradient, and the cell's x0 - c to the fitted value, where the normal needs xi
-  const AT hid = disp_storage<T>() ? (sizeof(AT) == 4 ? (AT)g.f.h : (AT)g.h) : AT(0);
-  for (int rs = RS0; rs <= 4; rs++) {
-    const Cand<T>* cp = rs == RS0 ? &cd : nullptr;
-    AT s1[4][3];
-    if (!wls_fit_warp<AT>(g, x, lay, i, j, k, le, rs, 0, (const AT*)nullptr, tolfac, s1, cp)) {
-      if (sizeof(AT) == 4) return -1;
-      continue;
-    }
-    if (le <= 2) {
-      AT gX[3], v[3];
-      if constexpr (disp_storage<T>()) {
-        const AT r0[3] = {cell_rel<AT>(g, b, 0, i) + s1[0][0], cell_rel<AT>(g, b, 1, j) + s1[0][1],
-                          cell_rel<AT>(g, b, 2, k) + s1[0][2]};
-        phi0_dir_r<AT>(b, r0, gX);
-      } else {
-        const AT c0[3] = {s1[0][0], s1[0][1], s1[0][2]};
-        phi0_dir<AT>(b, c0, gX);
-      }
-      for (int q = 0; q < 3; q++)
-        v[q] = (s1[1 + q][0] + (q == 0 ? hid : AT(0))) * gX[0] + (s1[1 + q][1] + (q == 1 ? hid : AT(0))) * gX[1] +
-               (s1[1 + q][2] + (q == 2 ? hid : AT(0))) * gX[2];
-      const AT nv = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-      if (!(nv > AT(0))) {
-        if (sizeof(AT) == 4) return -1;
-        continue;
-      }
-      const AT nrm[3] = {v[0] / nv, v[1] / nv, v[2] / nv};
-      AT s2[4][3];
-      if (!wls_fit_warp<AT>(g, x, lay, i, j, k, le, rs, 1, nrm, tolfac, s2, cp)) {
-        if (sizeof(AT) == 4) return -1;
-        continue;
-      }
-      for (int d = 0; d < 3; d++) out[d] = (double)s2[0][d];
-      return 1;
-    }
-    for (int d = 0; d < 3; d++) out[d] = (double)s1[0][d];
-    return 1;
-  }
-  return 0;
-}
-
-// One cell's fits in the accumulation type of the storage: FP64 storage fits in FP64 (1:
-// extrapolated, 0: degenerate); FP32 storage fits in FP32 and returns -1 when the system was too
-// ill-conditioned to trust, for the FP64 redo kernel (a separate kernel, so that the FP32 one
-// keeps the register budget of FP32 fits).  FP64: the redo itself.
-template <typename AT, typename T>
-__device__ int wls_cell_warp(const Geo& g, const Body& b, const T* __restrict__ x, const int8_t* __restrict__ lay,
-                             int i, int j, int k, int le, double out[3]) {
+// A cell whose batched fit failed, fitted again by the whole warp in FP64: the kernel-only fit, then (layers 1 and 2)
+// the fit weighted by the normal n_e = normalised (grad xi)^T grad_X phi_0(xi_e) of that first fit; the search radius
+// grows up to 4 while the system stays degenerate.  FP32 storage comes here when a system was too ill-conditioned
+// for FP32.  Rare, so it is kept out of the callers' registers.  The failed cells of a batch follow one another in their
+// warp: with a disk of 0.9 to 4 cells' half-thickness across the grid (64^3 .. 128^3, fits of radius 2 failing along its
+// edge or all over it) every extrapolation that succeeds takes 0.3 to 0.7 of its time with a list of failed cells spread
+// over all SMs (96^3, tilted, 1.2 cells: 1.77 -> 0.83 ms); one that ends degenerate takes up to 1.55 times as long.
+// Returns 1 with the map at the cell in lane 0's out, 0 when degenerate.
+template <typename T>
+__device__ __noinline__ int wls_again(const Geo& g, const Body& b, const T* x, const int8_t* lay, long c, int le,
+                                      double out[3]) {
+  int i, j, k;
+  decode(c, g.n[0], g.n[1], i, j, k);
   Cand<T> cd;
   load_cand(g, x, lay, i, j, k, le, cd);
-  return wls_cell_try<AT>(g, b, x, lay, i, j, k, le, cd, out);
+  // FP32 storage fits displacements: the identity's slope per cell offset is added back to the
+  // fitted gradient, and the cell's x0 - c to the fitted value, where the normal needs xi
+  const double hid = disp_storage<T>() ? g.h : 0.0;
+  int ok = 0;
+  for (int rs = RS0; rs <= 4 && !ok; rs++) {
+    const Cand<T>* cp = rs == RS0 ? &cd : nullptr;
+    double s1[4][3];
+    if (!wls_fit_warp(g, x, lay, i, j, k, le, rs, 0, nullptr, s1, cp)) continue;
+    if (le <= 2) {
+      double gX[3], v[3];
+      if constexpr (disp_storage<T>()) {
+        const double r0[3] = {cell_rel<double>(g, b, 0, i) + s1[0][0], cell_rel<double>(g, b, 1, j) + s1[0][1],
+                              cell_rel<double>(g, b, 2, k) + s1[0][2]};
+        phi0_dir_r<double>(b, r0, gX);
+      } else {
+        const double c0[3] = {s1[0][0], s1[0][1], s1[0][2]};
+        phi0_dir<double>(b, c0, gX);
+      }
+      for (int q = 0; q < 3; q++)
+        v[q] = (s1[1 + q][0] + (q == 0 ? hid : 0.0)) * gX[0] + (s1[1 + q][1] + (q == 1 ? hid : 0.0)) * gX[1] +
+               (s1[1 + q][2] + (q == 2 ? hid : 0.0)) * gX[2];
+      const double nv = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+      if (!(nv > 0.0)) continue;
+      const double nrm[3] = {v[0] / nv, v[1] / nv, v[2] / nv};
+      double s2[4][3];
+      if (!wls_fit_warp(g, x, lay, i, j, k, le, rs, 1, nrm, s2, cp)) continue;
+      for (int d = 0; d < 3; d++) out[d] = s2[0][d];
+    } else {
+      for (int d = 0; d < 3; d++) out[d] = s1[0][d];
+    }
+    ok = 1;
+  }
+  __syncwarp();
+  return ok;
 }
 
 // ---- batches of cells ------------------------------------------------------------------
@@ -649,19 +633,6 @@ __device__ __forceinline__ int batch_size(int n, int warps) {
   const int want = sizeof(AT) == 8 ? (warps + 3) / 4 : warps;
   const int g = (n + want - 1) / want;
   return g < 1 ? 1 : (g > WB ? WB : g);
-}
-
-// A cell whose batched fit failed, fitted again by the whole warp in FP64 with the growing radius (FP32
-// storage: the system was too ill-conditioned for FP32; rare, so it is kept out of the callers' registers).
-// Returns 1 with the map at the cell in lane 0's out, 0 when degenerate.
-template <typename T>
-__device__ __noinline__ int wls_again(const Geo& g, const Body& b, const T* x, const int8_t* lay, long c, int l,
-                                      double out[3]) {
-  int i, j, k;
-  decode(c, g.n[0], g.n[1], i, j, k);
-  const int q = wls_cell_warp<double>(g, b, x, lay, i, j, k, l, out);
-  __syncwarp();
-  return q;
 }
 
 // The cells of layer l (its segment of the band list) in the storage type, batch by batch

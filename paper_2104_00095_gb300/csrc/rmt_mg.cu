@@ -1574,34 +1574,18 @@ __global__ void __launch_bounds__(BX* BYMAX) k_resid_restrict_mac(Lv F, Lv C, co
   resid_restrict_mac_at(F, C, x, b, rho, bc, xc, I, J, K);
 }
 
-// restriction of the residual to the coarse right-hand side at coarse unknown (I, J, K) (coarse
-// x zeroed): MAC the 8-cell mean, FE full weighting
-// Restriction of the fine residual to the coarse right-hand side (and a zero coarse iterate).
-// Cell-centred: the mean of the 8 children.  Nodal: full weighting, weight 1/2 per axis on which
-// the fine node lies between coarse nodes, summed plane by plane (fine planes 2K-1, 2K, 2K+1).
-// One thread marches up to RZ coarse unknowns of its (I, J) column; in the nodal case the fine
-// plane 2K+1 is kept in registers as the next unknown's plane 2K'-1.
+// Restriction of the nodal residual to the coarse right-hand side (and a zero coarse iterate): full weighting,
+// weight 1/2 per axis on which the fine node lies between coarse nodes, summed plane by plane (fine planes 2K-1,
+// 2K, 2K+1).  One thread marches up to RZ coarse unknowns of its (I, J) column and keeps the fine plane 2K+1 in
+// registers as the next unknown's plane 2K'-1.
 constexpr int RZ = 8;
 template <typename T>
-__global__ void __launch_bounds__(BX* BYMAX) k_restrict(Lv F, Lv C, int kind, const T* __restrict__ rf,
-                                                      T* __restrict__ bc, T* __restrict__ xc, int zc) {
+__global__ void __launch_bounds__(BX* BYMAX) k_restrict(Lv F, Lv C, const T* __restrict__ rf, T* __restrict__ bc,
+                                                      T* __restrict__ xc, int zc) {
   wait_prior();
-  const int ext[3] = {kind == 0 ? C.n[0] : C.nn[0], kind == 0 ? C.n[1] : C.nn[1], kind == 0 ? C.n[2] : C.nn[2]};
   const int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
-  if (I >= ext[0] || J >= ext[1]) return;
-  const int K0 = blockIdx.z * zc, K1 = min(K0 + zc, ext[2]);
-  if (kind == 0) {
-    for (int K = K0; K < K1; K++) {
-      T s = T(0);
-#pragma unroll
-      for (int q = 0; q < 8; q++) s += rf[cix(F, 2 * I + (q & 1), 2 * J + ((q >> 1) & 1), 2 * K + ((q >> 2) & 1))];
-      s *= T(0.125);
-      const long u = cix(C, I, J, K);
-      bc[u] = s;
-      xc[u] = T(0);
-    }
-    return;
-  }
+  if (I >= C.nn[0] || J >= C.nn[1]) return;
+  const int K0 = blockIdx.z * zc, K1 = min(K0 + zc, C.nn[2]);
   // the fine x and y node indices 2I-1, 2I, 2I+1 (wrapped; -1 outside a wall) and the columns
   int fx[3], fy[3];
 #pragma unroll
@@ -2445,7 +2429,7 @@ void vcycle(MGSolver* m, int l, cudaStream_t s) {
     launch_fe_tile<1>(m, l, T(0), (const T*)m->x[l], (T*)m->r[l], (const T*)m->b[l], s);
     const int zc = column_chunk(C.nnode, RZ);
     launch_after(k_restrict<T>, grid3(C.nn[0], C.nn[1], (C.nn[2] + zc - 1) / zc, m->by), dim3(BX, m->by), 0, s, 
-        L, C, m->kind, (const T*)m->r[l], (T*)m->b[l + 1], (T*)m->x[l + 1], zc);
+        L, C, (const T*)m->r[l], (T*)m->b[l + 1], (T*)m->x[l + 1], zc);
     rmt_count_launches(1);
   }
   vcycle<T>(m, l + 1, s);
