@@ -140,7 +140,7 @@ __device__ bool solve4(AT A[4][4], AT B[4][3], AT X[4][3], AT tolfac) {
     for (int j = 0; j < k; j++) s -= L[k][j] * L[k][j] * D[j];
     D[k] = s;
     if (!(s > tol)) return false;
-    iD[k] = AT(1) / s;  // one division per pivot: each is some ten instructions
+    iD[k] = AT(1) / s;  // one division per pivot: each is some ten instructions; the rest are quot()s
     L[k][k] = AT(1);
     for (int i = k + 1; i < 4; i++) {
       AT t = A[i][k];
@@ -357,7 +357,7 @@ __device__ __noinline__ int wls_again(const Geo& g, const Body& b, const T* x, c
 //    16 + 8 + 4 + 2 + 1 additions for 22 totals instead of 110, added in the same tree.
 // One warp per cell with 66 multiplications and additions per candidate and fit and a solve by all
 // lanes took 136 us per layer and body of the 128^3 settling mixture in FP64, and 1.50 ms per
-// extrapolation of one body on 96^3 (0.66 now); with it a step of the mixture took 5.5 ms longer.
+// extrapolation of one body on 96^3 (0.60 now); with it a step of the mixture took 5.5 ms longer.
 constexpr int WB = 32;                 // cells of a batch at most
 constexpr int NSUM = 22, NPAD = 23;    // totals of a fit, padded against bank conflicts
 // 1 / sqrt(s), s = 0 .. 12 (the squared lengths of the 5^3 box's offsets)

@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(GX* GY, 2)
 // ---------------------------------------------------------------------------------
 // FP64: separate passes.  The FP64 units bound these kernels, and the ring of columns around a tile of the fused
 // kernel above costs more there than the passes over memory it saves (walls,
-// 128^3: fused 3.69 ms, separate 1.62 ms).
+// 128^3: fused 3.69 ms, separate 1.68 ms).
 
 // Limited slopes of the three velocity components along the three axes at every cell
 // (SI "Normal derivatives"); S[3 * d + a] = d u_a / d x_d.
@@ -349,7 +349,7 @@ struct Slopes9 {
 };
 // One component to a block (grid z: component, chunk of planes).  A thread marches up a column: along z each
 // inner limited difference is formed once and serves three slopes.  Ghosts across walls are folded into the
-// loads, so that the warps at a wall take the path of the others (128^3 with walls: 0.72 ms, a thread to a cell
+// loads, so that the warps at a wall take the path of the others (128^3 with walls: 0.80 ms, a thread to a cell
 // with a separate path at the walls 1.5 ms with the limiters of the time).
 __global__ void __launch_bounds__(TILE_X* TILE_Y) k_slopes64(Geo g, const double* __restrict__ u,
                                                              const __grid_constant__ Slopes9 S, int zc, int chunks) {

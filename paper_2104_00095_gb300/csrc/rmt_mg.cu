@@ -22,8 +22,8 @@
 // red-black Gauss-Seidel (7-point; one thread per same-colour cell pair along x) and weighted
 // Jacobi (27-point; one fused pass per sweep).  Transfers: 8-cell average / trilinear
 // (cell-centred), full weighting / trilinear (nodal).  Coarse densities are 8-cell means.
-// The coarsest level is solved by one block with conjugate gradients.  Norms use fixed-order
-// two-stage reductions, so results are deterministic.
+// The coarsest level is solved with conjugate gradients by one block or one cluster.  Sums are
+// added in a fixed order (threads, warps, blocks), so results are deterministic.
 #include <cooperative_groups.h>
 
 #include <cstdio>
@@ -1889,8 +1889,9 @@ __global__ void k_add_to64(const T* __restrict__ a, double* __restrict__ b, long
 // coarsest level: conjugate gradients (the operator is symmetric positive semi-definite with the
 // constants as null space; the right-hand side is made mean-free and so is the result).  Levels
 // that fit a cluster's registers and shared memory take k_coarse_solve (rmt_mg_coarse.cuh); the
-// one-block kernel below is for those that do not (an odd grid of more than 32^3 cells, which has
-// one level only).
+// one-block kernel below is for those that do not (coarse_cfg): more than 32768 unknowns, as in a grid
+// of twice an odd side from 66 on or of an odd side from 33 on, levels of few wide planes, and in FP64 the 7-point
+// level from 29^3 cells on, whose six coefficients in two precisions exceed a block's shared memory.
 constexpr int COARSE_TPB = 512;
 // relative tolerance of the coarsest solve: FP64 solves to 1e-10; an FP32 V-cycle needs its
 // coarse correction to well below its own convergence factor (about 0.1), and FP32 CG on the

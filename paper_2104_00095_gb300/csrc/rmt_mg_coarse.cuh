@@ -30,7 +30,8 @@ constexpr int COARSE_ONE = 1024;     // unknowns of a single-block solve (FP32)
 constexpr int COARSE_ONE64 = 256;    // ... FP64: its operator is bound by one SM's FP64 lanes
 constexpr int COARSE_UPT = 8;        // unknowns per thread at most
 constexpr int COARSE_WORK = 8;       // FP64: FP32 iterations of all passes together, in units of max_it
-// threads of a block: one unknown each up to 1024, else 4 or 8 on 512 (128 registers a thread)
+// threads of a block: one unknown each up to 1024 (64 registers), else 4 or 8 on 512 (128 registers; the 27-point
+// forms of 8 are given 64 and spill some 1.2 KB a thread)
 constexpr int COARSE_MAXT = 1024, COARSE_MULTT = 512;
 
 // split of a coarsest level over a cluster

@@ -16,7 +16,7 @@
 // body needs, and a body's window leaves most of the chip idle.  The halo repeats about twice
 // the slopes of a full tile; the choice of the upwind side before the state is formed, and a
 // face's state formed once for both its cells, take half of the states away.  All bodies of a step, three
-// passes for each and this: 20 bodies in 128^3 501 -> 170 us (FP64 1333 -> 594 us, bound by its arithmetic),
+// passes for each and this: 20 bodies in 128^3 501 -> 170 us (FP64 1333 -> 644 us, bound by its arithmetic),
 // 3 in 48^3 81 -> 31 us, 8 in 256^3 327 -> 230 us.
 #include "rmt_band.cuh"
 
